@@ -25,13 +25,16 @@ __global__ void k_idft(int N, int U, int n2, const double* __restrict__ G,
     }
 }
 
-__global__ void k_join(int N, int n, const double* q, const double* u, double* zb) {
+// q, u (internal numbering) -> end points (N x 2n, the caller's dof order)
+__global__ void k_join(int N, int n, int ni, const int* __restrict__ row_of, const double* __restrict__ q,
+                       const double* __restrict__ u, double* zb) {
     const size_t total = (size_t)N * n;
     for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
          idx += (size_t)gridDim.x * blockDim.x) {
         const size_t s = idx / n, i = idx % n;
-        zb[s * 2 * n + i] = q[idx];
-        zb[s * 2 * n + n + i] = u[idx];
+        const size_t r = s * ni + row_of[i];
+        zb[s * 2 * n + i] = q[r];
+        zb[s * 2 * n + n + i] = u[r];
     }
 }
 
@@ -53,54 +56,56 @@ __global__ void k_dft_res(int N, int U, int n2, const double* __restrict__ RG,
 // Jacobian products (Eq. 22, 23) from the stored tangents
 // ----------------------------------------------------------------------------
 
-// zout[s][i] = sum_{j < 2n} Phi_s[i][j] zin[s][j],  Phi_s = [X[:, :2n]; V[:, :2n]]; one warp per (s, i)
+// zout[s][i] = sum_{j < 2n} Phi_s[i][j] zin[s][j]; one warp per (s, i)
 template <typename T>
-__global__ void k_phi_apply(int N, int n, int P, const T* X, const T* V, const double* zin,
-                            double* zout) {
+__global__ void k_phi_apply(int N, PhiView<T> F, const double* zin, double* zout) {
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    const int n2 = 2 * n;
+    const int n2 = 2 * F.n;
     if (warp >= N * n2) return;
     const int s = warp / n2, i = warp % n2;
-    const T* row = (i < n ? X + ((size_t)s * n + i) * P : V + ((size_t)s * n + (i - n)) * P);
+    int g;
+    const T* row = F.row(s, i, g);
     const double* z = zin + (size_t)s * n2;
     double acc = 0.0;
-    for (int j = lane; j < n2; j += 32) acc += (double)row[j] * z[j];
+    for (int j = lane; j < 2 * F.pan.n[g]; j += 32) acc += (double)row[j] * z[F.col(g, j)];
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (lane == 0) zout[warp] = acc;
 }
 
 template <typename T>
-__global__ void k_domega_col(int N, int n, int P, const T* X, const T* V, double* zout) {
-    const int n2 = 2 * n;
+__global__ void k_domega_col(int N, PhiView<T> F, double* zout) {
+    const int n2 = 2 * F.n;
     const size_t total = (size_t)N * n2;
     for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
          idx += (size_t)gridDim.x * blockDim.x) {
-        const size_t s = idx / n2;
-        const int i = (int)(idx % n2);
-        const T* row = (i < n ? X + (s * n + i) * P : V + (s * n + (i - n)) * P);
-        zout[idx] = (double)row[2 * n];
+        int g;
+        const T* row = F.row((int)(idx / n2), (int)(idx % n2), g);
+        zout[idx] = (double)row[2 * F.pan.n[g]];
     }
 }
 
+// Phi_s and d zbar_s / d w_1 of trajectories s0 .. s0 + N - 1
 template <typename T>
-__global__ void k_phi_copy(int N, int n, int P, const T* X, const T* V, double* Phi, double* dzdw) {
-    const int n2 = 2 * n;
+__global__ void k_phi_copy(int N, int s0, PhiView<T> F, double* Phi, double* dzdw) {
+    const int n2 = 2 * F.n;
     const size_t total = (size_t)N * n2 * n2;
     for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
          idx += (size_t)gridDim.x * blockDim.x) {
         const size_t s = idx / ((size_t)n2 * n2);
         const int r = (int)((idx / n2) % n2), c = (int)(idx % n2);
-        const T* row = (r < n ? X + (s * n + r) * P : V + (s * n + (r - n)) * P);
-        if (Phi) Phi[idx] = (double)row[c];
-        if (dzdw && c == 0) dzdw[s * n2 + r] = (double)row[2 * n];
+        if (Phi) Phi[idx] = F.at(s0 + (int)s, r, c);
+        if (dzdw && c == 0) {
+            int g;
+            const T* row = F.row(s0 + (int)s, r, g);
+            dzdw[s * n2 + r] = (double)row[2 * F.pan.n[g]];
+        }
     }
 }
 
 // dense Eq. (22): J[(i,u),(j,v)] = sum_s RG[u][s] Phi_s[i][j] G[s][v] - delta
 template <typename T>
-__global__ void k_dense_jac(int N, int n, int U, int P, const T* X, const T* V,
-                            const double* RG, const double* G, double* J, size_t lda) {
-    const int n2 = 2 * n;
+__global__ void k_dense_jac(int N, int U, PhiView<T> F, const double* RG, const double* G, double* J, size_t lda) {
+    const int n2 = 2 * F.n;
     const size_t m = (size_t)n2 * U;
     const size_t total = m * m;
     for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
@@ -109,10 +114,7 @@ __global__ void k_dense_jac(int N, int n, int U, int P, const T* X, const T* V,
         const int i = (int)(row / U), uu = (int)(row % U);
         const int j = (int)(col / U), vv = (int)(col % U);
         double acc = 0.0;
-        for (int s = 0; s < N; ++s) {
-            const T* xr = (i < n ? X + ((size_t)s * n + i) * P : V + ((size_t)s * n + (i - n)) * P);
-            acc += RG[(size_t)uu * N + s] * (double)xr[j] * G[(size_t)s * U + vv];
-        }
+        for (int s = 0; s < N; ++s) acc += RG[(size_t)uu * N + s] * F.at(s, i, j) * G[(size_t)s * U + vv];
         J[row * lda + col] = acc - (row == col ? 1.0 : 0.0);
     }
 }
@@ -132,8 +134,8 @@ __global__ void k_pmat(int N, int U, const double* __restrict__ G, const double*
 
 // dense Jacobian of Eq. FSES_T: J[(s,i),(t,j)] = Pm[s][t] Phi_t[i][j] - delta (unknowns sample-major)
 template <typename T>
-__global__ void k_dense_jac_ht(int N, int n, int P, const T* X, const T* V, const double* Pm, double* J) {
-    const int n2 = 2 * n;
+__global__ void k_dense_jac_ht(int N, PhiView<T> F, const double* Pm, double* J) {
+    const int n2 = 2 * F.n;
     const size_t m = (size_t)N * n2;
     const size_t total = m * m;
     for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
@@ -141,8 +143,7 @@ __global__ void k_dense_jac_ht(int N, int n, int P, const T* X, const T* V, cons
         const size_t row = idx / m, col = idx % m;
         const int s = (int)(row / n2), i = (int)(row % n2);
         const int t = (int)(col / n2), j = (int)(col % n2);
-        const T* xr = (i < n ? X + ((size_t)t * n + i) * P : V + ((size_t)t * n + (i - n)) * P);
-        J[idx] = Pm[(size_t)s * N + t] * (double)xr[j] - (row == col ? 1.0 : 0.0);
+        J[idx] = Pm[(size_t)s * N + t] * F.at(t, i, j) - (row == col ? 1.0 : 0.0);
     }
 }
 
@@ -318,20 +319,21 @@ __global__ void k_lyap_weights(int N, int U, int dm1, const int* ktab, const dou
 
 // A[i][c] = sum_s w_s sum_j Psi_s[i][j] Q[j][c],  Psi = diag(1, w) Phi diag(1, 1/w)  (Eq. F3)
 template <typename T>
-__global__ void k_lyap_prop(int N, int n, int P, int h, double w, const T* X, const T* V,
-                            const double* wts, const double* Q, double* Aout) {
-    const int n2 = 2 * n;
+__global__ void k_lyap_prop(int N, int h, double w, PhiView<T> F, const double* wts, const double* Q, double* Aout) {
+    const int n = F.n, n2 = 2 * n;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (warp >= n2 * h) return;
     const int i = warp / h, c = warp % h;
     const double si = (i < n) ? 1.0 : w;
     double acc = 0.0;
     for (int s = 0; s < N; ++s) {
-        const T* row = (i < n ? X + ((size_t)s * n + i) * P : V + ((size_t)s * n + (i - n)) * P);
+        int g;
+        const T* row = F.row(s, i, g);
         double a2 = 0.0;
-        for (int j = lane; j < n2; j += 32) {
+        for (int k = lane; k < 2 * F.pan.n[g]; k += 32) {
+            const int j = F.col(g, k);
             const double sj = (j < n) ? 1.0 : 1.0 / w;
-            a2 += (double)row[j] * sj * Q[(size_t)j * h + c];
+            a2 += (double)row[k] * sj * Q[(size_t)j * h + c];
         }
         acc += wts[s] * a2;
     }
@@ -393,7 +395,7 @@ void launch_idft(fse_ctx* c, const double* Z, double* zb) {
 void launch_collect_end(fse_ctx* c) {
     const Params& p = c->p;
     const size_t tot = (size_t)p.N * p.n;
-    k_join<<<nblocks(tot, 256), 256, 0, c->stream>>>(p.N, p.n, c->d.q, c->d.u, c->d.zb);
+    k_join<<<nblocks(tot, 256), 256, 0, c->stream>>>(p.N, p.n, p.ni, c->d.row_of, c->d.q, c->d.u, c->d.zb);
 }
 
 void launch_dft_residual(fse_ctx* c, const double* zb, const double* Z0, double* R, int subtract) {
@@ -403,62 +405,56 @@ void launch_dft_residual(fse_ctx* c, const double* zb, const double* Z0, double*
                                                                       Z0, R, subtract);
 }
 
+template <typename T>
+static PhiView<T> phi_view(const fse_ctx* c) {
+    return {(const T*)c->d.X, (const T*)c->d.V, c->d.row_of, c->d.orig_of, c->p.n, c->p.pan};
+}
+
 void launch_phi_apply(fse_ctx* c, const double* zin, double* zout) {
     const Params& p = c->p;
     const size_t warps = (size_t)p.N * 2 * p.n;
     const int g = (int)((warps * 32 + 255) / 256);
     if (p.prec == FSE_MIXED_FP32)
-        k_phi_apply<float><<<g, 256, 0, c->stream>>>(p.N, p.n, p.ld, (const float*)c->d.X,
-                                                    (const float*)c->d.V, zin, zout);
+        k_phi_apply<float><<<g, 256, 0, c->stream>>>(p.N, phi_view<float>(c), zin, zout);
     else
-        k_phi_apply<double><<<g, 256, 0, c->stream>>>(p.N, p.n, p.ld, (const double*)c->d.X,
-                                                     (const double*)c->d.V, zin, zout);
+        k_phi_apply<double><<<g, 256, 0, c->stream>>>(p.N, phi_view<double>(c), zin, zout);
 }
 
 void launch_domega(fse_ctx* c, double* zout) {
     const Params& p = c->p;
     const size_t tot = (size_t)p.N * 2 * p.n;
     if (p.prec == FSE_MIXED_FP32)
-        k_domega_col<float><<<nblocks(tot, 256), 256, 0, c->stream>>>(p.N, p.n, p.ld, (const float*)c->d.X,
-                                                                  (const float*)c->d.V, zout);
+        k_domega_col<float><<<nblocks(tot, 256), 256, 0, c->stream>>>(p.N, phi_view<float>(c), zout);
     else
-        k_domega_col<double><<<nblocks(tot, 256), 256, 0, c->stream>>>(p.N, p.n, p.ld, (const double*)c->d.X,
-                                                                   (const double*)c->d.V, zout);
+        k_domega_col<double><<<nblocks(tot, 256), 256, 0, c->stream>>>(p.N, phi_view<double>(c), zout);
 }
 
-void launch_phi_copy(fse_ctx* c, double* Phi, double* dzdw) {
+static void phi_copy_range(fse_ctx* c, int s0, int count, double* Phi, double* dzdw) {
     const Params& p = c->p;
-    const size_t tot = (size_t)p.N * 4 * p.n * p.n;
+    const size_t tot = (size_t)count * 4 * p.n * p.n;
     if (p.prec == FSE_MIXED_FP32)
-        k_phi_copy<float><<<nblocks(tot, 256), 256, 0, c->stream>>>(p.N, p.n, p.ld, (const float*)c->d.X,
-                                                                (const float*)c->d.V, Phi, dzdw);
+        k_phi_copy<float><<<nblocks(tot, 256), 256, 0, c->stream>>>(count, s0, phi_view<float>(c), Phi, dzdw);
     else
-        k_phi_copy<double><<<nblocks(tot, 256), 256, 0, c->stream>>>(p.N, p.n, p.ld, (const double*)c->d.X,
-                                                                 (const double*)c->d.V, Phi, dzdw);
+        k_phi_copy<double><<<nblocks(tot, 256), 256, 0, c->stream>>>(count, s0, phi_view<double>(c), Phi, dzdw);
 }
 
-void launch_phi_copy_one(fse_ctx* c, int s, double* Phi, double* dzdw) {
-    const Params& p = c->p;
-    const size_t tot = (size_t)4 * p.n * p.n;
-    const size_t off = (size_t)s * p.n * p.ld;
-    if (p.prec == FSE_MIXED_FP32)
-        k_phi_copy<float><<<nblocks(tot, 256), 256, 0, c->stream>>>(1, p.n, p.ld, (const float*)c->d.X + off,
-                                                                (const float*)c->d.V + off, Phi, dzdw);
-    else
-        k_phi_copy<double><<<nblocks(tot, 256), 256, 0, c->stream>>>(1, p.n, p.ld, (const double*)c->d.X + off,
-                                                                 (const double*)c->d.V + off, Phi, dzdw);
-}
+void launch_phi_copy(fse_ctx* c, double* Phi, double* dzdw) { phi_copy_range(c, 0, c->p.N, Phi, dzdw); }
 
-void launch_dense_jac(fse_ctx* c, double* J) {
+void launch_phi_copy_one(fse_ctx* c, int s, double* Phi, double* dzdw) { phi_copy_range(c, s, 1, Phi, dzdw); }
+
+// dense Eq. (22) into an array of row stride lda
+static void dense_jac(fse_ctx* c, double* J, size_t lda) {
     const Params& p = c->p;
     const size_t m = (size_t)2 * p.n * p.U;
     if (p.prec == FSE_MIXED_FP32)
-        k_dense_jac<float><<<nblocks(m * m, 256, 64), 256, 0, c->stream>>>(
-            p.N, p.n, p.U, p.ld, (const float*)c->d.X, (const float*)c->d.V, c->d.RG, c->d.G, J, m);
+        k_dense_jac<float><<<nblocks(m * m, 256, 64), 256, 0, c->stream>>>(p.N, p.U, phi_view<float>(c), c->d.RG,
+                                                                           c->d.G, J, lda);
     else
-        k_dense_jac<double><<<nblocks(m * m, 256, 64), 256, 0, c->stream>>>(
-            p.N, p.n, p.U, p.ld, (const double*)c->d.X, (const double*)c->d.V, c->d.RG, c->d.G, J, m);
+        k_dense_jac<double><<<nblocks(m * m, 256, 64), 256, 0, c->stream>>>(p.N, p.U, phi_view<double>(c), c->d.RG,
+                                                                            c->d.G, J, lda);
 }
+
+void launch_dense_jac(fse_ctx* c, double* J) { dense_jac(c, J, (size_t)2 * c->p.n * c->p.U); }
 
 void launch_pmat(fse_ctx* c, double* Pm) {
     const Params& p = c->p;
@@ -469,22 +465,14 @@ void launch_dense_jac_ht(fse_ctx* c, const double* Pm, double* J) {
     const Params& p = c->p;
     const size_t m = (size_t)2 * p.n * p.N;
     if (p.prec == FSE_MIXED_FP32)
-        k_dense_jac_ht<float><<<nblocks(m * m, 256, 64), 256, 0, c->stream>>>(
-            p.N, p.n, p.ld, (const float*)c->d.X, (const float*)c->d.V, Pm, J);
+        k_dense_jac_ht<float><<<nblocks(m * m, 256, 64), 256, 0, c->stream>>>(p.N, phi_view<float>(c), Pm, J);
     else
-        k_dense_jac_ht<double><<<nblocks(m * m, 256, 64), 256, 0, c->stream>>>(
-            p.N, p.n, p.ld, (const double*)c->d.X, (const double*)c->d.V, Pm, J);
+        k_dense_jac_ht<double><<<nblocks(m * m, 256, 64), 256, 0, c->stream>>>(p.N, phi_view<double>(c), Pm, J);
 }
 
 void launch_bordered_jac(fse_ctx* c, const double* Rw, const double* tZ, double tail, double* B) {
-    const Params& p = c->p;
-    const size_t m = (size_t)2 * p.n * p.U;
-    if (p.prec == FSE_MIXED_FP32)
-        k_dense_jac<float><<<nblocks(m * m, 256, 64), 256, 0, c->stream>>>(
-            p.N, p.n, p.U, p.ld, (const float*)c->d.X, (const float*)c->d.V, c->d.RG, c->d.G, B, m + 1);
-    else
-        k_dense_jac<double><<<nblocks(m * m, 256, 64), 256, 0, c->stream>>>(
-            p.N, p.n, p.U, p.ld, (const double*)c->d.X, (const double*)c->d.V, c->d.RG, c->d.G, B, m + 1);
+    const size_t m = (size_t)2 * c->p.n * c->p.U;
+    dense_jac(c, B, m + 1);
     k_border<<<nblocks(m + 1, 256), 256, 0, c->stream>>>(m, Rw, tZ, tail, B);
 }
 
@@ -497,14 +485,8 @@ void launch_unknown_border(fse_ctx* c, int j, double w, const double* R, const d
 }
 
 void launch_dense_jac_bordered(fse_ctx* c, int u, const double* cols, const double* rows, double* B) {
-    const Params& p = c->p;
-    const size_t m = (size_t)2 * p.n * p.U;
-    if (p.prec == FSE_MIXED_FP32)
-        k_dense_jac<float><<<nblocks(m * m, 256, 64), 256, 0, c->stream>>>(
-            p.N, p.n, p.U, p.ld, (const float*)c->d.X, (const float*)c->d.V, c->d.RG, c->d.G, B, m + u);
-    else
-        k_dense_jac<double><<<nblocks(m * m, 256, 64), 256, 0, c->stream>>>(
-            p.N, p.n, p.U, p.ld, (const double*)c->d.X, (const double*)c->d.V, c->d.RG, c->d.G, B, m + u);
+    const size_t m = (size_t)2 * c->p.n * c->p.U;
+    dense_jac(c, B, m + u);
     k_border_multi<<<nblocks(m + u, 256), 256, 0, c->stream>>>(m, u, cols, rows, B);
 }
 
@@ -558,11 +540,9 @@ int lyapunov_run(fse_ctx* c, double w, int N_Ly, int h, double* sigma) {
         k_lyap_weights<<<nblocks(p.N, 128), 128, 0, c->stream>>>(p.N, p.U, p.d - 1, c->d.ktab, c->d.Gi,
                                                              ph[0], ph[1], ph[2], wts);
         if (p.prec == FSE_MIXED_FP32)
-            k_lyap_prop<float><<<g, 256, 0, c->stream>>>(p.N, p.n, p.ld, h, w, (const float*)c->d.X,
-                                                        (const float*)c->d.V, wts, Q, A);
+            k_lyap_prop<float><<<g, 256, 0, c->stream>>>(p.N, h, w, phi_view<float>(c), wts, Q, A);
         else
-            k_lyap_prop<double><<<g, 256, 0, c->stream>>>(p.N, p.n, p.ld, h, w, (const double*)c->d.X,
-                                                         (const double*)c->d.V, wts, Q, A);
+            k_lyap_prop<double><<<g, 256, 0, c->stream>>>(p.N, h, w, phi_view<double>(c), wts, Q, A);
         k_lyap_qr<<<1, 512, 0, c->stream>>>(m, h, A, Q, acc);
     }
     std::vector<double> hacc(h);
@@ -668,11 +648,9 @@ int lyapunov_run_noalloc(fse_ctx* c, double w, int N_Ly, int h, double* sigma) {
         k_lyap_weights<<<nblocks(p.N, 128), 128, 0, c->stream>>>(p.N, p.U, p.d - 1, c->d.ktab, c->d.Gi,
                                                              ph[0], ph[1], ph[2], wts);
         if (p.prec == FSE_MIXED_FP32)
-            k_lyap_prop<float><<<g, 256, 0, c->stream>>>(p.N, p.n, p.ld, h, w, (const float*)c->d.X,
-                                                        (const float*)c->d.V, wts, Q, A);
+            k_lyap_prop<float><<<g, 256, 0, c->stream>>>(p.N, h, w, phi_view<float>(c), wts, Q, A);
         else
-            k_lyap_prop<double><<<g, 256, 0, c->stream>>>(p.N, p.n, p.ld, h, w, (const double*)c->d.X,
-                                                         (const double*)c->d.V, wts, Q, A);
+            k_lyap_prop<double><<<g, 256, 0, c->stream>>>(p.N, h, w, phi_view<double>(c), wts, Q, A);
         k_lyap_qr<<<1, 512, 0, c->stream>>>(m, h, A, Q, acc);
     }
     double hacc[kNoallocAcc];

@@ -78,25 +78,30 @@ struct RowGroups {
     std::vector<int> map;    // E x R
 };
 
-static RowGroups group_rows(int n, const std::vector<int>& cptr, const std::vector<int>& ccol, int R) {
-    RowGroups G;
-    G.R = R;
-    std::map<std::vector<int>, int> open;
+// appends the groups of rows r0 .. r1 - 1 to G
+static void group_rows(int r0, int r1, const std::vector<int>& cptr, const std::vector<int>& ccol, RowGroups& G) {
+    const int R = G.R;
     std::vector<std::vector<int>> members;
-    for (int i = 0; i < n; ++i) {
-        std::vector<int> pat(ccol.begin() + cptr[i], ccol.begin() + cptr[i + 1]);
-        auto it = open.find(pat);
-        if (it != open.end()) {
-            std::vector<int>& mem = members[it->second];
+    std::vector<int> of(r1 - r0);   // group of each row
+    auto same = [&](int i, int j) {
+        return cptr[i + 1] - cptr[i] == cptr[j + 1] - cptr[j] &&
+               std::equal(ccol.begin() + cptr[i], ccol.begin() + cptr[i + 1], ccol.begin() + cptr[j]);
+    };
+    for (int i = r0; i < r1; ++i) {
+        // the group of the nearest earlier row with this pattern, if it is open
+        int j = i - 1;
+        while (j >= std::max(r0, i - 7) && !same(i, j)) --j;
+        if (j >= std::max(r0, i - 7)) {
+            std::vector<int>& mem = members[of[j - r0]];
             if ((int)mem.size() < R && i - mem[0] < 8) {
                 mem.push_back(i);
+                of[i - r0] = of[j - r0];
                 continue;
             }
         }
-        open[pat] = (int)members.size();
+        of[i - r0] = (int)members.size();
         members.push_back({i});
     }
-    G.ptr.push_back(0);
     for (const auto& mem : members) {
         const int i0 = mem[0], len = cptr[i0 + 1] - cptr[i0];
         for (int r = 0; r < R; ++r) G.rows.push_back(r < (int)mem.size() ? mem[r] : -1);
@@ -106,11 +111,287 @@ static RowGroups group_rows(int n, const std::vector<int>& cptr, const std::vect
         }
         G.ptr.push_back((int)G.col.size());
     }
-    return G;
 }
+
+// A numbering of the model's dofs: the caller's own (one panel), or by components (Panels in
+// fse_internal.h).
+struct Numbering {
+    std::vector<int> row_of, orig_of;   // dof -> internal row; internal row -> dof (-1: inert)
+    int ni = 0, b = 0;
+    fse::Panels pan;
+};
+
+// rows, strides and offsets of the panels once pan.nc, row0, n and b are set
+static void finish_panels(Numbering& N) {
+    fse::Panels& P = N.pan;
+    P.tot = 0;
+    N.b = 0;
+    for (int g = 0; g < P.nc; ++g) {
+        P.ld[g] = (2 * P.n[g] + 1 + 3) & ~3;
+        P.off[g] = P.tot;
+        P.tot += (size_t)P.n[g] * P.ld[g];
+        N.b = std::max(N.b, P.b[g]);
+    }
+}
+
+static Numbering own_numbering(int n, int b) {
+    Numbering N;
+    N.ni = n;
+    N.row_of.resize(n);
+    for (int i = 0; i < n; ++i) N.row_of[i] = i;
+    N.orig_of = N.row_of;
+    N.pan.n[0] = n;
+    N.pan.b[0] = b;
+    finish_panels(N);
+    return N;
+}
+
+// Numbering by components (pairs: every coupled pair of dofs, comp[i]: a label per component).  The
+// largest components get a panel each, the others share the last one; dofs keep their order inside
+// a component.  nc stays 0 where it does not pay: the panels' tangents (rows in whole blocks x
+// columns) are what every step streams and solves, and below a quarter saved the inert rows and the
+// shorter blocks cost about as much (n = 24: 3 panels of 32 rows against 1).
+static Numbering component_numbering(int n, const std::vector<std::pair<int, int>>& pairs, const std::vector<int>& comp) {
+    Numbering N;
+    N.pan.nc = 0;
+    std::vector<std::vector<int>> members;
+    std::map<int, int> index;
+    for (int i = 0; i < n; ++i) {
+        auto it = index.find(comp[i]);
+        if (it == index.end()) {
+            it = index.emplace(comp[i], (int)members.size()).first;
+            members.emplace_back();
+        }
+        members[it->second].push_back(i);
+    }
+    if (members.size() < 2) return N;
+    std::stable_sort(members.begin(), members.end(),
+                     [](const std::vector<int>& a, const std::vector<int>& b) { return a.size() > b.size(); });
+    const int nc = std::min<int>((int)members.size(), FSE_MAX_PANELS);
+    N.row_of.assign(n, 0);
+    int r = 0;
+    double area = 0.0;
+    for (int g = 0; g < nc; ++g) {
+        r = (r + FSE_BLK - 1) / FSE_BLK * FSE_BLK;
+        N.pan.row0[g] = r;
+        for (size_t k = g; k < (g + 1 < nc ? g + 1 : members.size()); ++k)
+            for (int i : members[k]) N.row_of[i] = r++;
+        N.pan.n[g] = r - N.pan.row0[g];
+        area += (double)((N.pan.n[g] + FSE_BLK - 1) / FSE_BLK * FSE_BLK) * (2 * N.pan.n[g] + 1);
+    }
+    if (area > 0.75 * ((n + FSE_BLK - 1) / FSE_BLK * FSE_BLK) * (2.0 * n + 1)) return N;
+    N.pan.nc = nc;
+    N.ni = r;
+    N.orig_of.assign(N.ni, -1);
+    for (int i = 0; i < n; ++i) N.orig_of[N.row_of[i]] = i;
+    for (const auto& pr : pairs) {
+        const int a = N.row_of[pr.first], b = N.row_of[pr.second];
+        int g = nc - 1;
+        while (a < N.pan.row0[g]) --g;
+        N.pan.b[g] = std::max(N.pan.b[g], std::abs(a - b));
+    }
+    finish_panels(N);
+    return N;
+}
+
+// CSR of the union pattern of M, D, K in a numbering (sorted columns; inert rows: M = K = 1), the
+// diagonal-major full band of M and the K_t pattern with its sources (element in sorted order, a, b)
+struct Matrices {
+    std::vector<int> cptr, ccol, kptr, kcol, ksoff, ksrc;
+    std::vector<double> cm, cd, ck, Mb;
+};
 
 // bytes of one group record: the ring slot (int, padded to 8 bytes), then 2R values
 static int group_record_bytes(int R, size_t tsz) { return (int)((8 + 2 * R * tsz + 15) / 16 * 16); }
+
+static Matrices build_matrices(const fse_model* m, const Numbering& N, int b_user, const std::vector<int>& et,
+                               const std::vector<int>& ed) {
+    Matrices X;
+    const int n = m->n, ni = N.ni, b = N.b;
+    X.cptr.assign(ni + 1, 0);
+    X.Mb.assign((size_t)(2 * b + 1) * ni, 0.0);
+    for (int r = 0; r < ni; ++r) {
+        const int i = N.orig_of[r];
+        if (i < 0) {
+            X.ccol.push_back(r);
+            X.cm.push_back(1.0);
+            X.cd.push_back(0.0);
+            X.ck.push_back(1.0);
+            X.Mb[(size_t)b * ni + r] = 1.0;
+        } else {
+            for (int j = std::max(0, i - b_user); j <= std::min(n - 1, i + b_user); ++j) {
+                const size_t o = (size_t)i * n + j;
+                if (m->M[o] == 0.0 && m->D[o] == 0.0 && m->K[o] == 0.0) continue;
+                const int c = N.row_of[j];
+                X.ccol.push_back(c);
+                X.cm.push_back(m->M[o]);
+                X.cd.push_back(m->D[o]);
+                X.ck.push_back(m->K[o]);
+                X.Mb[(size_t)(c - r + b) * ni + r] = m->M[o];
+            }
+        }
+        X.cptr[r + 1] = (int)X.ccol.size();
+    }
+    // CSR pattern of K_t: entry (dof_a, dof_b) for every element and local pair; each entry
+    // keeps its sources (element in sorted order, a, b) in increasing element order
+    std::vector<std::vector<std::pair<int, int>>> ktrow(ni);   // (col, source)
+    for (int k = 0; k < m->n_nl; ++k) {
+        const int nd = et[k] == 1 ? 1 : (et[k] == 2 ? 2 : 6);
+        for (int a = 0; a < nd; ++a)
+            for (int bb = 0; bb < nd; ++bb) {
+                const int ga = ed[(size_t)6 * k + a], gb = ed[(size_t)6 * k + bb];
+                if (ga >= 0 && gb >= 0) ktrow[N.row_of[ga]].push_back({N.row_of[gb], k * 36 + a * 6 + bb});
+            }
+    }
+    X.kptr.assign(ni + 1, 0);
+    X.ksoff.assign(1, 0);
+    for (int i = 0; i < ni; ++i) {
+        auto& r = ktrow[i];
+        std::stable_sort(r.begin(), r.end(), [](const std::pair<int, int>& x, const std::pair<int, int>& y) {
+            return x.first < y.first;
+        });
+        for (size_t q = 0; q < r.size(); ++q) {
+            if (q == 0 || r[q].first != r[q - 1].first) {
+                X.kcol.push_back(r[q].first);
+                X.ksoff.push_back(X.ksoff.back());
+            }
+            X.ksrc.push_back(r[q].second);
+            X.ksoff.back()++;
+        }
+        X.kptr[i + 1] = (int)X.kcol.size();
+    }
+    return X;
+}
+
+// sizes, row groups and passes of the tangent kernels for one numbering (p: n_el, prec, has_vel set)
+static RowGroups plan_tangents(Params& p, const Numbering& N, const Matrices& X, std::vector<int>& gpass,
+                               std::vector<int>& ginfo, std::vector<int>& grr) {
+    const size_t tsz = p.prec == FSE_MIXED_FP32 ? 4 : 8;
+    p.ni = N.ni;
+    p.b = N.b;
+    p.nnz = (int)X.ccol.size();
+    p.nnz_kt = (int)X.kcol.size();
+    p.nblk = (p.ni + FSE_BLK - 1) / FSE_BLK;
+    p.RECE = ((p.b + 3) & ~3) * FSE_BLK + FSE_BLK * FSE_BLK;
+    p.ND = (p.b + FSE_BLK - 1) / FSE_BLK;
+    // row groups: R chosen by the shared-memory wavefronts per 64-column pass of an entry
+    // (4 for the X and V elements, RB / 16 for the broadcast record).  Groups and passes of
+    // FSE_RHS_GPS groups stay inside a panel; the last pass of a panel is filled up with empty groups.
+    RowGroups grp;
+    double best = 0.0;
+    for (int R = 1; R <= FSE_RHS_MAXR; ++R) {
+        RowGroups cand;
+        fse::Panels pan = N.pan;
+        cand.R = R;
+        cand.ptr.push_back(0);
+        for (int g = 0; g < pan.nc; ++g) {
+            group_rows(pan.row0[g], pan.row0[g] + pan.n[g], X.cptr, X.ccol, cand);
+            while (g + 1 < pan.nc && (cand.ptr.size() - 1) % FSE_RHS_GPS) {
+                cand.rows.insert(cand.rows.end(), R, -1);
+                cand.ptr.push_back(cand.ptr.back());
+            }
+            pan.g1[g] = (int)cand.ptr.size() - 1;
+            pan.pass0[g + 1] = (pan.g1[g] + FSE_RHS_GPS - 1) / FSE_RHS_GPS;
+        }
+        const double cost = (double)cand.col.size() * (4.0 + group_record_bytes(R, tsz) / 16.0);
+        if (R == 1 || cost < best) {
+            best = cost;
+            grp = std::move(cand);
+            p.pan = pan;
+        }
+    }
+    p.R = grp.R;
+    p.ng = (int)grp.ptr.size() - 1;
+    p.nE = (int)grp.col.size();
+    p.RB = group_record_bytes(p.R, tsz);
+    // per pass: rows that must be staged (monotone inside a panel), entries, ring span
+    const int npass = p.pan.pass0[p.pan.nc];
+    std::vector<int> ghi(npass), gmin(npass);
+    const int dep = p.prec == FSE_MIXED_FP32 ? FSE_RHS_DEPTH_F32 : FSE_RHS_DEPTH_F64;
+    p.RW = 32;
+    p.ME = 0;
+    for (int g = 0; g < p.pan.nc; ++g) {
+        const int r0 = N.pan.row0[g], r1 = r0 + N.pan.n[g], q0 = p.pan.pass0[g], q1 = p.pan.pass0[g + 1];
+        int hi = 0;
+        for (int ps = q0; ps < q1; ++ps) {
+            const int a = ps * FSE_RHS_GPS, z = std::min(p.ng, a + FSE_RHS_GPS);
+            int mx = 0;
+            for (int k = a * p.R; k < z * p.R; ++k) mx = std::max(mx, grp.rows[k]);
+            hi = std::max(hi, std::min(r1, mx + N.pan.b[g] + 1));
+            ghi[ps] = hi;
+            gmin[ps] = grp.rows[(size_t)a * p.R];
+            p.ME = std::max(p.ME, grp.ptr[z] - grp.ptr[a]);
+        }
+        // rows are staged in 32-row TMA boxes: the ring (a multiple of 32 rows) holds from the
+        // first row a pass reads up to the last box staged for the passes in flight
+        for (int ps = q0; ps < q1; ++ps) {
+            const int top = (ghi[std::min(ps + dep, q1 - 1)] + 31) & ~31;
+            p.RW = std::max(p.RW, top - std::max(r0, gmin[ps] - N.pan.b[g]));
+        }
+    }
+    p.RW = (p.RW + 31) & ~31;
+    p.RWT = 1;
+    while (p.RWT < p.b + FSE_BLK) p.RWT <<= 1;
+    // per pass: {rows of the panel to stage, first entry, end entry, first K_t entry}, {K_t entries,
+    // first group, 0, 0}; the K_t slice of a pass starts at a multiple of 4 and has a multiple of 4
+    // entries (16-byte bulk copies); per group: {first entry relative to its pass, entries};
+    // per row: {row, K_t begin, K_t end (relative to the pass's slice), 0}
+    p.kt_ld = std::max(4, (p.nnz_kt + 3) & ~3);
+    gpass.assign((size_t)8 * npass, 0);
+    ginfo.assign((size_t)2 * ((p.ng + 1) & ~1), 0);
+    grr.assign((size_t)p.ng * p.R * 4, 0);
+    p.MK = 0;
+    for (int ps = 0; ps < npass; ++ps) {
+        const int g0 = ps * FSE_RHS_GPS, g1 = std::min(p.ng, g0 + FSE_RHS_GPS);
+        int k0 = p.nnz_kt, k1 = 0, pg = p.pan.nc - 1;
+        while (ps < p.pan.pass0[pg]) --pg;
+        for (int g = g0; g < g1; ++g)
+            for (int r = 0; r < p.R; ++r) {
+                const int i = grp.rows[(size_t)g * p.R + r];
+                if (i < 0) continue;
+                k0 = std::min(k0, X.kptr[i]);
+                k1 = std::max(k1, X.kptr[i + 1]);
+            }
+        const int kb = k1 > k0 ? (k0 & ~3) : 0;
+        const int kn = k1 > k0 ? ((k1 - kb + 3) & ~3) : 0;
+        p.MK = std::max(p.MK, kn);
+        int* d = &gpass[(size_t)8 * ps];
+        d[0] = ghi[ps] - N.pan.row0[pg];
+        d[1] = grp.ptr[g0];
+        d[2] = grp.ptr[g1];
+        d[3] = kb;
+        d[4] = kn;
+        d[5] = g0;
+        for (int g = g0; g < g1; ++g) {
+            ginfo[(size_t)2 * g] = grp.ptr[g] - grp.ptr[g0];
+            ginfo[(size_t)2 * g + 1] = grp.ptr[g + 1] - grp.ptr[g];
+            for (int r = 0; r < p.R; ++r) {
+                const size_t q = (size_t)g * p.R + r;
+                const int i = grp.rows[q];
+                grr[4 * q] = i;
+                grr[4 * q + 1] = i >= 0 ? X.kptr[i] - kb : 0;
+                grr[4 * q + 2] = i >= 0 ? X.kptr[i + 1] - kb : 0;
+            }
+        }
+    }
+    // panel Cholesky in the state kernel for FP32 factors with b <= 96 when its window fits
+    p.chol_blk = 0;
+    if (p.prec == FSE_MIXED_FP32 && p.b <= 96) {
+        p.chol_blk = 1;
+        if (fse::state_smem(p) > 220 * 1024) p.chol_blk = 0;
+    }
+    p.smem_state = fse::state_smem(p);
+    p.smem_rhs = fse::rhs_smem(p);
+    p.smem_trsm = fse::trsm_smem(p);
+    return grp;
+}
+
+// whether the kernels' on-chip working sets fit
+static bool plan_fits(const Params& p) {
+    const size_t lim = 220 * 1024, nb = p.b + 1;
+    return p.b <= FSE_MAX_BAND && p.smem_state <= lim && p.smem_rhs <= lim && p.smem_trsm <= lim &&
+           (nb + 9) * nb * sizeof(double) <= lim;
+}
 
 // cos and sin of the rotation angles 2 pi k~_l . rho of Eq. (14), l < L, for the context's rho
 static void rotation_tables(const fse_ctx* c, std::vector<double>& rc, std::vector<double>& rs) {
@@ -141,7 +422,7 @@ static void free_ctx(fse_ctx* c) {
                     c->d.ktab, c->d.LMc, c->d.LMr, c->d.LMinv, c->d.q, c->d.u, c->d.a, c->d.zb,
                     c->d.Lc, c->d.Lr, c->d.Linv, c->d.Dinv, c->d.Rf, c->d.Rb, c->d.Tf, c->d.Tb, c->d.X, c->d.V, c->d.Y, c->d.Z0, c->d.R,
                     c->d.vec, c->d.vec2, c->d.yb, c->d.status, c->d.iters, c->d.nref, c->d.flag, c->Jd, c->piv, c->kry, c->kdot,
-                    c->ht, c->unk, c->d.Sband, c->d.ktc_ptr, c->d.ktc_e, c->d.ktc_c, c->d.ktc_r};
+                    c->ht, c->unk, c->d.row_of, c->d.orig_of, c->d.Sband, c->d.ktc_ptr, c->d.ktc_e, c->d.ktc_c, c->d.ktc_r};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (auto& e : c->ev)
@@ -206,10 +487,14 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
         if (!std::isfinite(o->rho[j])) return set_err(nullptr, FSE_EINVAL, "rho not finite");
     // half-bandwidth from exact zeros and element spans
     int b = 0;
+    std::vector<std::pair<int, int>> pairs;   // coupled pairs of dofs
     for (int i = 0; i < n; ++i)
         for (int j = 0; j < n; ++j) {
             const size_t o2 = (size_t)i * n + j;
-            if (m->M[o2] != 0.0 || m->D[o2] != 0.0 || m->K[o2] != 0.0) b = std::max(b, std::abs(i - j));
+            if (m->M[o2] != 0.0 || m->D[o2] != 0.0 || m->K[o2] != 0.0) {
+                b = std::max(b, std::abs(i - j));
+                if (i != j) pairs.push_back({i, j});
+            }
         }
     for (int e = 0; e < m->n_nl; ++e) {
         const fse_nl_elem& el = m->nl[e];
@@ -219,15 +504,27 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
             if (el.dof[a] >= n || el.dof[a] < -1) return set_err(nullptr, FSE_EINVAL, "element dof out of range");
             if (el.type != 3 && el.dof[a] < 0) return set_err(nullptr, FSE_EINVAL, "spring dof must be >= 0");
             for (int c2 = 0; c2 < nd; ++c2)
-                if (el.dof[a] >= 0 && el.dof[c2] >= 0) b = std::max(b, std::abs(el.dof[a] - el.dof[c2]));
+                if (el.dof[a] >= 0 && el.dof[c2] >= 0) {
+                    b = std::max(b, std::abs(el.dof[a] - el.dof[c2]));
+                    if (el.dof[a] != el.dof[c2]) pairs.push_back({el.dof[a], el.dof[c2]});
+                }
         }
         if (el.type == 3 && !(el.p[1] > 0.0)) return set_err(nullptr, FSE_EINVAL, "beam element length must be > 0");
     }
+    // components of the coupling graph (union-find with path halving)
+    std::vector<int> comp(n);
+    for (int i = 0; i < n; ++i) comp[i] = i;
+    auto find = [&](int i) {
+        while (comp[i] != i) i = comp[i] = comp[comp[i]];
+        return i;
+    };
+    for (const auto& pr : pairs) comp[find(pr.first)] = find(pr.second);
+    for (int i = 0; i < n; ++i) comp[i] = find(i);
     fse_ctx* c = new (std::nothrow) fse_ctx();
     if (!c) return set_err(nullptr, FSE_ENOMEM, "host allocation failed");
     Params& p = c->p;
     p.n = n;
-    p.b = b;
+    p.b_user = b;
     p.d = o->d;
     p.e = m->e;
     p.N = (int)N;
@@ -237,7 +534,6 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
     p.U = (int)U;
     p.L = (int)(U - 1) / 2;
     p.S1 = o->S1;
-    p.P = 2 * n + 1;
     p.maxit = o->newton_maxit;
     p.prec = o->precision;
     p.tol = o->newton_tol;
@@ -245,7 +541,6 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
     for (int e = 0; e < m->n_nl; ++e)
         if (m->nl[e].type == FSE_NL_VDP) p.has_vel = true;
     const size_t tsz = p.prec == FSE_MIXED_FP32 ? 4 : 8;
-    const int nb = b + 1;
     for (int j = 0; j < o->d - 1; ++j) c->rho.push_back(o->rho[j]);
     if (device >= 0) {
         if (cudaSetDevice(device) != cudaSuccess) {
@@ -290,25 +585,6 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
     // rotation angles 2 pi k~_l . rho (Eq. 14)
     std::vector<double> rcv, rsv;
     rotation_tables(c, rcv, rsv);
-    // diagonal-major full band of M (for its factor) and the CSR of the union pattern of M, D, K
-    const int fb = 2 * b + 1;
-    std::vector<double> Mb((size_t)fb * n, 0.0);
-    std::vector<int> cptr(n + 1, 0), ccol;
-    std::vector<double> cm, cd, ck;
-    for (int i = 0; i < n; ++i) {
-        for (int j = std::max(0, i - b); j <= std::min(n - 1, i + b); ++j) {
-            const size_t o2 = (size_t)i * n + j;
-            Mb[(size_t)(j - i + b) * n + i] = m->M[o2];
-            if (m->M[o2] != 0.0 || m->D[o2] != 0.0 || m->K[o2] != 0.0) {
-                ccol.push_back(j);
-                cm.push_back(m->M[o2]);
-                cd.push_back(m->D[o2]);
-                ck.push_back(m->K[o2]);
-            }
-        }
-        cptr[i + 1] = (int)ccol.size();
-    }
-    p.nnz = (int)ccol.size();
     // colour the elements so that no two of a colour share a dof
     std::vector<int> color(m->n_nl, 0);
     std::vector<uint64_t> used(n, 0);
@@ -346,145 +622,50 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
         coff[color[order[k]] + 1]++;
     }
     for (int cl = 0; cl < ncol; ++cl) coff[cl + 1] += coff[cl];
-    // CSR pattern of K_t: entry (dof_a, dof_b) for every element and local pair; each entry
-    // keeps its sources (element in sorted order, a, b) in increasing element order
-    std::vector<std::vector<std::pair<int, int>>> ktrow(n);   // (col, source)
-    for (int k = 0; k < m->n_nl; ++k) {
-        const int nd = et[k] == 1 ? 1 : (et[k] == 2 ? 2 : 6);
-        for (int a = 0; a < nd; ++a)
-            for (int bb = 0; bb < nd; ++bb) {
-                const int ga = ed[(size_t)6 * k + a], gb = ed[(size_t)6 * k + bb];
-                if (ga >= 0 && gb >= 0) ktrow[ga].push_back({gb, k * 36 + a * 6 + bb});
-            }
-    }
-    std::vector<int> kptr(n + 1, 0), kcol, ksoff(1, 0), ksrc;
-    for (int i = 0; i < n; ++i) {
-        auto& r = ktrow[i];
-        std::stable_sort(r.begin(), r.end(), [](const std::pair<int, int>& x, const std::pair<int, int>& y) {
-            return x.first < y.first;
-        });
-        for (size_t q = 0; q < r.size(); ++q) {
-            if (q == 0 || r[q].first != r[q - 1].first) {
-                kcol.push_back(r[q].first);
-                ksoff.push_back(ksoff.back());
-            }
-            ksrc.push_back(r[q].second);
-            ksoff.back()++;
-        }
-        kptr[i + 1] = (int)kcol.size();
-    }
-    p.nnz_kt = (int)kcol.size();
-    p.nblk = (n + FSE_BLK - 1) / FSE_BLK;
-    p.RECE = ((b + 3) & ~3) * FSE_BLK + FSE_BLK * FSE_BLK;
-    p.ND = (b + FSE_BLK - 1) / FSE_BLK;
-    p.tc_ok = p.prec == FSE_MIXED_FP32 && b <= 96;
-    p.ld = (p.P + 3) & ~3;
-    // row groups: R chosen by the shared-memory wavefronts per 64-column pass of an entry
-    // (4 for the X and V elements, RB / 16 for the broadcast record)
-    RowGroups grp;
-    {
-        double best = 0.0;
-        for (int R = 1; R <= FSE_RHS_MAXR; ++R) {
-            RowGroups cand = group_rows(n, cptr, ccol, R);
-            const double cost = (double)cand.col.size() * (4.0 + group_record_bytes(R, tsz) / 16.0);
-            if (R == 1 || cost < best) {
-                best = cost;
-                grp = std::move(cand);
-            }
-        }
-    }
-    p.R = grp.R;
-    p.ng = (int)grp.ptr.size() - 1;
-    p.nE = (int)grp.col.size();
-    p.RB = group_record_bytes(p.R, tsz);
-    // per pass of FSE_RHS_GPS groups: rows that must be staged (monotone), entries, ring span
-    const int npass = (p.ng + FSE_RHS_GPS - 1) / FSE_RHS_GPS;
-    std::vector<int> ghi(npass), gmin(npass);
-    {
-        int hi = 0;
-        for (int ps = 0; ps < npass; ++ps) {
-            const int g0 = ps * FSE_RHS_GPS, g1 = std::min(p.ng, g0 + FSE_RHS_GPS);
-            int mx = 0;
-            for (int g = g0; g < g1; ++g)
-                for (int r = 0; r < p.R; ++r) mx = std::max(mx, grp.rows[(size_t)g * p.R + r]);
-            hi = std::max(hi, std::min(n, mx + b + 1));
-            ghi[ps] = hi;
-            gmin[ps] = grp.rows[(size_t)g0 * p.R];
-            p.ME = std::max(p.ME, grp.ptr[g1] - grp.ptr[g0]);
-        }
-        // rows are staged in 32-row TMA boxes: the ring (a multiple of 32 rows) holds from the
-        // first row a pass reads up to the last box staged for the passes in flight
-        const int dep = p.prec == FSE_MIXED_FP32 ? FSE_RHS_DEPTH_F32 : FSE_RHS_DEPTH_F64;
-        p.RW = 32;
-        for (int ps = 0; ps < npass; ++ps) {
-            const int top = (ghi[std::min(ps + dep, npass - 1)] + 31) & ~31;
-            p.RW = std::max(p.RW, top - std::max(0, gmin[ps] - b));
-        }
-        p.RW = (p.RW + 31) & ~31;
-    }
-    p.RWT = 1;
-    while (p.RWT < b + FSE_BLK) p.RWT <<= 1;
-    // per pass: {rows to stage, first entry, end entry, first K_t entry}, {K_t entries, first
-    // group, 0, 0}; the K_t slice of a pass starts at a multiple of 4 and has a multiple of 4
-    // entries (16-byte bulk copies); per group: {first entry relative to its pass, entries};
-    // per row: {row, K_t begin, K_t end (relative to the pass's slice), 0}
-    p.kt_ld = std::max(4, (p.nnz_kt + 3) & ~3);
-    std::vector<int> gpass((size_t)8 * npass, 0), ginfo((size_t)2 * ((p.ng + 1) & ~1), 0);
-    std::vector<int> grr((size_t)p.ng * p.R * 4, 0);
-    p.MK = 0;
-    for (int ps = 0; ps < npass; ++ps) {
-        const int g0 = ps * FSE_RHS_GPS, g1 = std::min(p.ng, g0 + FSE_RHS_GPS);
-        int k0 = p.nnz_kt, k1 = 0;
-        for (int g = g0; g < g1; ++g)
-            for (int r = 0; r < p.R; ++r) {
-                const int i = grp.rows[(size_t)g * p.R + r];
-                if (i < 0) continue;
-                k0 = std::min(k0, kptr[i]);
-                k1 = std::max(k1, kptr[i + 1]);
-            }
-        const int kb = k1 > k0 ? (k0 & ~3) : 0;
-        const int kn = k1 > k0 ? ((k1 - kb + 3) & ~3) : 0;
-        p.MK = std::max(p.MK, kn);
-        int* d = &gpass[(size_t)8 * ps];
-        d[0] = ghi[ps];
-        d[1] = grp.ptr[g0];
-        d[2] = grp.ptr[g1];
-        d[3] = kb;
-        d[4] = kn;
-        d[5] = g0;
-        for (int g = g0; g < g1; ++g) {
-            ginfo[(size_t)2 * g] = grp.ptr[g] - grp.ptr[g0];
-            ginfo[(size_t)2 * g + 1] = grp.ptr[g + 1] - grp.ptr[g];
-            for (int r = 0; r < p.R; ++r) {
-                const size_t q = (size_t)g * p.R + r;
-                const int i = grp.rows[q];
-                grr[4 * q] = i;
-                grr[4 * q + 1] = i >= 0 ? kptr[i] - kb : 0;
-                grr[4 * q + 2] = i >= 0 ? kptr[i + 1] - kb : 0;
-            }
-        }
-    }
-    std::vector<int> gslot(grp.col.size()), kslot(p.kt_ld, 0);
-    for (size_t q = 0; q < grp.col.size(); ++q) gslot[q] = grp.col[q] % p.RW;
-    for (size_t q = 0; q < kcol.size(); ++q) kslot[q] = kcol[q] % p.RW;
-    // panel Cholesky in the state kernel for FP32 factors with b <= 96 when its window fits
-    p.chol_blk = 0;
-    if (p.prec == FSE_MIXED_FP32 && b <= 96) {
-        p.chol_blk = 1;
-        if (fse::state_smem(p) > 220 * 1024) p.chol_blk = 0;
-    }
-    p.smem_state = fse::state_smem(p);
-    p.smem_rhs = fse::rhs_smem(p);
-    p.smem_trsm = fse::trsm_smem(p);
-    const size_t lim = 220 * 1024;
-    if (b > FSE_MAX_BAND || p.smem_state > lim || p.smem_rhs > lim || p.smem_trsm > lim ||
-        (size_t)(nb + 9) * nb * sizeof(double) > lim) {
+    // numbering, matrices and plan.  What is accepted is decided in the caller's numbering, so that the
+    // documented size limits do not depend on the components.
+    std::vector<int> gpass, ginfo, grr;
+    Numbering num = own_numbering(n, b);
+    Matrices mat = build_matrices(m, num, b, et, ed);
+    RowGroups grp = plan_tangents(p, num, mat, gpass, ginfo, grr);
+    if (!plan_fits(p)) {
         free_ctx(c);
         return set_err(nullptr, FSE_EINVAL, "n or half-bandwidth too large for the on-chip working set");
     }
+    p.tc_ok = p.prec == FSE_MIXED_FP32 && b <= 96;
+    {
+        Numbering by_comp = component_numbering(n, pairs, comp);
+        if (by_comp.pan.nc > 1) {
+            Params q = p;
+            Matrices mc = build_matrices(m, by_comp, b, et, ed);
+            std::vector<int> gp, gi, gr;
+            RowGroups gc = plan_tangents(q, by_comp, mc, gp, gi, gr);
+            if (plan_fits(q)) {
+                p = q;
+                num = std::move(by_comp);
+                mat = std::move(mc);
+                grp = std::move(gc);
+                gpass.swap(gp);
+                ginfo.swap(gi);
+                grr.swap(gr);
+            }
+        }
+    }
+    const int ni = p.ni, nb = p.b + 1, fb = 2 * p.b + 1;
+    const std::vector<int>&cptr = mat.cptr, &ccol = mat.ccol, &kptr = mat.kptr, &kcol = mat.kcol, &ksoff = mat.ksoff,
+          &ksrc = mat.ksrc;
+    const std::vector<double>&cm = mat.cm, &cd = mat.cd, &ck = mat.ck, &Mb = mat.Mb;
+    for (int& x : ed)
+        if (x >= 0) x = num.row_of[x];
+    std::vector<double> Fi((size_t)m->e * ni, 0.0);
+    for (int k = 0; k < m->e; ++k)
+        for (int i = 0; i < n; ++i) Fi[(size_t)k * ni + num.row_of[i]] = m->F[(size_t)k * n + i];
+    std::vector<int> gslot(grp.col.size()), kslot(p.kt_ld, 0);
+    for (size_t q = 0; q < grp.col.size(); ++q) gslot[q] = grp.col[q] % p.RW;
+    for (size_t q = 0; q < kcol.size(); ++q) kslot[q] = kcol[q] % p.RW;
     // device allocations
-    const size_t Nn = (size_t)N * n, band = (size_t)fb * n, lb = (size_t)n * nb;
-    const size_t sensz = (size_t)N * n * p.ld * tsz;
+    const size_t Nn = (size_t)N * ni, band = (size_t)fb * ni, lb = (size_t)ni * nb;
+    const size_t sensz = (size_t)N * p.pan.tot * tsz;
     const size_t ktsz = (size_t)N * p.kt_ld * tsz;
     const size_t dsz = (size_t)N * p.nblk * FSE_BLK * FSE_BLK * tsz;
     cudaError_t e = cudaSuccess;
@@ -492,12 +673,14 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
         if (e == cudaSuccess) e = dalloc(ptr, bytes);
     };
     A(&c->d.Mb, band * 8);
-    A(&c->d.F, (size_t)m->e * n * 8);
+    A(&c->d.row_of, (size_t)n * 4);
+    A(&c->d.orig_of, (size_t)ni * 4);
+    A(&c->d.F, Fi.size() * 8);
     A(&c->d.el_type, (size_t)std::max(1, m->n_nl) * 4);
     A(&c->d.el_dof, (size_t)std::max(1, m->n_nl) * 24);
     A(&c->d.el_p, (size_t)std::max(1, m->n_nl) * 48);
     A(&c->d.col_off, (size_t)(ncol + 1) * 4);
-    A(&c->d.cs_ptr, (size_t)(n + 1) * 4);
+    A(&c->d.cs_ptr, (size_t)(ni + 1) * 4);
     A(&c->d.cs_col, (size_t)p.nnz * 4);
     A(&c->d.g_pass, gpass.size() * 4);
     A(&c->d.g_info, ginfo.size() * 4);
@@ -512,20 +695,20 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
     A(&c->d.cs_s, (size_t)p.nnz * 8);
     A(&c->d.cs_A, (size_t)p.nnz * tsz);
     A(&c->d.cs_B, (size_t)p.nnz * tsz);
-    A(&c->d.kt_ptr, (size_t)(n + 1) * 4);
+    A(&c->d.kt_ptr, (size_t)(ni + 1) * 4);
     // panel factor: K_t entries of the lower triangle grouped by column
-    std::vector<int> ktc_ptr(n + 1, 0), ktc_e, ktc_c, ktc_r;
+    std::vector<int> ktc_ptr(ni + 1, 0), ktc_e, ktc_c, ktc_r;
     if (p.chol_blk) {
-        for (int i = 0; i < n; ++i)
+        for (int i = 0; i < ni; ++i)
             for (int e = kptr[i]; e < kptr[i + 1]; ++e)
                 if (kcol[e] <= i) ++ktc_ptr[kcol[e] + 1];
-        for (int j = 0; j < n; ++j) ktc_ptr[j + 1] += ktc_ptr[j];
-        const int nl = ktc_ptr[n];
+        for (int j = 0; j < ni; ++j) ktc_ptr[j + 1] += ktc_ptr[j];
+        const int nl = ktc_ptr[ni];
         ktc_e.assign(std::max(1, nl), 0);
         ktc_c.assign(std::max(1, nl), 0);
         ktc_r.assign(std::max(1, nl), 0);
         std::vector<int> fill(ktc_ptr.begin(), ktc_ptr.end() - 1);
-        for (int i = 0; i < n; ++i)
+        for (int i = 0; i < ni; ++i)
             for (int e = kptr[i]; e < kptr[i + 1]; ++e) {
                 const int j = kcol[e];
                 if (j > i) continue;
@@ -534,8 +717,8 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
                 ktc_c[k] = j;
                 ktc_r[k] = i - j;
             }
-        A(&c->d.Sband, (size_t)n * nb * 4);
-        A(&c->d.ktc_ptr, (size_t)(n + 1) * 4);
+        A(&c->d.Sband, lb * 4);
+        A(&c->d.ktc_ptr, (size_t)(ni + 1) * 4);
         A(&c->d.ktc_e, ktc_e.size() * 4);
         A(&c->d.ktc_c, ktc_c.size() * 4);
         A(&c->d.ktc_r, ktc_r.size() * 4);
@@ -559,12 +742,12 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
     A(&c->d.ktab, c->ktab_host.size() * 4);
     A(&c->d.LMc, lb * 8);
     A(&c->d.LMr, lb * 8);
-    A(&c->d.LMinv, (size_t)n * 8);
+    A(&c->d.LMinv, (size_t)ni * 8);
     A(&c->d.q, Nn * 8);
     A(&c->d.u, Nn * 8);
     A(&c->d.a, Nn * 8);
-    A(&c->d.zb, Nn * 16);
-    A(&c->d.yb, Nn * 16);
+    A(&c->d.zb, (size_t)N * n * 16);
+    A(&c->d.yb, (size_t)N * n * 16);
     A(&c->d.Lc, FSE_NBUF_F * (size_t)N * lb * tsz);
     A(&c->d.Lr, FSE_NBUF_F * (size_t)N * lb * tsz);
     A(&c->d.Linv, FSE_NBUF_F * Nn * tsz);
@@ -573,7 +756,7 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
     A(&c->d.Rf, FSE_NBUF_F * rsz);
     A(&c->d.Rb, FSE_NBUF_F * rsz);
     if (p.tc_ok) {
-        const size_t tcsz = (size_t)2 * N * (p.nblk + 1) * 8 * FSE_BLK * FSE_BLK * 4;   // two step parities
+        const size_t tcsz = (size_t)2 * N * (p.nblk + p.pan.nc) * 8 * FSE_BLK * FSE_BLK * 4;   // two step parities
         A(&c->d.Tf, tcsz);
         A(&c->d.Tb, tcsz);
     }
@@ -597,7 +780,9 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
     }
     cudaStream_t st = c->stream;
     cudaMemcpyAsync(c->d.Mb, Mb.data(), band * 8, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.F, m->F, (size_t)m->e * n * 8, cudaMemcpyHostToDevice, st);
+    cudaMemcpyAsync(c->d.row_of, num.row_of.data(), (size_t)n * 4, cudaMemcpyHostToDevice, st);
+    cudaMemcpyAsync(c->d.orig_of, num.orig_of.data(), (size_t)ni * 4, cudaMemcpyHostToDevice, st);
+    cudaMemcpyAsync(c->d.F, Fi.data(), Fi.size() * 8, cudaMemcpyHostToDevice, st);
     if (m->n_nl > 0) {
         cudaMemcpyAsync(c->d.el_type, et.data(), et.size() * 4, cudaMemcpyHostToDevice, st);
         cudaMemcpyAsync(c->d.el_dof, ed.data(), ed.size() * 4, cudaMemcpyHostToDevice, st);
@@ -637,6 +822,10 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
     cudaMemsetAsync(c->d.iters, 0, (size_t)N * 4, st);
     cudaMemsetAsync(c->d.nref, 0, (size_t)N * 4, st);
     cudaMemsetAsync(c->d.flag, 0, 16, st);
+    if (ni > n) {   // the column factors leave the inert rows out: L = 1 there
+        cudaMemsetAsync(c->d.Lr, 0, FSE_NBUF_F * (size_t)N * lb * tsz, st);
+        fse::launch_fill_ones(c, c->d.Linv, FSE_NBUF_F * Nn);
+    }
     cudaMemsetAsync(c->d.Rf, 0, FSE_NBUF_F * rsz, st);   // entries outside the band stay zero
     cudaMemsetAsync(c->d.Rb, 0, FSE_NBUF_F * rsz, st);
     if (fse::make_tangent_maps(c) != FSE_OK) {
@@ -676,7 +865,7 @@ extern "C" int fse_sizes(const fse_ctx* c, int* nu, int* U, int* N, int* n, int*
     if (U) *U = c->p.U;
     if (N) *N = c->p.N;
     if (n) *n = c->p.n;
-    if (band) *band = c->p.b;
+    if (band) *band = c->p.b_user;
     return FSE_OK;
 }
 

@@ -20,8 +20,29 @@
 #define FSE_RHS_DEPTH_F32 3
 #define FSE_RHS_DEPTH_F64 2
 #define FSE_MAX_BAND 224  // half-bandwidth limit of the blocked solves
+#define FSE_MAX_PANELS 4  // tangent panels (decoupled groups of dofs), at most
 
 namespace fse {
+
+// Internal numbering and tangent panels.  Dofs that no entry of M, D, K and no element couples form
+// separate components (a flat shell's bending, membrane and drilling dofs, say): a start direction of
+// one component never moves another, so the tangents X, V are block diagonal.  Setup renumbers the
+// dofs component by component, each panel (one large component, or several small ones together)
+// starting at a multiple of FSE_BLK rows; the rows that fill a panel up are inert (M = K = 1, no
+// coupling, no load: their state stays zero).  The half-bandwidth is then the largest one inside a
+// component, and panel g stores only its own n_g rows x (2 n_g + 1) directions [d/dq | d/du | d/dw_1].
+// A model with one component keeps its numbering: one panel, row0 = 0, n = ni.
+struct Panels {
+    int nc = 1;                      // panels
+    int row0[FSE_MAX_PANELS] = {};   // first internal row
+    int n[FSE_MAX_PANELS] = {};      // rows (without the inert ones)
+    int b[FSE_MAX_PANELS] = {};      // half-bandwidth inside the panel
+    int ld[FSE_MAX_PANELS] = {};     // row stride: 2 n + 1 rounded up to a multiple of 4
+    int pass0[FSE_MAX_PANELS + 1] = {};   // first pass of the right-hand-side kernel; its row groups
+    int g1[FSE_MAX_PANELS] = {};          // are pass0 * FSE_RHS_GPS .. g1 - 1
+    size_t off[FSE_MAX_PANELS] = {}; // first element of the panel in a trajectory's tangents
+    size_t tot = 0;                  // elements of one trajectory's X (or V)
+};
 
 // Storage used by the kernels (b = half-bandwidth, detected at setup):
 //  * M, D, K, S and the sensitivity operators are CSR on the union of the
@@ -33,8 +54,10 @@ namespace fse {
 //  * factor of K_eff, per trajectory: column band Lc[j*(b+1) + (i-j)], row band
 //    Lr[i*(b+1) + (j-i+b)], 1/L_jj, and the inverses of the 32x32 diagonal
 //    blocks Dinv[B][r][c] (lower triangular, identity padding past n).
-//  * tangents of trajectory s: X[s][i][t], V[s][i][t], i < n, t < P = 2n+1
-//    (d/dz0 for t < 2n, d/dw_1 for t = 2n), consecutive t contiguous.
+//  * tangents of trajectory s, panel g: X[s * tot + off_g + i * ld_g + t], i < n_g, t < 2 n_g + 1
+//    (d/dz0 of the panel's own dofs for t < 2 n_g, d/dw_1 for t = 2 n_g); V alike.
+//  Vectors of N x 2n and 2nU values are in the caller's dof order; q, u, a, the matrices, the
+//  elements and the factors are in the internal numbering (ni rows).
 
 struct Dev {
     // model (FP64)
@@ -91,8 +114,11 @@ struct Dev {
     double* LMc = nullptr;
     double* LMr = nullptr;
     double* LMinv = nullptr;
+    // internal numbering: row_of[i] the internal row of dof i (n), orig_of[r] the dof of row r (ni, -1: inert)
+    int* row_of = nullptr;
+    int* orig_of = nullptr;
     // trajectory state (FP64)
-    double* q = nullptr;     // N x n
+    double* q = nullptr;     // N x ni
     double* u = nullptr;
     double* a = nullptr;
     double* zb = nullptr;    // N x 2n  (start / end points)
@@ -110,12 +136,12 @@ struct Dev {
     void* Rf = nullptr;
     void* Rb = nullptr;
     // factor records of the tensor-core solves (FP32 tangents, b <= 96), per direction two
-    // buffers (step parity) of N x (nblk + 1) x 8192 floats: record sigma + 1 holds the B operands
-    // (hi | lo, K-major) of the MMAs issued after block sigma (fse_tc.cu)
+    // buffers (step parity) of N x (nblk + panels) x 8192 floats: record sigma + 1 of a panel holds the
+    // B operands (hi | lo, K-major) of the MMAs issued after its block sigma (fse_tc.cu)
     void* Tf = nullptr;
     void* Tb = nullptr;
     // tangents (sensitivity precision)
-    void* X = nullptr;       // N x n x ld (columns P..ld-1 are zero padding)
+    void* X = nullptr;       // N x pan.tot (columns 2 n_g + 1 .. ld_g - 1 are zero padding)
     void* V = nullptr;
     void* Y = nullptr;       // right-hand side / forward-substitution buffer
     // vectors
@@ -132,13 +158,16 @@ struct Dev {
 };
 
 struct Params {
-    int n = 0, b = 0, d = 0, e = 0, N = 0, U = 0, L = 0, S1 = 0, P = 0;
+    int n = 0, d = 0, e = 0, N = 0, U = 0, L = 0, S1 = 0;
+    int ni = 0;              // internal rows (n, or with several panels n plus the inert rows)
+    int b = 0;               // half-bandwidth in the internal numbering (the largest of the panels)
+    int b_user = 0;          // half-bandwidth of the caller's numbering (fse_sizes, size limits)
+    Panels pan;
     // trajectory shard: this context integrates samples s0 .. s0 + N - 1 of an N_glob-sample grid;
     // its DFT sums are then partial and complete only after the reduction across shards
     int N_glob = 0, s0 = 0;
     bool shard = false;
     int maxit = 0, prec = 0, ncolors = 0, n_el = 0, nnz = 0, nnz_kt = 0, nblk = 0;
-    int ld = 0;              // row stride of the tangent arrays: P rounded up to a multiple of 4
     int RW = 0;              // ring rows of the right-hand-side kernel (two passes + 2b)
     int R = 1, ng = 0, nE = 0, ME = 0, RB = 16;   // row groups: rows per group, groups, entries,
                                                   // entries per pass (max), record bytes
@@ -154,13 +183,18 @@ struct Params {
     size_t smem_state = 0, smem_rhs = 0, smem_trsm = 0;
 };
 
+struct TangentMaps {
+    CUtensorMap m[2 * FSE_MAX_PANELS];
+};
+
 }  // namespace fse
 
 struct fse_ctx {
     fse::Params p;
     fse::Dev d;
-    CUtensorMap tmX{};   // TMA maps of the tangent arrays X, V ([N][n][ld], boxes of 32 rows x the
-    CUtensorMap tmV{};   // right-hand-side kernel's column tile); the type carries its own alignment
+    // TMA maps of panel g of X (2 g) and V (2 g + 1): [N][n_g][ld_g], boxes of 32 rows x the
+    // right-hand-side kernel's column tile; the type carries its own alignment
+    fse::TangentMaps tm{};
     int device = 0;
     cudaStream_t stream = nullptr;   // state path + everything ordered
     cudaStream_t stream2 = nullptr;  // sensitivity kernels (overlap with the next state step)
@@ -253,6 +287,7 @@ inline void mark_device(std::atomic<unsigned long long>& done) {
     done.fetch_or(1ull << (dev & 63));
 }
 void launch_fill_tables(fse_ctx* c);
+void launch_fill_ones(fse_ctx* c, void* p, size_t count);   // `count` ones in the tangent precision
 void launch_build_ops(fse_ctx* c, double omega1);
 void launch_build_groups(fse_ctx* c);
 int launch_factor_M(fse_ctx* c);

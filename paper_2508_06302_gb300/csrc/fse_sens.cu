@@ -15,14 +15,18 @@
 // Tangent rows have stride ld (a multiple of 4); columns P..ld-1 stay zero.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "fse_common.cuh"
 
 namespace fse {
 
 struct SensArgs {
-    int n, b, P, ld, kt_ld, nblk, RW, RWT;
-    int ng, ME, RB, MK, RECE;
+    int n, b, kt_ld, nblk, RW, RWT;   // n internal rows, b the largest half-bandwidth of the panels
+    int ME, RB, MK, RECE;
     double a2c;
+    Panels pan;
+    int tile0[FSE_MAX_PANELS + 1];    // first column tile of each panel (tile0[nc]: all tiles)
     const int* kt_slot;
     int* err;   // set when a pipeline wait gives up
     const void *g_rec, *g_rr, *g_info, *g_pass, *kt_val, *romega;
@@ -30,16 +34,17 @@ struct SensArgs {
     void *X, *V, *Y;
 };
 
-template <typename T>
-struct Vec2;
-template <>
-struct Vec2<float> {
-    using type = float2;
+// the tangent panel of a column tile: the kernels below work on one panel as a banded system of its own
+struct PanelTile {
+    int g, row0, n, b, ld, P, tile;
 };
-template <>
-struct Vec2<double> {
-    using type = double2;
-};
+__device__ __forceinline__ PanelTile panel_tile(const SensArgs& A, int x) {
+    int g = 0;
+#pragma unroll
+    for (int k = 1; k < FSE_MAX_PANELS; ++k)
+        if (k < A.pan.nc && x >= A.tile0[k]) g = k;
+    return {g, A.pan.row0[g], A.pan.n[g], A.pan.b[g], A.pan.ld[g], 2 * A.pan.n[g] + 1, x - A.tile0[g]};
+}
 
 // 4 consecutive elements, 16-byte (float) / 2 x 16-byte (double) aligned
 template <typename T>
@@ -129,15 +134,16 @@ __host__ __device__ constexpr int rhs_record_bytes() {
 // read from memory once per step; the consumers read nothing else from global memory.
 template <typename T, int R>
 __global__ void __launch_bounds__(32 * (FSE_RHS_GPS + 1), 1)
-    k_sens_rhs(SensArgs A, const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmV) {
+    k_sens_rhs(SensArgs A, const __grid_constant__ TangentMaps tm) {
     constexpr int CW = sizeof(T) == 4 ? 64 : 32;   // columns per CTA
     constexpr int EL = CW / 32;                     // columns per lane
     constexpr int GPS = FSE_RHS_GPS;
     constexpr int NB = (sizeof(T) == 4 ? FSE_RHS_DEPTH_F32 : FSE_RHS_DEPTH_F64) + 1;   // buffers in flight
     constexpr int RB = rhs_record_bytes<T, R>();
     constexpr int RW4 = RB / 4;                     // 32-bit words per record
-    const int n = A.n, P = A.P, ld = A.ld, RW = A.RW, ng = A.ng, ME = A.ME, MK = A.MK;
-    const int s = blockIdx.y, t0 = blockIdx.x * CW;
+    const PanelTile pt = panel_tile(A, blockIdx.x);
+    const int P = pt.P, ld = pt.ld, RW = A.RW, ng = A.pan.g1[pt.g], ME = A.ME, MK = A.MK;
+    const int s = blockIdx.y, t0 = pt.tile * CW;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     __shared__ __align__(8) unsigned long long bar_full[NB], bar_empty[NB];
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -148,9 +154,9 @@ __global__ void __launch_bounds__(32 * (FSE_RHS_GPS + 1), 1)
     T* rX = reinterpret_cast<T*>(sm128);            // RW x CW (RW a multiple of 32)
     T* rV = rX + (size_t)RW * CW;
     unsigned char* bufs = reinterpret_cast<unsigned char*>(rV + (size_t)RW * CW);
-    const size_t base = (size_t)s * n * ld;
-    T* Y = reinterpret_cast<T*>(A.Y) + base;
-    const int npass = (ng + GPS - 1) / GPS;
+    // internal row i of the panel: Y[i * ld]
+    T* Y = reinterpret_cast<T*>(A.Y) + (size_t)s * A.pan.tot + A.pan.off[pt.g] - (size_t)pt.row0 * ld;
+    const int p0 = A.pan.pass0[pt.g], npass = A.pan.pass0[pt.g + 1] - p0;
     if (threadIdx.x == 0) {
         for (int k = 0; k < NB; ++k) {
             mbar_init(&bar_full[k], 1);
@@ -164,7 +170,8 @@ __global__ void __launch_bounds__(32 * (FSE_RHS_GPS + 1), 1)
         const unsigned char* rec = reinterpret_cast<const unsigned char*>(A.g_rec);
         const int4* rr_g = reinterpret_cast<const int4*>(A.g_rr);
         const int2* gi_g = reinterpret_cast<const int2*>(A.g_info);
-        const int4* pd = reinterpret_cast<const int4*>(A.g_pass);
+        const int4* pd = reinterpret_cast<const int4*>(A.g_pass) + 2 * p0;
+        const CUtensorMap *tmX = &tm.m[2 * pt.g], *tmV = tmX + 1;
         const T* ktv = reinterpret_cast<const T*>(A.kt_val) + (size_t)s * A.kt_ld;
         constexpr unsigned chunkbytes = 32u * CW * (unsigned)sizeof(T);   // one TMA box: 32 rows
         int loadedc = 0, q = 0;                                            // 32-row chunks staged
@@ -187,8 +194,9 @@ __global__ void __launch_bounds__(32 * (FSE_RHS_GPS + 1), 1)
             if (lane == 0) mbar_arrive_tx(&bar_full[slot], 2u * nch * chunkbytes + mbytes + rbytes + ibytes + kbytes);
             __syncwarp();
             for (int k = lane; k < 2 * nch; k += 32) {
-                const int arr = k & 1, r0 = 32 * (loadedc + (k >> 1));
-                tma_load3((arr ? rV : rX) + (size_t)(r0 % RW) * CW, arr ? &tmV : &tmX, t0, r0, s, &bar_full[slot]);
+                const int arr = k & 1, r0 = 32 * (loadedc + (k >> 1));   // row inside the panel
+                tma_load3((arr ? rV : rX) + (size_t)((pt.row0 + r0) % RW) * CW, arr ? tmV : tmX, t0, r0, s,
+                          &bar_full[slot]);
             }
             if (lane == 0) {
                 unsigned char* b2 = buf;
@@ -215,7 +223,7 @@ __global__ void __launch_bounds__(32 * (FSE_RHS_GPS + 1), 1)
         return;
     }
     // ---- consumers (shared memory read through explicit 32-bit shared addresses)
-    const T* rom = reinterpret_cast<const T*>(A.romega) + (size_t)s * n;
+    const T* rom = reinterpret_cast<const T*>(A.romega) + (size_t)s * A.n;
     const bool wcol = t0 + CW > P - 1;   // this CTA holds the w_1 column
     const unsigned sX = smem_addr(rX) + EL * lane * (unsigned)sizeof(T);
     const unsigned sV = smem_addr(rV) + EL * lane * (unsigned)sizeof(T);
@@ -224,7 +232,7 @@ __global__ void __launch_bounds__(32 * (FSE_RHS_GPS + 1), 1)
     for (int pass = 0; pass < npass; ++pass) {
         const int slot = pass % NB;
         if (!mbar_wait(&bar_full[slot], (pass / NB) & 1, A.err)) break;
-        const int g = pass * GPS + warp;
+        const int g = (p0 + pass) * GPS + warp;
         if (g < ng) {
             const unsigned buf = sB + (unsigned)(slot * bufsz);
             const int2 gi = lds_i2(buf + oGI + warp * 8);
@@ -382,8 +390,9 @@ struct TileLoader {   // MAXL >= b * 32 / 256
 // backward, X and V) are fetched into registers while the current block computes.
 template <typename T, bool FWD, int MAXL>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_trsm(SensArgs A) {
-    const int n = A.n, b = A.b, ld = A.ld, nb = b + 1, RM = A.RWT - 1;
-    const int s = blockIdx.y, t0 = blockIdx.x * 128;
+    const PanelTile pt = panel_tile(A, blockIdx.x);
+    const int n = pt.n, b = A.b, ld = pt.ld, nb = b + 1, RM = A.RWT - 1;
+    const int s = blockIdx.y, t0 = pt.tile * 128;
     const int tr = threadIdx.x >> 5, tc = threadIdx.x & 31;   // rows 4tr.., cols 4tc..
     const int t = t0 + 4 * tc;
     const bool tok = t < ld;
@@ -396,14 +405,14 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_trsm(SensArgs A
     Dt[0] = Lt[0] + (size_t)bpad * 32;
     Lt[1] = Dt[0] + 1024;
     Dt[1] = Lt[1] + (size_t)bpad * 32;
-    const T* Lband = reinterpret_cast<const T*>(FWD ? A.Lr : A.Lc) + (size_t)s * n * nb;
-    const T* Dv = reinterpret_cast<const T*>(A.Dinv) + (size_t)s * A.nblk * FSE_BLK * FSE_BLK;
-    const size_t base = (size_t)s * n * ld;
+    const T* Lband = reinterpret_cast<const T*>(FWD ? A.Lr : A.Lc) + ((size_t)s * A.n + pt.row0) * nb;
+    const T* Dv = reinterpret_cast<const T*>(A.Dinv) + ((size_t)s * A.nblk + pt.row0 / FSE_BLK) * FSE_BLK * FSE_BLK;
+    const size_t base = (size_t)s * A.pan.tot + A.pan.off[pt.g];
     T* Y = reinterpret_cast<T*>(A.Y) + base;
     T* X = reinterpret_cast<T*>(A.X) + base;
     T* V = reinterpret_cast<T*>(A.V) + base;
     const T a2 = T(A.a2c);
-    const int nblk = A.nblk;
+    const int nblk = (n + FSE_BLK - 1) / FSE_BLK;
     auto blk = [&](int q) { return FWD ? q : nblk - 1 - q; };
     auto load_rows = [&](const T* src, int B, T out[4][4]) {
         const int i0 = B * FSE_BLK;
@@ -441,7 +450,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_trsm(SensArgs A
         __syncthreads();                                  // tiles of block q are in Lt/Dt[buf]
         const T* L = Lt[buf];
         if (FWD) {
-            for (int c = max(0, b - i0); c < b; ++c) {
+            for (int c = b - min(i0, pt.b); c < b; ++c) {   // the panel's own band and rows
                 T yv[4], lv[4];
                 ld4(ring + (size_t)((i0 - b + c) & RM) * 128 + 4 * tc, yv);
                 ld4(L + c * 32 + 4 * tr, lv);
@@ -451,7 +460,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_trsm(SensArgs A
                     for (int cc = 0; cc < 4; ++cc) acc[rr][cc] -= lv[rr] * yv[cc];
             }
         } else {
-            const int cend = min(b, n - (i0 + FSE_BLK));
+            const int cend = min(pt.b, n - (i0 + FSE_BLK));
             for (int c = 0; c < cend; ++c) {
                 T xv[4], lv[4];
                 ld4(ring + (size_t)((i0 + FSE_BLK + c) & RM) * 128 + 4 * tc, xv);
@@ -577,7 +586,9 @@ __global__ void __launch_bounds__(256, 1) k_trsm8(SensArgs A) {
     constexpr int EL = 16 / sizeof(T);             // columns per lane
     constexpr int CW = 64 * EL;                    // columns per CTA
     constexpr int RT = 8;                          // rows per thread
-    const int n = A.n, b = A.b, ld = A.ld, RM = A.RWT - 1, RECE = A.RECE, nblk = A.nblk;
+    const PanelTile pt = panel_tile(A, blockIdx.x);
+    const int n = pt.n, b = A.b, bp = pt.b, ld = pt.ld, RM = A.RWT - 1, RECE = A.RECE;
+    const int nblk = (n + FSE_BLK - 1) / FSE_BLK;
     const int s = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // Row group of a warp: the zeros of the band tile and of the diagonal-block inverse are
     // skipped, so the row groups do unequal work (FWD: b - 8 rg band columns and 8 + 8 rg
@@ -586,7 +597,7 @@ __global__ void __launch_bounds__(256, 1) k_trsm8(SensArgs A) {
     const int cg = warp >> 2, rg = cg ? 3 - (warp & 3) : (warp & 3);
     const int r0 = RT * rg;                        // first row of this thread in the block
     const int cl = cg * (CW / 2) + EL * lane;      // first column of this thread in the tile
-    const int t = blockIdx.x * CW + cl;            // global column
+    const int t = pt.tile * CW + cl;               // column of the panel
     const bool tok = t < ld;
     __shared__ __align__(8) unsigned long long bar[2];
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -598,8 +609,9 @@ __global__ void __launch_bounds__(256, 1) k_trsm8(SensArgs A) {
     constexpr unsigned TS = sizeof(T);
     const unsigned sRing = smem_addr(ring) + cl * TS, sStg = smem_addr(stg), sRec0 = smem_addr(rec0);
     const unsigned recb = (unsigned)RECE * TS;
-    const T* R = reinterpret_cast<const T*>(FWD ? A.Rf : A.Rb) + (size_t)s * nblk * RECE;
-    const size_t base = (size_t)s * n * ld;
+    const T* R = reinterpret_cast<const T*>(FWD ? A.Rf : A.Rb) +
+                 ((size_t)s * A.nblk + pt.row0 / FSE_BLK) * RECE;
+    const size_t base = (size_t)s * A.pan.tot + A.pan.off[pt.g];
     T* Y = reinterpret_cast<T*>(A.Y) + base;
     T* X = reinterpret_cast<T*>(A.X) + base;
     T* V = reinterpret_cast<T*>(A.V) + base;
@@ -660,11 +672,11 @@ __global__ void __launch_bounds__(256, 1) k_trsm8(SensArgs A) {
         const bool wok = mbar_wait(&bar[buf], (q >> 1) & 1, A.err);
         const unsigned sL = sRec0 + (buf ? recb : 0u) + r0 * TS;     // this thread's 8 rows of the record
         // band part: rows of earlier (FWD) or later (BWD) blocks from the ring.  Record column c
-        // is zero for row r when c < r (FWD: L(i0 + r, i0 - b + c) lies outside the band) or when
-        // c > b - 32 + r (BWD: L(i0 + 32 + c, i0 + r)), so this thread's rows r0 .. r0 + 7 need
-        // c >= r0 (FWD) or c < b - 24 + r0 (BWD) only.
-        const int c0 = FWD ? max(max(0, b - i0), r0) : 0;
-        const int c1 = FWD ? b : min(min(b, n - (i0 + FSE_BLK)), b - FSE_BLK + RT + r0);
+        // is zero for row r when c < b - bp + r (FWD: L(i0 + r, i0 - b + c) lies outside the panel's
+        // band bp <= b) or when c > bp - 32 + r (BWD: L(i0 + 32 + c, i0 + r)), so this thread's rows
+        // r0 .. r0 + 7 need c >= b - bp + r0 (FWD) or c < bp - 24 + r0 (BWD) only.
+        const int c0 = FWD ? max(b - i0, b - bp + r0) : 0;
+        const int c1 = FWD ? b : min(min(bp, n - (i0 + FSE_BLK)), bp - FSE_BLK + RT + r0);
         // the operands of column c + 1 are read from shared memory before the products of column c
         auto ldc = [&](int c, T xv[EL], T lv[RT]) {
             const int rowg = FWD ? (i0 - b + c) : (i0 + FSE_BLK + c);
@@ -806,16 +818,19 @@ __global__ void __launch_bounds__(256, 1) k_trsm8(SensArgs A) {
 // the new step enters through u' = 2/D (q' - q_k') - u_k').  C_t lives on the K_t pattern; one
 // thread per tangent column, rows without velocity-tangent entries are skipped.
 template <typename T>
-__global__ void k_ct_rhs(int n, int ld, int kt_ld, double wa2, double w, const int* __restrict__ kt_ptr,
-                         const int* __restrict__ kt_col, const T* __restrict__ c1, const T* __restrict__ c0,
-                         const T* __restrict__ X, const T* __restrict__ V, T* Y) {
-    const int s = blockIdx.y;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void k_ct_rhs(SensArgs A, double wa2, double w, const int* __restrict__ kt_ptr,
+                         const int* __restrict__ kt_col, const T* __restrict__ c1, const T* __restrict__ c0) {
+    const PanelTile pt = panel_tile(A, blockIdx.x);
+    const int s = blockIdx.y, ld = pt.ld;
+    const int t = pt.tile * blockDim.x + threadIdx.x;
     if (t >= ld) return;
-    const size_t base = (size_t)s * n * ld;
-    const T* C1 = c1 + (size_t)s * kt_ld;
-    const T* C0 = c0 + (size_t)s * kt_ld;
-    for (int i = 0; i < n; ++i) {
+    const T* X = reinterpret_cast<const T*>(A.X);
+    const T* V = reinterpret_cast<const T*>(A.V);
+    T* Y = reinterpret_cast<T*>(A.Y);
+    const size_t base = (size_t)s * A.pan.tot + A.pan.off[pt.g] - (size_t)pt.row0 * ld;   // internal row i at i * ld
+    const T* C1 = c1 + (size_t)s * A.kt_ld;
+    const T* C0 = c0 + (size_t)s * A.kt_ld;
+    for (int i = pt.row0; i < pt.row0 + pt.n; ++i) {
         const int e0 = kt_ptr[i], e1 = kt_ptr[i + 1];
         if (e0 == e1) continue;
         double acc = 0.0;
@@ -827,17 +842,23 @@ __global__ void k_ct_rhs(int n, int ld, int kt_ld, double wa2, double w, const i
     }
 }
 
-// X_0 = [I 0 0], V_0 = [0 I 0], zero padding columns
+// X_0 = [I 0 0], V_0 = [0 I 0] in every panel (blockIdx.z), zero padding columns; one row of one
+// trajectory per block and step of the grid, 16 bytes a thread
 template <typename T>
-__global__ void k_sens_init(int N, int n, int ld, T* X, T* V) {
-    const size_t total = (size_t)N * n * ld;
-    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const size_t r = idx / ld;
-        const int t = (int)(idx % ld), i = (int)(r % n);
-        X[idx] = (t == i) ? T(1) : T(0);
-        V[idx] = (t == i + n) ? T(1) : T(0);
-    }
+__global__ void k_sens_init(int N, Panels pan, T* X, T* V) {
+    const int g = blockIdx.z, n = pan.n[g], ld = pan.ld[g], s = blockIdx.y;
+    const size_t base = (size_t)s * pan.tot + pan.off[g];
+    for (int i = blockIdx.x; i < n; i += gridDim.x)
+        for (int t = 4 * threadIdx.x; t < ld; t += 4 * blockDim.x) {
+            T x[4], v[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                x[k] = (t + k == i) ? T(1) : T(0);
+                v[k] = (t + k == i + n) ? T(1) : T(0);
+            }
+            st4(X + base + (size_t)i * ld + t, x);
+            st4(V + base + (size_t)i * ld + t, v);
+        }
 }
 
 // ----------------------------------------------------------------------------
@@ -873,17 +894,19 @@ int make_tangent_maps(fse_ctx* c) {
     const bool f32 = p.prec == FSE_MIXED_FP32;
     const size_t tsz = f32 ? 4 : 8;
     const cuuint32_t cw = f32 ? 64 : 32;
-    const cuuint64_t dims[3] = {(cuuint64_t)p.ld, (cuuint64_t)p.n, (cuuint64_t)p.N};
-    const cuuint64_t strides[2] = {(cuuint64_t)p.ld * tsz, (cuuint64_t)p.n * p.ld * tsz};
     const cuuint32_t box[3] = {cw, 32, 1};
     const cuuint32_t es[3] = {1, 1, 1};
     const CUtensorMapDataType dt = f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64;
-    for (int k = 0; k < 2; ++k) {
-        CUtensorMap* m = k ? &c->tmV : &c->tmX;
-        void* ptr = k ? c->d.V : c->d.X;
-        if (encode(m, dt, 3, ptr, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return FSE_ECUDA;
+    for (int g = 0; g < p.pan.nc; ++g) {
+        const cuuint64_t dims[3] = {(cuuint64_t)p.pan.ld[g], (cuuint64_t)p.pan.n[g], (cuuint64_t)p.N};
+        const cuuint64_t strides[2] = {(cuuint64_t)p.pan.ld[g] * tsz, (cuuint64_t)p.pan.tot * tsz};
+        for (int k = 0; k < 2; ++k) {
+            void* ptr = (char*)(k ? c->d.V : c->d.X) + p.pan.off[g] * tsz;
+            if (encode(&c->tm.m[2 * g + k], dt, 3, ptr, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                       CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+                return FSE_ECUDA;
+        }
     }
     return FSE_OK;
 }
@@ -901,17 +924,23 @@ void launch_build_groups(fse_ctx* c) {
                                                          (unsigned char*)c->d.g_rec);
 }
 
+// column tiles of cw columns over all panels (A.tile0), trajectories
+static dim3 tile_grid(const Params& p, SensArgs& A, int cw) {
+    A.tile0[0] = 0;
+    for (int g = 0; g < p.pan.nc; ++g) A.tile0[g + 1] = A.tile0[g] + (2 * p.pan.n[g] + 1 + cw - 1) / cw;
+    return dim3(A.tile0[p.pan.nc], p.N);
+}
+
 template <typename T, int R>
-static void rhs_launch(fse_ctx* c, const SensArgs& A, cudaStream_t st) {
+static void rhs_launch(fse_ctx* c, SensArgs& A, cudaStream_t st) {
     static std::atomic<unsigned long long> attr{0};
     if (needs_device_setup(attr)) {
         cudaFuncSetAttribute(k_sens_rhs<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
         mark_device(attr);
     }
     const Params& p = c->p;
-    constexpr int CW = sizeof(T) == 4 ? 64 : 32;
-    dim3 g((p.P + CW - 1) / CW, p.N);
-    k_sens_rhs<T, R><<<g, 32 * (FSE_RHS_GPS + 1), p.smem_rhs, st>>>(A, c->tmX, c->tmV);
+    const dim3 g = tile_grid(p, A, sizeof(T) == 4 ? 64 : 32);
+    k_sens_rhs<T, R><<<g, 32 * (FSE_RHS_GPS + 1), p.smem_rhs, st>>>(A, c->tm);
 }
 
 size_t trsm_smem(const Params& p) {
@@ -924,7 +953,7 @@ size_t trsm_smem(const Params& p) {
 }
 
 template <typename T>
-static void sens_launch(fse_ctx* c, const SensArgs& A, int phase, cudaStream_t st) {
+static void sens_launch(fse_ctx* c, SensArgs& A, int phase, cudaStream_t st) {
     const Params& p = c->p;
     static std::atomic<unsigned long long> attr{0};
     if (needs_device_setup(attr)) {
@@ -946,8 +975,7 @@ static void sens_launch(fse_ctx* c, const SensArgs& A, int phase, cudaStream_t s
             cudaFuncSetAttribute(k_trsm8<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
             mark_device(attr8);
         }
-        constexpr int CW = 64 * (16 / (int)sizeof(T));
-        dim3 g((p.P + CW - 1) / CW, p.N);
+        const dim3 g = tile_grid(p, A, 64 * (16 / (int)sizeof(T)));
         if (phase == 1)
             k_trsm8<T, true><<<g, 256, p.smem_trsm, st>>>(A);
         else
@@ -955,7 +983,7 @@ static void sens_launch(fse_ctx* c, const SensArgs& A, int phase, cudaStream_t s
     } else {
         // 96 < b <= FSE_MAX_BAND (224): the factor tile of b x 32 values over 256 threads needs
         // MAXL = 28 registers per thread
-        dim3 g((p.P + 127) / 128, p.N);
+        const dim3 g = tile_grid(p, A, 128);
         if (phase == 1)
             k_trsm<T, true, 28><<<g, 256, p.smem_trsm, st>>>(A);
         else
@@ -965,13 +993,13 @@ static void sens_launch(fse_ctx* c, const SensArgs& A, int phase, cudaStream_t s
 
 void launch_sens_init(fse_ctx* c, cudaStream_t st) {
     const Params& p = c->p;
-    const size_t tot = (size_t)p.N * p.n * p.ld;
+    int rows = 0;
+    for (int g = 0; g < p.pan.nc; ++g) rows = std::max(rows, p.pan.n[g]);
+    const dim3 grid(std::min(rows, 128), p.N, p.pan.nc);
     if (p.prec == FSE_MIXED_FP32)
-        k_sens_init<float><<<nblocks(tot, 256, 64), 256, 0, st>>>(p.N, p.n, p.ld, (float*)c->d.X,
-                                                                       (float*)c->d.V);
+        k_sens_init<float><<<grid, 128, 0, st>>>(p.N, p.pan, (float*)c->d.X, (float*)c->d.V);
     else
-        k_sens_init<double><<<nblocks(tot, 256, 64), 256, 0, st>>>(p.N, p.n, p.ld, (double*)c->d.X,
-                                                                        (double*)c->d.V);
+        k_sens_init<double><<<grid, 128, 0, st>>>(p.N, p.pan, (double*)c->d.X, (double*)c->d.V);
 }
 
 void launch_sens_phase(fse_ctx* c, int k, double w, int phase, cudaStream_t st) {
@@ -979,10 +1007,9 @@ void launch_sens_phase(fse_ctx* c, int k, double w, int phase, cudaStream_t st) 
     const size_t tsz = p.prec == FSE_MIXED_FP32 ? 4 : 8;
     const double Dl = 2.0 * M_PI / p.S1;
     SensArgs A;
-    A.n = p.n;
+    A.n = p.ni;
     A.b = p.b;
-    A.P = p.P;
-    A.ld = p.ld;
+    A.pan = p.pan;
     A.kt_ld = p.kt_ld;
     A.MK = p.MK;
     A.nblk = p.nblk;
@@ -990,7 +1017,6 @@ void launch_sens_phase(fse_ctx* c, int k, double w, int phase, cudaStream_t st) 
     A.RWT = p.RWT;
     A.RECE = p.RECE;
     A.a2c = 2.0 / Dl;
-    A.ng = p.ng;
     A.ME = p.ME;
     A.RB = p.RB;
     A.g_rr = c->d.g_rr;
@@ -1000,8 +1026,8 @@ void launch_sens_phase(fse_ctx* c, int k, double w, int phase, cudaStream_t st) 
     A.kt_slot = c->d.kt_slot;
     A.err = c->d.flag;
     const size_t ktsz = (size_t)p.N * p.kt_ld * tsz;
-    const size_t fsz = (size_t)p.N * p.n * (p.b + 1) * tsz;
-    const size_t vsz = (size_t)p.N * p.n * tsz;
+    const size_t fsz = (size_t)p.N * p.ni * (p.b + 1) * tsz;
+    const size_t vsz = (size_t)p.N * p.ni * tsz;
     const size_t dsz = (size_t)p.N * p.nblk * FSE_BLK * FSE_BLK * tsz;
     const int f = k % 2;
     A.kt_val = (const char*)c->d.kt_val + (k % FSE_NBUF_KT) * ktsz;   // K_t(q_k)
@@ -1024,16 +1050,14 @@ void launch_sens_phase(fse_ctx* c, int k, double w, int phase, cudaStream_t st) 
         const size_t csz = (size_t)p.N * p.kt_ld * tsz;
         const void* c1 = (const char*)c->d.ct_val + ((k + 1) % FSE_NBUF_KT) * csz;
         const void* c0 = (const char*)c->d.ct_val + (k % FSE_NBUF_KT) * csz;
-        const dim3 g((p.ld + 127) / 128, p.N);
+        const dim3 g = tile_grid(p, A, 128);   // the padding columns of a panel stay in its last tile or are zero
         const double wa2 = w * 2.0 / Dl;
         if (p.prec == FSE_MIXED_FP32)
-            k_ct_rhs<float><<<g, 128, 0, st>>>(p.n, p.ld, p.kt_ld, wa2, w, c->d.kt_ptr, c->d.kt_col,
-                                               (const float*)c1, (const float*)c0, (const float*)c->d.X,
-                                               (const float*)c->d.V, (float*)c->d.Y);
+            k_ct_rhs<float><<<g, 128, 0, st>>>(A, wa2, w, c->d.kt_ptr, c->d.kt_col, (const float*)c1,
+                                               (const float*)c0);
         else
-            k_ct_rhs<double><<<g, 128, 0, st>>>(p.n, p.ld, p.kt_ld, wa2, w, c->d.kt_ptr, c->d.kt_col,
-                                                (const double*)c1, (const double*)c0, (const double*)c->d.X,
-                                                (const double*)c->d.V, (double*)c->d.Y);
+            k_ct_rhs<double><<<g, 128, 0, st>>>(A, wa2, w, c->d.kt_ptr, c->d.kt_col, (const double*)c1,
+                                                (const double*)c0);
         return;
     }
     if (phase > 0 && use_tc(c)) {

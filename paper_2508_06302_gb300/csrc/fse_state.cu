@@ -638,6 +638,7 @@ __host__ __device__ inline size_t state_wspan(int nb, int blk) {
 
 struct StateArgs {
     int n, b, e, dm1, maxit, ncolors, n_el, nnz_kt, kt_ld, nblk, init;
+    Panels pan;
     int refactor;       // 0: keep the previous factors (residual-only steps, see launch_state_step)
     double tol, Dl, a0c, a1c, a2c, w, phi;
     double rho[FSE_MAX_D - 1];
@@ -679,7 +680,15 @@ __device__ int band_factor(const StateArgs& A, T* Ac, T* Lr, T* Linv, T* Dinv, T
         const ChbSource src{A.Sband, A.ktc_ptr, A.ktc_e, A.ktc_c, A.ktc_r, kt, ct, float(A.w * A.a2c)};
         return cta_band_cholesky_blk(Ac, Lr, Linv, Dinv, A.n, A.b, wnd, Rf, Rb, A.RECE, A.full_factor != 0, src);
     }
-    const int bad = band_cholesky<T>(Ac, Lr, Linv, A.n, A.b, wnd, stg, Rf, Rb, A.RECE);
+    // column by column: one panel after the other, so that inert rows cost no barrier (their L stays
+    // the identity that setup wrote)
+    int bad = 0;
+    for (int g = 0; g < A.pan.nc && !bad; ++g) {
+        const int r0 = A.pan.row0[g];
+        const size_t o = (size_t)r0 * (A.b + 1), ro = (size_t)(r0 / FSE_BLK) * A.RECE;
+        bad = band_cholesky<T>(Ac + o, Lr + o, Linv + r0, A.pan.n[g], A.b, wnd, stg, Rf + ro, Rb + ro, A.RECE);
+        __syncthreads();   // every thread has read the pivot flag before the next panel clears it
+    }
     if (!bad) cta_diag_inverses<T>(Lr, Linv, A.n, A.b, A.nblk, Dinv, wnd, Rf, Rb, A.RECE);
     return bad;
 }
@@ -1242,6 +1251,19 @@ void launch_fill_tables(fse_ctx* c) {
                                          c->d.G, c->d.Gi, c->d.RG);
 }
 
+template <typename T>
+__global__ void k_fill_ones(size_t n, T* p) {
+    for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n; k += (size_t)gridDim.x * blockDim.x)
+        p[k] = T(1);
+}
+
+void launch_fill_ones(fse_ctx* c, void* p, size_t count) {
+    if (c->p.prec == FSE_MIXED_FP32)
+        k_fill_ones<float><<<nblocks(count, 256), 256, 0, c->stream>>>(count, (float*)p);
+    else
+        k_fill_ones<double><<<nblocks(count, 256), 256, 0, c->stream>>>(count, (double*)p);
+}
+
 void launch_build_ops(fse_ctx* c, double w) {
     const Params& p = c->p;
     const double Dl = 2.0 * M_PI / p.S1;
@@ -1255,8 +1277,8 @@ void launch_build_ops(fse_ctx* c, double w) {
                                                       c->d.cs_s, (double*)c->d.cs_A, (double*)c->d.cs_B);
     if (p.chol_blk) {
         const int nb = p.b + 1;
-        cudaMemsetAsync(c->d.Sband, 0, (size_t)p.n * nb * 4, c->stream);
-        k_sband<<<nblocks(p.n, 128), 128, 0, c->stream>>>(p.n, nb, c->d.cs_ptr, c->d.cs_col, c->d.cs_s,
+        cudaMemsetAsync(c->d.Sband, 0, (size_t)p.ni * nb * 4, c->stream);
+        k_sband<<<nblocks(p.ni, 128), 128, 0, c->stream>>>(p.ni, nb, c->d.cs_ptr, c->d.cs_col, c->d.cs_s,
                                                           (float*)c->d.Sband);
     }
 }
@@ -1269,7 +1291,7 @@ int launch_factor_M(fse_ctx* c) {
     cudaMemsetAsync(flag, 0, sizeof(int), c->stream);
     const size_t smem = (size_t)(nb + 1 + FSE_CHOL_PF) * nb * sizeof(double);
     cudaFuncSetAttribute(k_factor_M, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_factor_M<<<1, 256, smem, c->stream>>>(p.n, p.b, c->d.Mb, c->d.LMc, c->d.LMr, c->d.LMinv, flag);
+    k_factor_M<<<1, 256, smem, c->stream>>>(p.ni, p.b, c->d.Mb, c->d.LMc, c->d.LMr, c->d.LMinv, flag);
     int h = 0;
     cudaMemcpyAsync(&h, flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
     cudaStreamSynchronize(c->stream);
@@ -1280,15 +1302,16 @@ size_t state_smem(const Params& p) {
     const int nb = p.b + 1;
     const size_t tsz = p.prec == FSE_MIXED_FP32 ? 4 : 8;
     const size_t wspan = state_wspan(nb, tsz == 4 ? p.chol_blk : 0);
-    return (size_t)(6 * p.n + FSE_BLK) * 8 + (wspan + (size_t)p.n) * tsz + (p.has_vel ? (size_t)p.n * 8 + 8 : 0);
+    return (size_t)(6 * p.ni + FSE_BLK) * 8 + (wspan + (size_t)p.ni) * tsz + (p.has_vel ? (size_t)p.ni * 8 + 8 : 0);
 }
 
 static StateArgs make_state_args(fse_ctx* c, double w, int init, int k) {
     const Params& p = c->p;
     const size_t tsz = p.prec == FSE_MIXED_FP32 ? 4 : 8;
     StateArgs A;
-    A.n = p.n;
+    A.n = p.ni;
     A.b = p.b;
+    A.pan = p.pan;
     A.e = p.e;
     A.dm1 = p.d - 1;
     A.maxit = p.maxit;
@@ -1326,8 +1349,8 @@ static StateArgs make_state_args(fse_ctx* c, double w, int init, int k) {
     A.has_vel = p.has_vel ? 1 : 0;
     A.ce = c->d.ce;
     const size_t ktsz = (size_t)p.N * p.kt_ld * tsz;
-    const size_t fsz = (size_t)p.N * p.n * (p.b + 1) * tsz;
-    const size_t vsz = (size_t)p.N * p.n * tsz;
+    const size_t fsz = (size_t)p.N * p.ni * (p.b + 1) * tsz;
+    const size_t vsz = (size_t)p.N * p.ni * tsz;
     const size_t dsz = (size_t)p.N * p.nblk * FSE_BLK * FSE_BLK * tsz;
     // state k (new state q_{k+1}) writes K_t(q_{k+1}) to buffer (k+1) % 3 and the factor to k % 2;
     // the init call (k = -1) writes buffer 0 and factor 1
@@ -1391,21 +1414,24 @@ static void state_launch(fse_ctx* c, const StateArgs& A, cudaStream_t st) {
     state_launch_k<T, false>(c, A, st);
 }
 
-__global__ void k_split(int N, int n, const double* zb, double* q, double* u) {
-    const size_t total = (size_t)N * n;
+// start points (N x 2n, the caller's dof order) -> q, u in the internal numbering; inert rows zero
+__global__ void k_split(int N, int n, int ni, const int* __restrict__ orig_of, const double* __restrict__ zb,
+                        double* q, double* u) {
+    const size_t total = (size_t)N * ni;
     for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
          idx += (size_t)gridDim.x * blockDim.x) {
-        const size_t s = idx / n, i = idx % n;
-        q[idx] = zb[s * 2 * n + i];
-        u[idx] = zb[s * 2 * n + n + i];
+        const size_t s = idx / ni;
+        const int i = orig_of[idx % ni];
+        q[idx] = i >= 0 ? zb[s * 2 * n + i] : 0.0;
+        u[idx] = i >= 0 ? zb[s * 2 * n + n + i] : 0.0;
     }
 }
 
 void launch_init_state(fse_ctx* c, double w) {
     ensure_constants();
     const Params& p = c->p;
-    const size_t tot = (size_t)p.N * p.n;
-    k_split<<<nblocks(tot, 256), 256, 0, c->stream>>>(p.N, p.n, c->d.zb, c->d.q, c->d.u);
+    const size_t tot = (size_t)p.N * p.ni;
+    k_split<<<nblocks(tot, 256), 256, 0, c->stream>>>(p.N, p.n, p.ni, c->d.orig_of, c->d.zb, c->d.q, c->d.u);
     StateArgs A = make_state_args(c, w, 1, -1);
     A.refactor = 1;
     if (p.prec == FSE_MIXED_FP32)

@@ -181,17 +181,23 @@ __device__ __forceinline__ void tmem_stage8(unsigned taddr, const float v[TC_HR]
 }
 
 struct TcArgs {
-    int n, ld, nblk, ND;
+    int nblk, ND;       // blocks of all panels; blocks a block couples to
     float a2c;
     int* err;
-    const float* rec;   // N x (nblk + 1) records of this direction
+    const float* rec;   // N x (nblk + panels) records of this direction, nblk_g + 1 for each panel
     float *X, *V, *Y;
+    Panels pan;
+    int tile0[FSE_MAX_PANELS];   // first column tile of each panel
 };
 
 template <bool FWD>
 __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_solve(TcArgs A) {
-    const int n = A.n, ld = A.ld, nblk = A.nblk, ND = A.ND;
-    const int s = blockIdx.y, t0 = blockIdx.x * TC_M;
+    int g = 0;   // this tile's panel, solved as a banded system of its own
+#pragma unroll
+    for (int k = 1; k < FSE_MAX_PANELS; ++k)
+        if (k < A.pan.nc && (int)blockIdx.x >= A.tile0[k]) g = k;
+    const int n = A.pan.n[g], ld = A.pan.ld[g], nblk = (n + FSE_BLK - 1) / FSE_BLK, ND = A.ND;
+    const int s = blockIdx.y, t0 = ((int)blockIdx.x - A.tile0[g]) * TC_M;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     extern __shared__ __align__(128) unsigned char smraw[];
     // A operand of the last solved block [hi | lo], staged right-hand sides [2][hi | lo], records [3]
@@ -207,11 +213,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_solve(TcArgs A) {
         rhs_free, drain;
     __shared__ unsigned s_taddr;
     __shared__ volatile int s_abort;
-    const size_t base = (size_t)s * n * ld;
+    const size_t base = (size_t)s * A.pan.tot + A.pan.off[g];
     float* Y = A.Y + base;
     float* X = A.X + base;
     float* V = A.V + base;
-    const float* R = A.rec + (size_t)s * (nblk + 1) * TC_REC;
+    const float* R = A.rec + ((size_t)s * (A.nblk + A.pan.nc) + A.pan.row0[g] / FSE_BLK + g) * TC_REC;
     auto blk = [&](int q) { return FWD ? q : nblk - 1 - q; };
     // TMEM column of the right-hand-side A operand of block t (hi; lo 32 columns further)
     auto rhs_slot = [&](int t) { return TC_COL_RHS + (unsigned)(t & 1) * 64u; };
@@ -419,9 +425,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_solve(TcArgs A) {
                      : "memory");
 }
 
-// Factor records of both directions for the tensor-core solves, one CTA per (target block in
-// processing order tau, trajectory, direction).  Processing order: forward blocks 0, 1, ..;
-// backward blocks nblk-1, nblk-2, ...  Record sigma + 1 holds the B operands of round sigma: the
+// Factor records of both directions for the tensor-core solves, one CTA per (target block,
+// trajectory, direction).  Processing order in a panel: forward blocks 0, 1, ..; backward from the
+// last one.  Record sigma + 1 holds the B operands of round sigma: the
 // 96-row coupling operand [-C(sigma+1, sigma); -C(sigma+2, sigma); -C(sigma+3, sigma)] and
 // D'(sigma+3); record 0 holds [D'(0); D'(1); D'(2)] in its coupling operand.  Each operand as
 // hi | lo in the K-major layout (element (r, k) = B[r][k], r the row of the target block, k the
@@ -430,18 +436,21 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_solve(TcArgs A) {
 //   backward: C(t, s)[r][k] = sum_j Dinv_t[j][r] L(32 s + k, 32 t + j),     D'(t) = Dinv_t^T
 // (t, s block indices of the processing positions; the rows and columns past n are zero, the
 // diagonal-block inverse is the identity there).
-__global__ void __launch_bounds__(256) k_tc_records(int n, int b, int nblk, int ND, const float* __restrict__ Lr,
-                                                    const float* __restrict__ Dinv, float* __restrict__ recF,
-                                                    float* __restrict__ recB) {
-    const int tau = blockIdx.x, s = blockIdx.y;
+__global__ void __launch_bounds__(256) k_tc_records(int n, int b, int nblk, int ND, Panels pan,
+                                                    const float* __restrict__ Lr, const float* __restrict__ Dinv,
+                                                    float* __restrict__ recF, float* __restrict__ recB) {
+    const int Bt = blockIdx.x, s = blockIdx.y;   // target block; its panel g and position tau in it
     const bool fwd = blockIdx.z == 0;
     const int nb = b + 1;
-    const int Bt = fwd ? tau : nblk - 1 - tau;
+    int g = 0;
+    while (g + 1 < pan.nc && Bt * FSE_BLK >= pan.row0[g + 1]) ++g;
+    const int B0 = pan.row0[g] / FSE_BLK, nbg = (pan.n[g] + FSE_BLK - 1) / FSE_BLK;
+    const int tau = fwd ? Bt - B0 : B0 + nbg - 1 - Bt;
     __shared__ float Dv[32][33];
     __shared__ float Lt[32][33];
     const float* Lband = Lr + (size_t)s * n * nb;
     const float* Dt = Dinv + ((size_t)s * nblk + Bt) * TC_MAT;
-    float* rec = (fwd ? recF : recB) + (size_t)s * (nblk + 1) * TC_REC;
+    float* rec = (fwd ? recF : recB) + ((size_t)s * (nblk + pan.nc) + B0 + g) * TC_REC;
     for (int x = threadIdx.x; x < TC_MAT; x += blockDim.x) Dv[x >> 5][x & 31] = Dt[x];
     __syncthreads();
     auto L = [&](int i, int j) -> float {
@@ -490,18 +499,18 @@ __global__ void __launch_bounds__(256) k_tc_records(int n, int b, int nblk, int 
 // ----------------------------------------------------------------------------
 
 // floats of one record buffer (one direction, one step parity)
-static size_t tc_records_floats(const Params& p) { return (size_t)p.N * (p.nblk + 1) * TC_REC; }
+static size_t tc_records_floats(const Params& p) { return (size_t)p.N * (p.nblk + p.pan.nc) * TC_REC; }
 
 void launch_tc_records(fse_ctx* c, int k, cudaStream_t st) {
     const Params& p = c->p;
     const int f = k % 2;
-    const size_t fsz = (size_t)p.N * p.n * (p.b + 1) * 4;
+    const size_t fsz = (size_t)p.N * p.ni * (p.b + 1) * 4;
     const size_t dsz = (size_t)p.N * p.nblk * FSE_BLK * FSE_BLK * 4;
     const float* Lr = reinterpret_cast<const float*>((const char*)c->d.Lr + f * fsz);
     const float* Dv = reinterpret_cast<const float*>((const char*)c->d.Dinv + f * dsz);
     const size_t ro = (size_t)f * tc_records_floats(p);
-    k_tc_records<<<dim3(p.nblk, p.N, 2), 256, 0, st>>>(p.n, p.b, p.nblk, p.ND, Lr, Dv, (float*)c->d.Tf + ro,
-                                                        (float*)c->d.Tb + ro);
+    k_tc_records<<<dim3(p.nblk, p.N, 2), 256, 0, st>>>(p.ni, p.b, p.nblk, p.ND, p.pan, Lr, Dv,
+                                                        (float*)c->d.Tf + ro, (float*)c->d.Tb + ro);
 }
 
 void launch_tc_solve(fse_ctx* c, int k, int phase, cudaStream_t st) {
@@ -513,16 +522,20 @@ void launch_tc_solve(fse_ctx* c, int k, int phase, cudaStream_t st) {
         mark_device(attr);
     }
     TcArgs A;
-    A.n = p.n;
-    A.ld = p.ld;
     A.nblk = p.nblk;
     A.ND = p.ND;
+    A.pan = p.pan;
     A.a2c = (float)(2.0 / (2.0 * M_PI / p.S1));
     A.err = c->d.flag;
     A.X = (float*)c->d.X;
     A.V = (float*)c->d.V;
     A.Y = (float*)c->d.Y;
-    dim3 g((p.ld + TC_M - 1) / TC_M, p.N);
+    int tiles = 0;
+    for (int k = 0; k < p.pan.nc; ++k) {
+        A.tile0[k] = tiles;
+        tiles += (p.pan.ld[k] + TC_M - 1) / TC_M;
+    }
+    const dim3 g(tiles, p.N);
     const size_t ro = (size_t)(k % 2) * tc_records_floats(p);
     if (phase == 1) {
         A.rec = (const float*)c->d.Tf + ro;
