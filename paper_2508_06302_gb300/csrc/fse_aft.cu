@@ -2,7 +2,10 @@
 // outer Newton solve and the Lyapunov exponents (App. F).
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <atomic>
 #include <cmath>
+#include <cstdint>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -38,38 +41,135 @@ __global__ void k_join(int N, int n, int ni, const int* __restrict__ row_of, con
     }
 }
 
-// out[i*U + c] = sum_s RG[c][s] zb[s][i] - (subtract ? Z0[i*U + c] : 0); one warp per output
-__global__ void k_dft_res(int N, int U, int n2, const double* __restrict__ RG,
-                          const double* __restrict__ zb, const double* __restrict__ Z0, double* out,
-                          int subtract) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    const int total = n2 * U;
-    if (warp >= total) return;
-    const int i = warp / U, c = warp % U;
-    double acc = 0.0;
-    for (int s = lane; s < N; s += 32) acc += RG[(size_t)c * N + s] * zb[(size_t)s * n2 + i];
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) out[warp] = acc - (subtract ? Z0[warp] : 0.0);
+// out[i*U + c] = sum_s RG[c][s] zb[s][i] - (subtract ? Z0[i*U + c] : 0): a thread takes one state i and
+// DFT_C coefficients, so that zb is read along i (coalesced, from L2 after the first coefficients) and RG
+// comes as broadcasts from shared memory, staged DFT_S samples at a time.  FP64 FMAs bound it (N U 2n:
+// 15 M for the 1872-dof shell, 24 us); one warp per output with the lanes over the samples read zb with a
+// stride of 2n.  Few coefficients a thread: the FP64 pipes of an SM's four partitions are only busy with
+// three or more warps on each (243-dof plate, 256 samples x 225 coefficients: 117 us with 116 blocks of
+// 128 x 8).  1872-dof shell 117 -> 33 us, plate 90 -> 66 us.
+constexpr int DFT_C = 2, DFT_S = 64, DFT_T = 128;
+__global__ void __launch_bounds__(DFT_T) k_dft_res(int N, int U, int n2, const double* __restrict__ RG,
+                                                   const double* __restrict__ zb, const double* __restrict__ Z0,
+                                                   double* out, int subtract) {
+    __shared__ double rg[DFT_S][DFT_C];
+    const int i = blockIdx.x * DFT_T + threadIdx.x, c0 = blockIdx.y * DFT_C;
+    double acc[DFT_C];
+#pragma unroll
+    for (int k = 0; k < DFT_C; ++k) acc[k] = 0.0;
+    for (int s0 = 0; s0 < N; s0 += DFT_S) {
+        const int ns = min(DFT_S, N - s0);
+        __syncthreads();
+        for (int x = threadIdx.x; x < ns * DFT_C; x += DFT_T) {
+            const int k = x / ns, s = x - k * ns;
+            rg[s][k] = c0 + k < U ? RG[(size_t)(c0 + k) * N + s0 + s] : 0.0;
+        }
+        __syncthreads();
+        if (i < n2) {
+#pragma unroll 8
+            for (int s = 0; s < ns; ++s) {
+                const double z = zb[(size_t)(s0 + s) * n2 + i];
+#pragma unroll
+                for (int k = 0; k < DFT_C; ++k) acc[k] += rg[s][k] * z;
+            }
+        }
+    }
+    if (i >= n2) return;
+    const size_t o = (size_t)i * U + c0;
+#pragma unroll
+    for (int k = 0; k < DFT_C; ++k)
+        if (c0 + k < U) out[o + k] = acc[k] - (subtract ? Z0[o + k] : 0.0);
 }
 
 // ----------------------------------------------------------------------------
 // Jacobian products (Eq. 22, 23) from the stored tangents
 // ----------------------------------------------------------------------------
 
-// zout[s][i] = sum_{j < 2n} Phi_s[i][j] zin[s][j]; one warp per (s, i)
+// 4 values as FP64.  FP32 -> FP64 conversions run at the FP64 rate (GB300: 2 a clock and SM), as dear as
+// the multiply-add that follows; moving the bits with integer instructions is exact for normal values,
+// and the conversion is kept for a vector that holds a zero, a subnormal, an infinity or a NaN.
+__device__ __forceinline__ double widen(unsigned b) {
+    return __hiloint2double((((int)b >> 3) & 0x8fffffff) + 0x38000000, (int)(b << 29));
+}
+__device__ __forceinline__ void ld4_fp64(const float* p, double v[4]) {
+    const float4 f = *reinterpret_cast<const float4*>(p);
+    const unsigned b[4] = {__float_as_uint(f.x), __float_as_uint(f.y), __float_as_uint(f.z), __float_as_uint(f.w)};
+    bool normal = true;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) normal = normal && ((b[k] + 0x00800000u) & 0x7fffffffu) > 0x00ffffffu;
+    if (normal) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = widen(b[k]);
+    } else {
+        v[0] = f.x;
+        v[1] = f.y;
+        v[2] = f.z;
+        v[3] = f.w;
+    }
+}
+__device__ __forceinline__ void ld4_fp64(const double* p, double v[4]) {
+    const double2 x = *reinterpret_cast<const double2*>(p), y = *reinterpret_cast<const double2*>(p + 2);
+    v[0] = x.x;
+    v[1] = x.y;
+    v[2] = y.x;
+    v[3] = y.y;
+}
+
+// zout[s][i] = sum_{j < 2n} Phi_s[i][j] zin[s][j].  A CTA takes PHI_ROWS rows of one panel of one
+// trajectory: the panel's part of zin goes to shared memory in the panel's column order, a warp takes the
+// X and V rows of two dofs (four dot products share each z).  Bound by the FP64 FMAs (FP32 tangents;
+// 349 M for the 1872-dof shell's 64 trajectories = 0.55 ms) or by reading the tangents.  A warp per row
+// with converting loads and z from global memory: 1.28 ms there, now 0.75 ms; 243-dof plate 485 -> 171 us.
+constexpr int PHI_ROWS = 16;
 template <typename T>
-__global__ void k_phi_apply(int N, PhiView<T> F, const double* zin, double* zout) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    const int n2 = 2 * F.n;
-    if (warp >= N * n2) return;
-    const int s = warp / n2, i = warp % n2;
-    int g;
-    const T* row = F.row(s, i, g);
-    const double* z = zin + (size_t)s * n2;
-    double acc = 0.0;
-    for (int j = lane; j < 2 * F.pan.n[g]; j += 32) acc += (double)row[j] * z[F.col(g, j)];
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) zout[warp] = acc;
+__global__ void __launch_bounds__(256) k_phi_apply(PhiView<T> F, const double* __restrict__ zin, double* zout) {
+    extern __shared__ double zs[];
+    int x = blockIdx.x, g = 0;
+    while (x >= (F.pan.n[g] + PHI_ROWS - 1) / PHI_ROWS) x -= (F.pan.n[g++] + PHI_ROWS - 1) / PHI_ROWS;
+    const int s = blockIdx.y, n = F.n, m = F.pan.n[g], ld = F.pan.ld[g], row0 = F.pan.row0[g];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const double* z = zin + (size_t)s * 2 * n;
+    for (int k = threadIdx.x; k < m; k += 256) {
+        const int j = F.orig_of[row0 + k];
+        zs[k] = z[j];
+        zs[m + k] = z[n + j];
+    }
+    __syncthreads();
+    const int ra = x * PHI_ROWS + 2 * warp, rb = ra + 1;
+    if (ra >= m) return;
+    const size_t base = (size_t)s * F.pan.tot + F.pan.off[g];
+    const size_t oa = base + (size_t)ra * ld, ob = rb < m ? oa + ld : oa;
+    const T* rows[4] = {F.X + oa, F.V + oa, F.X + ob, F.V + ob};
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    const int m4 = (2 * m) & ~3;
+    for (int j = 4 * lane; j < m4; j += 128) {
+        double zv[4], v[4][4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) ld4_fp64(rows[q] + j, v[q]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) zv[k] = zs[j + k];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) acc[q] += v[q][k] * zv[k];
+    }
+    for (int j = m4 + lane; j < 2 * m; j += 32)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q] += (double)rows[q][j] * zs[j];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+    if (lane == 0) {
+        double* o = zout + (size_t)s * 2 * n;
+        const int ia = F.orig_of[row0 + ra];
+        o[ia] = acc[0];
+        o[n + ia] = acc[1];
+        if (rb < m) {
+            const int ib = F.orig_of[row0 + rb];
+            o[ib] = acc[2];
+            o[n + ib] = acc[3];
+        }
+    }
 }
 
 template <typename T>
@@ -400,9 +500,8 @@ void launch_collect_end(fse_ctx* c) {
 
 void launch_dft_residual(fse_ctx* c, const double* zb, const double* Z0, double* R, int subtract) {
     const Params& p = c->p;
-    const size_t warps = (size_t)2 * p.n * p.U;
-    k_dft_res<<<(int)((warps * 32 + 255) / 256), 256, 0, c->stream>>>(p.N, p.U, 2 * p.n, c->d.RG, zb,
-                                                                      Z0, R, subtract);
+    const dim3 g((2 * p.n + DFT_T - 1) / DFT_T, (p.U + DFT_C - 1) / DFT_C);
+    k_dft_res<<<g, DFT_T, 0, c->stream>>>(p.N, p.U, 2 * p.n, c->d.RG, zb, Z0, R, subtract);
 }
 
 template <typename T>
@@ -410,14 +509,27 @@ static PhiView<T> phi_view(const fse_ctx* c) {
     return {(const T*)c->d.X, (const T*)c->d.V, c->d.row_of, c->d.orig_of, c->p.n, c->p.pan};
 }
 
-void launch_phi_apply(fse_ctx* c, const double* zin, double* zout) {
+template <typename T>
+static void phi_apply(fse_ctx* c, const double* zin, double* zout) {
+    static std::atomic<unsigned long long> attr{0};
+    if (needs_device_setup(attr)) {
+        cudaFuncSetAttribute(k_phi_apply<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+        mark_device(attr);
+    }
     const Params& p = c->p;
-    const size_t warps = (size_t)p.N * 2 * p.n;
-    const int g = (int)((warps * 32 + 255) / 256);
-    if (p.prec == FSE_MIXED_FP32)
-        k_phi_apply<float><<<g, 256, 0, c->stream>>>(p.N, phi_view<float>(c), zin, zout);
+    int tiles = 0, most = 0;
+    for (int g = 0; g < p.pan.nc; ++g) {
+        tiles += (p.pan.n[g] + PHI_ROWS - 1) / PHI_ROWS;
+        most = std::max(most, p.pan.n[g]);
+    }
+    k_phi_apply<T><<<dim3(tiles, p.N), 256, (size_t)2 * most * 8, c->stream>>>(phi_view<T>(c), zin, zout);
+}
+
+void launch_phi_apply(fse_ctx* c, const double* zin, double* zout) {
+    if (c->p.prec == FSE_MIXED_FP32)
+        phi_apply<float>(c, zin, zout);
     else
-        k_phi_apply<double><<<g, 256, 0, c->stream>>>(p.N, phi_view<double>(c), zin, zout);
+        phi_apply<double>(c, zin, zout);
 }
 
 void launch_domega(fse_ctx* c, double* zout) {
@@ -679,28 +791,45 @@ __global__ void k_axpby(size_t n, double a, const double* x, double b, double* y
         y[k] = a * x[k] + b * y[k];
 }
 
-// out[0] = sum x^2, out[1] = sum y^2 (y may be null); one block
-__global__ void k_norms2(size_t n, const double* x, const double* y, double* out) {
-    __shared__ double ra[1024], rb[1024];
-    double a = 0.0, b = 0.0;
-    for (size_t k = threadIdx.x; k < n; k += blockDim.x) {
-        a += x[k] * x[k];
-        if (y) b += y[k] * y[k];
-    }
-    ra[threadIdx.x] = a;
-    rb[threadIdx.x] = b;
+// out[i] = a_i . b_i for i < gridDim.y, a_i = a + i sa, b_i = b + i sb.  gridDim.x blocks share a dot
+// product; the last one to finish adds the partial sums in block order, so the result does not depend on
+// which that is.  part: gridDim.y x gridDim.x doubles, count: gridDim.y counters, zero before and after.
+__global__ void __launch_bounds__(256) k_dots(size_t n, const double* a, ptrdiff_t sa, const double* b, ptrdiff_t sb,
+                                              double* part, unsigned* count, double* out) {
+    __shared__ double red[8];
+    __shared__ bool last;
+    const int i = blockIdx.y, nb = gridDim.x;
+    const double *x = a + (ptrdiff_t)i * sa, *y = b + (ptrdiff_t)i * sb;
+    const size_t per = (n + nb - 1) / nb, k0 = blockIdx.x * per, k1 = min(n, k0 + per);
+    double acc = 0.0;
+#pragma unroll 4
+    for (size_t k = k0 + threadIdx.x; k < k1; k += 256) acc += x[k] * y[k];
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
-            ra[threadIdx.x] += ra[threadIdx.x + o];
-            rb[threadIdx.x] += rb[threadIdx.x + o];
-        }
-        __syncthreads();
-    }
     if (threadIdx.x == 0) {
-        out[0] = ra[0];
-        out[1] = rb[0];
+        double t = 0.0;
+        for (int w = 0; w < 8; ++w) t += red[w];
+        part[(size_t)i * nb + blockIdx.x] = t;
+        __threadfence();
+        last = atomicInc(&count[i], nb - 1) == (unsigned)nb - 1;
     }
+    __syncthreads();
+    if (last && threadIdx.x == 0) {
+        __threadfence();
+        double t = 0.0;
+        for (int k = 0; k < nb; ++k) t += __ldcg(part + (size_t)i * nb + k);
+        out[i] = t;
+    }
+}
+
+// x *= 1 / sqrt(norm2[0]) (left alone where that is not positive)
+__global__ void k_normalise(size_t n, const double* norm2, double* x) {
+    const double s = *norm2;
+    if (!(s > 0.0)) return;
+    const double f = 1.0 / sqrt(s);
+    for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n; k += (size_t)gridDim.x * blockDim.x)
+        x[k] *= f;
 }
 
 // z = mean + sum_k c_k basis[k]  (basis r x nu)
@@ -730,38 +859,41 @@ __global__ void k_pod_project(size_t nu, int r, const double* mean, const double
     if (threadIdx.x == 0) coef[(size_t)j * r + k] = red[0];
 }
 
-// out[i] = V_i . w, one block per Krylov vector
-__global__ void k_mdot(size_t n, const double* __restrict__ V, const double* __restrict__ w, double* out) {
-    const int i = blockIdx.x;
-    __shared__ double red[512];
-    double acc = 0.0;
-    const double* v = V + (size_t)i * n;
-    for (size_t x = threadIdx.x; x < n; x += blockDim.x) acc += v[x] * w[x];
-    red[threadIdx.x] = acc;
+// w += sign sum_{i<k} coef[i] V_i
+__global__ void __launch_bounds__(128) k_mupdate(size_t n, int k, const double* __restrict__ V,
+                                                 const double* __restrict__ coef, double sign, double* w) {
+    __shared__ double cs[257];   // k <= restart + 1
+    for (int i = threadIdx.x; i < k; i += 128) cs[i] = sign * coef[i];
     __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[i] = red[0];
-}
-
-// w += sum_{i<k} coef[i] V_i
-__global__ void k_mupdate(size_t n, int k, const double* __restrict__ V, const double* __restrict__ coef,
-                          double* w) {
-    for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < n; x += (size_t)gridDim.x * blockDim.x) {
+    for (size_t x = blockIdx.x * (size_t)128 + threadIdx.x; x < n; x += (size_t)gridDim.x * 128) {
         double acc = w[x];
-        for (int i = 0; i < k; ++i) acc += coef[i] * V[(size_t)i * n + x];
+#pragma unroll 8
+        for (int i = 0; i < k; ++i) acc += cs[i] * V[(size_t)i * n + x];
         w[x] = acc;
     }
 }
 
-void vec_mdot(fse_ctx* c, size_t n, int k, const double* V, const double* w, double* out_dev) {
-    k_mdot<<<k, 512, 0, c->stream>>>(n, V, w, out_dev);
+// One block per dot product left the GPU idle (31 us for 40 products of 26640 values, 2 us of reading):
+// blocks of about 4096 values, at most FSE_DOT_BLOCKS a product (10 us, launches and caches cold).
+static void dots(fse_ctx* c, size_t n, int k, const double* a, ptrdiff_t sa, const double* b, ptrdiff_t sb,
+                 double* out_dev) {
+    const int nb = (int)std::min<size_t>(FSE_DOT_BLOCKS, (n + 4095) / 4096);
+    for (int i = 0; i < k; i += FSE_DOT_VECS) {   // the partial sums hold FSE_DOT_VECS products at a time
+        const int m = std::min(FSE_DOT_VECS, k - i);
+        k_dots<<<dim3(nb, m), 256, 0, c->stream>>>(n, a + i * sa, sa, b + i * sb, sb, c->d.red, c->d.redc, out_dev + i);
+    }
 }
 
-void vec_mupdate(fse_ctx* c, size_t n, int k, const double* V, const double* coef_dev, double* w) {
-    k_mupdate<<<nblocks(n, 256), 256, 0, c->stream>>>(n, k, V, coef_dev, w);
+void vec_mdot(fse_ctx* c, size_t n, int k, const double* V, const double* w, double* out_dev) {
+    dots(c, n, k, V, (ptrdiff_t)n, w, 0, out_dev);
+}
+
+void vec_mupdate(fse_ctx* c, size_t n, int k, const double* V, const double* coef_dev, double sign, double* w) {
+    k_mupdate<<<nblocks(n, 128), 128, 0, c->stream>>>(n, k, V, coef_dev, sign, w);
+}
+
+void vec_normalise(fse_ctx* c, size_t n, const double* norm2_dev, double* x) {
+    k_normalise<<<nblocks(n, 256), 256, 0, c->stream>>>(n, norm2_dev, x);
 }
 
 void vec_axpby(fse_ctx* c, size_t n, double a, const double* x, double b, double* y) {
@@ -769,7 +901,9 @@ void vec_axpby(fse_ctx* c, size_t n, double a, const double* x, double b, double
 }
 
 void vec_norms2(fse_ctx* c, size_t n, const double* x, const double* y, double* out_dev) {
-    k_norms2<<<1, 1024, 0, c->stream>>>(n, x, y, out_dev);
+    if (!y) cudaMemsetAsync(out_dev + 1, 0, 8, c->stream);
+    const ptrdiff_t d = y ? ((intptr_t)y - (intptr_t)x) / 8 : 0;
+    dots(c, n, y ? 2 : 1, x, d, x, d, out_dev);
 }
 
 void pod_expand(fse_ctx* c, size_t nu, int r, const double* mean, const double* basis, const double* coef,

@@ -422,7 +422,7 @@ static void free_ctx(fse_ctx* c) {
                     c->d.ktab, c->d.LMc, c->d.LMr, c->d.LMinv, c->d.q, c->d.u, c->d.a, c->d.zb,
                     c->d.Lc, c->d.Lr, c->d.Linv, c->d.Dinv, c->d.Rf, c->d.Rb, c->d.Tf, c->d.Tb, c->d.X, c->d.V, c->d.Y, c->d.Z0, c->d.R,
                     c->d.vec, c->d.vec2, c->d.yb, c->d.status, c->d.iters, c->d.nref, c->d.flag, c->Jd, c->piv, c->kry, c->kdot,
-                    c->ht, c->unk, c->d.row_of, c->d.orig_of, c->d.Sband, c->d.ktc_ptr, c->d.ktc_e, c->d.ktc_c, c->d.ktc_r};
+                    c->ht, c->unk, c->d.row_of, c->d.orig_of, c->d.ap, c->d.red, c->d.redc, c->d.Sband, c->d.ktc_ptr, c->d.ktc_e, c->d.ktc_c, c->d.ktc_r};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (auto& e : c->ev)
@@ -768,6 +768,9 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
     A(&c->d.R, nu * 8);
     A(&c->d.vec, nu * 8);
     A(&c->d.vec2, nu * 8);
+    A(&c->d.ap, 2 * nu * 8);
+    A(&c->d.red, FSE_DOT_VECS * FSE_DOT_BLOCKS * 8);
+    A(&c->d.redc, FSE_DOT_VECS * 4);
     A(&c->d.status, (size_t)N * 4);
     A(&c->d.iters, (size_t)N * 4);
     A(&c->d.nref, (size_t)N * 4);
@@ -819,6 +822,7 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
     cudaMemcpyAsync(c->d.rs, rsv.data(), rsv.size() * 8, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(c->d.ktab, c->ktab_host.data(), c->ktab_host.size() * 4, cudaMemcpyHostToDevice, st);
     cudaMemsetAsync(c->d.status, 0, (size_t)N * 4, st);
+    cudaMemsetAsync(c->d.redc, 0, FSE_DOT_VECS * 4, st);
     cudaMemsetAsync(c->d.iters, 0, (size_t)N * 4, st);
     cudaMemsetAsync(c->d.nref, 0, (size_t)N * 4, st);
     cudaMemsetAsync(c->d.flag, 0, 16, st);
@@ -1066,15 +1070,42 @@ extern "C" int fse_jacobian_apply(fse_ctx* c, const double* v, double* Jv, int n
     if (!c->have_jac) return set_err(c, FSE_ENOJAC, "no Jacobian stored: call fse_residual_jacobian with want_jacobian=1");
     cudaSetDevice(c->device);
     const size_t nu = (size_t)2 * c->p.n * c->p.U;
-    for (int k = 0; k < nvec; ++k) {
-        cudaMemcpyAsync(c->d.vec, v + k * nu, nu * 8, cudaMemcpyHostToDevice, c->stream);
-        fse::launch_idft(c, c->d.vec, c->d.zb);
-        fse::launch_phi_apply(c, c->d.zb, c->d.yb);
-        const int rc = dft_sub(c, c->d.yb, c->d.vec, c->d.vec2);
-        if (rc) return rc;
-        cudaMemcpyAsync(Jv + k * nu, c->d.vec2, nu * 8, cudaMemcpyDeviceToHost, c->stream);
+    // Large vectors: the copies of one overlap the kernels of the next; they alternate between two input
+    // and output pairs (d.vec / d.vec2 and d.ap), results leave on the second stream.  Below 256 KB the
+    // copies take less than the events between the streams (36 dofs, 15 coefficients: 13 us more a call).
+    if (nvec < 2 || nu * 8 < (256u << 10)) {
+        for (int k = 0; k < nvec; ++k) {
+            cudaMemcpyAsync(c->d.vec, v + k * nu, nu * 8, cudaMemcpyHostToDevice, c->stream);
+            fse::launch_idft(c, c->d.vec, c->d.zb);
+            fse::launch_phi_apply(c, c->d.zb, c->d.yb);
+            const int rc = dft_sub(c, c->d.yb, c->d.vec, c->d.vec2);
+            if (rc) return rc;
+            cudaMemcpyAsync(Jv + k * nu, c->d.vec2, nu * 8, cudaMemcpyDeviceToHost, c->stream);
+        }
+        return cuda_check(c, cudaStreamSynchronize(c->stream), "jacobian_apply");
     }
-    return cuda_check(c, cudaStreamSynchronize(c->stream), "jacobian_apply");
+    double* in[2] = {c->d.vec, c->d.ap};
+    double* out[2] = {c->d.vec2, c->d.ap + nu};
+    int rc = FSE_OK;
+    auto fetch = [&](int k) {   // result k to the host
+        cudaStreamWaitEvent(c->stream2, c->ev[3 + (k & 1)], 0);
+        cudaMemcpyAsync(Jv + k * nu, out[k & 1], nu * 8, cudaMemcpyDeviceToHost, c->stream2);
+    };
+    for (int k = 0; k < nvec && rc == FSE_OK; ++k) {
+        // buffers k & 1: their last user, vector k - 2, has left (fetch below, ordered on stream2)
+        cudaEventRecord(c->ev[5], c->stream2);
+        cudaStreamWaitEvent(c->stream, c->ev[5], 0);
+        cudaMemcpyAsync(in[k & 1], v + k * nu, nu * 8, cudaMemcpyHostToDevice, c->stream);
+        fse::launch_idft(c, in[k & 1], c->d.zb);
+        fse::launch_phi_apply(c, c->d.zb, c->d.yb);
+        rc = dft_sub(c, c->d.yb, in[k & 1], out[k & 1]);
+        cudaEventRecord(c->ev[3 + (k & 1)], c->stream);
+        if (k > 0) fetch(k - 1);
+    }
+    if (rc == FSE_OK) fetch(nvec - 1);
+    const int rs = cuda_check(c, cudaStreamSynchronize(c->stream2), "jacobian_apply");
+    const int rt = cuda_check(c, cudaStreamSynchronize(c->stream), "jacobian_apply");
+    return rc ? rc : (rs ? rs : rt);
 }
 
 extern "C" int fse_jacobian_domega(fse_ctx* c, double* out) {
@@ -1202,7 +1233,7 @@ static int gmres_dev(fse_ctx* c, size_t n, const std::function<void(const double
         c->kdot = nullptr;
         c->kry_cap = 0;
         cudaError_t e = cudaMalloc(&c->kry, (size_t)(m + 1) * n * 8);
-        if (e == cudaSuccess) e = cudaMalloc(&c->kdot, (size_t)2 * (m + 2) * 8);
+        if (e == cudaSuccess) e = cudaMalloc(&c->kdot, (size_t)(2 * (256 + 2) + 2) * 8);   // restart <= 256
         if (e != cudaSuccess) return cuda_check(c, e, "GMRES basis");
         c->kry_cap = (size_t)(m + 1) * n;
     }
@@ -1227,7 +1258,8 @@ static int gmres_dev(fse_ctx* c, size_t n, const std::function<void(const double
         *relres_out = 0.0;
         return FSE_OK;
     }
-    std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m), hcol(m + 2), h2(m + 2);
+    std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m), hcol(m + 2),
+        h2(2 * (m + 2) + 1);
     bool first = true;
     while (it < maxit) {
         // r = b - J x  (x = 0 on the first cycle)
@@ -1252,25 +1284,21 @@ static int gmres_dev(fse_ctx* c, size_t n, const std::function<void(const double
             double* w = Vb + (size_t)(k + 1) * n;
             Av(Vb + (size_t)k * n, w);
             ++it;
-            // two passes of classical Gram-Schmidt against v_0..v_k
-            std::fill(hcol.begin(), hcol.end(), 0.0);
-            for (int pass = 0; pass < 2; ++pass) {
-                fse::vec_mdot(c, n, k + 1, Vb, w, hd);
-                cudaMemcpyAsync(h2.data(), hd, (size_t)(k + 1) * 8, cudaMemcpyDeviceToHost, c->stream);
-                rc = cuda_check(c, cudaStreamSynchronize(c->stream), "GMRES dots");
-                if (rc) return rc;
-                for (int i = 0; i <= k; ++i) {
-                    hcol[i] += h2[i];
-                    h2[i] = -h2[i];
-                }
-                cudaMemcpyAsync(hd + (m + 2), h2.data(), (size_t)(k + 1) * 8, cudaMemcpyHostToDevice, c->stream);
-                fse::vec_mupdate(c, n, k + 1, Vb, hd + (m + 2), w);
-            }
-            double hn = 0.0;
-            rc = norm2(w, &hn);
+            // two passes of classical Gram-Schmidt against v_0..v_k, the norm and the scaling on the
+            // device; the coefficients come to the host once
+            double *h1 = hd, *h2d = hd + (m + 2), *nd = hd + 2 * (m + 2);
+            fse::vec_mdot(c, n, k + 1, Vb, w, h1);
+            fse::vec_mupdate(c, n, k + 1, Vb, h1, -1.0, w);
+            fse::vec_mdot(c, n, k + 1, Vb, w, h2d);
+            fse::vec_mupdate(c, n, k + 1, Vb, h2d, -1.0, w);
+            fse::vec_norms2(c, n, w, nullptr, nd);
+            cudaMemcpyAsync(h2.data(), hd, (size_t)(2 * (m + 2) + 1) * 8, cudaMemcpyDeviceToHost, c->stream);
+            fse::vec_normalise(c, n, nd, w);
+            rc = cuda_check(c, cudaStreamSynchronize(c->stream), "GMRES dots");
             if (rc) return rc;
+            for (int i = 0; i <= k; ++i) hcol[i] = h2[i] + h2[m + 2 + i];
+            const double hn = std::sqrt(h2[2 * (m + 2)]);
             hcol[k + 1] = hn;
-            if (hn > 0.0) fse::vec_axpby(c, n, 0.0, w, 1.0 / hn, w);
             // apply the previous rotations, then a new one that zeroes hcol[k + 1]
             for (int i = 0; i < k; ++i) {
                 const double t = cs[i] * hcol[i] + sn[i] * hcol[i + 1];
@@ -1298,7 +1326,7 @@ static int gmres_dev(fse_ctx* c, size_t n, const std::function<void(const double
             y[i] = H[(size_t)i * m + i] != 0.0 ? t / H[(size_t)i * m + i] : 0.0;
         }
         cudaMemcpyAsync(hd + (m + 2), y.data(), (size_t)k * 8, cudaMemcpyHostToDevice, c->stream);
-        fse::vec_mupdate(c, n, k, Vb, hd + (m + 2), x);
+        fse::vec_mupdate(c, n, k, Vb, hd + (m + 2), 1.0, x);
         rc = cuda_check(c, cudaStreamSynchronize(c->stream), "GMRES update");
         if (rc) return rc;
         if (rel <= rtol) break;
@@ -1586,7 +1614,7 @@ extern "C" int fse_newton_step_unknown(fse_ctx* c, double* Z0, double w, double*
         auto Av = [c, m, u, cols, rows](const double* x, double* y) {
             jac_apply_dev(c, x, y);
             if (u) {
-                fse::vec_mupdate(c, m, u, cols, x + m, y);
+                fse::vec_mupdate(c, m, u, cols, x + m, 1.0, y);
                 fse::vec_mdot(c, m, u, rows, x, y + m);
             }
         };

@@ -20,6 +20,8 @@
 #define FSE_RHS_DEPTH_F32 3
 #define FSE_RHS_DEPTH_F64 2
 #define FSE_MAX_BAND 224  // half-bandwidth limit of the blocked solves
+#define FSE_DOT_VECS 64   // dot products of one launch, at most
+#define FSE_DOT_BLOCKS 64 // blocks of one dot product, at most
 #define FSE_MAX_PANELS 4  // tangent panels (decoupled groups of dofs), at most
 
 namespace fse {
@@ -150,6 +152,9 @@ struct Dev {
     double* vec = nullptr;   // scratch 2nU
     double* vec2 = nullptr;  // scratch 2nU
     double* yb = nullptr;    // N x 2n scratch
+    double* ap = nullptr;    // 2 x 2nU: second input / output pair of fse_jacobian_apply
+    double* red = nullptr;      // partial sums of the dot products, FSE_DOT_VECS x FSE_DOT_BLOCKS
+    unsigned* redc = nullptr;   // their counters, zero between launches
     int* status = nullptr;   // N
     int* iters = nullptr;    // N
     int* nref = nullptr;     // N  in-loop refactorisations of the per-step Newton
@@ -330,10 +335,12 @@ int lyapunov_run_noalloc(fse_ctx* c, double omega1, int N_Ly, int h, double* sig
 // vector helpers on the context stream (fse_aft.cu)
 void vec_axpby(fse_ctx* c, size_t n, double a, const double* x, double b, double* y);
 void vec_norms2(fse_ctx* c, size_t n, const double* x, const double* y, double* out_dev);
-// out[i] = V_i . w for i < k (V: k x n row-major), one block per vector
+// out[i] = V_i . w for i < k (V: k x n row-major)
 void vec_mdot(fse_ctx* c, size_t n, int k, const double* V, const double* w, double* out_dev);
-// w += sum_{i<k} coef[i] V_i  (coef on the device)
-void vec_mupdate(fse_ctx* c, size_t n, int k, const double* V, const double* coef_dev, double* w);
+// w += sign sum_{i<k} coef[i] V_i  (coef on the device)
+void vec_mupdate(fse_ctx* c, size_t n, int k, const double* V, const double* coef_dev, double sign, double* w);
+// x *= 1 / sqrt(norm2_dev[0])
+void vec_normalise(fse_ctx* c, size_t n, const double* norm2_dev, double* x);
 void pod_expand(fse_ctx* c, size_t nu, int r, const double* mean, const double* basis, const double* coef,
                 double* z);
 void pod_project(fse_ctx* c, size_t nu, int r, int m, const double* mean, const double* basis, const double* Z,
