@@ -1,5 +1,6 @@
 // AFT (Eq. 20, 21, 15, 16), structured Jacobian products (Eq. 22, 23), the dense
 // outer Newton solve and the Lyapunov exponents (App. F).
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -400,86 +401,158 @@ __global__ void k_back_subst(const double* A, double* x, int m) {
 // Lyapunov exponents (App. F)
 // ----------------------------------------------------------------------------
 
-// weights w_s(phi) = sum_c H_c(phi) Gamma^-1[c][s] of the trigonometric interpolant
-__global__ void k_lyap_weights(int N, int U, int dm1, const int* ktab, const double* Gi,
-                               double phi0, double phi1, double phi2, double* wts) {
+// weights w_s(phi) = sum_c H_c(phi) Gamma^-1[c][s] of the trigonometric interpolant; a warp per sample,
+// its lanes share the harmonics (sine and cosine in FP64 are the work)
+__global__ void __launch_bounds__(128) k_lyap_weights(int N, int U, int dm1, const int* __restrict__ ktab,
+                                                      const double* __restrict__ Gi, double phi0, double phi1,
+                                                      double phi2, double* wts) {
     const double ph[3] = {phi0, phi1, phi2};
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < N; s += gridDim.x * blockDim.x) {
-        double acc = Gi[s];
-        for (int c = 1; c < U; ++c) {
-            const int l = (c - 1) >> 1;
-            double arg = 0.0;
-            for (int j = 0; j < dm1; ++j) arg += (double)ktab[l * dm1 + j] * ph[j];
-            const double h = ((c - 1) & 1) ? sin(arg) : cos(arg);
-            acc += h * Gi[(size_t)c * N + s];
-        }
-        wts[s] = acc;
-    }
-}
-
-// A[i][c] = sum_s w_s sum_j Psi_s[i][j] Q[j][c],  Psi = diag(1, w) Phi diag(1, 1/w)  (Eq. F3)
-template <typename T>
-__global__ void k_lyap_prop(int N, int h, double w, PhiView<T> F, const double* wts, const double* Q, double* Aout) {
-    const int n = F.n, n2 = 2 * n;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (warp >= n2 * h) return;
-    const int i = warp / h, c = warp % h;
-    const double si = (i < n) ? 1.0 : w;
+    const int s = (blockIdx.x * 128 + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (s >= N) return;
     double acc = 0.0;
-    for (int s = 0; s < N; ++s) {
-        int g;
-        const T* row = F.row(s, i, g);
-        double a2 = 0.0;
-        for (int k = lane; k < 2 * F.pan.n[g]; k += 32) {
-            const int j = F.col(g, k);
-            const double sj = (j < n) ? 1.0 : 1.0 / w;
-            a2 += (double)row[k] * sj * Q[(size_t)j * h + c];
-        }
-        acc += wts[s] * a2;
+    for (int l = lane; 1 + 2 * l < U; l += 32) {
+        double arg = 0.0, sn, cs;
+        for (int j = 0; j < dm1; ++j) arg += (double)ktab[l * dm1 + j] * ph[j];
+        sincos(arg, &sn, &cs);
+        acc += cs * Gi[(size_t)(1 + 2 * l) * N + s] + sn * Gi[(size_t)(2 + 2 * l) * N + s];
     }
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) Aout[(size_t)i * h + c] = si * acc;
+    if (lane == 0) wts[s] = Gi[s] + acc;
 }
 
-// classical Gram-Schmidt with re-orthogonalisation, one CTA: Q R = A; acc[c] += ln R[c][c]
-__global__ void k_lyap_qr(int m, int h, double* A, double* Q, double* acc) {
-    __shared__ double red[1024];
-    __shared__ double coef[64];
+// A[i][c] = sum_j (sum_s w_s Psi_s[i][j]) Q[j][c],  Psi = diag(1, w) Phi diag(1, 1/w)  (Eq. F3): the
+// interpolated monodromy first, then its product, 4 n^2 (N + h) multiply-adds instead of 4 n^2 N h.  A
+// CTA takes LYP_R rows of X or V of one panel; LYP_C columns of the interpolated rows go to shared
+// memory, then thread (row, c) adds their products with column c < h <= 64 of Q.
+// 90-dof shell, 15 trajectories, h = 32: 92 -> 21 us.
+constexpr int LYP_R = 4, LYP_C = 128;
+template <typename T>
+__global__ void __launch_bounds__(256) k_lyap_prop(int N, int h, double w, PhiView<T> F, const double* __restrict__ wts,
+                                                   const double* __restrict__ Q, double* Aout) {
+    __shared__ double ms[LYP_R][LYP_C + 1];
+    __shared__ int cols[LYP_C];
+    int x = blockIdx.x, g = 0;
+    while (x >= (F.pan.n[g] + LYP_R - 1) / LYP_R) x -= (F.pan.n[g++] + LYP_R - 1) / LYP_R;
+    const int n = F.n, m = F.pan.n[g], ld = F.pan.ld[g], row0 = F.pan.row0[g], r0 = x * LYP_R;
+    const bool vel = blockIdx.y != 0;   // rows of V
+    const T* B = (vel ? F.V : F.X) + F.pan.off[g] + (size_t)r0 * ld;
+    const int tr = threadIdx.x >> 6, tc = threadIdx.x & 63;   // product: row, column of Q
+    double acc = 0.0;
+    for (int j0 = 0; j0 < 2 * m; j0 += LYP_C) {
+        const int nj = min(LYP_C, 2 * m - j0);
+        __syncthreads();
+        for (int e = threadIdx.x; e < LYP_R * LYP_C; e += 256) {
+            const int r = e / LYP_C, j = e % LYP_C;
+            double v = 0.0;
+            if (j < nj && r0 + r < m) {
+                const T* p = B + (size_t)r * ld + j0 + j;
+#pragma unroll 4
+                for (int s = 0; s < N; ++s) v += wts[s] * (double)p[(size_t)s * F.pan.tot];
+                if (j0 + j >= m) v /= w;
+            }
+            ms[r][j] = v;
+            if (r == 0 && j < nj) cols[j] = F.col(g, j0 + j);
+        }
+        __syncthreads();
+        if (tc < h)
+#pragma unroll 8
+            for (int j = 0; j < nj; ++j) acc += ms[tr][j] * Q[(size_t)cols[j] * h + tc];
+    }
+    if (tc < h && r0 + tr < m) {
+        const int i = F.orig_of[row0 + r0 + tr];
+        Aout[(size_t)(vel ? n + i : i) * h + tc] = vel ? w * acc : acc;
+    }
+}
+
+// Classical Gram-Schmidt with re-orthogonalisation, Q R = A; acc[c] += ln R[c][c].  One cluster: each of
+// its CTAs keeps a slice of the rows in shared memory (B, odd row pitch: a column of 32 rows and a row of
+// 32 columns both hit 32 banks), Q replacing A column by column; a column needs two sums over all rows
+// (the coefficients of each pass, the norm with the second), which the CTAs exchange through distributed
+// shared memory, one cluster barrier a sum.  The 2 m h^2 FP64 multiply-adds at 2 a clock and SM would take one SM 90 us
+// (m = 180, h = 32), so the rows are split even when few; a warp alone has a quarter of that rate (64
+// clocks an FP64 instruction), so sums are kept shallow and nothing is computed by more warps than need it.  With one CTA and a block-wide
+// reduction per coefficient this took 2.3 ms; now 172 us (90-dof shell, h = 32, launch included).  Slices that do not fit in shared memory
+// (beyond m h = 200 k values over 8 CTAs) work in place on A.
+constexpr int LYQ_T = 256, LYQ_W = LYQ_T / 32;
+__global__ void __launch_bounds__(LYQ_T) k_lyap_qr(int m, int h, int in_smem, double* A, double* Q, double* acc) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = cl.block_rank(), size = cl.num_blocks();   // size 1, 2, 4 or 8
+    extern __shared__ double sB[];
+    __shared__ double red[LYQ_W][64], coef[64], nrms[64], s_nrm2, part[2][8][64];   // part[event & 1][rank][k]
+    const int per = (m + size - 1) / size, i0 = min(m, rank * per), rows = min(m, i0 + per) - i0;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, bp = in_smem ? (h | 1) : h;
+    double* B = in_smem ? sB : A + (size_t)i0 * h;
+    if (in_smem)
+        for (int e = tid; e < rows * h; e += LYQ_T) B[(e / h) * bp + e % h] = A[(size_t)i0 * h + e];
+    for (int e = tid; e < 2 * 8 * 64; e += LYQ_T) (&part[0][0][0])[e] = 0.0;   // ranks past the cluster add 0
+    cl.sync();
+    int event = 0;
+    // v[0] + .. + v[7 stride] in pairs
+    auto sum8 = [](const double* v, int stride) {
+        return ((v[0] + v[stride]) + (v[2 * stride] + v[3 * stride])) +
+               ((v[4 * stride] + v[5 * stride]) + (v[6 * stride] + v[7 * stride]));
+    };
+    // coef[k] = sum over the warps' red[.][k] of all CTAs, k < cnt
+    auto exchange = [&](int cnt) {
+        __syncthreads();
+        if (tid < cnt) {
+            const double t = sum8(&red[0][tid], 64);
+            for (int r = 0; r < size; ++r) *cl.map_shared_rank(&part[event & 1][rank][tid], r) = t;
+        }
+        cl.sync();
+        if (tid < cnt) coef[tid] = sum8(&part[event & 1][0][tid], 64);
+        ++event;
+        __syncthreads();
+    };
     for (int c = 0; c < h; ++c) {
-        for (int pass = 0; pass < 2; ++pass) {
-            for (int k = 0; k < c; ++k) {
+        if (tid == 0) s_nrm2 = -1.0;
+        for (int pass = 0; pass < 2 && c > 0; ++pass) {
+            // pass 1 also sums the square of the column itself (k = c) that it is about to correct
+            for (int k = lane; k < c + pass; k += 32) {   // lanes across the columns, warps across the rows
                 double d = 0.0;
-                for (int i = threadIdx.x; i < m; i += blockDim.x) d += Q[(size_t)i * h + k] * A[(size_t)i * h + c];
-                red[threadIdx.x] = d;
-                __syncthreads();
-                for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-                    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-                    __syncthreads();
+                for (int i = warp; i < rows; i += LYQ_W) d += B[(size_t)i * bp + k] * B[(size_t)i * bp + c];
+                red[warp][k] = d;
+            }
+            exchange(c + pass);
+            if (pass == 1 && warp == LYQ_W - 1) {
+                // |a - Q y|^2 = |a|^2 - |y|^2 for orthonormal Q; y is what the first pass left, rounding
+                // as a rule, and where it is more the norm is summed again below
+                double y2 = lane < c ? coef[lane] * coef[lane] : 0.0;
+                if (lane + 32 < c) y2 += coef[lane + 32] * coef[lane + 32];
+                for (int o = 16; o > 0; o >>= 1) y2 += __shfl_xor_sync(0xffffffffu, y2, o);
+                if (lane == 0 && y2 <= 1e-8 * coef[c]) s_nrm2 = coef[c] - y2;
+            }
+            // four lanes a row
+            for (int i0 = 0; i0 < rows; i0 += LYQ_T / 4) {
+                const int i = i0 + (tid >> 2);
+                double v = 0.0;
+                if (i < rows)
+                    for (int k = tid & 3; k < c; k += 4) v += coef[k] * B[(size_t)i * bp + k];
+                if (i0 + 8 * warp < rows) {   // this warp has rows
+                    v += __shfl_xor_sync(0xffffffffu, v, 1);
+                    v += __shfl_xor_sync(0xffffffffu, v, 2);
+                    if (i < rows && (tid & 3) == 0) B[(size_t)i * bp + c] -= v;
                 }
-                if (threadIdx.x == 0) coef[k] = red[0];
-                __syncthreads();
-            }
-            for (int i = threadIdx.x; i < m; i += blockDim.x) {
-                double v = A[(size_t)i * h + c];
-                for (int k = 0; k < c; ++k) v -= coef[k] * Q[(size_t)i * h + k];
-                A[(size_t)i * h + c] = v;
             }
             __syncthreads();
         }
-        double d = 0.0;
-        for (int i = threadIdx.x; i < m; i += blockDim.x) d += A[(size_t)i * h + c] * A[(size_t)i * h + c];
-        red[threadIdx.x] = d;
-        __syncthreads();
-        for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-            if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+        if (s_nrm2 < 0.0) {   // the same in every thread of the cluster: coef is
+            double d = 0.0;
+            for (int i = tid; i < rows; i += LYQ_T) d += B[(size_t)i * bp + c] * B[(size_t)i * bp + c];
+            for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+            if (lane == 0) red[warp][0] = d;
+            exchange(1);
+            if (tid == 0) s_nrm2 = coef[0];
             __syncthreads();
         }
-        const double nrm = sqrt(red[0]);
-        __syncthreads();
-        for (int i = threadIdx.x; i < m; i += blockDim.x) Q[(size_t)i * h + c] = A[(size_t)i * h + c] / nrm;
-        if (threadIdx.x == 0) acc[c] += log(nrm);
+        for (int i = tid; i < rows; i += LYQ_T) B[(size_t)i * bp + c] /= sqrt(s_nrm2);
+        if (tid == LYQ_T - 1) nrms[c] = sqrt(s_nrm2);
         __syncthreads();
     }
+    for (int e = tid; e < rows * h; e += LYQ_T) Q[(size_t)i0 * h + e] = B[(size_t)(e / h) * bp + e % h];
+    if (rank == 0 && tid < h) acc[tid] += log(nrms[tid]);
+    cl.sync();   // no CTA leaves while another may still write to its shared memory
 }
 
 // ----------------------------------------------------------------------------
@@ -624,6 +697,51 @@ int dense_lu_solve(fse_ctx* c, double* A, double* bvec, int m) {
     return h ? FSE_ENONPOS_PIVOT : FSE_OK;
 }
 
+// N_Ly steps of the propagation from Q, with scratch A (2n x h), wts (N); acc[c] += sum of ln R[c][c]
+static int lyapunov_steps(fse_ctx* c, double w, int N_Ly, int h, double* Q, double* A, double* acc, double* wts) {
+    const Params& p = c->p;
+    const int m = 2 * p.n;
+    static std::atomic<unsigned long long> attr{0};
+    if (needs_device_setup(attr)) {
+        cudaFuncSetAttribute(k_lyap_qr, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        mark_device(attr);
+    }
+    // 8 CTAs (the portable cluster size) from 64 rows on: fewer rows a CTA than that are all barrier
+    int size = 1;
+    while (size < 8 && m / (2 * size) >= 8) size *= 2;
+    const size_t smem = (size_t)((m + size - 1) / size) * (h | 1) * 8;
+    const int in_smem = smem <= 200 * 1024;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(size);
+    cfg.blockDim = dim3(LYQ_T);
+    cfg.dynamicSmemBytes = in_smem ? smem : 0;
+    cfg.stream = c->stream;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = size;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int tiles = 0;
+    for (int g = 0; g < p.pan.nc; ++g) tiles += (p.pan.n[g] + LYP_R - 1) / LYP_R;
+    for (int i = 1; i <= N_Ly; ++i) {
+        double ph[3] = {0, 0, 0};
+        for (int j = 0; j < p.d - 1; ++j) ph[j] = 2.0 * (i - 1) * M_PI * c->rho[j];
+        k_lyap_weights<<<(p.N + 3) / 4, 128, 0, c->stream>>>(p.N, p.U, p.d - 1, c->d.ktab, c->d.Gi, ph[0], ph[1],
+                                                             ph[2], wts);
+        if (p.prec == FSE_MIXED_FP32)
+            k_lyap_prop<float><<<dim3(tiles, 2), 256, 0, c->stream>>>(p.N, h, w, phi_view<float>(c), wts, Q, A);
+        else
+            k_lyap_prop<double><<<dim3(tiles, 2), 256, 0, c->stream>>>(p.N, h, w, phi_view<double>(c), wts, Q, A);
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, k_lyap_qr, m, h, in_smem, A, Q, acc);
+        if (e != cudaSuccess) {
+            c->err = std::string("Lyapunov QR launch: ") + cudaGetErrorString(e);
+            return FSE_ECUDA;
+        }
+    }
+    return FSE_OK;
+}
+
 int lyapunov_run(fse_ctx* c, double w, int N_Ly, int h, double* sigma) {
     const Params& p = c->p;
     const int m = 2 * p.n;
@@ -644,19 +762,7 @@ int lyapunov_run(fse_ctx* c, double w, int N_Ly, int h, double* sigma) {
     for (int c2 = 0; c2 < h; ++c2) Q0[(size_t)c2 * h + c2] = 1.0;
     cudaMemcpyAsync(Q, Q0.data(), sizeof(double) * m * h, cudaMemcpyHostToDevice, c->stream);
     cudaMemsetAsync(acc, 0, sizeof(double) * h, c->stream);
-    const size_t warps = (size_t)m * h;
-    const int g = (int)((warps * 32 + 255) / 256);
-    for (int i = 1; i <= N_Ly; ++i) {
-        double ph[3] = {0, 0, 0};
-        for (int j = 0; j < p.d - 1; ++j) ph[j] = 2.0 * (i - 1) * M_PI * c->rho[j];
-        k_lyap_weights<<<nblocks(p.N, 128), 128, 0, c->stream>>>(p.N, p.U, p.d - 1, c->d.ktab, c->d.Gi,
-                                                             ph[0], ph[1], ph[2], wts);
-        if (p.prec == FSE_MIXED_FP32)
-            k_lyap_prop<float><<<g, 256, 0, c->stream>>>(p.N, h, w, phi_view<float>(c), wts, Q, A);
-        else
-            k_lyap_prop<double><<<g, 256, 0, c->stream>>>(p.N, h, w, phi_view<double>(c), wts, Q, A);
-        k_lyap_qr<<<1, 512, 0, c->stream>>>(m, h, A, Q, acc);
-    }
+    const int rc = lyapunov_steps(c, w, N_Ly, h, Q, A, acc, wts);
     std::vector<double> hacc(h);
     cudaMemcpyAsync(hacc.data(), acc, sizeof(double) * h, cudaMemcpyDeviceToHost, c->stream);
     cudaError_t e = cudaStreamSynchronize(c->stream);
@@ -664,6 +770,7 @@ int lyapunov_run(fse_ctx* c, double w, int N_Ly, int h, double* sigma) {
     cudaFree(A);
     cudaFree(acc);
     cudaFree(wts);
+    if (rc) return rc;
     if (e != cudaSuccess) {
         c->err = std::string("Lyapunov run: ") + cudaGetErrorString(e);
         return FSE_ECUDA;
@@ -752,19 +859,8 @@ int lyapunov_run_noalloc(fse_ctx* c, double w, int N_Ly, int h, double* sigma) {
     double* acc = base + 2 * kNoallocQ;
     double* wts = acc + kNoallocAcc;
     k_lyap_init<<<nblocks((size_t)m * h, 256), 256, 0, c->stream>>>(m, h, Q, acc);
-    const size_t warps = (size_t)m * h;
-    const int g = (int)((warps * 32 + 255) / 256);
-    for (int i = 1; i <= N_Ly; ++i) {
-        double ph[3] = {0, 0, 0};
-        for (int j = 0; j < p.d - 1; ++j) ph[j] = 2.0 * (i - 1) * M_PI * c->rho[j];
-        k_lyap_weights<<<nblocks(p.N, 128), 128, 0, c->stream>>>(p.N, p.U, p.d - 1, c->d.ktab, c->d.Gi,
-                                                             ph[0], ph[1], ph[2], wts);
-        if (p.prec == FSE_MIXED_FP32)
-            k_lyap_prop<float><<<g, 256, 0, c->stream>>>(p.N, h, w, phi_view<float>(c), wts, Q, A);
-        else
-            k_lyap_prop<double><<<g, 256, 0, c->stream>>>(p.N, h, w, phi_view<double>(c), wts, Q, A);
-        k_lyap_qr<<<1, 512, 0, c->stream>>>(m, h, A, Q, acc);
-    }
+    const int rs = lyapunov_steps(c, w, N_Ly, h, Q, A, acc, wts);
+    if (rs) return rs;
     double hacc[kNoallocAcc];
     cudaMemcpyAsync(hacc, acc, sizeof(double) * h, cudaMemcpyDeviceToHost, c->stream);
     const cudaError_t e = cudaStreamSynchronize(c->stream);
