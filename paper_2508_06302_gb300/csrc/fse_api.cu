@@ -113,6 +113,11 @@ static void group_rows(int r0, int r1, const std::vector<int>& cptr, const std::
     }
 }
 
+// dofs of a nonlinear element type (FSE_NL_*)
+static int host_elem_ndof(int type) {
+    return (type == FSE_NL_CUBIC_GROUND || type == FSE_NL_VDP) ? 1 : (type == FSE_NL_CUBIC_DIFF ? 2 : 6);
+}
+
 // A numbering of the model's dofs: the caller's own (one panel), or by components (Panels in
 // fse_internal.h).
 struct Numbering {
@@ -151,7 +156,9 @@ static Numbering own_numbering(int n, int b) {
 // a component.  nc stays 0 where it does not pay: the panels' tangents (rows in whole blocks x
 // columns) are what every step streams and solves, and below a quarter saved the inert rows and the
 // shorter blocks cost about as much (n = 24: 3 panels of 32 rows against 1).
-static Numbering component_numbering(int n, const std::vector<std::pair<int, int>>& pairs, const std::vector<int>& comp) {
+static Numbering component_numbering(const fse_model* m, const std::vector<std::pair<int, int>>& pairs,
+                                     const std::vector<int>& comp) {
+    const int n = m->n;
     Numbering N;
     N.pan.nc = 0;
     std::vector<std::vector<int>> members;
@@ -190,6 +197,14 @@ static Numbering component_numbering(int n, const std::vector<std::pair<int, int
         while (a < N.pan.row0[g]) --g;
         N.pan.b[g] = std::max(N.pan.b[g], std::abs(a - b));
     }
+    for (int g = 0; g < nc; ++g) N.pan.lin[g] = 1;
+    for (int e = 0; e < m->n_nl; ++e)
+        for (int a = 0; a < host_elem_ndof(m->nl[e].type); ++a)
+            if (m->nl[e].dof[a] >= 0) {
+                int g = nc - 1;
+                while (N.row_of[m->nl[e].dof[a]] < N.pan.row0[g]) --g;
+                N.pan.lin[g] = 0;
+            }
     finish_panels(N);
     return N;
 }
@@ -405,11 +420,6 @@ static void rotation_tables(const fse_ctx* c, std::vector<double>& rc, std::vect
         rc[l] = cos(th);
         rs[l] = sin(th);
     }
-}
-
-// dofs of a nonlinear element type (FSE_NL_*)
-static int host_elem_ndof(int type) {
-    return (type == FSE_NL_CUBIC_GROUND || type == FSE_NL_VDP) ? 1 : (type == FSE_NL_CUBIC_DIFF ? 2 : 6);
 }
 
 static void free_ctx(fse_ctx* c) {
@@ -634,7 +644,7 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
     }
     p.tc_ok = p.prec == FSE_MIXED_FP32 && b <= 96;
     {
-        Numbering by_comp = component_numbering(n, pairs, comp);
+        Numbering by_comp = component_numbering(m, pairs, comp);
         if (by_comp.pan.nc > 1) {
             Params q = p;
             Matrices mc = build_matrices(m, by_comp, b, et, ed);

@@ -104,16 +104,20 @@ __device__ __forceinline__ double csr_row(const int* __restrict__ ptr, const int
     return acc;
 }
 
-// max that propagates NaN from either argument (fmax drops it), so that a non-finite
-// value anywhere reaches the convergence test
-__device__ __forceinline__ double nanmax(double a, double b) { return (a > b || a != a) ? a : b; }
+// max(a, |b|) for a >= +0, NaN-propagating so that a non-finite value anywhere reaches the convergence
+// test: non-negative doubles are ordered like their bits (infinity and then NaN above the finite ones),
+// and integer compares do not occupy the slow FP64 pipe
+__device__ __forceinline__ double absmax(double a, double b) {
+    const long long x = __double_as_longlong(a), y = __double_as_longlong(b) & 0x7fffffffffffffffll;
+    return __longlong_as_double(x > y ? x : y);
+}
 
-// Block-wide max reduction of two values (blockDim.x multiple of 32, <= 1024), NaN-propagating.
+// Block-wide max reduction of two values >= +0 (blockDim.x multiple of 32, <= 1024), NaN-propagating.
 __device__ __forceinline__ void block_max2(double& a, double& b) {
     __shared__ double ra[32], rb[32];
     for (int o = 16; o > 0; o >>= 1) {
-        a = nanmax(a, __shfl_xor_sync(0xffffffffu, a, o));
-        b = nanmax(b, __shfl_xor_sync(0xffffffffu, b, o));
+        a = absmax(a, __shfl_xor_sync(0xffffffffu, a, o));
+        b = absmax(b, __shfl_xor_sync(0xffffffffu, b, o));
     }
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
     __syncthreads();
@@ -126,8 +130,8 @@ __device__ __forceinline__ void block_max2(double& a, double& b) {
     a = 0.0;
     b = 0.0;
     for (int k = 0; k < nw; ++k) {
-        a = nanmax(a, ra[k]);
-        b = nanmax(b, rb[k]);
+        a = absmax(a, ra[k]);
+        b = absmax(b, rb[k]);
     }
 }
 

@@ -39,6 +39,7 @@ struct Panels {
     int row0[FSE_MAX_PANELS] = {};   // first internal row
     int n[FSE_MAX_PANELS] = {};      // rows (without the inert ones)
     int b[FSE_MAX_PANELS] = {};      // half-bandwidth inside the panel
+    int lin[FSE_MAX_PANELS] = {};    // no nonlinear element: K_eff and its factor depend on w_1 alone
     int ld[FSE_MAX_PANELS] = {};     // row stride: 2 n + 1 rounded up to a multiple of 4
     int pass0[FSE_MAX_PANELS + 1] = {};   // first pass of the right-hand-side kernel; its row groups
     int g1[FSE_MAX_PANELS] = {};          // are pass0 * FSE_RHS_GPS .. g1 - 1

@@ -94,21 +94,55 @@ __global__ void k_sband(int n, int nb, const int* __restrict__ ptr, const int* _
 // columns of the band staged ahead of the Cholesky window (cp.async ring)
 #define FSE_CHOL_PF 8
 
+// L_jj = sqrt(p) and 1 / L_jj of a pivot, both correctly rounded.  FP64: Newton-Raphson for 1 / sqrt(p)
+// from the FP32 value (x <- x + x (1 - p x^2) / 2 doubles the 23 good bits twice), then Markstein's final
+// corrections (IBM J. Res. Dev. 34, 1990) of the square root, g + (p - g^2) / (2 sqrt p), and of the
+// reciprocal, x + x (1 - g x): half the FP64 instructions of sqrt and a division one after the other.
+// Outside the FP32 range the library's are used.
+__device__ __forceinline__ void pivot_root(float p, float& ljj, float& inv) {
+    ljj = sqrtf(p);
+    inv = 1.0f / ljj;
+}
+__device__ __forceinline__ void pivot_root(double p, double& ljj, double& inv) {
+    const unsigned e = (unsigned)__double2hiint(p) >> 20;   // biased exponent (p > 0)
+    if (e < 1023 - 100 || e >= 1023 + 100) {
+        ljj = sqrt(p);
+        inv = 1.0 / ljj;
+        return;
+    }
+    double x = (double)rsqrtf((float)p);
+    const double hp = 0.5 * p;
+    x = fma(fma(-hp * x, x, 0.5), x, x);
+    x = fma(fma(-hp * x, x, 0.5), x, x);
+    const double g = p * x;
+    ljj = fma(fma(-g, g, p), 0.5 * x, g);
+    inv = fma(fma(-ljj, x, 1.0), x, x);
+}
+// positive and finite, without FP64 compares
+__device__ __forceinline__ bool good_pivot(float p) { return p > 0.0f && p < INFINITY; }
+__device__ __forceinline__ bool good_pivot(double p) {
+    const long long v = __double_as_longlong(p);
+    return v > 0 && v < 0x7ff0000000000000ll;
+}
+
 // Banded Cholesky with a warp-cooperative trailing update.  The window holds the nb columns
 // j..j+b in nb + 1 shared slots (column c in slot c mod (nb + 1)).  Step j, between two barriers:
 //  (a) threads r < nb write column j - 1 of L out of its slot, refill that slot with column
 //      j + nb from the cp.async staging ring (entry r was staged by thread r) and stage
 //      column j + nb + PF - 1;
-//  (b) warp w updates columns j + cc, cc = w + 1, w + 1 + 8, ..., with lanes over the rows:
-//      A_(j+cc+rr, j+cc) -= A_(j+cc+rr, j) A_(j+cc, j) / A_(j, j), rr <= b - cc.
-// (a) and (b) touch different slots, so one barrier per column suffices.
+//  (b) columns j + cc, lanes over the rows: A_(j+cc+rr, j+cc) -= A_(j+cc+rr, j) A_(j+cc, j) / A_(j, j),
+//      rr <= b - cc: warp 0 takes cc = 1 and then forms the next pivot's root and reciprocal, warps
+//      1 .. 7 the other columns in turn.
+// (a) and (b) touch different slots, so one barrier per column suffices.  In FP64 the pivot chain and the
+// FP64 rate (a warp instruction holds its SM partition for 64 clocks) set the pace: with the square root
+// and the divisions in every warp a column took about 2.5 us.
 template <typename T>
 __device__ int cta_band_cholesky_w(T* Ac, T* Lr, T* Linv, int n, int b, T* wnd, T* stg, T* Rf, T* Rb, int RECE) {
     constexpr int PF = FSE_CHOL_PF;
     const int nb = b + 1, ns = nb + 1;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
-    __shared__ int bad;
-    if (tid == 0) bad = 0;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;   // 8 warps
+    __shared__ int s_bad[2];
+    __shared__ T s_inv[2], s_ljj[2];   // of column j at j & 1 (s_bad: its pivot is no good)
     for (int idx = tid; idx < nb * nb; idx += blockDim.x) {
         const int c = idx / nb;   // column c starts in slot c
         wnd[idx] = (c < n) ? Ac[(size_t)c * nb + (idx - c * nb)] : T(0);
@@ -139,46 +173,70 @@ __device__ int cta_band_cholesky_w(T* Ac, T* Lr, T* Linv, int n, int b, T* wnd, 
             for (int c = 0; c < b - jp; ++c) Lr[(size_t)jp * nb + c] = T(0);
         }
     };
+    // the pivot of column j, checked (warp 0)
+    auto next_pivot = [&](int j, T piv) {
+        const bool ok = good_pivot(piv);
+        T ljj, inv;
+        pivot_root(ok ? piv : T(1), ljj, inv);
+        if (lane == 0) {
+            s_ljj[j & 1] = ljj;
+            s_inv[j & 1] = inv;
+            s_bad[j & 1] = !ok;
+        }
+    };
     __syncthreads();
-    T ljj_prev = T(0), inv_prev = T(0);
+    if (warp == 0) next_pivot(0, wnd[0]);
+    __syncthreads();
     int slot = 0;   // slot of column j
     int j = 0;
     for (; j < n; ++j) {
+        if (s_bad[j & 1]) break;
         const T* colj = wnd + slot * nb;
-        const T piv = colj[0];
-        if (!(piv > T(0)) || !isfinite((double)piv)) {
-            if (tid == 0) bad = 1;
-            break;
-        }
-        const T ljj = sqrt(piv);
-        const T inv = T(1) / ljj;
-        const T inv2 = inv * inv;
+        const T inv = s_inv[j & 1], inv2 = inv * inv;
         const int sp = (slot == 0) ? ns - 1 : slot - 1;   // slot of column j - 1 = slot of column j + nb
         if (tid < nb) {
             T* colp = wnd + sp * nb;
-            if (j > 0) write_col(j - 1, colp, ljj_prev, inv_prev);
+            if (j > 0) write_col(j - 1, colp, s_ljj[(j - 1) & 1], s_inv[(j - 1) & 1]);
             cp_async_wait<PF - 2>();   // entry tid of column j + nb has landed
             const int jn = j + nb;
             colp[tid] = (jn < n) ? stg[(jn % PF) * nb + tid] : T(0);
             issue(jn + PF - 1);        // into the staging slot just read
         }
-        for (int cc = warp + 1; cc <= b; cc += nw) {
-            if (j + cc >= n) break;
+        const int ncc = min(b, n - 1 - j);   // columns j + 1 .. j + ncc are updated
+        auto update = [&](int cc, T g) {
             int sc = slot + cc;
             sc = (sc >= ns) ? sc - ns : sc;
             T* colc = wnd + sc * nb;
-            const T g = colj[cc] * inv2;
             for (int rr = lane; rr <= b - cc; rr += 32) colc[rr] -= colj[cc + rr] * g;
+        };
+        if (warp == 0) {
+            if (j + 1 < n) {
+                int sc = slot + 1;
+                sc = (sc >= ns) ? 0 : sc;
+                if (ncc >= 1) update(1, colj[1] * inv2);
+                __syncwarp();
+                next_pivot(j + 1, wnd[sc * nb]);
+            }
+        } else {
+            // this warp's columns cc = warp + 1 + 7 q: lane q forms the factor of the q-th
+            for (int q0 = 0; warp + 1 + 7 * q0 <= ncc; q0 += 32) {
+                const int mine = warp + 1 + 7 * (q0 + lane);
+                const T gl = mine <= ncc ? colj[mine] * inv2 : T(0);
+                for (int q = 0; q < 32; ++q) {
+                    const int cc = warp + 1 + 7 * (q0 + q);
+                    if (cc > ncc) break;
+                    update(cc, __shfl_sync(0xffffffffu, gl, q));
+                }
+            }
         }
         __syncthreads();
-        ljj_prev = ljj;
-        inv_prev = inv;
         slot = (slot + 1 == ns) ? 0 : slot + 1;
     }
-    if (j == n && tid < nb) write_col(n - 1, wnd + ((slot == 0) ? ns - 1 : slot - 1) * nb, ljj_prev, inv_prev);
+    if (j == n && tid < nb)
+        write_col(n - 1, wnd + ((slot == 0) ? ns - 1 : slot - 1) * nb, s_ljj[(n - 1) & 1], s_inv[(n - 1) & 1]);
     cp_async_wait<0>();
     __syncthreads();
-    return bad;
+    return j < n;
 }
 
 // Banded Cholesky with the window in registers (b + 1 <= 32 MAXK, nb <= 8 MAXS): warp w owns
@@ -324,6 +382,7 @@ __host__ __device__ constexpr size_t chol_blk_floats(int nb) {
 // all trajectories), the lower K_t entries by column, this trajectory's K_t and C_t values
 // (ct null without velocity-dependent elements) and w (2/Delta)
 struct ChbSource {
+    int col0;   // first column (internal row) of the panel that is factored
     const float* Sband;
     const int *ktc_ptr, *ktc_e, *ktc_c, *ktc_r;
     const float *kt, *ct;
@@ -492,7 +551,7 @@ __device__ int cta_band_cholesky_blk(float* Ac, float* Lr, float* Linv, float* D
                 const int e = src.ktc_e[k];
                 float v = src.kt[e];
                 if (src.ct) v += src.wa * src.ct[e];
-                chb_col(W, src.ktc_c[k], nb)[src.ktc_r[k]] += v;
+                chb_col(W, src.ktc_c[k] - src.col0, nb)[src.ktc_r[k]] += v;
             }
         }
     };
@@ -603,7 +662,8 @@ __device__ void cta_diag_inverses(const T* Lr, const T* Linv, int n, int b, int 
         for (int i = 0; i < FSE_BLK; ++i) {
             T acc = (i == lane) ? T(1) : T(0);
 #pragma unroll
-            for (int j = 0; j < i; ++j) acc -= Lt[i * FSE_BLK + j] * z[j];
+            for (int j = 0; j < i; ++j)
+                if (i - j <= b) acc -= Lt[i * FSE_BLK + j] * z[j];   // the same for the whole warp
             z[i] = acc * Lt[FSE_BLK * FSE_BLK + i];
         }
         T* D = Dinv + (size_t)B * FSE_BLK * FSE_BLK;
@@ -639,6 +699,7 @@ __host__ __device__ inline size_t state_wspan(int nb, int blk) {
 struct StateArgs {
     int n, b, e, dm1, maxit, ncolors, n_el, nnz_kt, kt_ld, nblk, init;
     Panels pan;
+    int skip_lin;       // linear panels keep their factors (steps k >= 1)
     int refactor;       // 0: keep the previous factors (residual-only steps, see launch_state_step)
     double tol, Dl, a0c, a1c, a2c, w, phi;
     double rho[FSE_MAX_D - 1];
@@ -671,32 +732,46 @@ struct StateArgs {
     int *status, *iters, *nref;
 };
 
-// factor of K_eff (column band Ac in place, row band, 1/L_jj, diagonal-block inverses and the
-// tangent-solve records); nonzero on a non-positive or non-finite pivot
+// whether the factor of panel g is formed in this step: the factors of linear panels are formed by the
+// initial call (parity buffer 1) and step 0 (buffer 0) and stay valid
+__device__ __forceinline__ bool panel_factored(const StateArgs& A, int g) { return !(A.skip_lin && A.pan.lin[g]); }
+
+// factor of K_eff, panel by panel (column band Ac in place, row band, 1/L_jj, diagonal-block inverses and
+// the tangent-solve records; inert rows cost no step: their L stays the identity that setup wrote);
+// nonzero on a non-positive or non-finite pivot
 template <typename T, bool BLK>
 __device__ int band_factor(const StateArgs& A, T* Ac, T* Lr, T* Linv, T* Dinv, T* wnd, T* stg, T* Rf, T* Rb,
                            const T* kt = nullptr, const T* ct = nullptr) {
-    if constexpr (BLK) {
-        const ChbSource src{A.Sband, A.ktc_ptr, A.ktc_e, A.ktc_c, A.ktc_r, kt, ct, float(A.w * A.a2c)};
-        return cta_band_cholesky_blk(Ac, Lr, Linv, Dinv, A.n, A.b, wnd, Rf, Rb, A.RECE, A.full_factor != 0, src);
-    }
-    // column by column: one panel after the other, so that inert rows cost no barrier (their L stays
-    // the identity that setup wrote)
     int bad = 0;
     for (int g = 0; g < A.pan.nc && !bad; ++g) {
-        const int r0 = A.pan.row0[g];
-        const size_t o = (size_t)r0 * (A.b + 1), ro = (size_t)(r0 / FSE_BLK) * A.RECE;
-        bad = band_cholesky<T>(Ac + o, Lr + o, Linv + r0, A.pan.n[g], A.b, wnd, stg, Rf + ro, Rb + ro, A.RECE);
+        if (!panel_factored(A, g)) continue;
+        const int r0 = A.pan.row0[g], n = A.pan.n[g], B0 = r0 / FSE_BLK;
+        const size_t o = (size_t)r0 * (A.b + 1), ro = (size_t)B0 * A.RECE, dof = (size_t)B0 * FSE_BLK * FSE_BLK;
+        if constexpr (BLK) {
+            const ChbSource src{r0,      A.Sband + o, A.ktc_ptr + r0, A.ktc_e, A.ktc_c,
+                                A.ktc_r, kt,          ct,             float(A.w * A.a2c)};
+            bad = cta_band_cholesky_blk(Ac + o, Lr + o, Linv + r0, Dinv + dof, n, A.b, wnd, Rf + ro, Rb + ro, A.RECE,
+                                        A.full_factor != 0, src);
+        } else {
+            bad = band_cholesky<T>(Ac + o, Lr + o, Linv + r0, n, A.b, wnd, stg, Rf + ro, Rb + ro, A.RECE);
+            if (!bad)
+                cta_diag_inverses<T>(Lr + o, Linv + r0, n, A.b, (n + FSE_BLK - 1) / FSE_BLK, Dinv + dof, wnd, Rf + ro,
+                                     Rb + ro, A.RECE);
+        }
         __syncthreads();   // every thread has read the pivot flag before the next panel clears it
     }
-    if (!bad) cta_diag_inverses<T>(Lr, Linv, A.n, A.b, A.nblk, Dinv, wnd, Rf, Rb, A.RECE);
     return bad;
 }
 
-__device__ __forceinline__ double forcing_i(const StateArgs& A, int s, int i, double phi) {
-    double e = A.F[i] * cos(phi);
-    for (int j = 1; j < A.e; ++j)
-        e += A.F[(size_t)j * A.n + i] * cos(A.phis[s * A.dm1 + (j - 1)] + A.rho[j - 1] * phi);
+// cosines of the forcing components of trajectory s at phi_1 = phi, one lane each (a cosine is some
+// hundred FP64 instructions: once per step, not once per dof)
+__device__ __forceinline__ void forcing_phases(const StateArgs& A, int s, double phi, double* cph) {
+    const int j = threadIdx.x - (blockDim.x - 32);   // the last warp
+    if (j >= 0 && j < A.e) cph[j] = cos(j == 0 ? phi : A.phis[s * A.dm1 + (j - 1)] + A.rho[j - 1] * phi);
+}
+__device__ __forceinline__ double forcing_i(const StateArgs& A, int i, const double* cph) {
+    double e = A.F[i] * cph[0];
+    for (int j = 1; j < A.e; ++j) e += A.F[(size_t)j * A.n + i] * cph[j];
     return e;
 }
 
@@ -734,13 +809,17 @@ __device__ void assemble_keff(const StateArgs& A, int s, const double* q, const 
                   ce ? ce + (size_t)el * 36 : nullptr);
     }
     if constexpr (BAND) {
-        for (int idx = threadIdx.x; idx < n * nb; idx += blockDim.x) Ac[idx] = T(0);
-        __syncthreads();
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            const int e1 = A.cs_ptr[i + 1];
-            for (int e = A.cs_ptr[i]; e < e1; ++e) {
-                const int j = A.cs_col[e];
-                if (j <= i) Ac[(size_t)j * nb + (i - j)] = T(A.cs_s[e]);
+        for (int g = 0; g < A.pan.nc; ++g) {
+            if (!panel_factored(A, g)) continue;   // its band holds the factor
+            const int r0 = A.pan.row0[g], r1 = r0 + A.pan.n[g];
+            for (int idx = r0 * nb + threadIdx.x; idx < r1 * nb; idx += blockDim.x) Ac[idx] = T(0);
+            __syncthreads();
+            for (int i = r0 + threadIdx.x; i < r1; i += blockDim.x) {
+                const int e1 = A.cs_ptr[i + 1];
+                for (int e = A.cs_ptr[i]; e < e1; ++e) {
+                    const int j = A.cs_col[e];
+                    if (j <= i) Ac[(size_t)j * nb + (i - j)] = T(A.cs_s[e]);
+                }
             }
         }
     }
@@ -1022,7 +1101,7 @@ __device__ void warp_band_solve_fp64(const double* __restrict__ Lc, const double
 
 // BLK: FP32 factor by 32-column panels (the launcher picks it when chol_blk is set)
 template <typename T, bool BLK>
-__global__ void __launch_bounds__(256) k_state(StateArgs A) {
+__global__ void __launch_bounds__(256, 2) k_state(StateArgs A) {
     static_assert(!BLK || sizeof(T) == 4, "panel Cholesky is FP32 only");
     const int s = blockIdx.x, n = A.n, b = A.b, nb = b + 1;
     const int tid = threadIdx.x, nt = blockDim.x;
@@ -1039,7 +1118,8 @@ __global__ void __launch_bounds__(256) k_state(StateArgs A) {
     double* sv = A.has_vel
                      ? reinterpret_cast<double*>((reinterpret_cast<size_t>(ysol + n) + 7) & ~static_cast<size_t>(7))
                      : nullptr;
-    __shared__ int s_conv, s_stat;
+    __shared__ int s_conv, s_stat, s_next;
+    __shared__ double s_cph[FSE_MAX_D];
     const size_t off = (size_t)s * n;
     const size_t foff = (size_t)s * n * nb;
     const size_t doff = (size_t)s * A.nblk * FSE_BLK * FSE_BLK;
@@ -1061,6 +1141,7 @@ __global__ void __launch_bounds__(256) k_state(StateArgs A) {
         s_stat = A.init ? 0 : A.status[s];
         s_conv = 0;
     }
+    forcing_phases(A, s, A.init ? 0.0 : A.phi, s_cph);
     for (int i = tid; i < n; i += nt) {
         sq[i] = A.q[off + i];
         su[i] = A.u[off + i];
@@ -1075,7 +1156,7 @@ __global__ void __launch_bounds__(256) k_state(StateArgs A) {
         vel_state();
         add_fnl(A, sq, sv, sr);
         for (int i = tid; i < n; i += nt)
-            sb[i] = forcing_i(A, s, i, 0.0) - A.w * csr_row(A.cs_ptr, A.cs_col, A.cs_d, i, su) -
+            sb[i] = forcing_i(A, i, s_cph) - A.w * csr_row(A.cs_ptr, A.cs_col, A.cs_d, i, su) -
                     csr_row(A.cs_ptr, A.cs_col, A.cs_k, i, sq) - sr[i];
         __syncthreads();
         if (tid < 32) warp_band_solve_fp64(A.LMc, A.LMr, A.LMinv, n, b, sb);
@@ -1085,8 +1166,8 @@ __global__ void __launch_bounds__(256) k_state(StateArgs A) {
         for (int i = tid; i < n; i += nt) {
             sa[i] = sb[i] * iw2;
             A.a[off + i] = sa[i];
-            zmax = nanmax(zmax, nanmax(fabs(sq[i]), fabs(su[i])));
-            amax = nanmax(amax, fabs(sa[i]));
+            zmax = absmax(absmax(zmax, sq[i]), su[i]);
+            amax = absmax(amax, sa[i]);
         }
         block_max2(zmax, amax);
         // a non-finite start point (from Z(0)) is reported as such, not as a failed factorisation
@@ -1107,7 +1188,7 @@ __global__ void __launch_bounds__(256) k_state(StateArgs A) {
         __syncthreads();
         const double w2 = A.w * A.w;
         for (int i = tid; i < n; i += nt)
-            sb[i] = forcing_i(A, s, i, A.phi) + w2 * csr_row(A.cs_ptr, A.cs_col, A.cs_m, i, sr) +
+            sb[i] = forcing_i(A, i, s_cph) + w2 * csr_row(A.cs_ptr, A.cs_col, A.cs_m, i, sr) +
                     A.w * csr_row(A.cs_ptr, A.cs_col, A.cs_d, i, sqn);
         __syncthreads();
         for (int i = tid; i < n; i += nt) sqn[i] = sq[i];   // predictor: the previous displacement
@@ -1133,23 +1214,32 @@ __global__ void __launch_bounds__(256) k_state(StateArgs A) {
             for (int i = tid; i < n; i += nt) {
                 const double v = sqn[i] - sr[i];
                 sqn[i] = v;
-                dmax = nanmax(dmax, fabs(sr[i]));
-                qmax = nanmax(qmax, fabs(v));
+                dmax = absmax(dmax, sr[i]);
+                qmax = absmax(qmax, v);
             }
             block_max2(dmax, qmax);
-            if (!isfinite(dmax) || !isfinite(qmax)) {
+            // thread 0 decides for all (FP64 compares): 0 go on, 1 converged, 2 not finite, 3 refactor.
+            // An FP32 factor limits the chord contraction by itself: one refactorisation per step is
+            // enough to tell nonlinearity from rounding, more would only repeat it
+            if (tid == 0) {
+                const bool allow = sizeof(T) == 8 || nref == 0;
+                s_next = (!isfinite(dmax) || !isfinite(qmax))                                    ? 2
+                         : (A.tol > 0.0 && dmax <= A.tol * qmax)                                 ? 1
+                         : (prev > 0.0 && dmax > 0.1 * prev && it + 1 < A.maxit && allow) ? 3
+                                                                                                 : 0;
+            }
+            __syncthreads();
+            const int next = s_next;
+            if (next == 2) {
                 if (tid == 0) s_stat = FSE_ENAN;
                 break;
             }
-            if (A.tol > 0.0 && dmax <= A.tol * qmax) {
+            if (next == 1) {
                 if (tid == 0) s_conv = 1;
                 ++it;
                 break;
             }
-            // an FP32 factor limits the chord contraction by itself: one refactorisation per
-            // step is enough to tell nonlinearity from rounding, more would only repeat it
-            const bool allow = sizeof(T) == 8 || nref == 0;
-            if (prev > 0.0 && dmax > 0.1 * prev && it + 1 < A.maxit && allow) {
+            if (next == 3) {
                 ++nref;
                 vel_iterate();
                 assemble_keff<T, !BLK>(A, s, sqn, sv, oLc, kt_out, ct_out);
@@ -1312,6 +1402,7 @@ static StateArgs make_state_args(fse_ctx* c, double w, int init, int k) {
     A.n = p.ni;
     A.b = p.b;
     A.pan = p.pan;
+    A.skip_lin = k >= 1;
     A.e = p.e;
     A.dm1 = p.d - 1;
     A.maxit = p.maxit;
