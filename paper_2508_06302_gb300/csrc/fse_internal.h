@@ -19,6 +19,7 @@
 // passes of the right-hand-side kernel in flight ahead of the one computed (FP32 / FP64 tangents)
 #define FSE_RHS_DEPTH_F32 3
 #define FSE_RHS_DEPTH_F64 2
+#define FSE_DIRECT_BAND 32  // half-bandwidth up to which FP64 tangents are solved row by row (k_direct)
 #define FSE_MAX_BAND 224  // half-bandwidth limit of the blocked solves
 #define FSE_DOT_VECS 64   // dot products of one launch, at most
 #define FSE_DOT_BLOCKS 64 // blocks of one dot product, at most
@@ -329,6 +330,9 @@ void launch_tc_solve(fse_ctx* c, int k, int phase, cudaStream_t st);
 // tangents of a long period drift (on the 1872-dof shell the monodromy of a 1000-step period
 // differs from the SIMT one by 1e-2, enough to stall Newton's convergence)
 inline bool use_tc(const fse_ctx* c) { return c->p.tc_ok && c->solve_kind == FSE_SOLVE_TC; }
+// FP64 tangents with narrow panels are solved row by row from the bands of the factor, without block
+// records
+inline bool use_direct(const fse::Params& p) { return p.prec == FSE_FP64 && p.b <= FSE_DIRECT_BAND; }
 int lyapunov_run(fse_ctx* c, double omega1, int N_Ly, int h, double* sigma);
 // same propagation with the static device scratch of fse_aft.cu (no allocation)
 int lyapunov_run_noalloc(fse_ctx* c, double omega1, int N_Ly, int h, double* sigma);

@@ -30,7 +30,7 @@ struct SensArgs {
     const int* kt_slot;
     int* err;   // set when a pipeline wait gives up
     const void *g_rec, *g_rr, *g_info, *g_pass, *kt_val, *romega;
-    const void *Lc, *Lr, *Dinv, *Rf, *Rb;
+    const void *Lc, *Lr, *Linv, *Dinv, *Rf, *Rb;
     void *X, *V, *Y;
 };
 
@@ -812,6 +812,136 @@ __global__ void __launch_bounds__(256, 1) k_trsm8(SensArgs A) {
     }
 }
 
+// Direct banded substitution in FP64, a thread per direction.  FP64 multiply-adds are what these solves
+// cost (2 a clock and SM), and the blocked form spends them on the zeros of its 32 x 32 diagonal-block
+// inverses and on whole tiles of 128 directions; column by column a row takes just b + 1.  The window of
+// B >= b rows that the solved row still updates sits in registers and moves down by one with each update
+// (w[k] <- w[k + 1] - L x), so nothing is copied.  The factor's columns (FWD, L_(i+k, i)) or rows (BWD,
+// L_(i, i-k)) of the next 32 rows come to shared memory by cp.async while 32 rows are solved, as rows
+// [1 / L_ii | L_1 .. L_B] (zeros past b) that a thread reads 16 bytes at a time before it uses them;
+// right-hand sides, X_k and V_k are loaded DSR rows ahead.
+// 447-dof beam, b = 5, 64 trajectories: 1.03 / 1.14 -> 0.32 / 0.46 ms (forward / backward with the V
+// update; 0.25 / 0.33 of FP64 work); 360-dof shell 0.34 / 0.31 -> 0.30 / 0.35 ms; 72-dof plate, 19
+// trajectories, 87 / 90 -> 68 / 104 us alone (too few warps for the FP64 pipes, fewer SMs taken from the
+// state kernel: 228 -> 192 us a step).
+constexpr int DSR = 4;    // rows loaded ahead
+constexpr int DSC = 32;   // rows of the factor staged at a time
+template <int B, bool FWD>
+__device__ void direct_solve(const SensArgs& A, const PanelTile& pt, int s, int t, double* stg) {
+    constexpr int BP = (B + 2) & ~1;   // row pitch, even
+    const int n = pt.n, b = A.b, pb = pt.b, nb = b + 1, ld = pt.ld;
+    const bool tok = t < ld;
+    const size_t fo = (size_t)s * A.n + pt.row0;
+    const double* Lb = reinterpret_cast<const double*>(FWD ? A.Lc : A.Lr) + fo * nb;
+    const double* Li = reinterpret_cast<const double*>(A.Linv) + fo;
+    const size_t base = (size_t)s * A.pan.tot + A.pan.off[pt.g] + (tok ? t : 0);
+    double* Y = reinterpret_cast<double*>(A.Y) + base;
+    double* X = reinterpret_cast<double*>(A.X) + base;
+    double* V = reinterpret_cast<double*>(A.V) + base;
+    const double a2 = A.a2c;
+    const int nch = (n + DSC - 1) / DSC;
+    for (int e = threadIdx.x; e < 2 * DSC * BP; e += 128) stg[e] = 0.0;
+    __syncthreads();
+    // chunk q of the processing order (BWD: from the last row down): its rows in memory are c0 ..
+    auto first_row = [&](int q) { return FWD ? DSC * q : max(0, n - DSC * (q + 1)); };
+    auto stage = [&](int q) {
+        if (q < nch) {
+            const int c0 = first_row(q), nr = min(DSC, n - DSC * q);
+            double* d = stg + (q & 1) * DSC * BP;
+            const int i = threadIdx.x >> 2;   // four threads a row
+            if (i < nr) {
+                const double* src = Lb + (size_t)(c0 + i) * nb;
+                for (int k = 1 + (threadIdx.x & 3); k <= pb; k += 4)
+                    cp_async_elem(d + i * BP + k, src + (FWD ? k : b - k));
+                if ((threadIdx.x & 3) == 0) cp_async_elem(d + i * BP, Li + c0 + i);
+            }
+        }
+        cp_async_commit();
+    };
+    double w[B + 1];
+#pragma unroll
+    for (int k = 0; k <= B; ++k) w[k] = 0.0;
+    double yn[DSR], xn[DSR], vn[DSR];
+    auto load = [&](int r, int u) {   // processing row r into slot u
+        if (tok && r < n) {
+            const size_t o = (size_t)(FWD ? r : n - 1 - r) * ld;
+            yn[u] = Y[o];
+            if (!FWD) {
+                xn[u] = X[o];
+                vn[u] = V[o];
+            }
+        }
+    };
+#pragma unroll
+    for (int u = 0; u < DSR; ++u) yn[u] = xn[u] = vn[u] = 0.0;
+    stage(0);
+#pragma unroll
+    for (int u = 0; u < DSR; ++u) load(u, u);
+    int r = 0;
+    for (int q = 0; q < nch; ++q) {
+        stage(q + 1);   // into the buffer of chunk q - 1, finished at the barrier below
+        cp_async_wait1();
+        __syncthreads();
+        const int c0 = first_row(q), nr = min(DSC, n - DSC * q);
+        const double* L = stg + (q & 1) * DSC * BP;
+        for (int k0 = 0; k0 < nr; k0 += DSR) {
+#pragma unroll
+            for (int u = 0; u < DSR; ++u) {
+                if (k0 + u < nr) {
+                    const int i = FWD ? k0 + u : nr - 1 - k0 - u;   // row of the chunk
+                    double l[BP];
+#pragma unroll
+                    for (int k = 0; k < BP; k += 2) {
+                        const double2 v = *reinterpret_cast<const double2*>(L + i * BP + k);
+                        l[k] = v.x;
+                        l[k + 1] = v.y;
+                    }
+                    const double x = fma(w[0], l[0], yn[u] * l[0]);
+#pragma unroll
+                    for (int k = 0; k < B; ++k) w[k] = fma(-l[k + 1], x, w[k + 1]);
+                    if (tok) {
+                        const size_t o = (size_t)(c0 + i) * ld;
+                        if (FWD) {
+                            Y[o] = x;
+                        } else {
+                            X[o] = x;
+                            V[o] = fma(a2, x - xn[u], -vn[u]);
+                        }
+                    }
+                    load(r + DSR, u);
+                    ++r;
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// window sizes: one register window per half-bandwidth would be 32 kernels; every fourth from 8 on
+template <bool FWD>
+__global__ void __launch_bounds__(128) k_direct(SensArgs A) {
+    extern __shared__ __align__(16) double dstg[];
+    const PanelTile pt = panel_tile(A, blockIdx.x);
+    const int t = pt.tile * 128 + threadIdx.x, s = blockIdx.y;
+    switch (pt.b <= 8 ? pt.b : (pt.b + 3) & ~3) {
+        case 0: direct_solve<0, FWD>(A, pt, s, t, dstg); break;
+        case 1: direct_solve<1, FWD>(A, pt, s, t, dstg); break;
+        case 2: direct_solve<2, FWD>(A, pt, s, t, dstg); break;
+        case 3: direct_solve<3, FWD>(A, pt, s, t, dstg); break;
+        case 4: direct_solve<4, FWD>(A, pt, s, t, dstg); break;
+        case 5: direct_solve<5, FWD>(A, pt, s, t, dstg); break;
+        case 6: direct_solve<6, FWD>(A, pt, s, t, dstg); break;
+        case 7: direct_solve<7, FWD>(A, pt, s, t, dstg); break;
+        case 8: direct_solve<8, FWD>(A, pt, s, t, dstg); break;
+        case 12: direct_solve<12, FWD>(A, pt, s, t, dstg); break;
+        case 16: direct_solve<16, FWD>(A, pt, s, t, dstg); break;
+        case 20: direct_solve<20, FWD>(A, pt, s, t, dstg); break;
+        case 24: direct_solve<24, FWD>(A, pt, s, t, dstg); break;
+        case 28: direct_solve<28, FWD>(A, pt, s, t, dstg); break;
+        default: direct_solve<FSE_DIRECT_BAND, FWD>(A, pt, s, t, dstg); break;
+    }
+}
+
 // Velocity-dependent elements (C_t = d f_nl / d qdot != 0): the right-hand side of the tangent
 // step gains (w 2/D C_t(k+1)) X_k + w (C_t(k+1) - C_t(k)) V_k (the linearised equation of motion of
 // step k eliminates the acceleration tangent as in the C_t = 0 case, and the velocity tangent of
@@ -968,6 +1098,13 @@ static void sens_launch(fse_ctx* c, SensArgs& A, int phase, cudaStream_t st) {
             case 3: rhs_launch<T, 3>(c, A, st); break;
             default: rhs_launch<T, 4>(c, A, st); break;
         }
+    } else if (use_direct(p)) {
+        const dim3 g = tile_grid(p, A, 128);
+        const size_t smem = (size_t)2 * DSC * (p.b <= 8 ? p.b + 2 : ((p.b + 3) & ~3) + 2) * 8;
+        if (phase == 1)
+            k_direct<true><<<g, 128, smem, st>>>(A);
+        else
+            k_direct<false><<<g, 128, smem, st>>>(A);
     } else if (p.b <= 96) {
         static std::atomic<unsigned long long> attr8{0};
         if (needs_device_setup(attr8)) {
@@ -1034,6 +1171,7 @@ void launch_sens_phase(fse_ctx* c, int k, double w, int phase, cudaStream_t st) 
     A.romega = (const char*)c->d.romega + f * vsz;
     A.Lc = (const char*)c->d.Lc + f * fsz;                             // factor of K_eff(q_{k+1})
     A.Lr = (const char*)c->d.Lr + f * fsz;
+    A.Linv = (const char*)c->d.Linv + f * vsz;
     A.Dinv = (const char*)c->d.Dinv + f * dsz;
     const size_t rsz = (size_t)p.N * p.nblk * p.RECE * tsz;
     A.Rf = (const char*)c->d.Rf + f * rsz;

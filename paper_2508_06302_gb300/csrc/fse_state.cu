@@ -720,7 +720,7 @@ struct StateArgs {
     double *q, *u, *a;
     const void *cLc, *cLr, *cLinv, *cDinv;   // chord factor (regular steps)
     void *oLc, *oLr, *oLinv, *oDinv;         // factor of K_eff at the new state
-    void *oRf, *oRb;                         // its block records for the tangent solves
+    void *oRf, *oRb;                         // its block records for the tangent solves (null: not used)
     const void *cRf, *cRb;                   // records of the chord factor (panel factor: the chord
                                              // solves read them instead of the bands)
     int full_factor;                         // panel factor: also write the bands, 1/L_jj and the block
@@ -753,10 +753,11 @@ __device__ int band_factor(const StateArgs& A, T* Ac, T* Lr, T* Linv, T* Dinv, T
             bad = cta_band_cholesky_blk(Ac + o, Lr + o, Linv + r0, Dinv + dof, n, A.b, wnd, Rf + ro, Rb + ro, A.RECE,
                                         A.full_factor != 0, src);
         } else {
-            bad = band_cholesky<T>(Ac + o, Lr + o, Linv + r0, n, A.b, wnd, stg, Rf + ro, Rb + ro, A.RECE);
+            T *rf = Rf ? Rf + ro : nullptr, *rb = Rb ? Rb + ro : nullptr;
+            bad = band_cholesky<T>(Ac + o, Lr + o, Linv + r0, n, A.b, wnd, stg, rf, rb, A.RECE);
             if (!bad)
-                cta_diag_inverses<T>(Lr + o, Linv + r0, n, A.b, (n + FSE_BLK - 1) / FSE_BLK, Dinv + dof, wnd, Rf + ro,
-                                     Rb + ro, A.RECE);
+                cta_diag_inverses<T>(Lr + o, Linv + r0, n, A.b, (n + FSE_BLK - 1) / FSE_BLK, Dinv + dof, wnd, rf, rb,
+                                     A.RECE);
         }
         __syncthreads();   // every thread has read the pivot flag before the next panel clears it
     }
@@ -1127,8 +1128,8 @@ __global__ void __launch_bounds__(256, 2) k_state(StateArgs A) {
     T* oLr = reinterpret_cast<T*>(A.oLr) + foff;
     T* oLi = reinterpret_cast<T*>(A.oLinv) + off;
     T* oDi = reinterpret_cast<T*>(A.oDinv) + doff;
-    T* oRf = reinterpret_cast<T*>(A.oRf) + (size_t)s * A.nblk * A.RECE;
-    T* oRb = reinterpret_cast<T*>(A.oRb) + (size_t)s * A.nblk * A.RECE;
+    T* oRf = A.oRf ? reinterpret_cast<T*>(A.oRf) + (size_t)s * A.nblk * A.RECE : nullptr;
+    T* oRb = A.oRb ? reinterpret_cast<T*>(A.oRb) + (size_t)s * A.nblk * A.RECE : nullptr;
     T* kt_out = reinterpret_cast<T*>(A.kt_out) + (size_t)s * A.kt_ld;
     T* ct_out = A.has_vel ? reinterpret_cast<T*>(A.ct_out) + (size_t)s * A.kt_ld : nullptr;
     // sv = w u at the state (sq, su), or, in the step, at u(q) = 2/Delta (q - q_k) - u_k
@@ -1467,8 +1468,8 @@ static StateArgs make_state_args(fse_ctx* c, double w, int init, int k) {
     A.oLinv = (char*)c->d.Linv + fo * vsz;
     A.oDinv = (char*)c->d.Dinv + fo * dsz;
     const size_t rsz = (size_t)p.N * p.nblk * p.RECE * tsz;
-    A.oRf = (char*)c->d.Rf + fo * rsz;
-    A.oRb = (char*)c->d.Rb + fo * rsz;
+    A.oRf = use_direct(p) ? nullptr : (char*)c->d.Rf + fo * rsz;
+    A.oRb = use_direct(p) ? nullptr : (char*)c->d.Rb + fo * rsz;
     A.cRf = (char*)c->d.Rf + fi * rsz;
     A.cRb = (char*)c->d.Rb + fi * rsz;
     A.full_factor = use_tc(c) ? 1 : 0;
