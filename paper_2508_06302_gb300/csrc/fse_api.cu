@@ -425,7 +425,7 @@ static void rotation_tables(const fse_ctx* c, std::vector<double>& rc, std::vect
 static void free_ctx(fse_ctx* c) {
     if (!c) return;
     void* ptrs[] = {c->d.Mb, c->d.F, c->d.el_type, c->d.el_dof, c->d.el_p, c->d.col_off,
-                    c->d.cs_ptr, c->d.cs_col, c->d.kt_slot, c->d.g_pass, c->d.g_info, c->d.g_rr, c->d.g_map, c->d.g_slot,
+                    c->d.cs_ptr, c->d.cs_col, c->d.sl_ptr, c->d.sl_col, c->d.sl_map, c->d.sl_m, c->d.sl_d, c->d.sl_s, c->d.kt_slot, c->d.g_pass, c->d.g_info, c->d.g_rr, c->d.g_map, c->d.g_slot,
                     c->d.g_rec, c->d.cs_m, c->d.cs_d, c->d.cs_k, c->d.cs_s, c->d.cs_A,
                     c->d.cs_B, c->d.kt_ptr, c->d.kt_col, c->d.kt_soff, c->d.kt_src, c->d.ke,
                     c->d.kt_val, c->d.ce, c->d.ct_val, c->d.romega, c->d.phis, c->d.G, c->d.Gi, c->d.RG, c->d.rc, c->d.rs,
@@ -670,6 +670,23 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
     std::vector<double> Fi((size_t)m->e * ni, 0.0);
     for (int k = 0; k < m->e; ++k)
         for (int i = 0; i < n; ++i) Fi[(size_t)k * ni + num.row_of[i]] = m->F[(size_t)k * n + i];
+    // slices of 32 rows
+    std::vector<int> slptr(p.nblk + 1, 0), slcol, slmap;
+    std::vector<double> slm, sld;
+    for (int B = 0; B < p.nblk; ++B) {
+        int len = 0;
+        for (int i = B * FSE_BLK; i < std::min(ni, (B + 1) * FSE_BLK); ++i) len = std::max(len, cptr[i + 1] - cptr[i]);
+        for (int k = 0; k < len; ++k)
+            for (int i = B * FSE_BLK; i < (B + 1) * FSE_BLK; ++i) {
+                const int e = i < ni && k < cptr[i + 1] - cptr[i] ? cptr[i] + k : -1;
+                slmap.push_back(e);
+                slcol.push_back(e >= 0 ? ccol[e] : std::min(i, ni - 1));
+                slm.push_back(e >= 0 ? cm[e] : 0.0);
+                sld.push_back(e >= 0 ? cd[e] : 0.0);
+            }
+        slptr[B + 1] = (int)slcol.size();
+    }
+    p.nsl = (int)slcol.size();
     std::vector<int> gslot(grp.col.size()), kslot(p.kt_ld, 0);
     for (size_t q = 0; q < grp.col.size(); ++q) gslot[q] = grp.col[q] % p.RW;
     for (size_t q = 0; q < kcol.size(); ++q) kslot[q] = kcol[q] % p.RW;
@@ -703,6 +720,12 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
     A(&c->d.cs_d, (size_t)p.nnz * 8);
     A(&c->d.cs_k, (size_t)p.nnz * 8);
     A(&c->d.cs_s, (size_t)p.nnz * 8);
+    A(&c->d.sl_ptr, slptr.size() * 4);
+    A(&c->d.sl_col, (size_t)p.nsl * 4);
+    A(&c->d.sl_map, (size_t)p.nsl * 4);
+    A(&c->d.sl_m, (size_t)p.nsl * 8);
+    A(&c->d.sl_d, (size_t)p.nsl * 8);
+    A(&c->d.sl_s, (size_t)p.nsl * 8);
     A(&c->d.cs_A, (size_t)p.nnz * tsz);
     A(&c->d.cs_B, (size_t)p.nnz * tsz);
     A(&c->d.kt_ptr, (size_t)(ni + 1) * 4);
@@ -815,6 +838,11 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
     cudaMemcpyAsync(c->d.cs_m, cm.data(), cm.size() * 8, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(c->d.cs_d, cd.data(), cd.size() * 8, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(c->d.cs_k, ck.data(), ck.size() * 8, cudaMemcpyHostToDevice, st);
+    cudaMemcpyAsync(c->d.sl_ptr, slptr.data(), slptr.size() * 4, cudaMemcpyHostToDevice, st);
+    cudaMemcpyAsync(c->d.sl_col, slcol.data(), slcol.size() * 4, cudaMemcpyHostToDevice, st);
+    cudaMemcpyAsync(c->d.sl_map, slmap.data(), slmap.size() * 4, cudaMemcpyHostToDevice, st);
+    cudaMemcpyAsync(c->d.sl_m, slm.data(), slm.size() * 8, cudaMemcpyHostToDevice, st);
+    cudaMemcpyAsync(c->d.sl_d, sld.data(), sld.size() * 8, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(c->d.kt_ptr, kptr.data(), kptr.size() * 4, cudaMemcpyHostToDevice, st);
     if (p.chol_blk) {
         cudaMemcpyAsync(c->d.ktc_ptr, ktc_ptr.data(), ktc_ptr.size() * 4, cudaMemcpyHostToDevice, st);

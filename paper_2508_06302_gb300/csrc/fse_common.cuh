@@ -104,6 +104,31 @@ __device__ __forceinline__ double csr_row(const int* __restrict__ ptr, const int
     return acc;
 }
 
+// The same over rows in slices of 32 (SELL): entry k of the slice's row l at ptr[i / 32] + 32 k + l, the
+// slice filled up with zeros to its longest row, so that a warp's loads are contiguous.  The entries are
+// added in the row's order, as above.
+__device__ __forceinline__ double sell_row(const int* __restrict__ ptr, const int* __restrict__ col,
+                                           const double* __restrict__ val, int i, const double* x) {
+    const int e1 = ptr[(i >> 5) + 1];
+    double acc = 0.0;
+#pragma unroll 4
+    for (int e = ptr[i >> 5] + (i & 31); e < e1; e += 32) acc += val[e] * x[col[e]];
+    return acc;
+}
+// two matrices of the pattern at once: a = A x, b = B y
+__device__ __forceinline__ void sell_row2(const int* __restrict__ ptr, const int* __restrict__ col,
+                                          const double* __restrict__ va, const double* __restrict__ vb, int i,
+                                          const double* x, const double* y, double& a, double& b) {
+    const int e1 = ptr[(i >> 5) + 1];
+    a = b = 0.0;
+#pragma unroll 4
+    for (int e = ptr[i >> 5] + (i & 31); e < e1; e += 32) {
+        const int j = col[e];
+        a += va[e] * x[j];
+        b += vb[e] * y[j];
+    }
+}
+
 // max(a, |b|) for a >= +0, NaN-propagating so that a non-finite value anywhere reaches the convergence
 // test: non-negative doubles are ordered like their bits (infinity and then NaN above the finite ones),
 // and integer compares do not occupy the slow FP64 pipe

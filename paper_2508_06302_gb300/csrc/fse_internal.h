@@ -78,6 +78,10 @@ struct Dev {
     double* cs_d = nullptr;
     double* cs_k = nullptr;
     double* cs_s = nullptr;  // S of Eq. (E7) for the current w_1 (FP64)
+    // M, D, S again in slices of 32 rows (sell_row in fse_common.cuh) for the products of the state
+    // kernel; sl_map: CSR entry of each (-1: filling)
+    int *sl_ptr = nullptr, *sl_col = nullptr, *sl_map = nullptr;
+    double *sl_m = nullptr, *sl_d = nullptr, *sl_s = nullptr;
     void* cs_A = nullptr;    // w^2 4/D^2 M + w 2/D D - K (sensitivity precision)
     void* cs_B = nullptr;    // w^2 4/D M
     // CSR of the K_t pattern and the element-tangent sources of each entry
@@ -174,7 +178,7 @@ struct Params {
     // its DFT sums are then partial and complete only after the reduction across shards
     int N_glob = 0, s0 = 0;
     bool shard = false;
-    int maxit = 0, prec = 0, ncolors = 0, n_el = 0, nnz = 0, nnz_kt = 0, nblk = 0;
+    int maxit = 0, prec = 0, ncolors = 0, n_el = 0, nnz = 0, nsl = 0, nnz_kt = 0, nblk = 0;
     int RW = 0;              // ring rows of the right-hand-side kernel (two passes + 2b)
     int R = 1, ng = 0, nE = 0, ME = 0, RB = 16;   // row groups: rows per group, groups, entries,
                                                   // entries per pass (max), record bytes

@@ -76,6 +76,12 @@ __global__ void k_build_ops(int nnz, double cm, double cd, double cb, const doub
     }
 }
 
+// the slices of S from its CSR values
+__global__ void k_slices(int nsl, const int* __restrict__ map, const double* __restrict__ S, double* sl) {
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nsl; e += gridDim.x * blockDim.x)
+        sl[e] = map[e] >= 0 ? S[map[e]] : 0.0;
+}
+
 // lower column band of S in FP32 for the panel factor: Sband[j (b + 1) + i - j] = S_ij, i >= j (zero
 // elsewhere: the caller clears it first); one thread per row
 __global__ void k_sband(int n, int nb, const int* __restrict__ ptr, const int* __restrict__ col,
@@ -94,6 +100,7 @@ __global__ void k_sband(int n, int nb, const int* __restrict__ ptr, const int* _
 // columns of the band staged ahead of the Cholesky window (cp.async ring)
 #define FSE_CHOL_PF 8
 
+__device__ __forceinline__ bool pivot_in_range(double p);   // p > 0, 2^-100 <= p < 2^100
 // L_jj = sqrt(p) and 1 / L_jj of a pivot, both correctly rounded.  FP64: Newton-Raphson for 1 / sqrt(p)
 // from the FP32 value (x <- x + x (1 - p x^2) / 2 doubles the 23 good bits twice), then Markstein's final
 // corrections (IBM J. Res. Dev. 34, 1990) of the square root, g + (p - g^2) / (2 sqrt p), and of the
@@ -104,8 +111,7 @@ __device__ __forceinline__ void pivot_root(float p, float& ljj, float& inv) {
     inv = 1.0f / ljj;
 }
 __device__ __forceinline__ void pivot_root(double p, double& ljj, double& inv) {
-    const unsigned e = (unsigned)__double2hiint(p) >> 20;   // biased exponent (p > 0)
-    if (e < 1023 - 100 || e >= 1023 + 100) {
+    if (!pivot_in_range(p)) {
         ljj = sqrt(p);
         inv = 1.0 / ljj;
         return;
@@ -117,6 +123,43 @@ __device__ __forceinline__ void pivot_root(double p, double& ljj, double& inv) {
     const double g = p * x;
     ljj = fma(fma(-g, g, p), 0.5 * x, g);
     inv = fma(fma(-ljj, x, 1.0), x, x);
+}
+// FP64 <-> FP32 by integer instructions (values in the FP32 range; conversions run at the FP64 rate)
+__device__ __forceinline__ float narrow_bits(double p) {   // truncated
+    const unsigned hi = (unsigned)__double2hiint(p), lo = (unsigned)__double2loint(p);
+    return __uint_as_float((hi & 0x80000000u) | (((hi & 0x7fffffffu) - 0x38000000u) << 3) | (lo >> 29));
+}
+__device__ __forceinline__ double widen_bits(float f) {
+    const int b = __float_as_int(f);
+    return __hiloint2double(((b >> 3) & 0x8fffffff) + 0x38000000, (int)((unsigned)b << 29));
+}
+__device__ __forceinline__ bool pivot_in_range(double p) {
+    const unsigned e = (unsigned)__double2hiint(p) >> 20;
+    return e >= 1023 - 100 && e < 1023 + 100;
+}
+// 1 / p = x (1 + t): x the FP32 reciprocal, t = e + e^2 with e = 1 - p x (|e| < 2^-22, so the dropped e^3
+// is below the last bit); a product c / p is then c x + c x t, two FP64 operations behind x
+__device__ __forceinline__ void pivot_split_rcp(float p, float& x, float& t) {
+    x = 1.0f / p;
+    t = 0.0f;
+}
+__device__ __forceinline__ void pivot_split_rcp(double p, double& x, double& t) {
+    if (!pivot_in_range(p)) {
+        x = 1.0 / p;
+        t = 0.0;
+        return;
+    }
+    x = widen_bits(1.0f / narrow_bits(p));
+    const double e = fma(-p, x, 1.0);
+    t = fma(e, e, e);
+}
+// 1 / sqrt(p) = y (1 + e / 2 + 3 e^2 / 8) with y the FP32 value and e = 1 - p y^2
+__device__ __forceinline__ float pivot_rsqrt(float p) { return 1.0f / sqrtf(p); }
+__device__ __forceinline__ double pivot_rsqrt(double p) {
+    if (!pivot_in_range(p)) return 1.0 / sqrt(p);
+    const double y = widen_bits(rsqrtf(narrow_bits(p)));
+    const double e = fma(-p * y, y, 1.0);
+    return fma(y, e * fma(e, 0.375, 0.5), y);
 }
 // positive and finite, without FP64 compares
 __device__ __forceinline__ bool good_pivot(float p) { return p > 0.0f && p < INFINITY; }
@@ -131,18 +174,23 @@ __device__ __forceinline__ bool good_pivot(double p) {
 //      j + nb from the cp.async staging ring (entry r was staged by thread r) and stage
 //      column j + nb + PF - 1;
 //  (b) columns j + cc, lanes over the rows: A_(j+cc+rr, j+cc) -= A_(j+cc+rr, j) A_(j+cc, j) / A_(j, j),
-//      rr <= b - cc: warp 0 takes cc = 1 and then forms the next pivot's root and reciprocal, warps
-//      1 .. 7 the other columns in turn.
-// (a) and (b) touch different slots, so one barrier per column suffices.  In FP64 the pivot chain and the
-// FP64 rate (a warp instruction holds its SM partition for 64 clocks) set the pace: with the square root
-// and the divisions in every warp a column took about 2.5 us.
-template <typename T>
+//      rr <= b - cc: warp 0 takes cc = 1 and then prepares the next pivot, warps 1 .. 7 the other
+//      columns in turn.
+// (a) and (b) touch different slots, so one barrier per column suffices.  In FP64 the pivot chain (an FP64
+// result takes some 125 clocks) and the FP64 rate (a warp instruction holds its SM partition for 64 clocks)
+// set the pace.  With the square root and the divisions in every warp a column took about 2.5 us; with
+// correctly rounded root and reciprocal formed once, 1.2 us; with SPLIT, where the update multiplies by an
+// unevaluated reciprocal and warp 7 forms 1 / L_jj beside it, 1.0 us (half-bandwidth 32).  Half-bandwidths
+// up to 8 keep the rounded form: there FP64 contexts serve nearly undamped beams, whose accelerations are
+// limited by the rounding of this factor's solves, and they keep their bits.
+template <typename T, bool SPLIT>
 __device__ int cta_band_cholesky_w(T* Ac, T* Lr, T* Linv, int n, int b, T* wnd, T* stg, T* Rf, T* Rb, int RECE) {
     constexpr int PF = FSE_CHOL_PF;
     const int nb = b + 1, ns = nb + 1;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;   // 8 warps
     __shared__ int s_bad[2];
-    __shared__ T s_inv[2], s_ljj[2];   // of column j at j & 1 (s_bad: its pivot is no good)
+    // of column j at j & 1 (s_bad: its pivot is no good; SPLIT: 1 / pivot = s_x (1 + s_t))
+    __shared__ T s_inv[2], s_ljj[2], s_x[2], s_t[2];
     for (int idx = tid; idx < nb * nb; idx += blockDim.x) {
         const int c = idx / nb;   // column c starts in slot c
         wnd[idx] = (c < n) ? Ac[(size_t)c * nb + (idx - c * nb)] : T(0);
@@ -176,11 +224,14 @@ __device__ int cta_band_cholesky_w(T* Ac, T* Lr, T* Linv, int n, int b, T* wnd, 
     // the pivot of column j, checked (warp 0)
     auto next_pivot = [&](int j, T piv) {
         const bool ok = good_pivot(piv);
-        T ljj, inv;
-        pivot_root(ok ? piv : T(1), ljj, inv);
+        T u, v;
+        if (SPLIT)
+            pivot_split_rcp(ok ? piv : T(1), u, v);
+        else
+            pivot_root(ok ? piv : T(1), u, v);
         if (lane == 0) {
-            s_ljj[j & 1] = ljj;
-            s_inv[j & 1] = inv;
+            (SPLIT ? s_x : s_ljj)[j & 1] = u;
+            (SPLIT ? s_t : s_inv)[j & 1] = v;
             s_bad[j & 1] = !ok;
         }
     };
@@ -192,7 +243,13 @@ __device__ int cta_band_cholesky_w(T* Ac, T* Lr, T* Linv, int n, int b, T* wnd, 
     for (; j < n; ++j) {
         if (s_bad[j & 1]) break;
         const T* colj = wnd + slot * nb;
-        const T inv = s_inv[j & 1], inv2 = inv * inv;
+        // c / pivot for entries c of column j
+        const T pu = SPLIT ? s_x[j & 1] : s_inv[j & 1], pv = SPLIT ? s_t[j & 1] : pu * pu;
+        auto over_pivot = [&](T c) {
+            if (!SPLIT) return c * pv;
+            const T g = c * pu;
+            return fma(g, pv, g);
+        };
         const int sp = (slot == 0) ? ns - 1 : slot - 1;   // slot of column j - 1 = slot of column j + nb
         if (tid < nb) {
             T* colp = wnd + sp * nb;
@@ -213,7 +270,7 @@ __device__ int cta_band_cholesky_w(T* Ac, T* Lr, T* Linv, int n, int b, T* wnd, 
             if (j + 1 < n) {
                 int sc = slot + 1;
                 sc = (sc >= ns) ? 0 : sc;
-                if (ncc >= 1) update(1, colj[1] * inv2);
+                if (ncc >= 1) update(1, over_pivot(colj[1]));
                 __syncwarp();
                 next_pivot(j + 1, wnd[sc * nb]);
             }
@@ -221,11 +278,18 @@ __device__ int cta_band_cholesky_w(T* Ac, T* Lr, T* Linv, int n, int b, T* wnd, 
             // this warp's columns cc = warp + 1 + 7 q: lane q forms the factor of the q-th
             for (int q0 = 0; warp + 1 + 7 * q0 <= ncc; q0 += 32) {
                 const int mine = warp + 1 + 7 * (q0 + lane);
-                const T gl = mine <= ncc ? colj[mine] * inv2 : T(0);
+                const T gl = mine <= ncc ? over_pivot(colj[mine]) : T(0);
                 for (int q = 0; q < 32; ++q) {
                     const int cc = warp + 1 + 7 * (q0 + q);
                     if (cc > ncc) break;
                     update(cc, __shfl_sync(0xffffffffu, gl, q));
+                }
+            }
+            if (SPLIT && warp == 7) {
+                const T piv = colj[0], inv = pivot_rsqrt(piv);
+                if (lane == 0) {
+                    s_inv[j & 1] = inv;
+                    s_ljj[j & 1] = piv * inv;
                 }
             }
         }
@@ -637,7 +701,8 @@ __device__ int band_cholesky(T* Ac, T* Lr, T* Linv, int n, int b, T* wnd, T* stg
             if (nb <= 96) return cta_band_cholesky_r<T, 12, 3>(Ac, Lr, Linv, n, b, wnd, stg, Rf, Rb, RECE);
         }
     }
-    return cta_band_cholesky_w<T>(Ac, Lr, Linv, n, b, wnd, stg, Rf, Rb, RECE);
+    if (sizeof(T) == 8 && b > 8) return cta_band_cholesky_w<T, true>(Ac, Lr, Linv, n, b, wnd, stg, Rf, Rb, RECE);
+    return cta_band_cholesky_w<T, false>(Ac, Lr, Linv, n, b, wnd, stg, Rf, Rb, RECE);
 }
 
 // inverses of the 32 x 32 diagonal blocks of L (one warp per block, one lane per column);
@@ -700,12 +765,15 @@ struct StateArgs {
     int n, b, e, dm1, maxit, ncolors, n_el, nnz_kt, kt_ld, nblk, init;
     Panels pan;
     int skip_lin;       // linear panels keep their factors (steps k >= 1)
+    int sens;           // the evaluation propagates tangents
     int refactor;       // 0: keep the previous factors (residual-only steps, see launch_state_step)
     double tol, Dl, a0c, a1c, a2c, w, phi;
     double rho[FSE_MAX_D - 1];
     const double *F, *phis;
     const int *cs_ptr, *cs_col;
     const double *cs_m, *cs_d, *cs_k, *cs_s;
+    const int *sl_ptr, *sl_col;              // M, D, S in slices of 32 rows
+    const double *sl_m, *sl_d, *sl_s;
     const int *el_type, *el_dof, *col_off;
     const double* el_p;
     const int *kt_ptr, *kt_col, *kt_soff, *kt_src;
@@ -983,91 +1051,69 @@ __device__ void cta_blocked_solve(const T* __restrict__ Lc, const T* __restrict_
 // The same solve for the panel factor (FP32, b <= 96), from the tangent-solve records of the
 // factor: forward record of block B [L(i0 + r, i0 - b + c) at c * 32 + r | Dinv^T at
 // (bpad + k) * 32 + r], backward record [L(i0 + 32 + c, i0 + r) at c * 32 + r | Dinv]; entries
-// outside the band are zero there.  Each block's record (RECE floats) is copied to shared memory
-// by 16-byte cp.async while the previous block computes, into rows padded to 36 floats (ws: two
-// such buffers): the 32 lanes of a warp (4 rows r x 8 record rows c) then read 32 different
-// banks, 4 c + r.
+// outside the band are zero there.  The 2 nblk records are one sequence, forward blocks up and then
+// backward blocks down; each (RECE floats) is copied to shared memory by 16-byte cp.async three blocks
+// ahead (a record comes from L2 or memory and takes longer than a block: with one block ahead a block
+// step took 1200 clocks), into rows padded to 36 floats (ws: four such buffers): the 32 lanes of a warp
+// (4 rows r x 8 record rows c) then read 32 different banks, 4 c + r.
 __device__ void cta_record_solve(const float* __restrict__ Rf, const float* __restrict__ Rb, int RECE, int n, int b,
                                  int nblk, double* r, float* y, float* tmp, float* ws) {
     constexpr int MC = 12;     // band entries per lane (b <= 96)
     constexpr int MAXU = 4;    // 16-byte chunks per thread (RECE <= (96 + 32) * 32 = 4 * 4 * 256)
-    constexpr int RP = 36;
+    constexpr int RP = 36, NBUF = 4;
     const int tid = threadIdx.x, row = tid >> 3, l8 = tid & 7;   // 32 rows x 8 lanes
     const int nrr = RECE / FSE_BLK, dr = nrr - FSE_BLK;          // record rows; first row of the block inverse
-    float* rs[2] = {ws, ws + nrr * RP};
-    auto fetch = [&](const float* R, float* d) {   // record R into the padded buffer d
+    const int nq = 2 * nblk;
+    auto fetch = [&](int q) {   // record q of the sequence into buffer q mod 4
+        if (q < nq) {
+            const float* R = q < nblk ? Rf + (size_t)q * RECE : Rb + (size_t)(nq - 1 - q) * RECE;
+            float* d = ws + (size_t)(q % NBUF) * nrr * RP;
 #pragma unroll
-        for (int u = 0; u < MAXU; ++u) {
-            const int ch = tid + 256 * u;   // floats 4 ch .. 4 ch + 3: record row ch / 8
-            if (4 * ch < RECE) cp_async16(d + (ch >> 3) * RP + 4 * (ch & 7), R + 4 * ch, 16);
+            for (int u = 0; u < MAXU; ++u) {
+                const int ch = tid + 256 * u;   // floats 4 ch .. 4 ch + 3: record row ch / 8
+                if (4 * ch < RECE) cp_async16(d + (ch >> 3) * RP + 4 * (ch & 7), R + 4 * ch, 16);
+            }
         }
         cp_async_commit();
     };
+    for (int q = 0; q < NBUF - 1; ++q) fetch(q);
     for (int i = tid; i < n; i += blockDim.x) y[i] = float(r[i]);
-    // forward: y_B = Dinv_B (r_B - L_{B,<} y_<)
-    fetch(Rf, rs[0]);
-    cp_async_wait0();
+    cp_async_wait<NBUF - 2>();
     __syncthreads();
-    for (int B = 0; B < nblk; ++B) {
-        const int i0 = B * FSE_BLK, i = i0 + row;
-        const float* R = rs[B & 1];
-        if (B + 1 < nblk) fetch(Rf + (size_t)(B + 1) * RECE, rs[(B + 1) & 1]);   // last read at block B - 1
+    for (int q = 0; q < nq; ++q) {
+        const bool fwd = q < nblk;
+        const int B = fwd ? q : nq - 1 - q, i0 = B * FSE_BLK, i = i0 + row;
+        const float* R = ws + (size_t)(q % NBUF) * nrr * RP;
+        fetch(q + NBUF - 1);   // into the buffer last read at step q - 1
+        // forward: y_B = Dinv_B (r_B - L_{B,<} y_<); backward: x_B = Dinv_B^T (y_B - L_{>,B}^T x_>)
+        const int j0 = fwd ? i0 - b : i0 + FSE_BLK;   // row of record row c: j0 + c, in [0, n)
         float part = 0.f;
 #pragma unroll
-        for (int q = 0; q < MC; ++q) {
-            const int c = l8 + 8 * q, j = i0 - b + c;
-            if (c < b && j >= 0) part += R[c * RP + row] * y[j];
+        for (int u = 0; u < MC; ++u) {
+            if (8 * u >= b) break;
+            const int c = l8 + 8 * u, j = j0 + c;
+            if (c < b && j >= 0 && j < n) part += R[c * RP + row] * y[j];
         }
         part += __shfl_xor_sync(0xffffffffu, part, 4);
         part += __shfl_xor_sync(0xffffffffu, part, 2);
         part += __shfl_xor_sync(0xffffffffu, part, 1);
         if (l8 == 0) tmp[row] = (i < n) ? y[i] - part : 0.f;
         __syncthreads();
-        float yv = 0.f;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int k = l8 + 8 * q;
-            yv += R[(dr + k) * RP + row] * tmp[k];
-        }
-        yv += __shfl_xor_sync(0xffffffffu, yv, 4);
-        yv += __shfl_xor_sync(0xffffffffu, yv, 2);
-        yv += __shfl_xor_sync(0xffffffffu, yv, 1);
-        if (l8 == 0 && i < n) y[i] = yv;
-        cp_async_wait0();
-        __syncthreads();
-    }
-    // backward: x_B = Dinv_B^T (y_B - L_{>,B}^T x_>)
-    fetch(Rb + (size_t)(nblk - 1) * RECE, rs[0]);
-    cp_async_wait0();
-    __syncthreads();
-    for (int q2 = 0; q2 < nblk; ++q2) {
-        const int B = nblk - 1 - q2, i0 = B * FSE_BLK, i = i0 + row;
-        const float* R = rs[q2 & 1];
-        if (B > 0) fetch(Rb + (size_t)(B - 1) * RECE, rs[(q2 + 1) & 1]);
-        float part = 0.f;
-#pragma unroll
-        for (int q = 0; q < MC; ++q) {
-            const int c = l8 + 8 * q, k = i0 + FSE_BLK + c;
-            if (c < b && k < n) part += R[c * RP + row] * y[k];
-        }
-        part += __shfl_xor_sync(0xffffffffu, part, 4);
-        part += __shfl_xor_sync(0xffffffffu, part, 2);
-        part += __shfl_xor_sync(0xffffffffu, part, 1);
-        if (l8 == 0) tmp[row] = (i < n) ? y[i] - part : 0.f;
-        __syncthreads();
+        // Dinv is lower triangular and stored whole: forward k <= row, backward k >= row
         float xv = 0.f;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int k = row + l8 + 8 * q;
+        for (int u = 0; u < 4; ++u) {
+            const int k = fwd ? l8 + 8 * u : row + l8 + 8 * u;
             if (k < FSE_BLK) xv += R[(dr + k) * RP + row] * tmp[k];
         }
         xv += __shfl_xor_sync(0xffffffffu, xv, 4);
         xv += __shfl_xor_sync(0xffffffffu, xv, 2);
         xv += __shfl_xor_sync(0xffffffffu, xv, 1);
         if (l8 == 0 && i < n) y[i] = xv;
-        cp_async_wait0();
+        cp_async_wait<NBUF - 2>();   // record q + 1 has landed
         __syncthreads();
     }
+    cp_async_wait0();
     for (int i = tid; i < n; i += blockDim.x) r[i] = (double)y[i];
     __syncthreads();
 }
@@ -1188,9 +1234,11 @@ __global__ void __launch_bounds__(256, 2) k_state(StateArgs A) {
         }
         __syncthreads();
         const double w2 = A.w * A.w;
-        for (int i = tid; i < n; i += nt)
-            sb[i] = forcing_i(A, i, s_cph) + w2 * csr_row(A.cs_ptr, A.cs_col, A.cs_m, i, sr) +
-                    A.w * csr_row(A.cs_ptr, A.cs_col, A.cs_d, i, sqn);
+        for (int i = tid; i < n; i += nt) {
+            double am, ad;
+            sell_row2(A.sl_ptr, A.sl_col, A.sl_m, A.sl_d, i, sr, sqn, am, ad);
+            sb[i] = forcing_i(A, i, s_cph) + w2 * am + A.w * ad;
+        }
         __syncthreads();
         for (int i = tid; i < n; i += nt) sqn[i] = sq[i];   // predictor: the previous displacement
         __syncthreads();
@@ -1203,7 +1251,7 @@ __global__ void __launch_bounds__(256, 2) k_state(StateArgs A) {
             __syncthreads();
         };
         for (it = 0; it < A.maxit; ++it) {
-            for (int i = tid; i < n; i += nt) sr[i] = csr_row(A.cs_ptr, A.cs_col, A.cs_s, i, sqn) - sb[i];
+            for (int i = tid; i < n; i += nt) sr[i] = sell_row(A.sl_ptr, A.sl_col, A.sl_s, i, sqn) - sb[i];
             __syncthreads();
             vel_iterate();
             add_fnl(A, sqn, sv, sr);
@@ -1275,11 +1323,13 @@ __global__ void __launch_bounds__(256, 2) k_state(StateArgs A) {
             A.a[off + i] = an;
         }
         __syncthreads();
-        // w_1 column: -2 w M (a_k + a_{k+1}) - D (u_k + u_{k+1})
+        // w_1 column: -2 w M (a_k + a_{k+1}) - D (u_k + u_{k+1}); only tangents read it
         T* rom = reinterpret_cast<T*>(A.romega) + off;
-        for (int i = tid; i < n; i += nt)
-            rom[i] = T(-2.0 * A.w * csr_row(A.cs_ptr, A.cs_col, A.cs_m, i, sr) -
-                       csr_row(A.cs_ptr, A.cs_col, A.cs_d, i, sb));
+        for (int i = tid; A.sens && i < n; i += nt) {
+            double am, ad;
+            sell_row2(A.sl_ptr, A.sl_col, A.sl_m, A.sl_d, i, sr, sb, am, ad);
+            rom[i] = T(-2.0 * A.w * am - ad);
+        }
         __syncthreads();
     }
     // effective stiffness at the new state, its banded Cholesky factor and block inverses
@@ -1287,7 +1337,7 @@ __global__ void __launch_bounds__(256, 2) k_state(StateArgs A) {
     if (A.refactor) {
         vel_state();
         assemble_keff<T, !BLK>(A, s, sq, sv, oLc, kt_out, ct_out);
-        if (A.has_vel && !A.init) {
+        if (A.has_vel && A.sens && !A.init) {
             // velocity-dependent elements add - C_t(k+1) u_{k+1} - C_t(k) u_k to the w_1 column
             // (d f / d w_1 = C_t u at both ends of the step); sb holds u_k + u_{k+1}, su u_{k+1}
             __syncthreads();
@@ -1327,7 +1377,7 @@ __global__ void k_factor_M(int n, int b, const double* Mb, double* LMc, double* 
         LMc[idx] = (i < n) ? Mb[(size_t)(b - r) * n + i] : 0.0;
     }
     __syncthreads();
-    const int bad = cta_band_cholesky_w<double>(LMc, LMr, LMinv, n, b, wndM, stgM, nullptr, nullptr, 0);
+    const int bad = cta_band_cholesky_w<double, false>(LMc, LMr, LMinv, n, b, wndM, stgM, nullptr, nullptr, 0);
     if (threadIdx.x == 0) *flag = bad;
 }
 
@@ -1366,6 +1416,7 @@ void launch_build_ops(fse_ctx* c, double w) {
     else
         k_build_ops<double><<<g, 256, 0, c->stream>>>(p.nnz, cm, cd, cb, c->d.cs_m, c->d.cs_d, c->d.cs_k,
                                                       c->d.cs_s, (double*)c->d.cs_A, (double*)c->d.cs_B);
+    k_slices<<<nblocks(p.nsl, 256), 256, 0, c->stream>>>(p.nsl, c->d.sl_map, c->d.cs_s, c->d.sl_s);
     if (p.chol_blk) {
         const int nb = p.b + 1;
         cudaMemsetAsync(c->d.Sband, 0, (size_t)p.ni * nb * 4, c->stream);
@@ -1429,6 +1480,11 @@ static StateArgs make_state_args(fse_ctx* c, double w, int init, int k) {
     A.cs_d = c->d.cs_d;
     A.cs_k = c->d.cs_k;
     A.cs_s = c->d.cs_s;
+    A.sl_ptr = c->d.sl_ptr;
+    A.sl_col = c->d.sl_col;
+    A.sl_m = c->d.sl_m;
+    A.sl_d = c->d.sl_d;
+    A.sl_s = c->d.sl_s;
     A.el_type = c->d.el_type;
     A.el_dof = c->d.el_dof;
     A.col_off = c->d.col_off;
@@ -1525,6 +1581,7 @@ void launch_init_state(fse_ctx* c, double w) {
     const size_t tot = (size_t)p.N * p.ni;
     k_split<<<nblocks(tot, 256), 256, 0, c->stream>>>(p.N, p.n, p.ni, c->d.orig_of, c->d.zb, c->d.q, c->d.u);
     StateArgs A = make_state_args(c, w, 1, -1);
+    A.sens = 0;   // the initial call has no step to differentiate
     A.refactor = 1;
     if (p.prec == FSE_MIXED_FP32)
         state_launch<float>(c, A, c->stream);
@@ -1539,6 +1596,7 @@ void launch_init_state(fse_ctx* c, double w) {
 // of k_state still reacts to a slow contraction.
 void launch_state_step(fse_ctx* c, int k, double w, cudaStream_t st, bool sens) {
     StateArgs A = make_state_args(c, w, 0, k);
+    A.sens = sens ? 1 : 0;
     A.refactor = (sens || k < 2 || (k & 3) < 2) ? 1 : 0;
     if (c->p.prec == FSE_MIXED_FP32)
         state_launch<float>(c, A, st);
