@@ -420,26 +420,29 @@ __device__ int cta_band_cholesky_r(T* Ac, T* Lr, T* Linv, int n, int b, T* colbu
 
 // Panel (blocked, right-looking) banded Cholesky for FP32 factors, b <= 96, 256 threads.
 // K_eff = L L^T is factored by panels of 32 columns j0 .. j0 + 31:
-//   [L11; L21] = the panel's columns, factored column by column: L11 = chol(A11) for the
-//                32 x 32 diagonal block and L21 = A21 L11^-T for the rows j0 + 32 .. j0 + 31 + b
+//   [L11; L21] = the panel's columns: L11 = chol(A11) for the 32 x 32 diagonal block and
+//                L21 = A21 L11^-T for the rows j0 + 32 .. j0 + 31 + b
 //   A22 -= L21 L21^T   the trailing band
-// The panel is factored by warps 0-4 without a barrier: each factors its own copy of the
-// diagonal block through shuffles and sweeps one row of its own with the same column operations
-// (the rows below the block; for warp 4, rows that start as the identity and end as the columns
-// of L11^-1, the diagonal-block inverse the tangent solves use: x L11^T = e_c gives x = column c
-// of L11^-1).  The trailing update (4 x 4 register tiles, all warps) and two CTA barriers come
-// once per panel, against one barrier per column in the unblocked form.  Warps 5-7 write the
-// previous panel's columns of L out (column band, row band, Linv, block inverse and the tangent-
-// solve records) while the panel is factored; warps 4-7 then stage the columns that the next panel
-// updates first, as the band of S (one FP32 copy for all trajectories) plus the trajectory's K_t
-// and C_t entries of those columns: K_eff is never assembled in global memory.
+// Sweep (warps 0-4, chb_panel): warp 0 factors the diagonal block in four sub-panels of 8 columns, a row
+// per lane, and hands each sub-panel of L11 on through shared memory; warps 1-4 apply it to a row of
+// their own (the <= 96 rows below the block; for warp 4 rows that start as the identity and end as the
+// columns of L11^-1, the diagonal-block inverse the tangent solves use: x L11^T = e_c gives x = column c
+// of L11^-1).  Meanwhile warps 5-7 stage the columns that this panel's update is the first to touch, as
+// the band of S (one FP32 copy for all trajectories) plus the trajectory's K_t and C_t entries of those
+// columns: K_eff is never assembled in global memory.  Then, after one CTA barrier, all warps update the
+// trailing band (4 x 4 register tiles) and copy L21 and L11^-1 to the solve records, which are plain
+// blocks of them; a second barrier ends the panel.
+// A panel is a chain of 32 pivots, so the sweep is what counts.  With every warp factoring its own copy of
+// the block (32 steps over 64 registers, a broadcast through shared memory each) a panel took 28 k clocks
+// on the 1872-dof shell, 18-26 k of them the sweep and as many the scattered write-out beside it; its
+// residual evaluation of 48 steps went from 33.1 to 26.2 ms.
 // Shared workspace (floats): a ring of CHB_R columns of the band (column c in slot c mod CHB_R,
-// entry c + r at r), L21 transposed [32][CHB_RP], L11^-1 of two panels [2][32][33], 1/L_jj of
-// two panels, per panel warp two buffers of the current column of L11.
+// entry c + r at r), L21 transposed [32][CHB_RP], L11^-1 [32][33], 1/L_jj [32], L11 [32][CHB_LP].
 constexpr int CHB_R = 160;    // >= b + 64 columns are live at once
 constexpr int CHB_RP = 100;   // row pitch of the transposed L21 (>= b, a multiple of 4)
+constexpr int CHB_LP = 36;    // pitch of L11: [row][column], rows 16-byte aligned
 __host__ __device__ constexpr size_t chol_blk_floats(int nb) {
-    return (size_t)CHB_R * nb + 32 * CHB_RP + 2 * 32 * 33 + 64 + 5 * 64;
+    return (size_t)CHB_R * nb + 32 * CHB_RP + 32 * 33 + 32 * CHB_LP + 32;
 }
 
 // where the panel factor takes K_eff = S + K_t + w (2/Delta) C_t from: the lower band of S (FP32,
@@ -456,74 +459,128 @@ struct ChbSource {
 // column c of the ring: W + (c mod CHB_R) nb
 __device__ __forceinline__ float* chb_col(float* W, int c, int nb) { return W + (size_t)(c % CHB_R) * nb; }
 
-// The panel factor and the trailing update are separate (not inlined) functions: inlined into the
-// panel loop, their 32-entry register arrays were kept in local memory.
-//
-// Panel at column j0 (threads 0-159, five warps, no barrier): every warp factors its own copy of
-// the diagonal block (lane i: row j0 + i, the identity past n) with shuffles, and applies the
-// same column operations to one row of its own: warps 1-3 the rows j0 + 32 .. j0 + 127 below the
-// block (rows past j0 + 31 + nr are zero), warp 4 the identity rows that become the columns of
-// L11^-1.  li[k] gets 1 / L_kk; L goes back into the ring, L21 transposed into P, L11^-1 into
-// Zo[i * 33 + c].  Returns false (warp 0) on a non-positive or non-finite pivot.  (Forming the
-// pivots once and sharing each column through shared memory and a barrier per column measured
-// 3-4x slower: the barrier chain set the pace.)
-__device__ __noinline__ bool chb_panel(int W_o, int li_o, int P_o, int Zo_o, int cb_o, int j0, int jb, int nr, int b,
-                                       int nb) {
-    extern __shared__ float chb_dyn[];   // the kernel's dynamic shared memory: plain shared loads and stores
-    float *W = chb_dyn + W_o, *li = chb_dyn + li_o, *P = chb_dyn + P_o, *Zo = chb_dyn + Zo_o;
-    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
-    float* cbw = chb_dyn + cb_o + w * 64;   // this warp's two buffers for the current column of L11
-    const int ib = 32 * (w - 1) + lane;   // warps 1-3: row j0 + 32 + ib
-    const bool below = w >= 1 && w <= 3 && ib < nr, ident = w == 4;
-    float d[32], a[32];
+// row of 32 registers v -= x[0..7] . (columns K .. K + 7 of rows K + 8 .. 31 of L11): the rank-8 update of a
+// row by a sub-panel; L11 rows are read as broadcasts, 16 bytes at a time
+template <int K>
+__device__ __forceinline__ void chb_rank8(float (&v)[32], const float* L11) {
 #pragma unroll
-    for (int k = 0; k < 32; ++k) {
-        d[k] = (k <= lane && lane < jb && lane - k <= b) ? chb_col(W, j0 + k, nb)[lane - k] : (k == lane ? 1.f : 0.f);
-        a[k] = below ? ((32 + ib - k <= b) ? chb_col(W, j0 + k, nb)[32 + ib - k] : 0.f) : ((ident && k == lane) ? 1.f : 0.f);
+    for (int m = K + 8; m < 32; ++m) {
+        const float4 p = *reinterpret_cast<const float4*>(L11 + m * CHB_LP + K);
+        const float4 q = *reinterpret_cast<const float4*>(L11 + m * CHB_LP + K + 4);
+        float t = v[m];
+        t = fmaf(-v[K], p.x, t);
+        t = fmaf(-v[K + 1], p.y, t);
+        t = fmaf(-v[K + 2], p.z, t);
+        t = fmaf(-v[K + 3], p.w, t);
+        t = fmaf(-v[K + 4], q.x, t);
+        t = fmaf(-v[K + 5], q.y, t);
+        t = fmaf(-v[K + 6], q.z, t);
+        t = fmaf(-v[K + 7], q.w, t);
+        v[m] = t;
     }
+}
+// sub-panel K of the diagonal block (warp 0, lane = row): 8 pivots, each column's entries for the other
+// columns of the sub-panel by shuffles
+template <int K>
+__device__ __forceinline__ bool chb_diag8(float (&d)[32], float* L11, float* li, int lane) {
     bool ok = true;
 #pragma unroll
-    for (int k = 0; k < 32; ++k) {
+    for (int k = K; k < K + 8; ++k) {
         const float piv = __shfl_sync(0xffffffffu, d[k], k);
         ok = ok && (piv > 0.f) && (piv < INFINITY);
         const float inv = rsqrtf(piv);   // 1 / L_kk (FP32 factor: refined by the FP64 residual)
-        const float lk = (lane == k) ? piv * inv : (lane > k ? d[k] * inv : 0.f);
+        const float lk = lane >= k ? d[k] * inv : 0.f;   // lane k: piv / sqrt(piv)
         d[k] = lk;
-        a[k] *= inv;
-        if (w == 0 && lane == k) li[k] = inv;
-        // column k goes through the warp's buffer (k & 1) and comes back as broadcast 16-byte
-        // loads: a quarter of the shared-memory operations of one shuffle per entry.  The
-        // buffer written at step k + 1 was last read at step k - 1, before this __syncwarp.
-        float* cbk = cbw + (k & 1) * 32;
-        cbk[lane] = lk;
-        __syncwarp();
-        const float4* c4 = reinterpret_cast<const float4*>(cbk);
+        if (lane == k) li[k] = inv;
 #pragma unroll
-        for (int g = (k + 1) / 4; g < 8; ++g) {
-            const float4 v = c4[g];   // L(j0 + 4g .. j0 + 4g + 3, j0 + k)
-            const float lv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int m = 4 * g + u;
-                if (m > k) {
-                    d[m] = fmaf(-lk, lv[u], d[m]);
-                    a[m] = fmaf(-a[k], lv[u], a[m]);
-                }
-            }
-        }
+        for (int m = k + 1; m < K + 8; ++m) d[m] = fmaf(-lk, __shfl_sync(0xffffffffu, lk, m), d[m]);
     }
-#pragma unroll
-    for (int k = 0; k < 32; ++k) {
-        if (w == 0) {
-            if (k <= lane && lane < jb && lane - k <= b) chb_col(W, j0 + k, nb)[lane - k] = d[k];
-        } else if (below) {
-            if (32 + ib - k <= b) chb_col(W, j0 + k, nb)[32 + ib - k] = a[k];
-            P[k * CHB_RP + ib] = a[k];
-        } else if (ident) {
-            Zo[k * 33 + lane] = a[k];
-        }
-    }
+    *reinterpret_cast<float4*>(L11 + lane * CHB_LP + K) = make_float4(d[K], d[K + 1], d[K + 2], d[K + 3]);
+    *reinterpret_cast<float4*>(L11 + lane * CHB_LP + K + 4) = make_float4(d[K + 4], d[K + 5], d[K + 6], d[K + 7]);
     return ok;
+}
+// the same sub-panel for a row below the block (or an identity row): 8 substitutions
+template <int K>
+__device__ __forceinline__ void chb_row8(float (&a)[32], const float* L11, const float* li) {
+#pragma unroll
+    for (int k = K; k < K + 8; ++k) {
+        float t = a[k];
+#pragma unroll
+        for (int j = K; j < k; ++j) t = fmaf(-a[j], L11[k * CHB_LP + j], t);
+        a[k] = t * li[k];
+    }
+}
+
+// named barriers 2 .. 5: sub-panel K / 8 of L11 is in shared memory (warp 0 arrives, warps 1-4 wait)
+__device__ __forceinline__ void chb_arrive(int id) { asm volatile("bar.arrive %0, 160;\n" ::"r"(id) : "memory"); }
+__device__ __forceinline__ void chb_wait(int id) { asm volatile("bar.sync %0, 160;\n" ::"r"(id) : "memory"); }
+
+// The panel at column j0 (threads 0-159).  Rows past n of the diagonal block are the identity, rows past
+// j0 + 31 + nr below it zero.  L21 goes transposed into P, L11^-1 into Zo[i * 33 + c], 1 / L_kk into li, and
+// with `back` L11 and L21 also into the ring.  Returns false (warp 0) on a non-positive or non-finite
+// pivot.  Separate, not inlined: inlined into the panel loop its register arrays went to local memory.
+__device__ __noinline__ bool chb_panel(int W_o, int li_o, int P_o, int Zo_o, int L_o, int j0, int jb, int nr, int b,
+                                       int nb, bool back) {
+    extern __shared__ float chb_dyn[];   // the kernel's dynamic shared memory: plain shared loads and stores
+    float *W = chb_dyn + W_o, *li = chb_dyn + li_o, *P = chb_dyn + P_o, *Zo = chb_dyn + Zo_o, *L11 = chb_dyn + L_o;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float v[32];
+    if (w == 0) {
+#pragma unroll
+        for (int k = 0; k < 32; ++k)
+            v[k] = (k <= lane && lane < jb && lane - k <= b) ? chb_col(W, j0 + k, nb)[lane - k] : (k == lane ? 1.f : 0.f);
+        bool ok = chb_diag8<0>(v, L11, li, lane);
+        __syncwarp();
+        chb_arrive(2);
+        chb_rank8<0>(v, L11);
+        ok = chb_diag8<8>(v, L11, li, lane) && ok;
+        __syncwarp();
+        chb_arrive(3);
+        chb_rank8<8>(v, L11);
+        ok = chb_diag8<16>(v, L11, li, lane) && ok;
+        __syncwarp();
+        chb_arrive(4);
+        chb_rank8<16>(v, L11);
+        ok = chb_diag8<24>(v, L11, li, lane) && ok;
+        __syncwarp();
+        chb_arrive(5);
+        if (back) {
+#pragma unroll
+            for (int k = 0; k < 32; ++k)
+                if (k <= lane && lane < jb && lane - k <= b) chb_col(W, j0 + k, nb)[lane - k] = v[k];
+        }
+        return ok;
+    }
+    const int ib = 32 * (w - 1) + lane;   // warps 1-3: row j0 + 32 + ib
+    const bool ident = w == 4, below = !ident && ib < nr;
+#pragma unroll
+    for (int k = 0; k < 32; ++k)
+        v[k] = below ? ((32 + ib - k <= b) ? chb_col(W, j0 + k, nb)[32 + ib - k] : 0.f) : ((ident && k == lane) ? 1.f : 0.f);
+    chb_wait(2);
+    chb_row8<0>(v, L11, li);
+    chb_rank8<0>(v, L11);
+    chb_wait(3);
+    chb_row8<8>(v, L11, li);
+    chb_rank8<8>(v, L11);
+    chb_wait(4);
+    chb_row8<16>(v, L11, li);
+    chb_rank8<16>(v, L11);
+    chb_wait(5);
+    chb_row8<24>(v, L11, li);
+    if (ident) {
+#pragma unroll
+        for (int k = 0; k < 32; ++k) Zo[k * 33 + lane] = v[k];
+    } else {
+#pragma unroll
+        for (int k = 0; k < 32; ++k)
+            if (ib < CHB_RP) P[k * CHB_RP + ib] = v[k];   // zero past nr: the records take whole blocks
+        if (back && below) {
+#pragma unroll
+            for (int k = 0; k < 32; ++k)
+                if (32 + ib - k <= b) chb_col(W, j0 + k, nb)[32 + ib - k] = v[k];
+        }
+    }
+    return true;
 }
 
 // A22 -= L21 L21^T over the nr x nr lower triangle of the trailing band: 4 x 4 tiles (ti, tc),
@@ -565,17 +622,17 @@ __device__ __noinline__ void chb_update(int W_o, int P_o, int j0, int nr, int nb
 
 __device__ int cta_band_cholesky_blk(float* Ac, float* Lr, float* Linv, float* Dinv, int n, int b, float* ws,
                                      float* Rf, float* Rb, int RECE, bool full, const ChbSource& src) {
-    const int nb = b + 1;
+    const int nb = b + 1, nblk = (n + FSE_BLK - 1) / FSE_BLK;
     const int tid = threadIdx.x, warp = tid >> 5;
-    float* W = ws;
-    float* P = W + (size_t)CHB_R * nb;   // P[k * CHB_RP + i'] = L(j0 + 32 + i', j0 + k)
-    float* Z = P + 32 * CHB_RP;          // panel q: Z[(q & 1) * 1056 + i * 33 + c] = (L11^-1)(i, c)
-    float* Li = Z + 2 * 32 * 33;         // 1/L_jj of panels of even / odd index
-    float* cb = Li + 64;                 // per panel warp, two buffers of the current column of L11
+    float* L11 = ws;                     // 16-byte aligned parts first
+    float* P = L11 + 32 * CHB_LP;        // P[k * CHB_RP + i'] = L(j0 + 32 + i', j0 + k)
+    float* Z = P + 32 * CHB_RP;          // Z[i * 33 + c] = (L11^-1)(i, c)
+    float* li = Z + 32 * 33;             // 1/L_jj
+    float* W = li + 32;
     // offsets (floats) of the workspace parts in the dynamic shared memory, for the panel bodies
     extern __shared__ float chb_dyn[];
-    const int o_W = (int)(W - chb_dyn), o_P = (int)(P - chb_dyn), o_Z = (int)(Z - chb_dyn), o_Li = (int)(Li - chb_dyn),
-              o_cb = (int)(cb - chb_dyn);
+    const int o_W = (int)(W - chb_dyn), o_P = (int)(P - chb_dyn), o_Z = (int)(Z - chb_dyn), o_li = (int)(li - chb_dyn),
+              o_L = (int)(L11 - chb_dyn);
     __shared__ int bad;
     if (tid == 0) bad = 0;
     // rows i < b of the row band have no columns j < 0
@@ -585,7 +642,7 @@ __device__ int cta_band_cholesky_blk(float* Ac, float* Lr, float* Linv, float* D
     }
     // columns [c0, c1) of K_eff into the ring (zero past n): the band of S, then this trajectory's
     // K_t (and C_t) entries of those columns; threads t0 .. t0 + nthr - 1, either the whole CTA or
-    // warps 4-7, which synchronise on named barrier 1 between the two
+    // warps 5-7, which synchronise on named barrier 1 between the two
     auto stage = [&](int c0, int c1, int t0, int nthr) {
         const int cnt = max(0, c1 - c0) * nb;
         const float* g = src.Sband + (size_t)c0 * nb;
@@ -608,7 +665,7 @@ __device__ int cta_band_cholesky_blk(float* Ac, float* Lr, float* Linv, float* D
         if (nthr == 256)
             __syncthreads();
         else
-            asm volatile("bar.sync 1, 128;\n" ::: "memory");
+            asm volatile("bar.sync 1, 96;\n" ::: "memory");
         if (c1 > c0) {
             const int k1 = src.ktc_ptr[c1];
             for (int k = src.ktc_ptr[c0] + tid - t0; k < k1; k += nthr) {
@@ -619,74 +676,74 @@ __device__ int cta_band_cholesky_blk(float* Ac, float* Lr, float* Linv, float* D
             }
         }
     };
-    // write panel q's columns of L out of the ring; threads t0 .. t0 + nthr - 1
-    auto write_panel = [&](int q, int t0, int nthr) {
-        const int j0 = 32 * q, jb = min(32, n - j0), t = tid - t0;
-        const float* li = Li + (q & 1) * 32;
-        const float* Zq = Z + (q & 1) * 32 * 33;
-        for (int k = 0; full && k < jb; ++k) {   // column band, contiguous
-            const float* src = chb_col(W, j0 + k, nb);
-            float* dst = Ac + (size_t)(j0 + k) * nb;
-            for (int r = t; r < nb; r += nthr) dst[r] = (j0 + k + r < n) ? src[r] : 0.f;
+    // panel q's L21 and L11^-1 to the records (from P and Z: 16-byte stores of whole blocks, zeros where the
+    // band ends), and with `full` its columns to the bands; threads in descending order, since the update
+    // gives the first ones more tiles
+    const int dofs = RECE - FSE_BLK * FSE_BLK;
+    auto write_panel = [&](int q) {
+        const int t = 255 - tid;
+        float* rb = Rb + (size_t)q * RECE;
+        float* rf = Rf + (size_t)q * RECE;
+        // backward record [c][k] = L(j0 + 32 + c, j0 + k)
+        for (int e = t; e < b * 8; e += 256) {
+            const int c = e >> 3, k = 4 * (e & 7);
+            const float* p = P + k * CHB_RP + c;
+            reinterpret_cast<float4*>(rb)[e] = make_float4(p[0], p[CHB_RP], p[2 * CHB_RP], p[3 * CHB_RP]);
         }
-        const int rows = min(n, j0 + 32 + b) - j0;
-        // row band and backward records, j fastest (records only: the rows below the block)
-        for (int idx = t + (full ? 0 : 32 * FSE_BLK); idx < rows * 32; idx += nthr) {
-            const int ip = idx >> 5, k = idx & 31, i = j0 + ip, j = j0 + k, r = ip - k;
-            if (k >= jb || r < 0 || r > b) continue;
-            const float v = chb_col(W, j, nb)[r];
-            if (full) Lr[(size_t)i * nb + (b - r)] = v;
-            if (Rb && ip >= 32) Rb[(size_t)q * RECE + (ip - 32) * FSE_BLK + k] = v;
-        }
-        if (Rf) {
-            const int rb = rows - 32;   // rows below the diagonal block
-            for (int k = 0; k < jb; ++k) {   // forward records, i fastest
-                const int j = j0 + k;
-                const float* src = chb_col(W, j, nb);
-                for (int ii = t; ii < rb; ii += nthr) {
-                    const int i = j0 + 32 + ii, r = i - j, i0 = i & ~(FSE_BLK - 1);
-                    if (r <= b) Rf[(size_t)(i >> 5) * RECE + (j - i0 + b) * FSE_BLK + (i - i0)] = src[r];
-                }
+        // forward records of the blocks u = 1, 2, .. below: [b - 32 u + k][r] = L(j0 + 32 u + r, j0 + k)
+        for (int u = 1; 32 * (u - 1) < b && q + u < nblk; ++u) {
+            const int k0 = max(0, 32 * u - b);
+            float4* o = reinterpret_cast<float4*>(Rf + (size_t)(q + u) * RECE + (b - 32 * u) * FSE_BLK);
+            for (int e = t + 8 * k0; e < 256; e += 256) {
+                const int k = e >> 3, r = 4 * (e & 7);
+                o[e] = *reinterpret_cast<const float4*>(P + k * CHB_RP + 32 * (u - 1) + r);
             }
         }
-        for (int k = t; full && k < jb; k += nthr) Linv[j0 + k] = li[k];
-        float* D = Dinv + (size_t)q * FSE_BLK * FSE_BLK;
-        const int dofs = RECE - FSE_BLK * FSE_BLK;
-        for (int idx = t; idx < FSE_BLK * FSE_BLK; idx += nthr) {
-            const int i = idx >> 5, c = idx & 31;
-            const float z = Zq[i * 33 + c];
-            if (full) D[idx] = z;
-            if (Rf && Rb) {
-                Rb[(size_t)q * RECE + dofs + idx] = z;                 // backward record: Dinv
-                Rf[(size_t)q * RECE + dofs + c * FSE_BLK + i] = z;     // forward record: Dinv^T
+        // the inverse: as it is behind the backward record, transposed behind the forward one
+        {
+            const int i = t >> 3, c = 4 * (t & 7);
+            const float* z = Z + i * 33 + c;
+            reinterpret_cast<float4*>(rb + dofs)[t] = make_float4(z[0], z[1], z[2], z[3]);
+            const float* zt = Z + c * 33 + i;   // Dinv^T row i = column i of Dinv
+            reinterpret_cast<float4*>(rf + dofs)[t] = make_float4(zt[0], zt[33], zt[66], zt[99]);
+        }
+        if (full) {
+            const int j0 = 32 * q, jb = min(32, n - j0);
+            for (int k = 0; k < jb; ++k) {   // column band, contiguous
+                const float* col = chb_col(W, j0 + k, nb);
+                float* dst = Ac + (size_t)(j0 + k) * nb;
+                for (int r = t; r < nb; r += 256) dst[r] = (j0 + k + r < n) ? col[r] : 0.f;
             }
+            const int rows = min(n, j0 + 32 + b) - j0;
+            for (int idx = t; idx < rows * 32; idx += 256) {   // row band, j fastest
+                const int ip = idx >> 5, k = idx & 31, r = ip - k;
+                if (k < jb && r >= 0 && r <= b) Lr[(size_t)(j0 + ip) * nb + (b - r)] = chb_col(W, j0 + k, nb)[r];
+            }
+            for (int k = t; k < jb; k += 256) Linv[j0 + k] = li[k];
+            for (int idx = t; idx < FSE_BLK * FSE_BLK; idx += 256)
+                Dinv[(size_t)q * FSE_BLK * FSE_BLK + idx] = Z[(idx >> 5) * 33 + (idx & 31)];
         }
     };
     stage(0, min(n, 32 + b), 0, 256);
     __syncthreads();
-    const int npan = (n + FSE_BLK - 1) / FSE_BLK;
     int p = 0;
-    for (; p < npan; ++p) {
+    for (; p < nblk; ++p) {
         const int j0 = 32 * p, jb = min(32, n - j0);
         const int nr = max(0, min(n, j0 + 32 + b) - (j0 + 32));   // rows of L21 (<= b)
         if (tid < 160) {
-            const bool ok = chb_panel(o_W, o_Li + (p & 1) * 32, o_P, o_Z + (p & 1) * 32 * 33, o_cb, j0, jb, nr, b, nb);
+            const bool ok = chb_panel(o_W, o_li, o_P, o_Z, o_L, j0, jb, nr, b, nb, full);
             if (tid == 0 && !ok) bad = 1;
-        } else if (p > 0) {
-            write_panel(p - 1, 160, 96);
+        } else {
+            // columns first updated by this panel's successor; their ring slots held panels < p
+            const int c0 = 32 * (p + 1) + b;
+            stage(min(n, c0), min(n, c0 + 32), 160, 96);
         }
         __syncthreads();
         if (bad) break;
-        // columns first updated by panel p + 1; their ring slots held panels < p, written out above
-        if (warp >= 4) {
-            const int c0 = 32 * (p + 1) + b;
-            stage(min(n, c0), min(n, c0 + 32), 128, 128);
-        }
         chb_update(o_W, o_P, j0, nr, nb);
+        write_panel(p);
         __syncthreads();
     }
-    if (p == npan) write_panel(npan - 1, 0, 256);
-    __syncthreads();
     return bad;
 }
 
@@ -716,6 +773,7 @@ __device__ void cta_diag_inverses(const T* Lr, const T* Linv, int n, int b, int 
     for (int B = warp; B < nblk; B += nw) {
         const int i0 = B * FSE_BLK;
         __syncwarp();
+#pragma unroll 16
         for (int idx = lane; idx < FSE_BLK * FSE_BLK; idx += 32) {
             const int i = idx >> 5, j = idx & 31, gi = i0 + i, c = j - i + b;   // row band of L(gi, i0 + j)
             Lt[idx] = (gi < n && j < i && c >= 0) ? Lr[(size_t)gi * nb + c] : T(0);
@@ -1147,8 +1205,9 @@ __device__ void warp_band_solve_fp64(const double* __restrict__ Lc, const double
 }
 
 // BLK: FP32 factor by 32-column panels (the launcher picks it when chol_blk is set)
-template <typename T, bool BLK>
-__global__ void __launch_bounds__(256, 2) k_state(StateArgs A) {
+// MINB CTAs fit on an SM: see state_launch_n
+template <typename T, bool BLK, int MINB>
+__global__ void __launch_bounds__(256, MINB) k_state(StateArgs A) {
     static_assert(!BLK || sizeof(T) == 4, "panel Cholesky is FP32 only");
     const int s = blockIdx.x, n = A.n, b = A.b, nb = b + 1;
     const int tid = threadIdx.x, nt = blockDim.x;
@@ -1542,24 +1601,40 @@ static StateArgs make_state_args(fse_ctx* c, double w, int init, int k) {
     return A;
 }
 
-template <typename T, bool BLK>
+template <typename T, bool BLK, int MINB>
 static void state_launch_k(fse_ctx* c, const StateArgs& A, cudaStream_t st) {
     static std::atomic<unsigned long long> attr_set{0};
     if (needs_device_setup(attr_set)) {
-        cudaFuncSetAttribute(k_state<T, BLK>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+        cudaFuncSetAttribute(k_state<T, BLK, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
         mark_device(attr_set);
     }
-    k_state<T, BLK><<<c->p.N, 256, c->p.smem_state, st>>>(A);
+    k_state<T, BLK, MINB><<<c->p.N, 256, c->p.smem_state, st>>>(A);
+}
+template <typename T, bool BLK>
+static void state_launch_n(fse_ctx* c, const StateArgs& A, cudaStream_t st) {
+    // MINB = 2 (at most 128 registers, some spilled) halves the waves of more trajectories than SMs (243-dof
+    // plate, 256 trajectories) and leaves the FP64 tangent kernels of the previous step room on the same
+    // SMs (447-dof beam, 64 trajectories: 108 ms for 48 steps, 117 with 1; the FP32 ones fill an SM's shared
+    // memory: 540-dof shell 8.9 ms with 2, 7.5 with 1); MINB = 1 keeps the solves in registers where
+    // neither matters (447-dof beam: chord solve 54 us, 93 with 2).  Two fit: shared memory of an SM
+    // is 228 KB with 1 KB kept for each CTA, the static parts take about 2 KB.
+    const Params& p = c->p;
+    size_t ctas = p.N;
+    for (int g = 0; sizeof(T) == 8 && A.sens && g < p.pan.nc; ++g) ctas += (size_t)p.N * ((2 * p.pan.n[g] + 128) / 128);
+    if ((int)std::min<size_t>(ctas, 1 << 30) > num_sms() && 2 * (p.smem_state + 3 * 1024) <= 228 * 1024)
+        state_launch_k<T, BLK, 2>(c, A, st);
+    else
+        state_launch_k<T, BLK, 1>(c, A, st);
 }
 template <typename T>
 static void state_launch(fse_ctx* c, const StateArgs& A, cudaStream_t st) {
     if constexpr (sizeof(T) == 4) {
         if (A.chol_blk) {
-            state_launch_k<float, true>(c, A, st);
+            state_launch_n<float, true>(c, A, st);
             return;
         }
     }
-    state_launch_k<T, false>(c, A, st);
+    state_launch_n<T, false>(c, A, st);
 }
 
 // start points (N x 2n, the caller's dof order) -> q, u in the internal numbering; inert rows zero
