@@ -311,88 +311,199 @@ __global__ void k_border_multi(size_t m, int u, const double* __restrict__ cols,
 // dense LU with partial pivoting (FP64) for the outer Newton step
 // ----------------------------------------------------------------------------
 
-__global__ void k_lu_pivot(double* A, double* bvec, int* piv, int m, int k, int* flag) {
-    __shared__ double sv[1024];
-    __shared__ int si[1024];
-    double best = -1.0;
-    int bi = k;
-    for (int i = k + threadIdx.x; i < m; i += blockDim.x) {
-        const double v = fabs(A[(size_t)i * m + k]);
-        if (v > best) {
-            best = v;
-            bi = i;
+// Blocked right-looking LU of A (m x m, row-major) with the right-hand side b carried along as one more
+// column; L is not kept beyond its panel.  Per panel of LU_NB columns: k_lu_panel (one CTA: pivots, row
+// exchanges and elimination inside the panel), k_lu_rows (the exchanges and L11^-1 on the columns to the
+// right and b), k_lu_update (A22 -= L21 U12, b2 -= L21 u).  A rank-1 update of the whole matrix and three
+// launches per column took 15 us a column on 540 unknowns; now the panel's chain of pivot searches sets
+// the pace: 540 unknowns @LU@.
+// FP64 multiply-adds (m^3 / 3) are the floor of large systems.
+constexpr int LU_NB = 16;
+
+// largest |value| and its smallest row: keys are the bits of |v| (ordered like the values; NaN as 0, so
+// that it is never a pivot while another entry is not)
+__device__ __forceinline__ long long lu_key(double v) {
+    const long long k = __double_as_longlong(v) & 0x7fffffffffffffffll;
+    return k > 0x7ff0000000000000ll ? 0 : k;
+}
+
+// panel rows k .. m - 1, columns k .. k + nb - 1; in shared memory (row pitch LU_NB + 1) when it fits
+__global__ void __launch_bounds__(512) k_lu_panel(double* A, int* piv, int m, int k, int nb, int in_smem, int* flag) {
+    extern __shared__ double sp[];
+    __shared__ long long skey[16];
+    __shared__ int srow[16], s_piv;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, rows = m - k;
+    double* P = in_smem ? sp : A + (size_t)k * m + k;
+    const size_t pitch = in_smem ? LU_NB + 1 : m;
+    if (in_smem) {
+        for (int e = tid; e < rows * LU_NB; e += 512) {
+            const int r = e / LU_NB, c = e % LU_NB;
+            if (c < nb) P[r * pitch + c] = A[(size_t)(k + r) * m + k + c];
         }
+        __syncthreads();
     }
-    sv[threadIdx.x] = best;
-    si[threadIdx.x] = bi;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
-            const double v2 = sv[threadIdx.x + o];
-            const int i2 = si[threadIdx.x + o];
-            if (v2 > sv[threadIdx.x] || (v2 == sv[threadIdx.x] && i2 < si[threadIdx.x])) {
-                sv[threadIdx.x] = v2;
-                si[threadIdx.x] = i2;
+    for (int j = 0; j < nb; ++j) {
+        long long best = -1;
+        int bi = j;
+        for (int r = j + tid; r < rows; r += 512) {
+            const long long v = lu_key(P[r * pitch + j]);
+            if (v > best) {
+                best = v;
+                bi = r;
+            }
+        }
+        auto reduce = [&](int width) {
+            for (int o = width / 2; o > 0; o >>= 1) {
+                const long long v = __shfl_xor_sync(0xffffffffu, best, o);
+                const int i = __shfl_xor_sync(0xffffffffu, bi, o);
+                if (v > best || (v == best && i < bi)) {
+                    best = v;
+                    bi = i;
+                }
+            }
+        };
+        reduce(32);
+        if (lane == 0) {
+            skey[warp] = best;
+            srow[warp] = bi;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            best = lane < 16 ? skey[lane] : -1;
+            bi = lane < 16 ? srow[lane] : j;
+            reduce(32);
+            // exchange rows j and bi of the panel: one lane a column
+            if (bi != j && lane < nb) {
+                const double t = P[j * pitch + lane];
+                P[j * pitch + lane] = P[bi * pitch + lane];
+                P[bi * pitch + lane] = t;
+            }
+            if (lane == 0) {
+                s_piv = bi;
+                piv[k + j] = k + bi;
+                if (best <= 0) *flag = 1;
             }
         }
         __syncthreads();
-    }
-    const int p = si[0];
-    if (threadIdx.x == 0) {
-        piv[k] = p;
-        if (!(sv[0] > 0.0)) *flag = 1;
-    }
-    if (p != k) {
-        for (int c = threadIdx.x; c < m; c += blockDim.x) {
-            const double t = A[(size_t)k * m + c];
-            A[(size_t)k * m + c] = A[(size_t)p * m + c];
-            A[(size_t)p * m + c] = t;
+        const double pv = P[j * pitch + j];
+        for (int r = j + 1 + tid; r < rows; r += 512) {
+            double* p = P + r * pitch;
+            const double l = p[j] / pv;
+            p[j] = l;
+            for (int c = j + 1; c < nb; ++c) p[c] -= l * P[j * pitch + c];
         }
-        if (threadIdx.x == 0) {
-            const double t = bvec[k];
-            bvec[k] = bvec[p];
-            bvec[p] = t;
-        }
-    }
-}
-
-__global__ void k_lu_update(double* A, double* bvec, int m, int k) {
-    const double pv = A[(size_t)k * m + k];
-    const int rows = m - k - 1;
-    const size_t total = (size_t)rows * (m - k);
-    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const int i = k + 1 + (int)(idx / (m - k));
-        const int c = k + (int)(idx % (m - k));
-        const double l = A[(size_t)i * m + k] / pv;
-        if (c == k) {
-            // the multiplier is written after all reads of column k by this row are done
-            continue;
-        }
-        A[(size_t)i * m + c] -= l * A[(size_t)k * m + c];
-        if (c == k + 1) bvec[i] -= l * bvec[k];
-    }
-}
-
-__global__ void k_lu_mult(double* A, int m, int k) {
-    const double pv = A[(size_t)k * m + k];
-    for (int i = k + 1 + blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x)
-        A[(size_t)i * m + k] /= pv;
-}
-
-__global__ void k_back_subst(const double* A, double* x, int m) {
-    // single block, sequential over rows, parallel dot products
-    __shared__ double red[1024];
-    for (int i = m - 1; i >= 0; --i) {
-        double acc = 0.0;
-        for (int c = i + 1 + threadIdx.x; c < m; c += blockDim.x) acc += A[(size_t)i * m + c] * x[c];
-        red[threadIdx.x] = acc;
         __syncthreads();
-        for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-            if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-            __syncthreads();
+    }
+    if (in_smem)
+        for (int e = tid; e < rows * LU_NB; e += 512) {
+            const int r = e / LU_NB, c = e % LU_NB;
+            if (c < nb) A[(size_t)(k + r) * m + k + c] = P[r * pitch + c];
         }
-        if (threadIdx.x == 0) x[i] = (x[i] - red[0]) / A[(size_t)i * m + i];
+}
+
+// columns k + nb .. m - 1 of A and b (column m): the panel's row exchanges, then L11^-1 (unit lower)
+__global__ void __launch_bounds__(128) k_lu_rows(double* A, double* b, const int* __restrict__ piv, int m, int k,
+                                                 int nb) {
+    __shared__ double L[LU_NB][LU_NB];
+    __shared__ int pr[LU_NB];
+    for (int e = threadIdx.x; e < nb * nb; e += 128) L[e / nb][e % nb] = A[(size_t)(k + e / nb) * m + k + e % nb];
+    if (threadIdx.x < nb) pr[threadIdx.x] = piv[k + threadIdx.x];
+    __syncthreads();
+    const int c = k + nb + blockIdx.x * 128 + threadIdx.x;
+    if (c > m) return;
+    double* col = c < m ? A + c : b;
+    const size_t st = c < m ? m : 1;
+    for (int j = 0; j < nb; ++j)
+        if (pr[j] != k + j) {
+            const double t = col[(size_t)(k + j) * st];
+            col[(size_t)(k + j) * st] = col[(size_t)pr[j] * st];
+            col[(size_t)pr[j] * st] = t;
+        }
+    double u[LU_NB];
+#pragma unroll
+    for (int j = 0; j < LU_NB; ++j) u[j] = j < nb ? col[(size_t)(k + j) * st] : 0.0;
+#pragma unroll
+    for (int j = 1; j < LU_NB; ++j) {
+        if (j >= nb) break;
+#pragma unroll
+        for (int i = 0; i < j; ++i) u[j] -= L[j][i] * u[i];
+        col[(size_t)(k + j) * st] = u[j];
+    }
+}
+
+// A22 -= L21 U12, 64 x 64 tiles, 4 x 4 values a thread; the first column of tiles also updates b
+__global__ void __launch_bounds__(256) k_lu_update(double* A, double* b, int m, int k, int nb) {
+    __shared__ double L[LU_NB][65], U[LU_NB][64];   // L transposed
+    const int r0 = k + nb + blockIdx.y * 64, c0 = k + nb + blockIdx.x * 64;
+    for (int e = threadIdx.x; e < 64 * LU_NB; e += 256) {
+        const int r = e / LU_NB, j = e % LU_NB;
+        L[j][r] = (r0 + r < m && j < nb) ? A[(size_t)(r0 + r) * m + k + j] : 0.0;
+        const int j2 = e / 64, c = e % 64;
+        U[j2][c] = (c0 + c < m && j2 < nb) ? A[(size_t)(k + j2) * m + c0 + c] : 0.0;
+    }
+    __syncthreads();
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;   // columns tx + 16 v, rows ty + 16 u
+    double acc[4][4] = {};
+#pragma unroll
+    for (int j = 0; j < LU_NB; ++j) {
+        double l[4], u[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            l[q] = L[j][ty + 16 * q];
+            u[q] = U[j][tx + 16 * q];
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) acc[q][v] += l[q] * u[v];
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const int r = r0 + ty + 16 * q, c = c0 + tx + 16 * v;
+            if (r < m && c < m) A[(size_t)r * m + c] -= acc[q][v];
+        }
+    if (blockIdx.x == 0 && threadIdx.x < 64 && r0 + threadIdx.x < m) {
+        double t = b[r0 + threadIdx.x];
+        for (int j = 0; j < nb; ++j) t -= L[j][threadIdx.x] * b[k + j];
+        b[r0 + threadIdx.x] = t;
+    }
+}
+
+// U x = b in place, one CTA: blocks of 32 rows from the last up; warp 0 solves the 32 x 32 triangle (a
+// row per lane, reciprocals of the diagonal formed together), then all threads subtract its columns from
+// the rows above, two lanes a row
+__global__ void __launch_bounds__(1024) k_back_subst(const double* __restrict__ A, double* x, int m) {
+    __shared__ double xs[32], T[32][33];
+    const int tid = threadIdx.x, lane = tid & 31;
+    for (int k1 = m; k1 > 0; k1 -= 32) {
+        const int k0 = max(0, k1 - 32), nb = k1 - k0;
+        {
+            const int r = tid >> 5;
+            T[r][lane] = (r < nb && lane < nb) ? A[(size_t)(k0 + r) * m + k0 + lane] : (r == lane ? 1.0 : 0.0);
+        }
+        __syncthreads();
+        if (tid < 32) {
+            double v = lane < nb ? x[k0 + lane] : 0.0;
+            const double inv = 1.0 / T[lane][lane];
+            for (int i = 31; i >= 0; --i) {
+                const double xi = __shfl_sync(0xffffffffu, v * inv, i);
+                if (lane == i) v = xi;
+                if (lane < i) v -= T[lane][i] * xi;
+            }
+            xs[lane] = v;
+            if (lane < nb) x[k0 + lane] = v;
+        }
+        __syncthreads();
+        for (int r0 = 0; r0 < k0; r0 += 512) {
+            const int r = r0 + (tid >> 1);
+            double t = 0.0;
+            if (r < k0)
+                for (int j = tid & 1; j < nb; j += 2) t += A[(size_t)r * m + k0 + j] * xs[j];
+            t += __shfl_xor_sync(0xffffffffu, t, 1);
+            if (r < k0 && !(tid & 1)) x[r] -= t;
+        }
         __syncthreads();
     }
 }
@@ -678,13 +789,19 @@ void launch_dense_jac_bordered(fse_ctx* c, int u, const double* cols, const doub
 int dense_lu_solve(fse_ctx* c, double* A, double* bvec, int m) {
     int* flag = c->d.flag + 1;   // zero-pivot flag: the context's second status word
     cudaMemsetAsync(flag, 0, sizeof(int), c->stream);
-    for (int k = 0; k < m; ++k) {
-        k_lu_pivot<<<1, 1024, 0, c->stream>>>(A, bvec, c->piv, m, k, flag);
-        if (k + 1 < m) {
-            const size_t tot = (size_t)(m - k - 1) * (m - k);
-            k_lu_update<<<nblocks(tot, 256, 32), 256, 0, c->stream>>>(A, bvec, m, k);
-            k_lu_mult<<<nblocks(m - k - 1, 256), 256, 0, c->stream>>>(A, m, k);
-        }
+    static std::atomic<unsigned long long> attr{0};
+    if (needs_device_setup(attr)) {
+        cudaFuncSetAttribute(k_lu_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        mark_device(attr);
+    }
+    for (int k = 0; k < m; k += LU_NB) {
+        const int nb = std::min(LU_NB, m - k), rest = m - k - nb;
+        const size_t smem = (size_t)(m - k) * (LU_NB + 1) * 8;
+        const int in_smem = smem <= 200 * 1024;
+        k_lu_panel<<<1, 512, in_smem ? smem : 0, c->stream>>>(A, c->piv, m, k, nb, in_smem, flag);
+        k_lu_rows<<<(rest + 1 + 127) / 128, 128, 0, c->stream>>>(A, bvec, c->piv, m, k, nb);
+        if (rest > 0)
+            k_lu_update<<<dim3((rest + 63) / 64, (rest + 63) / 64), 256, 0, c->stream>>>(A, bvec, m, k, nb);
     }
     k_back_subst<<<1, 1024, 0, c->stream>>>(A, bvec, m);
     int h = 0;
