@@ -429,7 +429,7 @@ static void free_ctx(fse_ctx* c) {
                     c->d.g_rec, c->d.cs_m, c->d.cs_d, c->d.cs_k, c->d.cs_s, c->d.cs_A,
                     c->d.cs_B, c->d.kt_ptr, c->d.kt_col, c->d.kt_soff, c->d.kt_src, c->d.ke,
                     c->d.kt_val, c->d.ce, c->d.ct_val, c->d.romega, c->d.phis, c->d.G, c->d.Gi, c->d.RG, c->d.rc, c->d.rs,
-                    c->d.ktab, c->d.LMc, c->d.LMr, c->d.LMinv, c->d.q, c->d.u, c->d.a, c->d.zb,
+                    c->d.ktab, c->d.LMc, c->d.LMr, c->d.LMinv, c->d.LMd, c->d.q, c->d.u, c->d.a, c->d.zb,
                     c->d.Lc, c->d.Lr, c->d.Linv, c->d.Dinv, c->d.Rf, c->d.Rb, c->d.Tf, c->d.Tb, c->d.X, c->d.V, c->d.Y, c->d.Z0, c->d.R,
                     c->d.vec, c->d.vec2, c->d.yb, c->d.status, c->d.iters, c->d.nref, c->d.flag, c->Jd, c->piv, c->kry, c->kdot,
                     c->ht, c->unk, c->d.row_of, c->d.orig_of, c->d.ap, c->d.red, c->d.redc, c->d.Sband, c->d.ktc_ptr, c->d.ktc_e, c->d.ktc_c, c->d.ktc_r};
@@ -776,6 +776,7 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
     A(&c->d.LMc, lb * 8);
     A(&c->d.LMr, lb * 8);
     A(&c->d.LMinv, (size_t)ni * 8);
+    A(&c->d.LMd, (size_t)p.nblk * FSE_BLK * FSE_BLK * 8);
     A(&c->d.q, Nn * 8);
     A(&c->d.u, Nn * 8);
     A(&c->d.a, Nn * 8);

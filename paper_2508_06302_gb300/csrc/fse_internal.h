@@ -122,6 +122,7 @@ struct Dev {
     double* LMc = nullptr;
     double* LMr = nullptr;
     double* LMinv = nullptr;
+    double* LMd = nullptr;   // inverses of its 32 x 32 diagonal blocks
     // internal numbering: row_of[i] the internal row of dof i (n), orig_of[r] the dof of row r (ni, -1: inert)
     int* row_of = nullptr;
     int* orig_of = nullptr;

@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <type_traits>
 
 #include "fse_common.cuh"
 
@@ -842,7 +843,7 @@ struct StateArgs {
     void* ct_out;       // N x kt_ld, C_t at the new state (same pattern and ring as K_t)
     const void* ct_prev;   // N x kt_ld, C_t at the previous state
     void* romega;       // N x n, w_1-column term of this step (regular steps)
-    const double *LMc, *LMr, *LMinv;
+    const double *LMc, *LMr, *LMinv, *LMd;
     double *q, *u, *a;
     const void *cLc, *cLr, *cLinv, *cDinv;   // chord factor (regular steps)
     void *oLc, *oLr, *oLinv, *oDinv;         // factor of K_eff at the new state
@@ -980,14 +981,14 @@ __device__ void assemble_keff(const StateArgs& A, int s, const double* q, const 
 // off-diagonal band part as dot products (32 rows x 8 lanes); diagonal blocks through their
 // stored inverses.  For b <= 96 the next block's band entries and inverse are loaded into
 // registers while the current block computes.
-template <typename T>
-__device__ void cta_blocked_solve(const T* __restrict__ Lc, const T* __restrict__ Lr,
-                                  const T* __restrict__ Dinv, int n, int b, int nblk, double* r, T* y,
-                                  T* tmp) {
-    constexpr int MC = 12;                                     // band entries per lane (b <= 96)
+// MC: band entries per lane, b <= 8 MC (or b > 96, without the register prefetch).
+template <typename T, int MC>
+__device__ __forceinline__ void cta_blocked_solve_mc(const T* __restrict__ Lc, const T* __restrict__ Lr,
+                                                     const T* __restrict__ Dinv, int n, int b, int nblk, double* r,
+                                                     T* y, T* tmp) {
     const int nb = b + 1;
     const int row = threadIdx.x >> 3, l8 = threadIdx.x & 7;   // 32 rows x 8 lanes
-    const bool pf = b <= 8 * MC;
+    const bool pf = MC < 12 || b <= 8 * MC;
     for (int i = threadIdx.x; i < n; i += blockDim.x) y[i] = T(r[i]);
     __syncthreads();
     T lcur[MC], lnxt[MC], dcur[4], dnxt[4];
@@ -1106,6 +1107,19 @@ __device__ void cta_blocked_solve(const T* __restrict__ Lc, const T* __restrict_
     __syncthreads();
 }
 
+// the register buffers as short as the band allows: twelve entries a lane, two buffers of FP64 pairs, do
+// not fit beside a second CTA's registers
+template <typename T>
+__device__ void cta_blocked_solve(const T* __restrict__ Lc, const T* __restrict__ Lr, const T* __restrict__ Dinv, int n,
+                                  int b, int nblk, double* r, T* y, T* tmp) {
+    if (b <= 8)
+        cta_blocked_solve_mc<T, 1>(Lc, Lr, Dinv, n, b, nblk, r, y, tmp);
+    else if (b <= 32)
+        cta_blocked_solve_mc<T, 4>(Lc, Lr, Dinv, n, b, nblk, r, y, tmp);
+    else
+        cta_blocked_solve_mc<T, 12>(Lc, Lr, Dinv, n, b, nblk, r, y, tmp);
+}
+
 // The same solve for the panel factor (FP32, b <= 96), from the tangent-solve records of the
 // factor: forward record of block B [L(i0 + r, i0 - b + c) at c * 32 + r | Dinv^T at
 // (bpad + k) * 32 + r], backward record [L(i0 + 32 + c, i0 + r) at c * 32 + r | Dinv]; entries
@@ -1145,13 +1159,27 @@ __device__ void cta_record_solve(const float* __restrict__ Rf, const float* __re
         fetch(q + NBUF - 1);   // into the buffer last read at step q - 1
         // forward: y_B = Dinv_B (r_B - L_{B,<} y_<); backward: x_B = Dinv_B^T (y_B - L_{>,B}^T x_>)
         const int j0 = fwd ? i0 - b : i0 + FSE_BLK;   // row of record row c: j0 + c, in [0, n)
+        // operands first, then the sum: with a branch per entry the loads of a lane waited for one another
         float part = 0.f;
+        auto band = [&](auto cnt) {
+            constexpr int C = decltype(cnt)::value;
+            float lv[C], yv[C];
 #pragma unroll
-        for (int u = 0; u < MC; ++u) {
-            if (8 * u >= b) break;
-            const int c = l8 + 8 * u, j = j0 + c;
-            if (c < b && j >= 0 && j < n) part += R[c * RP + row] * y[j];
-        }
+            for (int u = 0; u < C; ++u) {
+                const int c = l8 + 8 * u, j = j0 + c;
+                const bool in = c < b && j >= 0 && j < n;
+                lv[u] = in ? R[c * RP + row] : 0.f;
+                yv[u] = in ? y[j] : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < C; ++u) part += lv[u] * yv[u];
+        };
+        if (b <= 32)
+            band(std::integral_constant<int, 4>());
+        else if (b <= 48)
+            band(std::integral_constant<int, 6>());
+        else
+            band(std::integral_constant<int, MC>());
         part += __shfl_xor_sync(0xffffffffu, part, 4);
         part += __shfl_xor_sync(0xffffffffu, part, 2);
         part += __shfl_xor_sync(0xffffffffu, part, 1);
@@ -1202,6 +1230,17 @@ __device__ void warp_band_solve_fp64(const double* __restrict__ Lc, const double
         }
         __syncwarp();
     }
+}
+
+// M x = r for the consistent start.  Half-bandwidths above 8: the blocked solve with the inverses of the
+// factor's diagonal blocks (1872 rows: 3.5 ms column by column in one warp, 0.3 ms); beams keep the
+// column form, a few columns' work, and with it the bits of their start.
+__device__ __noinline__ void mass_solve(const double* LMc, const double* LMr, const double* LMinv, const double* LMd,
+                                        int n, int b, int nblk, double* r, double* y, double* tmp) {
+    if (b > 8)
+        cta_blocked_solve<double>(LMc, LMr, LMd, n, b, nblk, r, y, tmp);
+    else if (threadIdx.x < 32)
+        warp_band_solve_fp64(LMc, LMr, LMinv, n, b, r);
 }
 
 // BLK: FP32 factor by 32-column panels (the launcher picks it when chol_blk is set)
@@ -1265,7 +1304,7 @@ __global__ void __launch_bounds__(256, MINB) k_state(StateArgs A) {
             sb[i] = forcing_i(A, i, s_cph) - A.w * csr_row(A.cs_ptr, A.cs_col, A.cs_d, i, su) -
                     csr_row(A.cs_ptr, A.cs_col, A.cs_k, i, sq) - sr[i];
         __syncthreads();
-        if (tid < 32) warp_band_solve_fp64(A.LMc, A.LMr, A.LMinv, n, b, sb);
+        mass_solve(A.LMc, A.LMr, A.LMinv, A.LMd, n, b, A.nblk, sb, sqn, sr + n);
         __syncthreads();
         const double iw2 = 1.0 / (A.w * A.w);
         double zmax = 0.0, amax = 0.0;
@@ -1426,7 +1465,7 @@ __global__ void __launch_bounds__(256, MINB) k_state(StateArgs A) {
 // mass factor at setup
 // ----------------------------------------------------------------------------
 
-__global__ void k_factor_M(int n, int b, const double* Mb, double* LMc, double* LMr, double* LMinv,
+__global__ void k_factor_M(int n, int b, const double* Mb, double* LMc, double* LMr, double* LMinv, double* LMd,
                            int* flag) {
     extern __shared__ double wndM[];
     const int nb = b + 1;
@@ -1437,6 +1476,7 @@ __global__ void k_factor_M(int n, int b, const double* Mb, double* LMc, double* 
     }
     __syncthreads();
     const int bad = cta_band_cholesky_w<double, false>(LMc, LMr, LMinv, n, b, wndM, stgM, nullptr, nullptr, 0);
+    if (!bad) cta_diag_inverses<double>(LMr, LMinv, n, b, (n + FSE_BLK - 1) / FSE_BLK, LMd, wndM);
     if (threadIdx.x == 0) *flag = bad;
 }
 
@@ -1490,9 +1530,10 @@ int launch_factor_M(fse_ctx* c) {
     const int nb = p.b + 1;
     int* flag = c->d.flag + 2;   // non-positive pivot of M: the context's third status word
     cudaMemsetAsync(flag, 0, sizeof(int), c->stream);
-    const size_t smem = (size_t)(nb + 1 + FSE_CHOL_PF) * nb * sizeof(double);
+    const size_t smem = std::max((size_t)(nb + 1 + FSE_CHOL_PF) * nb, (size_t)8 * (FSE_BLK * FSE_BLK + FSE_BLK)) *
+                        sizeof(double);
     cudaFuncSetAttribute(k_factor_M, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_factor_M<<<1, 256, smem, c->stream>>>(p.ni, p.b, c->d.Mb, c->d.LMc, c->d.LMr, c->d.LMinv, flag);
+    k_factor_M<<<1, 256, smem, c->stream>>>(p.ni, p.b, c->d.Mb, c->d.LMc, c->d.LMr, c->d.LMinv, c->d.LMd, flag);
     int h = 0;
     cudaMemcpyAsync(&h, flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
     cudaStreamSynchronize(c->stream);
@@ -1571,6 +1612,7 @@ static StateArgs make_state_args(fse_ctx* c, double w, int init, int k) {
     A.LMc = c->d.LMc;
     A.LMr = c->d.LMr;
     A.LMinv = c->d.LMinv;
+    A.LMd = c->d.LMd;
     A.q = c->d.q;
     A.u = c->d.u;
     A.a = c->d.a;
