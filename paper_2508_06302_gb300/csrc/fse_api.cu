@@ -308,7 +308,10 @@ static RowGroups plan_tangents(Params& p, const Numbering& N, const Matrices& X,
             pan.g1[g] = (int)cand.ptr.size() - 1;
             pan.pass0[g + 1] = (pan.g1[g] + FSE_RHS_GPS - 1) / FSE_RHS_GPS;
         }
-        const double cost = (double)cand.col.size() * (4.0 + group_record_bytes(R, tsz) / 16.0);
+        // FP32: shared-memory wavefronts; FP64: its multiply-adds (16 clocks of an SM each) far outweigh
+        // them, and the ones on the zeros of incomplete groups with them
+        const double cost = (double)cand.col.size() *
+                            (4.0 + group_record_bytes(R, tsz) / 16.0 + (tsz == 8 ? 2.0 * 16.0 * R : 0.0));
         if (R == 1 || cost < best) {
             best = cost;
             grp = std::move(cand);

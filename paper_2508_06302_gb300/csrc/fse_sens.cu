@@ -570,8 +570,12 @@ __device__ __forceinline__ void fma2(unsigned long long& d, unsigned long long a
 }
 
 // Blocked banded substitution with 8 x EL register tiles (b <= 96): one CTA = one trajectory
-// x CW = 64 EL directions (256 in FP32, 128 in FP64), 8 warps = 4 row groups of 8 rows x 2
-// column halves.  Each shared-memory read of a solved row feeds 8 rows.  The factor of the
+// x CW = 32 EL NH directions (128 NH in FP32, 64 NH in FP64), 4 NH warps = 4 row groups of 8 rows x NH
+// column groups.  NH = 1 where the ring is 64 rows (b <= 32): two or three CTAs share an SM and one
+// computes while another waits at its two barriers a block or for its rows (243-dof plate, FP32, 256
+// trajectories: forward 92 -> 77 us, backward 117 -> 104).  NH = 2 for wider bands, where the ring of 128
+// rows leaves room for no third CTA and the doubled record traffic costs more (1872-dof shell, b = 44:
+// 0.52 / 0.68 ms with 2, 0.53 / 0.74 with 1).  Each shared-memory read of a solved row feeds 8 rows.  The factor of the
 // block (its band tile and the diagonal-block inverse, one contiguous record written by the
 // state kernel) comes by one bulk copy per block, double-buffered on mbarriers; the next
 // block's right-hand side rows are loaded into registers while the current block computes.
@@ -581,22 +585,23 @@ __device__ __forceinline__ void fma2(unsigned long long& d, unsigned long long a
 // FP32: the products run as packed pairs of rows (fma.rn.f32x2, two IEEE FMAs per instruction,
 // the same results as scalar FMAs with half the issue slots); the ring holds -x so that the band
 // update is one packed FMA per pair.
-template <typename T, bool FWD>
-__global__ void __launch_bounds__(256, 1) k_trsm8(SensArgs A) {
+template <typename T, bool FWD, int NH>
+__global__ void __launch_bounds__(128 * NH, 3 - NH) k_trsm8(SensArgs A) {
     constexpr int EL = 16 / sizeof(T);             // columns per lane
-    constexpr int CW = 64 * EL;                    // columns per CTA
+    constexpr int CW = 32 * EL * NH;               // columns per CTA
     constexpr int RT = 8;                          // rows per thread
     const PanelTile pt = panel_tile(A, blockIdx.x);
     const int n = pt.n, b = A.b, bp = pt.b, ld = pt.ld, RM = A.RWT - 1, RECE = A.RECE;
     const int nblk = (n + FSE_BLK - 1) / FSE_BLK;
     const int s = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // Row group of a warp: the zeros of the band tile and of the diagonal-block inverse are
-    // skipped, so the row groups do unequal work (FWD: b - 8 rg band columns and 8 + 8 rg
-    // diagonal ones); the second column half takes the row groups in reverse order, so the
-    // two warps that share a scheduler (warp and warp + 4) always do the same work in total.
-    const int cg = warp >> 2, rg = cg ? 3 - (warp & 3) : (warp & 3);
+    // skipped, so the row groups do unequal work in each part (FWD: b - 8 rg band columns and 8 + 8 rg
+    // diagonal ones); the second column half, or every other CTA, takes them in reverse order, so that
+    // the warps that share a scheduler do the same work in total.
+    const int cg = NH == 2 ? warp >> 2 : 0;
+    const int rg = (NH == 2 ? cg : blockIdx.x & 1) ? 3 - (warp & 3) : warp & 3;
     const int r0 = RT * rg;                        // first row of this thread in the block
-    const int cl = cg * (CW / 2) + EL * lane;      // first column of this thread in the tile
+    const int cl = cg * 32 * EL + EL * lane;       // first column of this thread in the tile
     const int t = pt.tile * CW + cl;               // column of the panel
     const bool tok = t < ld;
     __shared__ __align__(8) unsigned long long bar[2];
@@ -1073,13 +1078,32 @@ static void rhs_launch(fse_ctx* c, SensArgs& A, cudaStream_t st) {
     k_sens_rhs<T, R><<<g, 32 * (FSE_RHS_GPS + 1), p.smem_rhs, st>>>(A, c->tm);
 }
 
+// working set of the solves with NH = 2 column groups (the size limit of fse_setup)
 size_t trsm_smem(const Params& p) {
     const size_t tsz = p.prec == FSE_MIXED_FP32 ? 4 : 8;
-    if (p.b <= 96) {   // k_trsm8: ring + staging block of CW = 64 x 16 / tsz columns + 2 records
+    if (p.b <= 96) {
         const size_t cw = 64 * (16 / tsz);
         return ((size_t)p.RWT * cw + (size_t)FSE_BLK * cw + 2 * (size_t)p.RECE) * tsz;
     }
     return ((size_t)p.RWT * 128 + 2 * ((size_t)((p.b + 3) & ~3) * 32 + 1024)) * tsz;
+}
+
+template <typename T, int NH>
+static void trsm8_launch(fse_ctx* c, SensArgs& A, int phase, cudaStream_t st) {
+    static std::atomic<unsigned long long> attr{0};
+    if (needs_device_setup(attr)) {
+        cudaFuncSetAttribute(k_trsm8<T, true, NH>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+        cudaFuncSetAttribute(k_trsm8<T, false, NH>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+        mark_device(attr);
+    }
+    const Params& p = c->p;
+    const size_t cw = 32 * NH * (16 / sizeof(T));   // ring + staging block of cw columns + 2 records
+    const dim3 g = tile_grid(p, A, (int)cw);
+    const size_t smem = ((size_t)p.RWT * cw + (size_t)FSE_BLK * cw + 2 * (size_t)p.RECE) * sizeof(T);
+    if (phase == 1)
+        k_trsm8<T, true, NH><<<g, 128 * NH, smem, st>>>(A);
+    else
+        k_trsm8<T, false, NH><<<g, 128 * NH, smem, st>>>(A);
 }
 
 template <typename T>
@@ -1106,17 +1130,10 @@ static void sens_launch(fse_ctx* c, SensArgs& A, int phase, cudaStream_t st) {
         else
             k_direct<false><<<g, 128, smem, st>>>(A);
     } else if (p.b <= 96) {
-        static std::atomic<unsigned long long> attr8{0};
-        if (needs_device_setup(attr8)) {
-            cudaFuncSetAttribute(k_trsm8<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-            cudaFuncSetAttribute(k_trsm8<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-            mark_device(attr8);
-        }
-        const dim3 g = tile_grid(p, A, 64 * (16 / (int)sizeof(T)));
-        if (phase == 1)
-            k_trsm8<T, true><<<g, 256, p.smem_trsm, st>>>(A);
+        if (p.RWT <= 64)
+            trsm8_launch<T, 1>(c, A, phase, st);
         else
-            k_trsm8<T, false><<<g, 256, p.smem_trsm, st>>>(A);
+            trsm8_launch<T, 2>(c, A, phase, st);
     } else {
         // 96 < b <= FSE_MAX_BAND (224): the factor tile of b x 32 values over 256 threads needs
         // MAXL = 28 registers per thread
