@@ -827,14 +827,20 @@ __global__ void __launch_bounds__(128 * NH, 3 - NH) k_trsm8(SensArgs A) {
 // right-hand sides, X_k and V_k are loaded DSR rows ahead.
 // 447-dof beam, b = 5, 64 trajectories: 1.03 / 1.14 -> 0.32 / 0.46 ms (forward / backward with the V
 // update; 0.25 / 0.33 of FP64 work); 360-dof shell 0.34 / 0.31 -> 0.30 / 0.35 ms; 72-dof plate, 19
-// trajectories, 87 / 90 -> 68 / 104 us alone (too few warps for the FP64 pipes, fewer SMs taken from the
-// state kernel: 228 -> 192 us a step).
+// trajectories, 87 / 90 -> 62 / 80 us (H = 2; 68 / 104 with H = 1).
+// H lanes share a direction, each with a part of the window (the solved row and the first entry of the
+// next part travel by shuffle).  A warp's FP64 instructions are 64 clocks apart on its SM partition, so
+// with fewer warps than partitions a row costs b + 2 of them however idle the rest of the chip is; H = 2
+// halves that (72-dof plate, hyper-time form: 16.9 -> 13.7 ms a call).
 constexpr int DSR = 4;    // rows loaded ahead
 constexpr int DSC = 32;   // rows of the factor staged at a time
-template <int B, bool FWD>
-__device__ void direct_solve(const SensArgs& A, const PanelTile& pt, int s, int t, double* stg) {
-    constexpr int BP = (B + 2) & ~1;   // row pitch, even
+template <int B, bool FWD, int H>
+__device__ void direct_solve(const SensArgs& A, const PanelTile& pt, int s, double* stg) {
+    constexpr int W = (B + H - 1) / H;       // window entries of a lane: h W .. h W + W - 1
+    constexpr int BP = (H * W + 2) & ~1;     // row pitch, even
     const int n = pt.n, b = A.b, pb = pt.b, nb = b + 1, ld = pt.ld;
+    const int h = H == 1 ? 0 : threadIdx.x & 1;
+    const int t = pt.tile * (128 / H) + threadIdx.x / H;
     const bool tok = t < ld;
     const size_t fo = (size_t)s * A.n + pt.row0;
     const double* Lb = reinterpret_cast<const double*>(FWD ? A.Lc : A.Lr) + fo * nb;
@@ -863,9 +869,9 @@ __device__ void direct_solve(const SensArgs& A, const PanelTile& pt, int s, int 
         }
         cp_async_commit();
     };
-    double w[B + 1];
+    double w[W + 1];   // w[W]: first entry of the next part
 #pragma unroll
-    for (int k = 0; k <= B; ++k) w[k] = 0.0;
+    for (int k = 0; k <= W; ++k) w[k] = 0.0;
     double yn[DSR], xn[DSR], vn[DSR];
     auto load = [&](int r, int u) {   // processing row r into slot u
         if (tok && r < n) {
@@ -894,23 +900,37 @@ __device__ void direct_solve(const SensArgs& A, const PanelTile& pt, int s, int 
             for (int u = 0; u < DSR; ++u) {
                 if (k0 + u < nr) {
                     const int i = FWD ? k0 + u : nr - 1 - k0 - u;   // row of the chunk
-                    double l[BP];
+                    double l[W + 1], x;
+                    if constexpr (H == 1) {
+                        double lv[BP];
 #pragma unroll
-                    for (int k = 0; k < BP; k += 2) {
-                        const double2 v = *reinterpret_cast<const double2*>(L + i * BP + k);
-                        l[k] = v.x;
-                        l[k + 1] = v.y;
+                        for (int k = 0; k < BP; k += 2) {
+                            const double2 v = *reinterpret_cast<const double2*>(L + i * BP + k);
+                            lv[k] = v.x;
+                            lv[k + 1] = v.y;
+                        }
+#pragma unroll
+                        for (int k = 0; k <= W; ++k) l[k] = lv[k];
+                        x = fma(w[0], l[0], yn[u] * l[0]);
+                    } else {
+                        l[0] = L[i * BP];
+#pragma unroll
+                        for (int k = 1; k <= W; ++k) l[k] = L[i * BP + h * W + k];
+                        x = fma(w[0], l[0], yn[u] * l[0]);   // the first part's is the solved row
+                        x = __shfl_sync(0xffffffffu, x, (threadIdx.x & 31) & ~1);
+                        const double nx = __shfl_sync(0xffffffffu, w[0], (threadIdx.x & 31) | 1);
+                        w[W] = h == 0 ? nx : 0.0;
                     }
-                    const double x = fma(w[0], l[0], yn[u] * l[0]);
 #pragma unroll
-                    for (int k = 0; k < B; ++k) w[k] = fma(-l[k + 1], x, w[k + 1]);
+                    for (int k = 0; k < W; ++k) w[k] = fma(-l[k + 1], x, w[k + 1]);
                     if (tok) {
                         const size_t o = (size_t)(c0 + i) * ld;
                         if (FWD) {
-                            Y[o] = x;
+                            if (h == 0) Y[o] = x;
                         } else {
-                            X[o] = x;
-                            V[o] = fma(a2, x - xn[u], -vn[u]);
+                            const double v = fma(a2, x - xn[u], -vn[u]);
+                            if (h == 0) X[o] = x;
+                            if (h == H - 1) V[o] = v;
                         }
                     }
                     load(r + DSR, u);
@@ -923,27 +943,27 @@ __device__ void direct_solve(const SensArgs& A, const PanelTile& pt, int s, int 
 }
 
 // window sizes: one register window per half-bandwidth would be 32 kernels; every fourth from 8 on
-template <bool FWD>
+template <bool FWD, int H>
 __global__ void __launch_bounds__(128) k_direct(SensArgs A) {
     extern __shared__ __align__(16) double dstg[];
     const PanelTile pt = panel_tile(A, blockIdx.x);
-    const int t = pt.tile * 128 + threadIdx.x, s = blockIdx.y;
+    const int s = blockIdx.y;
     switch (pt.b <= 8 ? pt.b : (pt.b + 3) & ~3) {
-        case 0: direct_solve<0, FWD>(A, pt, s, t, dstg); break;
-        case 1: direct_solve<1, FWD>(A, pt, s, t, dstg); break;
-        case 2: direct_solve<2, FWD>(A, pt, s, t, dstg); break;
-        case 3: direct_solve<3, FWD>(A, pt, s, t, dstg); break;
-        case 4: direct_solve<4, FWD>(A, pt, s, t, dstg); break;
-        case 5: direct_solve<5, FWD>(A, pt, s, t, dstg); break;
-        case 6: direct_solve<6, FWD>(A, pt, s, t, dstg); break;
-        case 7: direct_solve<7, FWD>(A, pt, s, t, dstg); break;
-        case 8: direct_solve<8, FWD>(A, pt, s, t, dstg); break;
-        case 12: direct_solve<12, FWD>(A, pt, s, t, dstg); break;
-        case 16: direct_solve<16, FWD>(A, pt, s, t, dstg); break;
-        case 20: direct_solve<20, FWD>(A, pt, s, t, dstg); break;
-        case 24: direct_solve<24, FWD>(A, pt, s, t, dstg); break;
-        case 28: direct_solve<28, FWD>(A, pt, s, t, dstg); break;
-        default: direct_solve<FSE_DIRECT_BAND, FWD>(A, pt, s, t, dstg); break;
+        case 0: direct_solve<0, FWD, H>(A, pt, s, dstg); break;
+        case 1: direct_solve<1, FWD, H>(A, pt, s, dstg); break;
+        case 2: direct_solve<2, FWD, H>(A, pt, s, dstg); break;
+        case 3: direct_solve<3, FWD, H>(A, pt, s, dstg); break;
+        case 4: direct_solve<4, FWD, H>(A, pt, s, dstg); break;
+        case 5: direct_solve<5, FWD, H>(A, pt, s, dstg); break;
+        case 6: direct_solve<6, FWD, H>(A, pt, s, dstg); break;
+        case 7: direct_solve<7, FWD, H>(A, pt, s, dstg); break;
+        case 8: direct_solve<8, FWD, H>(A, pt, s, dstg); break;
+        case 12: direct_solve<12, FWD, H>(A, pt, s, dstg); break;
+        case 16: direct_solve<16, FWD, H>(A, pt, s, dstg); break;
+        case 20: direct_solve<20, FWD, H>(A, pt, s, dstg); break;
+        case 24: direct_solve<24, FWD, H>(A, pt, s, dstg); break;
+        case 28: direct_solve<28, FWD, H>(A, pt, s, dstg); break;
+        default: direct_solve<FSE_DIRECT_BAND, FWD, H>(A, pt, s, dstg); break;
     }
 }
 
@@ -1123,12 +1143,19 @@ static void sens_launch(fse_ctx* c, SensArgs& A, int phase, cudaStream_t st) {
             default: rhs_launch<T, 4>(c, A, st); break;
         }
     } else if (use_direct(p)) {
-        const dim3 g = tile_grid(p, A, 128);
-        const size_t smem = (size_t)2 * DSC * (p.b <= 8 ? p.b + 2 : ((p.b + 3) & ~3) + 2) * 8;
-        if (phase == 1)
-            k_direct<true><<<g, 128, smem, st>>>(A);
-        else
-            k_direct<false><<<g, 128, smem, st>>>(A);
+        const size_t smem = (size_t)2 * DSC * (p.b <= 8 ? p.b + 3 : ((p.b + 3) & ~3) + 2) * 8;
+        dim3 g = tile_grid(p, A, 128);
+        if (p.b > 4 && (int)(g.x * g.y) <= num_sms()) {   // at most one warp a partition: two lanes a direction
+            g = tile_grid(p, A, 64);
+            if (phase == 1)
+                k_direct<true, 2><<<g, 128, smem, st>>>(A);
+            else
+                k_direct<false, 2><<<g, 128, smem, st>>>(A);
+        } else if (phase == 1) {
+            k_direct<true, 1><<<g, 128, smem, st>>>(A);
+        } else {
+            k_direct<false, 1><<<g, 128, smem, st>>>(A);
+        }
     } else if (p.b <= 96) {
         if (p.RWT <= 64)
             trsm8_launch<T, 1>(c, A, phase, st);

@@ -102,8 +102,10 @@ __global__ void k_sband(int n, int nb, const int* __restrict__ ptr, const int* _
 #define FSE_CHOL_PF 8
 
 __device__ __forceinline__ bool pivot_in_range(double p);   // p > 0, 2^-100 <= p < 2^100
-// L_jj = sqrt(p) and 1 / L_jj of a pivot, both correctly rounded.  FP64: Newton-Raphson for 1 / sqrt(p)
-// from the FP32 value (x <- x + x (1 - p x^2) / 2 doubles the 23 good bits twice), then Markstein's final
+__device__ __forceinline__ float narrow_bits(double p);
+__device__ __forceinline__ double widen_bits(float f);
+// L_jj = sqrt(p) and 1 / L_jj of a pivot, both correctly rounded.  FP64: the FP32 value of 1 / sqrt(p) with
+// the first two terms of its series in e = 1 - p x^2 (22 good bits become 66), then Markstein's final
 // corrections (IBM J. Res. Dev. 34, 1990) of the square root, g + (p - g^2) / (2 sqrt p), and of the
 // reciprocal, x + x (1 - g x): half the FP64 instructions of sqrt and a division one after the other.
 // Outside the FP32 range the library's are used.
@@ -117,10 +119,9 @@ __device__ __forceinline__ void pivot_root(double p, double& ljj, double& inv) {
         inv = 1.0 / ljj;
         return;
     }
-    double x = (double)rsqrtf((float)p);
-    const double hp = 0.5 * p;
-    x = fma(fma(-hp * x, x, 0.5), x, x);
-    x = fma(fma(-hp * x, x, 0.5), x, x);
+    double x = widen_bits(rsqrtf(narrow_bits(p)));
+    const double e = fma(-p * x, x, 1.0);
+    x = fma(x, e * fma(e, 0.375, 0.5), x);
     const double g = p * x;
     ljj = fma(fma(-g, g, p), 0.5 * x, g);
     inv = fma(fma(-ljj, x, 1.0), x, x);
@@ -1370,7 +1371,10 @@ __global__ void __launch_bounds__(256, MINB) k_state(StateArgs A) {
             // enough to tell nonlinearity from rounding, more would only repeat it
             if (tid == 0) {
                 const bool allow = sizeof(T) == 8 || nref == 0;
-                s_next = (!isfinite(dmax) || !isfinite(qmax))                                    ? 2
+                const auto finite = [](double v) {   // v >= +0, by its exponent
+                    return __double2hiint(v) < 0x7ff00000;
+                };
+                s_next = (!finite(dmax) || !finite(qmax))                                        ? 2
                          : (A.tol > 0.0 && dmax <= A.tol * qmax)                                 ? 1
                          : (prev > 0.0 && dmax > 0.1 * prev && it + 1 < A.maxit && allow) ? 3
                                                                                                  : 0;
