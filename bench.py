@@ -214,10 +214,67 @@ def step_work(m, N, band, ld, prec_bytes):
     }
 
 
+def tangent_panels(m, most=4):
+    """The decoupled groups of dofs the tangents are kept in (csrc/fse_internal.h, Panels): components of
+    the coupling graph, up to three of at least n / 16 dofs a panel each, the others together in the last;
+    one panel where less than a quarter of the tangent block would be saved.  Per panel (rows, half-bandwidth, nonzeros of
+    the M, D, K pattern, nonzeros of the K_t pattern)."""
+    n = m.n
+    pat = (m.M != 0) | (m.D != 0) | (m.K != 0)
+    ii, jj = np.nonzero(pat)
+    kt = set()
+    for e in range(m.n_nl):
+        dofs = [int(x) for x in m.nl_dof[e] if x >= 0]
+        kt.update((a, b) for a in dofs for b in dofs)
+    comp = list(range(n))
+
+    def find(i):
+        while comp[i] != i:
+            comp[i] = comp[comp[i]]
+            i = comp[i]
+        return i
+    for a, b in list(zip(ii.tolist(), jj.tolist())) + list(kt):
+        comp[find(a)] = find(b)
+    members = {}
+    for i in range(n):
+        members.setdefault(find(i), []).append(i)
+    groups = sorted(members.values(), key=len, reverse=True)
+    own = 0
+    while own < most - 1 and own < len(groups) and 16 * len(groups[own]) >= n:
+        own += 1
+    groups = [[g] for g in groups[:own]] + ([groups[own:]] if own < len(groups) else [])
+    blocks = lambda k: -(-k // 32) * 32  # noqa: E731
+    rows = [sum(len(c) for c in g) for g in groups]
+    if sum(blocks(r) * (2 * r + 1) for r in rows) > 0.75 * blocks(n) * (2 * n + 1):
+        groups, rows = [[list(range(n))]], [n]
+    out = []
+    for g, r in zip(groups, rows):
+        pos = {i: k for k, i in enumerate(i for c in g for i in c)}
+        inside = [(a, b) for a, b in zip(ii.tolist(), jj.tolist()) if a in pos]
+        kin = [(a, b) for a, b in kt if a in pos]
+        band = max((abs(pos[a] - pos[b]) for a, b in inside + kin), default=0)
+        out.append((r, band, len(inside), len(kin)))
+    return out
+
+
+def panel_work(m, N, prec_bytes):
+    """step_work of the tangents as they are kept, panel by panel: a panel of n rows has 2n + 1 columns
+    and its own half-bandwidth; entries between panels are zero and neither stored nor computed."""
+    out = {"sens_rhs": [0.0, 0.0], "sens_fwd": [0.0, 0.0], "sens_bwd": [0.0, 0.0]}
+    w = prec_bytes
+    for n, b, nnz, nnz_kt in tangent_panels(m):
+        P, tri = 2 * n + 1, n * b - b * (b + 1) / 2
+        for k, fl, words in (("sens_rhs", 2.0 * (2 * nnz + nnz_kt), 3.0), ("sens_fwd", 2.0 * tri, 2.0),
+                             ("sens_bwd", 2.0 * tri + 3.0 * n, 5.0)):
+            out[k][0] += fl * P * N
+            out[k][1] += words * n * P * w * N
+    return {k: tuple(v) for k, v in out.items()}
+
+
 def step_rates(work, traj_steps_per_s, N, hbm_gbs, fp64_tflops=None, bf16_tflops=None):
     """Whole-step rates of the tangent propagation from the measured throughput: the algorithmic
     bytes and flops of the three sensitivity kernels per Newmark step of all N trajectories
-    (`step_work`), over the time of one such step, against the HBM peak and as multiples of the
+    (`panel_work`), over the time of one such step, against the HBM peak and as multiples of the
     FP64 and BF16 tensor peaks (the tangent flops are FP32, so the FP64 ratio exceeds 1; the state
     step's FP64 work, the DFTs and the outer solves are not counted)."""
     t = N / traj_steps_per_s
@@ -578,7 +635,7 @@ def main():
     b = ctx.band
     n, N = m.n, wl.N
     wb = 4 if args.precision == "mixed_fp32" else 8
-    work = step_work(m, N, b, 0, wb)
+    work = panel_work(m, N, wb)
     sm_mhz = clk.get("sm_mhz") or peaks.get("sm_max_mhz", 2070.0)
     lanes = 128 if wb == 4 else 2            # FP32 / FP64 SIMT lanes per SM (FP64: 1/64 of FP32)
     n_sm = torch.cuda.get_device_properties(local).multi_processor_count

@@ -151,9 +151,8 @@ static Numbering own_numbering(int n, int b) {
     return N;
 }
 
-// Numbering by components (pairs: every coupled pair of dofs, comp[i]: a label per component).  The
-// largest components get a panel each, the others share the last one; dofs keep their order inside
-// a component.  nc stays 0 where it does not pay: the panels' tangents (rows in whole blocks x
+// Numbering by components (pairs: every coupled pair of dofs, comp[i]: a label per component).  Large
+// components get a panel each, the others share the last one; dofs keep their order inside a component.  nc stays 0 where it does not pay: the panels' tangents (rows in whole blocks x
 // columns) are what every step streams and solves, and below a quarter saved the inert rows and the
 // shorter blocks cost about as much (n = 24: 3 panels of 32 rows against 1).
 static Numbering component_numbering(const fse_model* m, const std::vector<std::pair<int, int>>& pairs,
@@ -174,7 +173,11 @@ static Numbering component_numbering(const fse_model* m, const std::vector<std::
     if (members.size() < 2) return N;
     std::stable_sort(members.begin(), members.end(),
                      [](const std::vector<int>& a, const std::vector<int>& b) { return a.size() > b.size(); });
-    const int nc = std::min<int>((int)members.size(), FSE_MAX_PANELS);
+    // a panel of its own for components of at least n / 16 dofs (three of them at most), one for the rest
+    int nc = 0;
+    while (nc < FSE_MAX_PANELS - 1 && nc < (int)members.size() && 16 * members[nc].size() >= (size_t)n) ++nc;
+    if (nc < (int)members.size()) ++nc;
+    if (nc < 2) return N;
     N.row_of.assign(n, 0);
     int r = 0;
     double area = 0.0;
