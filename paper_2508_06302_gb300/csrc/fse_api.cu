@@ -431,14 +431,14 @@ static void rotation_tables(const fse_ctx* c, std::vector<double>& rc, std::vect
 static void free_ctx(fse_ctx* c) {
     if (!c) return;
     void* ptrs[] = {c->d.Mb, c->d.F, c->d.el_type, c->d.el_dof, c->d.el_p, c->d.col_off,
-                    c->d.cs_ptr, c->d.cs_col, c->d.sl_ptr, c->d.sl_col, c->d.sl_map, c->d.sl_m, c->d.sl_d, c->d.sl_s, c->d.kt_slot, c->d.g_pass, c->d.g_info, c->d.g_rr, c->d.g_map, c->d.g_slot,
+                    c->d.cs_ptr, c->d.cs_col, c->d.sl_ptr, c->d.sl_m, c->d.kt_slot, c->d.g_pass, c->d.g_info, c->d.g_rr, c->d.g_map, c->d.g_slot,
                     c->d.g_rec, c->d.cs_m, c->d.cs_d, c->d.cs_k, c->d.cs_s, c->d.cs_A,
                     c->d.cs_B, c->d.kt_ptr, c->d.kt_col, c->d.kt_soff, c->d.kt_src, c->d.ke,
                     c->d.kt_val, c->d.ce, c->d.ct_val, c->d.romega, c->d.phis, c->d.G, c->d.Gi, c->d.RG, c->d.rc, c->d.rs,
                     c->d.ktab, c->d.LMc, c->d.LMr, c->d.LMinv, c->d.LMd, c->d.q, c->d.u, c->d.a, c->d.zb,
                     c->d.Lc, c->d.Lr, c->d.Linv, c->d.Dinv, c->d.Rf, c->d.Rb, c->d.Tf, c->d.Tb, c->d.X, c->d.V, c->d.Y, c->d.Z0, c->d.R,
                     c->d.vec, c->d.vec2, c->d.yb, c->d.status, c->d.iters, c->d.nref, c->d.flag, c->Jd, c->piv, c->kry, c->kdot,
-                    c->ht, c->unk, c->d.row_of, c->d.orig_of, c->d.ap, c->d.red, c->d.redc, c->d.Sband, c->d.ktc_ptr, c->d.ktc_e, c->d.ktc_c, c->d.ktc_r};
+                    c->ht, c->unk, c->d.row_of, c->d.ap, c->d.Sband, c->d.ktc_ptr, c->d.ktc_e, c->d.ktc_c, c->d.ktc_r};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (auto& e : c->ev)
@@ -706,8 +706,7 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
         if (e == cudaSuccess) e = dalloc(ptr, bytes);
     };
     A(&c->d.Mb, band * 8);
-    A(&c->d.row_of, (size_t)n * 4);
-    A(&c->d.orig_of, (size_t)ni * 4);
+    A(&c->d.row_of, (size_t)(n + ni) * 4);
     A(&c->d.F, Fi.size() * 8);
     A(&c->d.el_type, (size_t)std::max(1, m->n_nl) * 4);
     A(&c->d.el_dof, (size_t)std::max(1, m->n_nl) * 24);
@@ -726,12 +725,16 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
     A(&c->d.cs_d, (size_t)p.nnz * 8);
     A(&c->d.cs_k, (size_t)p.nnz * 8);
     A(&c->d.cs_s, (size_t)p.nnz * 8);
+    // small arrays share allocations and copies (each costs several microseconds of setup): the index
+    // arrays of the slices [ptr | col | map], their values [m | d | s], the dof maps [row_of | orig_of], and
+    // the products' second pair with the partial sums and counters of the dot products
+    slptr.insert(slptr.end(), slcol.begin(), slcol.end());
+    slptr.insert(slptr.end(), slmap.begin(), slmap.end());
+    slm.insert(slm.end(), sld.begin(), sld.end());
+    std::vector<int> dofmap(num.row_of);
+    dofmap.insert(dofmap.end(), num.orig_of.begin(), num.orig_of.end());
     A(&c->d.sl_ptr, slptr.size() * 4);
-    A(&c->d.sl_col, (size_t)p.nsl * 4);
-    A(&c->d.sl_map, (size_t)p.nsl * 4);
-    A(&c->d.sl_m, (size_t)p.nsl * 8);
-    A(&c->d.sl_d, (size_t)p.nsl * 8);
-    A(&c->d.sl_s, (size_t)p.nsl * 8);
+    A(&c->d.sl_m, (size_t)3 * p.nsl * 8);
     A(&c->d.cs_A, (size_t)p.nnz * tsz);
     A(&c->d.cs_B, (size_t)p.nnz * tsz);
     A(&c->d.kt_ptr, (size_t)(ni + 1) * 4);
@@ -808,9 +811,7 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
     A(&c->d.R, nu * 8);
     A(&c->d.vec, nu * 8);
     A(&c->d.vec2, nu * 8);
-    A(&c->d.ap, 2 * nu * 8);
-    A(&c->d.red, FSE_DOT_VECS * FSE_DOT_BLOCKS * 8);
-    A(&c->d.redc, FSE_DOT_VECS * 4);
+    A(&c->d.ap, (2 * nu + FSE_DOT_VECS * FSE_DOT_BLOCKS) * 8 + FSE_DOT_VECS * 4);
     A(&c->d.status, (size_t)N * 4);
     A(&c->d.iters, (size_t)N * 4);
     A(&c->d.nref, (size_t)N * 4);
@@ -821,10 +822,16 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
         free_ctx(c);
         return rc;
     }
+    c->d.orig_of = c->d.row_of + n;
+    c->d.sl_col = c->d.sl_ptr + p.nblk + 1;
+    c->d.sl_map = c->d.sl_col + p.nsl;
+    c->d.sl_d = c->d.sl_m + p.nsl;
+    c->d.sl_s = c->d.sl_d + p.nsl;
+    c->d.red = c->d.ap + 2 * nu;
+    c->d.redc = (unsigned*)(c->d.red + FSE_DOT_VECS * FSE_DOT_BLOCKS);
     cudaStream_t st = c->stream;
     cudaMemcpyAsync(c->d.Mb, Mb.data(), band * 8, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.row_of, num.row_of.data(), (size_t)n * 4, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.orig_of, num.orig_of.data(), (size_t)ni * 4, cudaMemcpyHostToDevice, st);
+    cudaMemcpyAsync(c->d.row_of, dofmap.data(), dofmap.size() * 4, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(c->d.F, Fi.data(), Fi.size() * 8, cudaMemcpyHostToDevice, st);
     if (m->n_nl > 0) {
         cudaMemcpyAsync(c->d.el_type, et.data(), et.size() * 4, cudaMemcpyHostToDevice, st);
@@ -846,10 +853,7 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
     cudaMemcpyAsync(c->d.cs_d, cd.data(), cd.size() * 8, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(c->d.cs_k, ck.data(), ck.size() * 8, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(c->d.sl_ptr, slptr.data(), slptr.size() * 4, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.sl_col, slcol.data(), slcol.size() * 4, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.sl_map, slmap.data(), slmap.size() * 4, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(c->d.sl_m, slm.data(), slm.size() * 8, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.sl_d, sld.data(), sld.size() * 8, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(c->d.kt_ptr, kptr.data(), kptr.size() * 4, cudaMemcpyHostToDevice, st);
     if (p.chol_blk) {
         cudaMemcpyAsync(c->d.ktc_ptr, ktc_ptr.data(), ktc_ptr.size() * 4, cudaMemcpyHostToDevice, st);
