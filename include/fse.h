@@ -94,6 +94,8 @@ typedef struct fse_ctx fse_ctx;
  * harmonic table (App. B), the sample grid and Gamma / Gamma^-1 (App. D), the
  * rotation R(rho) (Eq. 14) and the banded forms of M, D, K (the half-bandwidth
  * b is detected from the exact zeros of M, D, K and the element dof spans).
+ * Dofs that nothing couples (a flat shell's bending and membrane dofs, say) are found at setup and
+ * their tangents kept apart internally; arguments, results and limits are in the caller's numbering.
  * Allocates all device memory of the context.  Errors: FSE_EINVAL for bad
  * sizes, the sampling rule S_j >= 2 H_j + 1 (Sec. 3.1), e > d, an element dof
  * out of range or a non-positive-definite M (FSE_ENONPOS_PIVOT); FSE_ENOMEM.
