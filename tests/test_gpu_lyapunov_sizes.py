@@ -12,7 +12,8 @@ pytestmark = pytest.mark.gpu
 
 CASES = [  # dofs of the chain, samples, exponents, precision
     (1, 1, 1, "fp64"), (3, 3, 5, "fp64"), (8, 5, 16, "mixed_fp32"), (9, 5, 17, "fp64"), (16, 3, 31, "fp64"),
-    (33, 5, 33, "mixed_fp32"), (40, 3, 64, "fp64"), (67, 3, 2, "fp64"), (2100, 3, 64, "fp64"),
+    (33, 5, 33, "mixed_fp32"), (40, 3, 64, "fp64"), (67, 3, 2, "fp64"), (1500, 3, 64, "mixed_fp32"),
+    (2100, 3, 64, "fp64"),
 ]
 
 
