@@ -48,30 +48,37 @@ __global__ void k_join(int N, int n, int ni, const int* __restrict__ row_of, con
 // 15 M for the 1872-dof shell, 24 us); one warp per output with the lanes over the samples read zb with a
 // stride of 2n.  Few coefficients a thread: the FP64 pipes of an SM's four partitions are only busy with
 // three or more warps on each (243-dof plate, 256 samples x 225 coefficients: 117 us with 116 blocks of
-// 128 x 8).  1872-dof shell 117 -> 33 us, plate 90 -> 66 us.
+// 128 x 8).  1872-dof shell 117 -> 33 us, plate 90 -> 66 us with one chain of additions a coefficient; with
+// four, and six additions over the lanes in k_phi_apply, eight products of the shell take 7.5 ms, not 8.0.
 constexpr int DFT_C = 2, DFT_S = 64, DFT_T = 128;
 __global__ void __launch_bounds__(DFT_T) k_dft_res(int N, int U, int n2, const double* __restrict__ RG,
                                                    const double* __restrict__ zb, const double* __restrict__ Z0,
                                                    double* out, int subtract) {
     __shared__ double rg[DFT_S][DFT_C];
     const int i = blockIdx.x * DFT_T + threadIdx.x, c0 = blockIdx.y * DFT_C;
-    double acc[DFT_C];
+    double acc[DFT_C][4];   // four chains a coefficient: an FP64 sum takes 125 clocks an addend
 #pragma unroll
-    for (int k = 0; k < DFT_C; ++k) acc[k] = 0.0;
+    for (int k = 0; k < DFT_C; ++k)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[k][q] = 0.0;
     for (int s0 = 0; s0 < N; s0 += DFT_S) {
         const int ns = min(DFT_S, N - s0);
         __syncthreads();
-        for (int x = threadIdx.x; x < ns * DFT_C; x += DFT_T) {
-            const int k = x / ns, s = x - k * ns;
-            rg[s][k] = c0 + k < U ? RG[(size_t)(c0 + k) * N + s0 + s] : 0.0;
+        for (int x = threadIdx.x; x < DFT_S * DFT_C; x += DFT_T) {   // zeros past the last sample
+            const int k = x / DFT_S, s = x % DFT_S;
+            rg[s][k] = c0 + k < U && s < ns ? RG[(size_t)(c0 + k) * N + s0 + s] : 0.0;
         }
         __syncthreads();
         if (i < n2) {
-#pragma unroll 8
-            for (int s = 0; s < ns; ++s) {
-                const double z = zb[(size_t)(s0 + s) * n2 + i];
+#pragma unroll 2
+            for (int s = 0; s < ns; s += 4) {
+                double z[4];
 #pragma unroll
-                for (int k = 0; k < DFT_C; ++k) acc[k] += rg[s][k] * z;
+                for (int q = 0; q < 4; ++q) z[q] = s + q < ns ? zb[(size_t)(s0 + s + q) * n2 + i] : 0.0;
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+#pragma unroll
+                    for (int k = 0; k < DFT_C; ++k) acc[k][q] += rg[s + q][k] * z[q];
             }
         }
     }
@@ -79,7 +86,8 @@ __global__ void __launch_bounds__(DFT_T) k_dft_res(int N, int U, int n2, const d
     const size_t o = (size_t)i * U + c0;
 #pragma unroll
     for (int k = 0; k < DFT_C; ++k)
-        if (c0 + k < U) out[o + k] = acc[k] - (subtract ? Z0[o + k] : 0.0);
+        if (c0 + k < U)
+            out[o + k] = ((acc[k][0] + acc[k][1]) + (acc[k][2] + acc[k][3])) - (subtract ? Z0[o + k] : 0.0);
 }
 
 // ----------------------------------------------------------------------------
@@ -157,19 +165,18 @@ __global__ void __launch_bounds__(256) k_phi_apply(PhiView<T> F, const double* _
     for (int j = m4 + lane; j < 2 * m; j += 32)
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[q] += (double)rows[q][j] * zs[j];
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-        for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
-    if (lane == 0) {
-        double* o = zout + (size_t)s * 2 * n;
-        const int ia = F.orig_of[row0 + ra];
-        o[ia] = acc[0];
-        o[n + ia] = acc[1];
-        if (rb < m) {
-            const int ib = F.orig_of[row0 + rb];
-            o[ib] = acc[2];
-            o[n + ib] = acc[3];
-        }
+    // sums over the lanes, six FP64 additions instead of 20: halves of the warp keep two sums each, then
+    // quarters one, so that lanes 8 q .. 8 q + 7 end with sum q
+    const bool up = lane & 16, up2 = lane & 8;
+    double k0 = up ? acc[2] : acc[0], k1 = up ? acc[3] : acc[1];
+    k0 += __shfl_xor_sync(0xffffffffu, up ? acc[0] : acc[2], 16);
+    k1 += __shfl_xor_sync(0xffffffffu, up ? acc[1] : acc[3], 16);
+    double t = up2 ? k1 : k0;
+    t += __shfl_xor_sync(0xffffffffu, up2 ? k0 : k1, 8);
+    for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((lane & 7) == 0) {
+        const int q = lane >> 3, r = q < 2 ? ra : rb;   // X and V row of ra, of rb
+        if (r < m) zout[(size_t)s * 2 * n + (q & 1) * n + F.orig_of[row0 + r]] = t;
     }
 }
 
