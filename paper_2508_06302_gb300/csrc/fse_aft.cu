@@ -586,11 +586,20 @@ __global__ void __launch_bounds__(256) k_lyap_prop(int N, int h, double w, PhiVi
 // its CTAs keeps a slice of the rows in shared memory (B, odd row pitch: a column of 32 rows and a row of
 // 32 columns both hit 32 banks), Q replacing A column by column; a column needs two sums over all rows
 // (the coefficients of each pass, the norm with the second), which the CTAs exchange through distributed
-// shared memory, one cluster barrier a sum.  The 2 m h^2 FP64 multiply-adds at 2 a clock and SM would take one SM 90 us
-// (m = 180, h = 32), so the rows are split even when few; a warp alone has a quarter of that rate (64
-// clocks an FP64 instruction), so sums are kept shallow and nothing is computed by more warps than need it.  With one CTA and a block-wide
-// reduction per coefficient this took 2.3 ms; now 172 us (90-dof shell, h = 32, launch included).  Slices that do not fit in shared memory
-// (beyond m h = 200 k values over 8 CTAs) work in place on A.
+// shared memory, one cluster barrier a sum.  The 2 m h^2 FP64 multiply-adds at 2 a clock and SM would take
+// one SM 90 us (m = 180, h = 32), so the rows are split even when few; a warp alone has a quarter of that
+// rate (64 clocks an FP64 instruction), so sums are kept shallow and nothing is computed by more warps than
+// need it.  With one CTA and a block-wide reduction per coefficient this took 2.3 ms; now 172 us (90-dof
+// shell, h = 32, launch included).  Slices that do not fit in shared memory (beyond m h = 200 k values over
+// 8 CTAs) work in place on A.
+//
+// Barriers between the writes and reads of each shared word: red -> the first barrier of exchange, and its
+// readers are done at the cluster barrier; part -> the cluster barrier, its slot not written again before
+// the cluster barrier of the next exchange; coef -> the last barrier of exchange, its readers are done at
+// the barrier that ends the pass (or the norm branch); s_nrm2 = -1 -> the barriers of pass 0 (c > 0 only:
+// column 0 has no passes and its branch does not ask), s_nrm2 = |a|^2 -> the barrier that ends pass 1 or
+// the norm branch, its readers are done at the barrier that ends the column, as the readers of B are;
+// nrms -> that barrier.
 constexpr int LYQ_T = 256, LYQ_W = LYQ_T / 32;
 __global__ void __launch_bounds__(LYQ_T) k_lyap_qr(int m, int h, int in_smem, double* A, double* Q, double* acc) {
     namespace cg = cooperative_groups;
@@ -624,7 +633,7 @@ __global__ void __launch_bounds__(LYQ_T) k_lyap_qr(int m, int h, int in_smem, do
         __syncthreads();
     };
     for (int c = 0; c < h; ++c) {
-        if (tid == 0) s_nrm2 = -1.0;
+        if (c > 0 && tid == 0) s_nrm2 = -1.0;
         for (int pass = 0; pass < 2 && c > 0; ++pass) {
             // pass 1 also sums the square of the column itself (k = c) that it is about to correct
             for (int k = lane; k < c + pass; k += 32) {   // lanes across the columns, warps across the rows
@@ -655,7 +664,8 @@ __global__ void __launch_bounds__(LYQ_T) k_lyap_qr(int m, int h, int in_smem, do
             }
             __syncthreads();
         }
-        if (s_nrm2 < 0.0) {   // the same in every thread of the cluster: coef is
+        // the same in every thread of the cluster: coef is, and column 0 does not read the flag
+        if (c == 0 || s_nrm2 < 0.0) {
             double d = 0.0;
             for (int i = tid; i < rows; i += LYQ_T) d += B[(size_t)i * bp + c] * B[(size_t)i * bp + c];
             for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
