@@ -190,9 +190,13 @@ __device__ int cta_band_cholesky_w(T* Ac, T* Lr, T* Linv, int n, int b, T* wnd, 
     constexpr int PF = FSE_CHOL_PF;
     const int nb = b + 1, ns = nb + 1;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;   // 8 warps
+    // of column j at j & 1, written by warp 0 in step j - 1 and read in step j, the barrier of step j - 1
+    // between (s_bad: its pivot is no good; SPLIT: 1 / pivot = s_x (1 + s_t))
     __shared__ int s_bad[2];
-    // of column j at j & 1 (s_bad: its pivot is no good; SPLIT: 1 / pivot = s_x (1 + s_t))
-    __shared__ T s_inv[2], s_ljj[2], s_x[2], s_t[2];
+    __shared__ T s_x[2], s_t[2];
+    // of column j at j & 3: read in step j + 1 too (write_col), when warp 0 writes column j + 2's without a
+    // barrier between; written in step j - 1, or with SPLIT by warp 7 in step j
+    __shared__ T s_inv[4], s_ljj[4];
     for (int idx = tid; idx < nb * nb; idx += blockDim.x) {
         const int c = idx / nb;   // column c starts in slot c
         wnd[idx] = (c < n) ? Ac[(size_t)c * nb + (idx - c * nb)] : T(0);
@@ -232,8 +236,8 @@ __device__ int cta_band_cholesky_w(T* Ac, T* Lr, T* Linv, int n, int b, T* wnd, 
         else
             pivot_root(ok ? piv : T(1), u, v);
         if (lane == 0) {
-            (SPLIT ? s_x : s_ljj)[j & 1] = u;
-            (SPLIT ? s_t : s_inv)[j & 1] = v;
+            *(SPLIT ? s_x + (j & 1) : s_ljj + (j & 3)) = u;
+            *(SPLIT ? s_t + (j & 1) : s_inv + (j & 3)) = v;
             s_bad[j & 1] = !ok;
         }
     };
@@ -246,7 +250,7 @@ __device__ int cta_band_cholesky_w(T* Ac, T* Lr, T* Linv, int n, int b, T* wnd, 
         if (s_bad[j & 1]) break;
         const T* colj = wnd + slot * nb;
         // c / pivot for entries c of column j
-        const T pu = SPLIT ? s_x[j & 1] : s_inv[j & 1], pv = SPLIT ? s_t[j & 1] : pu * pu;
+        const T pu = SPLIT ? s_x[j & 1] : s_inv[j & 3], pv = SPLIT ? s_t[j & 1] : pu * pu;
         auto over_pivot = [&](T c) {
             if (!SPLIT) return c * pv;
             const T g = c * pu;
@@ -255,7 +259,7 @@ __device__ int cta_band_cholesky_w(T* Ac, T* Lr, T* Linv, int n, int b, T* wnd, 
         const int sp = (slot == 0) ? ns - 1 : slot - 1;   // slot of column j - 1 = slot of column j + nb
         if (tid < nb) {
             T* colp = wnd + sp * nb;
-            if (j > 0) write_col(j - 1, colp, s_ljj[(j - 1) & 1], s_inv[(j - 1) & 1]);
+            if (j > 0) write_col(j - 1, colp, s_ljj[(j - 1) & 3], s_inv[(j - 1) & 3]);
             cp_async_wait<PF - 2>();   // entry tid of column j + nb has landed
             const int jn = j + nb;
             colp[tid] = (jn < n) ? stg[(jn % PF) * nb + tid] : T(0);
@@ -290,8 +294,8 @@ __device__ int cta_band_cholesky_w(T* Ac, T* Lr, T* Linv, int n, int b, T* wnd, 
             if (SPLIT && warp == 7) {
                 const T piv = colj[0], inv = pivot_rsqrt(piv);
                 if (lane == 0) {
-                    s_inv[j & 1] = inv;
-                    s_ljj[j & 1] = piv * inv;
+                    s_inv[j & 3] = inv;
+                    s_ljj[j & 3] = piv * inv;
                 }
             }
         }
@@ -299,7 +303,7 @@ __device__ int cta_band_cholesky_w(T* Ac, T* Lr, T* Linv, int n, int b, T* wnd, 
         slot = (slot + 1 == ns) ? 0 : slot + 1;
     }
     if (j == n && tid < nb)
-        write_col(n - 1, wnd + ((slot == 0) ? ns - 1 : slot - 1) * nb, s_ljj[(n - 1) & 1], s_inv[(n - 1) & 1]);
+        write_col(n - 1, wnd + ((slot == 0) ? ns - 1 : slot - 1) * nb, s_ljj[(n - 1) & 3], s_inv[(n - 1) & 3]);
     cp_async_wait<0>();
     __syncthreads();
     return j < n;
