@@ -875,8 +875,11 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
     cudaMemsetAsync(c->d.iters, 0, (size_t)N * 4, st);
     cudaMemsetAsync(c->d.nref, 0, (size_t)N * 4, st);
     cudaMemsetAsync(c->d.flag, 0, 16, st);
-    if (ni > n) {   // the column factors leave the inert rows out: L = 1 there
+    if (ni > n) {
+        // the column factors leave the inert rows out, the chord solves pass over them: L = 1 there, with no
+        // entries in the row band nor in the column band (which reaches into the next panel's rows)
         cudaMemsetAsync(c->d.Lr, 0, FSE_NBUF_F * (size_t)N * lb * tsz, st);
+        cudaMemsetAsync(c->d.Lc, 0, FSE_NBUF_F * (size_t)N * lb * tsz, st);
         fse::launch_fill_ones(c, c->d.Linv, FSE_NBUF_F * Nn);
     }
     cudaMemsetAsync(c->d.Rf, 0, FSE_NBUF_F * rsz, st);   // entries outside the band stay zero
