@@ -42,52 +42,55 @@ __global__ void k_join(int N, int n, int ni, const int* __restrict__ row_of, con
     }
 }
 
-// out[i*U + c] = sum_s RG[c][s] zb[s][i] - (subtract ? Z0[i*U + c] : 0): a thread takes one state i and
-// DFT_C coefficients, so that zb is read along i (coalesced, from L2 after the first coefficients) and RG
-// comes as broadcasts from shared memory, staged DFT_S samples at a time.  FP64 FMAs bound it (N U 2n:
-// 15 M for the 1872-dof shell, 24 us); one warp per output with the lanes over the samples read zb with a
-// stride of 2n.  Few coefficients a thread: the FP64 pipes of an SM's four partitions are only busy with
-// three or more warps on each (243-dof plate, 256 samples x 225 coefficients: 117 us with 116 blocks of
-// 128 x 8).  1872-dof shell 117 -> 33 us, plate 90 -> 66 us with one chain of additions a coefficient; with
-// four, and six additions over the lanes in k_phi_apply, eight products of the shell take 7.5 ms, not 8.0.
-constexpr int DFT_C = 2, DFT_S = 64, DFT_T = 128;
-__global__ void __launch_bounds__(DFT_T) k_dft_res(int N, int U, int n2, const double* __restrict__ RG,
-                                                   const double* __restrict__ zb, const double* __restrict__ Z0,
-                                                   double* out, int subtract) {
-    __shared__ double rg[DFT_S][DFT_C];
-    const int i = blockIdx.x * DFT_T + threadIdx.x, c0 = blockIdx.y * DFT_C;
-    double acc[DFT_C][4];   // four chains a coefficient: an FP64 sum takes 125 clocks an addend
-#pragma unroll
-    for (int k = 0; k < DFT_C; ++k)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[k][q] = 0.0;
-    for (int s0 = 0; s0 < N; s0 += DFT_S) {
-        const int ns = min(DFT_S, N - s0);
-        __syncthreads();
-        for (int x = threadIdx.x; x < DFT_S * DFT_C; x += DFT_T) {   // zeros past the last sample
-            const int k = x / DFT_S, s = x % DFT_S;
-            rg[s][k] = c0 + k < U && s < ns ? RG[(size_t)(c0 + k) * N + s0 + s] : 0.0;
-        }
-        __syncthreads();
-        if (i < n2) {
-#pragma unroll 2
-            for (int s = 0; s < ns; s += 4) {
-                double z[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) z[q] = s + q < ns ? zb[(size_t)(s0 + s + q) * n2 + i] : 0.0;
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-#pragma unroll
-                    for (int k = 0; k < DFT_C; ++k) acc[k][q] += rg[s + q][k] * z[q];
-            }
+// out[i*U + c] = sum_s RG[c][s] zb[s][i] - (subtract ? Z0[i*U + c] : 0), in two forms (the launcher chooses).
+// FP64 work bounds large ones (N U 2n multiply-adds: 15 M for the 1872-dof shell, 24 us), the chain of one
+// sum and the launch the small ones, so the samples of a sum are always dealt out.
+//
+// W warps share 32 states i and one coefficient c: lanes along i (zb coalesced, RG a broadcast), each warp a
+// slice of the samples, partial sums through shared memory.  1872-dof shell (64 samples, 63 coefficients)
+// 113 us with one warp per output and its lanes over the samples (zb with a stride of 2n), 31 now; 243-dof
+// plate (256 x 225) 88 -> 53; 36 states, 63 x 63, 2.8 us (15.7 with a thread per state and pair of
+// coefficients over all samples).
+template <int W>
+__global__ void __launch_bounds__(32 * W) k_dft_warps(int N, int U, int n2, const double* __restrict__ RG,
+                                                      const double* __restrict__ zb, const double* __restrict__ Z0,
+                                                      double* out, int subtract) {
+    __shared__ double part[W][32];
+    const int tiles = (n2 + 31) / 32, c = blockIdx.x / tiles;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, i = (blockIdx.x % tiles) * 32 + lane;
+    const int per = (N + W - 1) / W, s0 = warp * per, s1 = min(N, s0 + per);
+    double a = 0.0, b = 0.0;
+    if (i < n2) {
+        const double *z = zb + i, *r = RG + (size_t)c * N;
+        for (int s = s0; s < s1; s += 2) {
+            const bool two = s + 1 < s1;
+            a += r[s] * z[(size_t)s * n2];
+            b += (two ? r[s + 1] : 0.0) * (two ? z[(size_t)(s + 1) * n2] : 0.0);
         }
     }
-    if (i >= n2) return;
-    const size_t o = (size_t)i * U + c0;
+    part[warp][lane] = a + b;
+    __syncthreads();
+    if (warp == 0 && i < n2) {
+        double t = 0.0;
 #pragma unroll
-    for (int k = 0; k < DFT_C; ++k)
-        if (c0 + k < U)
-            out[o + k] = ((acc[k][0] + acc[k][1]) + (acc[k][2] + acc[k][3])) - (subtract ? Z0[o + k] : 0.0);
+        for (int w = 0; w < W; ++w) t += part[w][lane];
+        const size_t o = (size_t)i * U + c;
+        out[o] = t - (subtract ? Z0[o] : 0.0);
+    }
+}
+
+// one warp per output, lanes over the samples: for few states, where most lanes of the form above would be
+// idle (4 states, 1024 samples x 961 coefficients: 11 us against 60)
+__global__ void __launch_bounds__(256) k_dft_lanes(int N, int U, int n2, const double* __restrict__ RG,
+                                                   const double* __restrict__ zb, const double* __restrict__ Z0,
+                                                   double* out, int subtract) {
+    const int warp = (blockIdx.x * 256 + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (warp >= n2 * U) return;
+    const int i = warp / U, c = warp % U;
+    double acc = 0.0;
+    for (int s = lane; s < N; s += 32) acc += RG[(size_t)c * N + s] * zb[(size_t)s * n2 + i];
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) out[warp] = acc - (subtract ? Z0[warp] : 0.0);
 }
 
 // ----------------------------------------------------------------------------
@@ -116,22 +119,58 @@ __device__ __forceinline__ void ld4_fp64(const float* p, double v[4]) {
         v[3] = f.w;
     }
 }
-__device__ __forceinline__ void ld4_fp64(const double* p, double v[4]) {
-    const double2 x = *reinterpret_cast<const double2*>(p), y = *reinterpret_cast<const double2*>(p + 2);
-    v[0] = x.x;
-    v[1] = x.y;
-    v[2] = y.x;
-    v[3] = y.y;
+// zout[s][i] = sum_{j < 2n} Phi_s[i][j] zin[s][j], in two forms (launch_phi_apply chooses).
+//
+// G lanes take one row of X or V (B = 1), or both rows of a dof, which share each z (B = 2); z comes from
+// global memory, in the panel's column order through orig_of where there are panels.  FP64 multiply-adds
+// bound large ones (447-dof beam, 64 trajectories: 51 M = 81 us, 107 measured), the length of a lane's chain and
+// the launch small ones: 72 dofs, 64 trajectories, FP64: 7.4 us with 32 lanes a row, 5.3 with 16, 12.5 with
+// a staged z as below.
+template <typename T, int G, int B>
+__global__ void __launch_bounds__(256) k_phi_rows(int N, PhiView<T> F, const double* __restrict__ zin, double* zout) {
+    const int n = F.n, per = B == 2 ? n : 2 * n, total = N * per;
+    const int gid = (int)(((size_t)blockIdx.x * 256 + threadIdx.x) / G), l = threadIdx.x % G;
+    const int id = min(gid, total - 1);   // lanes past the last row repeat it: all take part in the shuffles
+    const int s = id / per, i = id % per, dof = i < n ? i : i - n;
+    const double* z = zin + (size_t)s * 2 * n;
+    const T* first = (B == 2 || i < n) ? F.X : F.V;
+    double a = 0.0, b = 0.0;
+    if (F.pan.nc == 1) {   // the caller's numbering
+        const size_t o = (size_t)s * F.pan.tot + (size_t)dof * F.pan.ld[0];
+        const T *x = first + o, *v = F.V + o;
+        for (int j = l; j < 2 * n; j += G) {
+            const double zj = z[j];
+            a += (double)x[j] * zj;
+            if (B == 2) b += (double)v[j] * zj;
+        }
+    } else {
+        const int r = F.row_of[dof], g = F.panel(r), m = F.pan.n[g], row0 = F.pan.row0[g];
+        const size_t o = (size_t)s * F.pan.tot + F.pan.off[g] + (size_t)(r - row0) * F.pan.ld[g];
+        const T *x = first + o, *v = F.V + o;
+        for (int j = l; j < 2 * m; j += G) {
+            const double zj = z[F.col(g, j)];
+            a += (double)x[j] * zj;
+            if (B == 2) b += (double)v[j] * zj;
+        }
+    }
+    if (B == 2) {   // halves of the group keep one sum each
+        const bool up = l & (G / 2);
+        const double other = __shfl_xor_sync(0xffffffffu, up ? a : b, G / 2);
+        a = (up ? b : a) + other;
+    }
+#pragma unroll
+    for (int o = G / 2 / B; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if (gid < total && l % (G / B) == 0) zout[(size_t)s * 2 * n + i + (l ? n : 0)] = a;
 }
 
-// zout[s][i] = sum_{j < 2n} Phi_s[i][j] zin[s][j].  A CTA takes PHI_ROWS rows of one panel of one
-// trajectory: the panel's part of zin goes to shared memory in the panel's column order, a warp takes the
-// X and V rows of two dofs (four dot products share each z).  Bound by the FP64 FMAs (FP32 tangents;
-// 349 M for the 1872-dof shell's 64 trajectories = 0.55 ms) or by reading the tangents.  A warp per row
-// with converting loads and z from global memory: 1.28 ms there, now 0.75 ms; 243-dof plate 485 -> 171 us.
+// FP32 tangents of some size: a conversion at the FP64 rate for every multiply-add doubles the work, so
+// values are widened by bit moves, and four dot products share each z.  A CTA takes PHI_ROWS rows of one
+// panel of one trajectory: the panel's part of zin goes to shared memory in the panel's column order, a warp
+// takes the X and V rows of two dofs.  Bound by the FP64 FMAs (349 M for the 1872-dof shell's 64
+// trajectories = 0.55 ms) or by reading the tangents.  Converting loads and a warp per row: 1.28 ms there,
+// 0.75 ms this way; 243-dof plate, 256 trajectories, 484 -> 143 us.
 constexpr int PHI_ROWS = 16;
-template <typename T>
-__global__ void __launch_bounds__(256) k_phi_apply(PhiView<T> F, const double* __restrict__ zin, double* zout) {
+__global__ void __launch_bounds__(256) k_phi_apply(PhiView<float> F, const double* __restrict__ zin, double* zout) {
     extern __shared__ double zs[];
     int x = blockIdx.x, g = 0;
     while (x >= (F.pan.n[g] + PHI_ROWS - 1) / PHI_ROWS) x -= (F.pan.n[g++] + PHI_ROWS - 1) / PHI_ROWS;
@@ -148,7 +187,7 @@ __global__ void __launch_bounds__(256) k_phi_apply(PhiView<T> F, const double* _
     if (ra >= m) return;
     const size_t base = (size_t)s * F.pan.tot + F.pan.off[g];
     const size_t oa = base + (size_t)ra * ld, ob = rb < m ? oa + ld : oa;
-    const T* rows[4] = {F.X + oa, F.V + oa, F.X + ob, F.V + ob};
+    const float* rows[4] = {F.X + oa, F.V + oa, F.X + ob, F.V + ob};
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
     const int m4 = (2 * m) & ~3;
     for (int j = 4 * lane; j < m4; j += 128) {
@@ -701,8 +740,23 @@ void launch_collect_end(fse_ctx* c) {
 
 void launch_dft_residual(fse_ctx* c, const double* zb, const double* Z0, double* R, int subtract) {
     const Params& p = c->p;
-    const dim3 g((2 * p.n + DFT_T - 1) / DFT_T, (p.U + DFT_C - 1) / DFT_C);
-    k_dft_res<<<g, DFT_T, 0, c->stream>>>(p.N, p.U, 2 * p.n, c->d.RG, zb, Z0, R, subtract);
+    const int N = p.N, U = p.U, n2 = 2 * p.n, tiles = (n2 + 31) / 32;
+    // FP64 issue slots of one coefficient: a warp per output takes N / 32 and some three for the sum over
+    // its lanes, a tile of 32 states N.  Below 24 states the first form also has the shorter chains (18
+    // states, 63 x 63: 2.4 us, 2.7 for the tiles; 24: 3.0 and 2.65); from 128 on its strided reads cost more
+    // than any idle lane (144 states, 1024 x 961: 497 us, 264).
+    if (n2 < 24 || (n2 < 128 && (long long)n2 * ((N + 31) / 32 + 3) < (long long)tiles * N)) {
+        const size_t lanes = (size_t)32 * n2 * U;
+        k_dft_lanes<<<(unsigned)((lanes + 255) / 256), 256, 0, c->stream>>>(N, U, n2, c->d.RG, zb, Z0, R, subtract);
+        return;
+    }
+    // eight warps a tile while the tiles are few (24 states, 196 x 169: 5.3 us, 7.0 with four; 1872-dof shell
+    // 34 and 31)
+    const unsigned g = (unsigned)tiles * U;
+    if (g < 2u * num_sms())
+        k_dft_warps<8><<<g, 256, 0, c->stream>>>(N, U, n2, c->d.RG, zb, Z0, R, subtract);
+    else
+        k_dft_warps<4><<<g, 128, 0, c->stream>>>(N, U, n2, c->d.RG, zb, Z0, R, subtract);
 }
 
 template <typename T>
@@ -710,27 +764,50 @@ static PhiView<T> phi_view(const fse_ctx* c) {
     return {(const T*)c->d.X, (const T*)c->d.V, c->d.row_of, c->d.orig_of, c->p.n, c->p.pan};
 }
 
-template <typename T>
-static void phi_apply(fse_ctx* c, const double* zin, double* zout) {
-    static std::atomic<unsigned long long> attr{0};
-    if (needs_device_setup(attr)) {
-        cudaFuncSetAttribute(k_phi_apply<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-        mark_device(attr);
-    }
-    const Params& p = c->p;
-    int tiles = 0, most = 0;
-    for (int g = 0; g < p.pan.nc; ++g) {
-        tiles += (p.pan.n[g] + PHI_ROWS - 1) / PHI_ROWS;
-        most = std::max(most, p.pan.n[g]);
-    }
-    k_phi_apply<T><<<dim3(tiles, p.N), 256, (size_t)2 * most * 8, c->stream>>>(phi_view<T>(c), zin, zout);
+template <typename T, int G, int B>
+static void phi_rows(fse_ctx* c, const double* zin, double* zout) {
+    const size_t lanes = (size_t)c->p.N * (B == 2 ? 1 : 2) * c->p.n * G;
+    k_phi_rows<T, G, B><<<(unsigned)((lanes + 255) / 256), 256, 0, c->stream>>>(c->p.N, phi_view<T>(c), zin, zout);
 }
 
 void launch_phi_apply(fse_ctx* c, const double* zin, double* zout) {
-    if (c->p.prec == FSE_MIXED_FP32)
-        phi_apply<float>(c, zin, zout);
-    else
-        phi_apply<double>(c, zin, zout);
+    const Params& p = c->p;
+    int tiles = 0, most = 0;
+    double work = 0.0;   // multiply-adds
+    for (int g = 0; g < p.pan.nc; ++g) {
+        tiles += (p.pan.n[g] + PHI_ROWS - 1) / PHI_ROWS;
+        most = std::max(most, p.pan.n[g]);
+        work += 4.0 * p.N * p.pan.n[g] * p.pan.n[g];
+    }
+    const bool f32 = p.prec == FSE_MIXED_FP32, many = (long long)2 * p.n * p.N >= 1024;
+    // The staged form needs enough work and enough CTAs to pay for the trip of z through shared memory
+    // (FP32, us staged / by rows: 120 dofs, 32 trajectories, 1.8 M: 7.9 / 11.4; 72, 64, 1.3 M: 10.5 / 8.0; 624, 3,
+    // 4.7 M: 20 / 25; 360, 3, 1.6 M: 13 / 9; 936, 1, 3.5 M: 28 / 19).
+    if (f32 && ((work >= 1.5e6 && p.N >= 8) || (work >= 4e6 && p.N >= 3))) {
+        static std::atomic<unsigned long long> attr{0};
+        if (needs_device_setup(attr)) {
+            cudaFuncSetAttribute(k_phi_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+            mark_device(attr);
+        }
+        k_phi_apply<<<dim3(tiles, p.N), 256, (size_t)2 * most * 8, c->stream>>>(phi_view<float>(c), zin, zout);
+        return;
+    }
+    // By rows: 16 lanes a row while rows are short (their chains stay short) and many enough to fill the
+    // GPU, else 32 (FP64, us with 16 / 32: 243 dofs, 64 trajectories 37 / 66; 200, 3: 4.3 / 3.3; FP32: 54, 16:
+    // 3.2 / 4.4; 200, 9: 9.3 / 8.3).  Long FP64 rows of several trajectories in pairs: 447 dofs, 16: 30.8, 34.9 one
+    // by one; 936, 16: 107 and 110 (3 trajectories: no difference; one: 11.8 and 10.1).
+    if (f32) {
+        if (many && 2 * most <= 256)
+            phi_rows<float, 16, 1>(c, zin, zout);
+        else
+            phi_rows<float, 32, 1>(c, zin, zout);
+    } else if (2 * most > 512 && p.N >= 9) {
+        phi_rows<double, 32, 2>(c, zin, zout);
+    } else if (many && 2 * most <= 512) {
+        phi_rows<double, 16, 1>(c, zin, zout);
+    } else {
+        phi_rows<double, 32, 1>(c, zin, zout);
+    }
 }
 
 void launch_domega(fse_ctx* c, double* zout) {
