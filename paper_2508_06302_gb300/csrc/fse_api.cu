@@ -430,15 +430,12 @@ static void rotation_tables(const fse_ctx* c, std::vector<double>& rc, std::vect
 
 static void free_ctx(fse_ctx* c) {
     if (!c) return;
-    void* ptrs[] = {c->d.Mb, c->d.F, c->d.el_type, c->d.el_dof, c->d.el_p, c->d.col_off,
-                    c->d.cs_ptr, c->d.cs_col, c->d.sl_ptr, c->d.sl_m, c->d.kt_slot, c->d.g_pass, c->d.g_info, c->d.g_rr, c->d.g_map, c->d.g_slot,
-                    c->d.g_rec, c->d.cs_m, c->d.cs_d, c->d.cs_k, c->d.cs_s, c->d.cs_A,
-                    c->d.cs_B, c->d.kt_ptr, c->d.kt_col, c->d.kt_soff, c->d.kt_src, c->d.ke,
-                    c->d.kt_val, c->d.ce, c->d.ct_val, c->d.romega, c->d.phis, c->d.G, c->d.Gi, c->d.RG, c->d.rc, c->d.rs,
-                    c->d.ktab, c->d.LMc, c->d.LMr, c->d.LMinv, c->d.LMd, c->d.q, c->d.u, c->d.a, c->d.zb,
+    void* ptrs[] = {c->d.image, c->d.g_rec, c->d.cs_s, c->d.sl_s, c->d.cs_A,
+                    c->d.cs_B, c->d.ke, c->d.kt_val, c->d.ce, c->d.ct_val, c->d.romega, c->d.G, c->d.Gi, c->d.RG,
+                    c->d.LMc, c->d.LMr, c->d.LMinv, c->d.LMd, c->d.q, c->d.u, c->d.a, c->d.zb,
                     c->d.Lc, c->d.Lr, c->d.Linv, c->d.Dinv, c->d.Rf, c->d.Rb, c->d.Tf, c->d.Tb, c->d.X, c->d.V, c->d.Y, c->d.Z0, c->d.R,
                     c->d.vec, c->d.vec2, c->d.yb, c->d.status, c->d.iters, c->d.nref, c->d.flag, c->Jd, c->piv, c->kry, c->kdot,
-                    c->ht, c->unk, c->d.row_of, c->d.ap, c->d.Sband, c->d.ktc_ptr, c->d.ktc_e, c->d.ktc_c, c->d.ktc_r};
+                    c->ht, c->unk, c->d.ap, c->d.Sband};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (auto& e : c->ev)
@@ -667,7 +664,7 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
             }
         }
     }
-    const int ni = p.ni, nb = p.b + 1, fb = 2 * p.b + 1;
+    const int ni = p.ni, nb = p.b + 1;
     const std::vector<int>&cptr = mat.cptr, &ccol = mat.ccol, &kptr = mat.kptr, &kcol = mat.kcol, &ksoff = mat.ksoff,
           &ksrc = mat.ksrc;
     const std::vector<double>&cm = mat.cm, &cd = mat.cd, &ck = mat.ck, &Mb = mat.Mb;
@@ -697,7 +694,7 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
     for (size_t q = 0; q < grp.col.size(); ++q) gslot[q] = grp.col[q] % p.RW;
     for (size_t q = 0; q < kcol.size(); ++q) kslot[q] = kcol[q] % p.RW;
     // device allocations
-    const size_t Nn = (size_t)N * ni, band = (size_t)fb * ni, lb = (size_t)ni * nb;
+    const size_t Nn = (size_t)N * ni, lb = (size_t)ni * nb;
     const size_t sensz = (size_t)N * p.pan.tot * tsz;
     const size_t ktsz = (size_t)N * p.kt_ld * tsz;
     const size_t dsz = (size_t)N * p.nblk * FSE_BLK * FSE_BLK * tsz;
@@ -705,39 +702,11 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
     auto A = [&](auto** ptr, size_t bytes) {
         if (e == cudaSuccess) e = dalloc(ptr, bytes);
     };
-    A(&c->d.Mb, band * 8);
-    A(&c->d.row_of, (size_t)(n + ni) * 4);
-    A(&c->d.F, Fi.size() * 8);
-    A(&c->d.el_type, (size_t)std::max(1, m->n_nl) * 4);
-    A(&c->d.el_dof, (size_t)std::max(1, m->n_nl) * 24);
-    A(&c->d.el_p, (size_t)std::max(1, m->n_nl) * 48);
-    A(&c->d.col_off, (size_t)(ncol + 1) * 4);
-    A(&c->d.cs_ptr, (size_t)(ni + 1) * 4);
-    A(&c->d.cs_col, (size_t)p.nnz * 4);
-    A(&c->d.g_pass, gpass.size() * 4);
-    A(&c->d.g_info, ginfo.size() * 4);
-    A(&c->d.g_rr, (size_t)p.ng * p.R * 16);
-    A(&c->d.g_map, (size_t)p.nE * p.R * 4);
-    A(&c->d.g_slot, (size_t)p.nE * 4);
     A(&c->d.g_rec, (size_t)p.nE * p.RB);
-    A(&c->d.kt_slot, (size_t)p.kt_ld * 4);
-    A(&c->d.cs_m, (size_t)p.nnz * 8);
-    A(&c->d.cs_d, (size_t)p.nnz * 8);
-    A(&c->d.cs_k, (size_t)p.nnz * 8);
     A(&c->d.cs_s, (size_t)p.nnz * 8);
-    // small arrays share allocations and copies (each costs several microseconds of setup): the index
-    // arrays of the slices [ptr | col | map], their values [m | d | s], the dof maps [row_of | orig_of], and
-    // the products' second pair with the partial sums and counters of the dot products
-    slptr.insert(slptr.end(), slcol.begin(), slcol.end());
-    slptr.insert(slptr.end(), slmap.begin(), slmap.end());
-    slm.insert(slm.end(), sld.begin(), sld.end());
-    std::vector<int> dofmap(num.row_of);
-    dofmap.insert(dofmap.end(), num.orig_of.begin(), num.orig_of.end());
-    A(&c->d.sl_ptr, slptr.size() * 4);
-    A(&c->d.sl_m, (size_t)3 * p.nsl * 8);
+    A(&c->d.sl_s, (size_t)p.nsl * 8);
     A(&c->d.cs_A, (size_t)p.nnz * tsz);
     A(&c->d.cs_B, (size_t)p.nnz * tsz);
-    A(&c->d.kt_ptr, (size_t)(ni + 1) * 4);
     // panel factor: K_t entries of the lower triangle grouped by column
     std::vector<int> ktc_ptr(ni + 1, 0), ktc_e, ktc_c, ktc_r;
     if (p.chol_blk) {
@@ -760,14 +729,60 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
                 ktc_r[k] = i - j;
             }
         A(&c->d.Sband, lb * 4);
-        A(&c->d.ktc_ptr, (size_t)(ni + 1) * 4);
-        A(&c->d.ktc_e, ktc_e.size() * 4);
-        A(&c->d.ktc_c, ktc_c.size() * 4);
-        A(&c->d.ktc_r, ktc_r.size() * 4);
     }
-    A(&c->d.kt_col, (size_t)std::max(1, p.nnz_kt) * 4);
-    A(&c->d.kt_soff, (size_t)(p.nnz_kt + 1) * 4);
-    A(&c->d.kt_src, (size_t)std::max<size_t>(1, ksrc.size()) * 4);
+    // What the host lays out for the kernels shares one allocation and one copy, each array on 256 bytes as
+    // if allocated by itself (array by array, some 30 of them, allocating, copying and freeing took about a
+    // third of the setup of a small model).
+    struct Part {
+        void** ptr;
+        const void* src;
+        size_t bytes, off;
+    };
+    std::vector<Part> parts;
+    size_t image_bytes = 0;
+    auto host = [&](auto** ptr, const auto& v) {
+        parts.push_back({(void**)ptr, v.data(), v.size() * sizeof(v[0]), image_bytes});
+        image_bytes += std::max<size_t>(256, (parts.back().bytes + 255) & ~(size_t)255);
+    };
+    host(&c->d.Mb, Mb);
+    host(&c->d.row_of, num.row_of);
+    host(&c->d.orig_of, num.orig_of);
+    host(&c->d.F, Fi);
+    host(&c->d.el_type, et);
+    host(&c->d.el_dof, ed);
+    host(&c->d.el_p, ep);
+    host(&c->d.col_off, coff);
+    host(&c->d.cs_ptr, cptr);
+    host(&c->d.cs_col, ccol);
+    host(&c->d.cs_m, cm);
+    host(&c->d.cs_d, cd);
+    host(&c->d.cs_k, ck);
+    host(&c->d.sl_ptr, slptr);
+    host(&c->d.sl_col, slcol);
+    host(&c->d.sl_map, slmap);
+    host(&c->d.sl_m, slm);
+    host(&c->d.sl_d, sld);
+    host(&c->d.g_pass, gpass);
+    host(&c->d.g_info, ginfo);
+    host(&c->d.g_rr, grr);
+    host(&c->d.g_map, grp.map);
+    host(&c->d.g_slot, gslot);
+    host(&c->d.kt_slot, kslot);
+    host(&c->d.kt_ptr, kptr);
+    host(&c->d.kt_col, kcol);
+    host(&c->d.kt_soff, ksoff);
+    host(&c->d.kt_src, ksrc);
+    if (p.chol_blk) {
+        host(&c->d.ktc_ptr, ktc_ptr);
+        host(&c->d.ktc_e, ktc_e);
+        host(&c->d.ktc_c, ktc_c);
+        host(&c->d.ktc_r, ktc_r);
+    }
+    host(&c->d.phis, phis);
+    host(&c->d.rc, rcv);
+    host(&c->d.rs, rsv);
+    host(&c->d.ktab, c->ktab_host);
+    A(&c->d.image, image_bytes);
     A(&c->d.ke, (size_t)N * std::max(1, m->n_nl) * 36 * 8);
     A(&c->d.kt_val, FSE_NBUF_KT * ktsz);
     if (p.has_vel) {
@@ -775,13 +790,9 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
         A(&c->d.ct_val, FSE_NBUF_KT * ktsz);
     }
     A(&c->d.romega, (size_t)2 * Nn * tsz);
-    A(&c->d.phis, (size_t)N * dm1 * 8);
     A(&c->d.G, (size_t)N * U * 8);
     A(&c->d.Gi, (size_t)N * U * 8);
     A(&c->d.RG, (size_t)N * U * 8);
-    A(&c->d.rc, rcv.size() * 8);
-    A(&c->d.rs, rsv.size() * 8);
-    A(&c->d.ktab, c->ktab_host.size() * 4);
     A(&c->d.LMc, lb * 8);
     A(&c->d.LMr, lb * 8);
     A(&c->d.LMinv, (size_t)ni * 8);
@@ -822,54 +833,17 @@ static int setup_impl(const fse_model* m, const fse_opts* o, long long s_begin, 
         free_ctx(c);
         return rc;
     }
-    c->d.orig_of = c->d.row_of + n;
-    c->d.sl_col = c->d.sl_ptr + p.nblk + 1;
-    c->d.sl_map = c->d.sl_col + p.nsl;
-    c->d.sl_d = c->d.sl_m + p.nsl;
-    c->d.sl_s = c->d.sl_d + p.nsl;
     c->d.red = c->d.ap + 2 * nu;
     c->d.redc = (unsigned*)(c->d.red + FSE_DOT_VECS * FSE_DOT_BLOCKS);
     cudaStream_t st = c->stream;
-    cudaMemcpyAsync(c->d.Mb, Mb.data(), band * 8, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.row_of, dofmap.data(), dofmap.size() * 4, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.F, Fi.data(), Fi.size() * 8, cudaMemcpyHostToDevice, st);
-    if (m->n_nl > 0) {
-        cudaMemcpyAsync(c->d.el_type, et.data(), et.size() * 4, cudaMemcpyHostToDevice, st);
-        cudaMemcpyAsync(c->d.el_dof, ed.data(), ed.size() * 4, cudaMemcpyHostToDevice, st);
-        cudaMemcpyAsync(c->d.el_p, ep.data(), ep.size() * 8, cudaMemcpyHostToDevice, st);
+    std::vector<unsigned char> image(image_bytes);
+    for (const Part& x : parts) {
+        *x.ptr = c->d.image + x.off;
+        if (x.bytes) std::memcpy(image.data() + x.off, x.src, x.bytes);
     }
-    cudaMemcpyAsync(c->d.col_off, coff.data(), coff.size() * 4, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.cs_ptr, cptr.data(), cptr.size() * 4, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.cs_col, ccol.data(), ccol.size() * 4, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.g_pass, gpass.data(), gpass.size() * 4, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.g_info, ginfo.data(), ginfo.size() * 4, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.g_rr, grr.data(), grr.size() * 4, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.g_map, grp.map.data(), grp.map.size() * 4, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.g_slot, gslot.data(), gslot.size() * 4, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.kt_slot, kslot.data(), kslot.size() * 4, cudaMemcpyHostToDevice, st);
+    cudaMemcpyAsync(c->d.image, image.data(), image_bytes, cudaMemcpyHostToDevice, st);
     cudaMemsetAsync(c->d.kt_val, 0, FSE_NBUF_KT * ktsz, st);
     if (p.has_vel) cudaMemsetAsync(c->d.ct_val, 0, FSE_NBUF_KT * ktsz, st);
-    cudaMemcpyAsync(c->d.cs_m, cm.data(), cm.size() * 8, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.cs_d, cd.data(), cd.size() * 8, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.cs_k, ck.data(), ck.size() * 8, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.sl_ptr, slptr.data(), slptr.size() * 4, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.sl_m, slm.data(), slm.size() * 8, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.kt_ptr, kptr.data(), kptr.size() * 4, cudaMemcpyHostToDevice, st);
-    if (p.chol_blk) {
-        cudaMemcpyAsync(c->d.ktc_ptr, ktc_ptr.data(), ktc_ptr.size() * 4, cudaMemcpyHostToDevice, st);
-        cudaMemcpyAsync(c->d.ktc_e, ktc_e.data(), ktc_e.size() * 4, cudaMemcpyHostToDevice, st);
-        cudaMemcpyAsync(c->d.ktc_c, ktc_c.data(), ktc_c.size() * 4, cudaMemcpyHostToDevice, st);
-        cudaMemcpyAsync(c->d.ktc_r, ktc_r.data(), ktc_r.size() * 4, cudaMemcpyHostToDevice, st);
-    }
-    if (p.nnz_kt > 0) {
-        cudaMemcpyAsync(c->d.kt_col, kcol.data(), kcol.size() * 4, cudaMemcpyHostToDevice, st);
-        cudaMemcpyAsync(c->d.kt_src, ksrc.data(), ksrc.size() * 4, cudaMemcpyHostToDevice, st);
-    }
-    cudaMemcpyAsync(c->d.kt_soff, ksoff.data(), ksoff.size() * 4, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.phis, phis.data(), phis.size() * 8, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.rc, rcv.data(), rcv.size() * 8, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.rs, rsv.data(), rsv.size() * 8, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(c->d.ktab, c->ktab_host.data(), c->ktab_host.size() * 4, cudaMemcpyHostToDevice, st);
     cudaMemsetAsync(c->d.status, 0, (size_t)N * 4, st);
     cudaMemsetAsync(c->d.redc, 0, FSE_DOT_VECS * 4, st);
     cudaMemsetAsync(c->d.iters, 0, (size_t)N * 4, st);

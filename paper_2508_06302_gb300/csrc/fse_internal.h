@@ -64,6 +64,7 @@ struct Panels {
 //  elements and the factors are in the internal numbering (ni rows).
 
 struct Dev {
+    unsigned char* image = nullptr;   // one allocation for all arrays that the host laid out at setup
     // model (FP64)
     double* Mb = nullptr;    // full band of M (setup factor)
     double* F = nullptr;     // e x n
