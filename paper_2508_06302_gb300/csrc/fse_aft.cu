@@ -47,10 +47,10 @@ __global__ void k_join(int N, int n, int ni, const int* __restrict__ row_of, con
 // sum and the launch the small ones, so the samples of a sum are always dealt out.
 //
 // W warps share 32 states i and one coefficient c: lanes along i (zb coalesced, RG a broadcast), each warp a
-// slice of the samples, partial sums through shared memory.  1872-dof shell (64 samples, 63 coefficients)
-// 113 us with one warp per output and its lanes over the samples (zb with a stride of 2n), 31 now; 243-dof
-// plate (256 x 225) 88 -> 53; 36 states, 63 x 63, 2.8 us (15.7 with a thread per state and pair of
-// coefficients over all samples).
+// slice of the samples, partial sums through shared memory; the loads of four samples go out together (one
+// by one a slice of 25 is a chain of 13 trips to L2: 10.8 us at 24 states, 196 x 169, now 6.5).  Against one
+// warp per output with its lanes over the samples (zb with a stride of 2n): 447-dof beam (64 samples x 63)
+// 30.7 -> 10.2 us, 243-dof plate (256 x 225) 90 -> 54, 72-dof plate (81 x 81) 10.7 -> 5.3.
 template <int W>
 __global__ void __launch_bounds__(32 * W) k_dft_warps(int N, int U, int n2, const double* __restrict__ RG,
                                                       const double* __restrict__ zb, const double* __restrict__ Z0,
@@ -62,11 +62,21 @@ __global__ void __launch_bounds__(32 * W) k_dft_warps(int N, int U, int n2, cons
     double a = 0.0, b = 0.0;
     if (i < n2) {
         const double *z = zb + i, *r = RG + (size_t)c * N;
-        for (int s = s0; s < s1; s += 2) {
-            const bool two = s + 1 < s1;
-            a += r[s] * z[(size_t)s * n2];
-            b += (two ? r[s + 1] : 0.0) * (two ? z[(size_t)(s + 1) * n2] : 0.0);
+        int s = s0;
+#pragma unroll 2
+        for (; s + 4 <= s1; s += 4) {   // four samples' loads at a time
+            double zv[4], rv[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                zv[q] = z[(size_t)(s + q) * n2];
+                rv[q] = r[s + q];
+            }
+            a += rv[0] * zv[0];
+            b += rv[1] * zv[1];
+            a += rv[2] * zv[2];
+            b += rv[3] * zv[3];
         }
+        for (; s < s1; ++s) a += r[s] * z[(size_t)s * n2];
     }
     part[warp][lane] = a + b;
     __syncthreads();
