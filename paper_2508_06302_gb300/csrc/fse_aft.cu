@@ -387,7 +387,7 @@ __device__ __forceinline__ long long lu_key(double v) {
 __global__ void __launch_bounds__(512) k_lu_panel(double* A, int* piv, int m, int k, int nb, int in_smem, int* flag) {
     extern __shared__ double sp[];
     __shared__ long long skey[16];
-    __shared__ int srow[16], s_piv;
+    __shared__ int srow[16];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, rows = m - k;
     double* P = in_smem ? sp : A + (size_t)k * m + k;
     const size_t pitch = in_smem ? LU_NB + 1 : m;
@@ -435,7 +435,6 @@ __global__ void __launch_bounds__(512) k_lu_panel(double* A, int* piv, int m, in
                 P[bi * pitch + lane] = t;
             }
             if (lane == 0) {
-                s_piv = bi;
                 piv[k + j] = k + bi;
                 if (best <= 0) *flag = 1;
             }

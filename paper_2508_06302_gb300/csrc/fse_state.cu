@@ -835,7 +835,7 @@ struct StateArgs {
     double rho[FSE_MAX_D - 1];
     const double *F, *phis;
     const int *cs_ptr, *cs_col;
-    const double *cs_m, *cs_d, *cs_k, *cs_s;
+    const double *cs_d, *cs_k, *cs_s;
     const int *sl_ptr, *sl_col;              // M, D, S in slices of 32 rows
     const double *sl_m, *sl_d, *sl_s;
     const int *el_type, *el_dof, *col_off;
@@ -850,7 +850,7 @@ struct StateArgs {
     void* romega;       // N x n, w_1-column term of this step (regular steps)
     const double *LMc, *LMr, *LMinv, *LMd;
     double *q, *u, *a;
-    const void *cLc, *cLr, *cLinv, *cDinv;   // chord factor (regular steps)
+    const void *cLc, *cLr, *cDinv;           // chord factor (regular steps)
     void *oLc, *oLr, *oLinv, *oDinv;         // factor of K_eff at the new state
     void *oRf, *oRb;                         // its block records for the tangent solves (null: not used)
     const void *cRf, *cRb;                   // records of the chord factor (panel factor: the chord
@@ -1584,7 +1584,6 @@ static StateArgs make_state_args(fse_ctx* c, double w, int init, int k) {
     A.phis = c->d.phis;
     A.cs_ptr = c->d.cs_ptr;
     A.cs_col = c->d.cs_col;
-    A.cs_m = c->d.cs_m;
     A.cs_d = c->d.cs_d;
     A.cs_k = c->d.cs_k;
     A.cs_s = c->d.cs_s;
@@ -1626,7 +1625,6 @@ static StateArgs make_state_args(fse_ctx* c, double w, int init, int k) {
     A.a = c->d.a;
     A.cLc = (char*)c->d.Lc + fi * fsz;
     A.cLr = (char*)c->d.Lr + fi * fsz;
-    A.cLinv = (char*)c->d.Linv + fi * vsz;
     A.cDinv = (char*)c->d.Dinv + fi * dsz;
     A.oLc = (char*)c->d.Lc + fo * fsz;
     A.oLr = (char*)c->d.Lr + fo * fsz;
