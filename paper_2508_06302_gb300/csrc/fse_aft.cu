@@ -751,10 +751,12 @@ void launch_dft_residual(fse_ctx* c, const double* zb, const double* Z0, double*
     const Params& p = c->p;
     const int N = p.N, U = p.U, n2 = 2 * p.n, tiles = (n2 + 31) / 32;
     // FP64 issue slots of one coefficient: a warp per output takes N / 32 and some three for the sum over
-    // its lanes, a tile of 32 states N.  Below 24 states the first form also has the shorter chains (18
-    // states, 63 x 63: 2.4 us, 2.7 for the tiles; 24: 3.0 and 2.65); from 128 on its strided reads cost more
-    // than any idle lane (144 states, 1024 x 961: 497 us, 264).
-    if (n2 < 24 || (n2 < 128 && (long long)n2 * ((N + 31) / 32 + 3) < (long long)tiles * N)) {
+    // its lanes, a tile of 32 states N.  Few states have the shorter chains in the first form (18 states,
+    // 63 x 63: 2.4 us, 2.7 for the tiles; 24: 3.0 and 2.65; with at most a sample a lane up to 48: 36 states, 16
+    // x 15, 3.17 and 3.26); from 128 on its strided reads cost more than any idle lane (144 states, 1024 x 961:
+    // 497 us, 264).
+    if (n2 < 24 || (n2 < 48 && N <= 32) ||
+        (n2 < 128 && (long long)n2 * ((N + 31) / 32 + 3) < (long long)tiles * N)) {
         const size_t lanes = (size_t)32 * n2 * U;
         k_dft_lanes<<<(unsigned)((lanes + 255) / 256), 256, 0, c->stream>>>(N, U, n2, c->d.RG, zb, Z0, R, subtract);
         return;
