@@ -152,9 +152,10 @@ static Numbering own_numbering(int n, int b) {
 }
 
 // Numbering by components (pairs: every coupled pair of dofs, comp[i]: a label per component).  Large
-// components get a panel each, the others share the last one; dofs keep their order inside a component.  nc stays 0 where it does not pay: the panels' tangents (rows in whole blocks x
-// columns) are what every step streams and solves, and below a quarter saved the inert rows and the
-// shorter blocks cost about as much (n = 24: 3 panels of 32 rows against 1).
+// components get a panel each, the others share the last one; dofs keep their order inside a component.  nc
+// stays 0 where it does not pay: the panels' tangents (rows in whole blocks x columns) are what every step
+// streams and solves, and below a quarter saved the inert rows and the shorter blocks cost about as much
+// (n = 24: 3 panels of 32 rows against 1).
 static Numbering component_numbering(const fse_model* m, const std::vector<std::pair<int, int>>& pairs,
                                      const std::vector<int>& comp) {
     const int n = m->n;
@@ -395,7 +396,11 @@ static RowGroups plan_tangents(Params& p, const Numbering& N, const Matrices& X,
             }
         }
     }
-    // panel Cholesky in the state kernel for FP32 factors with b <= 96 when its window fits
+    // panel Cholesky in the state kernel for FP32 factors with b <= 96 when its window fits; b is that of the
+    // panels, so divided models of a caller's half-bandwidth beyond 96 take it too.  It adds K_t to S in FP32
+    // (rounded twice) and multiplies by rsqrtf: against FP64 monodromies their FP32 ones come out no worse
+    // for it (36 runs of four shells of half-bandwidth 98 to 110, 8 to 24 steps: 0.93 of the error of the
+    // undivided column form on average, 0.72 to 1.18; 1.03 with the column form on the panels).
     p.chol_blk = 0;
     if (p.prec == FSE_MIXED_FP32 && p.b <= 96) {
         p.chol_blk = 1;
@@ -430,12 +435,12 @@ static void rotation_tables(const fse_ctx* c, std::vector<double>& rc, std::vect
 
 static void free_ctx(fse_ctx* c) {
     if (!c) return;
-    void* ptrs[] = {c->d.image, c->d.g_rec, c->d.cs_s, c->d.sl_s, c->d.cs_A,
-                    c->d.cs_B, c->d.ke, c->d.kt_val, c->d.ce, c->d.ct_val, c->d.romega, c->d.G, c->d.Gi, c->d.RG,
-                    c->d.LMc, c->d.LMr, c->d.LMinv, c->d.LMd, c->d.q, c->d.u, c->d.a, c->d.zb,
-                    c->d.Lc, c->d.Lr, c->d.Linv, c->d.Dinv, c->d.Rf, c->d.Rb, c->d.Tf, c->d.Tb, c->d.X, c->d.V, c->d.Y, c->d.Z0, c->d.R,
-                    c->d.vec, c->d.vec2, c->d.yb, c->d.status, c->d.iters, c->d.nref, c->d.flag, c->Jd, c->piv, c->kry, c->kdot,
-                    c->ht, c->unk, c->d.ap, c->d.Sband};
+    void* ptrs[] = {c->d.image, c->d.g_rec, c->d.cs_s, c->d.sl_s, c->d.cs_A, c->d.cs_B, c->d.ke, c->d.kt_val,
+                    c->d.ce, c->d.ct_val, c->d.romega, c->d.G, c->d.Gi, c->d.RG, c->d.LMc, c->d.LMr, c->d.LMinv,
+                    c->d.LMd, c->d.q, c->d.u, c->d.a, c->d.zb, c->d.Lc, c->d.Lr, c->d.Linv, c->d.Dinv, c->d.Rf,
+                    c->d.Rb, c->d.Tf, c->d.Tb, c->d.X, c->d.V, c->d.Y, c->d.Z0, c->d.R, c->d.vec, c->d.vec2,
+                    c->d.yb, c->d.status, c->d.iters, c->d.nref, c->d.flag, c->Jd, c->piv, c->kry, c->kdot, c->ht,
+                    c->unk, c->d.ap, c->d.Sband};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (auto& e : c->ev)
