@@ -20,6 +20,7 @@ import subprocess
 import tempfile
 import sys
 import time
+from typing import NamedTuple
 
 ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
@@ -182,8 +183,20 @@ def measured_peaks():
     return {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "sm_max_mhz": 2070.0}, "fallback"
 
 
+class Panel(NamedTuple):
+    """A group of dofs whose tangents are kept together: rows, half-bandwidth, nonzeros of the M, D, K
+    pattern and of the K_t pattern."""
+    n: int
+    band: int
+    nnz: int
+    nnz_kt: int
+
+
 def csr_counts(m):
-    """Nonzeros of the union pattern of M, D, K and of the K_t pattern of the nonlinear elements."""
+    """Nonzeros of the union pattern of M, D, K and of the K_t pattern of the nonlinear elements (of a
+    model or of a Panel)."""
+    if isinstance(m, Panel):
+        return m.nnz, m.nnz_kt
     nnz = int(np.count_nonzero((m.M != 0) | (m.D != 0) | (m.K != 0)))
     kt = set()
     for e in range(m.n_nl):
@@ -217,8 +230,7 @@ def step_work(m, N, band, ld, prec_bytes):
 def tangent_panels(m, most=4):
     """The decoupled groups of dofs the tangents are kept in (csrc/fse_internal.h, Panels): components of
     the coupling graph, up to three of at least n / 16 dofs a panel each, the others together in the last;
-    one panel where less than a quarter of the tangent block would be saved.  Per panel (rows, half-bandwidth, nonzeros of
-    the M, D, K pattern, nonzeros of the K_t pattern)."""
+    one panel where less than a quarter of the tangent block would be saved.  A list of Panel."""
     n = m.n
     pat = (m.M != 0) | (m.D != 0) | (m.K != 0)
     ii, jj = np.nonzero(pat)
@@ -253,22 +265,15 @@ def tangent_panels(m, most=4):
         inside = [(a, b) for a, b in zip(ii.tolist(), jj.tolist()) if a in pos]
         kin = [(a, b) for a, b in kt if a in pos]
         band = max((abs(pos[a] - pos[b]) for a, b in inside + kin), default=0)
-        out.append((r, band, len(inside), len(kin)))
+        out.append(Panel(r, band, len(inside), len(kin)))
     return out
 
 
 def panel_work(m, N, prec_bytes):
     """step_work of the tangents as they are kept, panel by panel: a panel of n rows has 2n + 1 columns
     and its own half-bandwidth; entries between panels are zero and neither stored nor computed."""
-    out = {"sens_rhs": [0.0, 0.0], "sens_fwd": [0.0, 0.0], "sens_bwd": [0.0, 0.0]}
-    w = prec_bytes
-    for n, b, nnz, nnz_kt in tangent_panels(m):
-        P, tri = 2 * n + 1, n * b - b * (b + 1) / 2
-        for k, fl, words in (("sens_rhs", 2.0 * (2 * nnz + nnz_kt), 3.0), ("sens_fwd", 2.0 * tri, 2.0),
-                             ("sens_bwd", 2.0 * tri + 3.0 * n, 5.0)):
-            out[k][0] += fl * P * N
-            out[k][1] += words * n * P * w * N
-    return {k: tuple(v) for k, v in out.items()}
+    parts = [step_work(p, N, p.band, 0, prec_bytes) for p in tangent_panels(m)]
+    return {k: tuple(sum(p[k][i] for p in parts) for i in (0, 1)) for k in parts[0]}
 
 
 def step_rates(work, traj_steps_per_s, N, hbm_gbs, fp64_tflops=None, bf16_tflops=None):
