@@ -762,19 +762,19 @@ void launch_dft_residual(fse_ctx* c, const double* zb, const double* Z0, double*
     const int N = p.N, U = p.U, n2 = 2 * p.n, tiles = (n2 + 31) / 32;
     // FP64 issue slots of one coefficient: a warp per output takes N / 32 and some three for the sum over
     // its lanes, a tile of 32 states N.  Few states have the shorter chains in the first form (18 states,
-    // 63 x 63: 2.4 us, 2.7 for the tiles; 24: 3.0 and 2.65; with at most a sample a lane up to 48: 36 states, 16
-    // x 15, 3.17 and 3.26); from 128 on its strided reads cost more than any idle lane (144 states, 1024 x 961:
-    // 497 us, 264).
+    // 63 x 63: 2.5 us, 2.8 for the tiles; 24: 3.0 and 2.8; with at most a sample a lane up to 48: 36 states, 25
+    // x 25, 2.1 and 2.2); from 128 on its strided reads cost more than any idle lane (144 states, 1024 x 961:
+    // 498 us, 263).
     if (n2 < 24 || (n2 < 48 && N <= 32) ||
         (n2 < 128 && (long long)n2 * ((N + 31) / 32 + 3) < (long long)tiles * N)) {
         const size_t lanes = (size_t)32 * n2 * U;
         k_dft_lanes<<<(unsigned)((lanes + 255) / 256), 256, 0, c->stream>>>(N, U, n2, c->d.RG, zb, Z0, R, subtract);
         return;
     }
-    // eight warps a tile while the tiles are few (24 states, 196 x 169: 5.3 us, 7.0 with four; 1872-dof shell
-    // 34 and 31)
+    // eight warps a tile while the tiles are few and each warp has two samples or more (24 states, 196 x 169:
+    // 5.3 us, 5.9 with four; 72 states, 16 x 15: 2.2 and 1.9; 1872-dof shell 34 and 30)
     const unsigned g = (unsigned)tiles * U;
-    if (g < 2u * num_sms())
+    if (g < 2u * num_sms() && N > 16)
         k_dft_warps<8><<<g, 256, 0, c->stream>>>(N, U, n2, c->d.RG, zb, Z0, R, subtract);
     else
         k_dft_warps<4><<<g, 128, 0, c->stream>>>(N, U, n2, c->d.RG, zb, Z0, R, subtract);
