@@ -1113,10 +1113,10 @@ int lyapunov_run_noalloc(fse_ctx* c, double w, int N_Ly, int h, double* sigma) {
 
 namespace fse {
 
-// y = a x + b y
+// y = a x + b y; with b = 0 what y held (nothing yet, or a NaN of an earlier call) does not take part
 __global__ void k_axpby(size_t n, double a, const double* x, double b, double* y) {
     for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n; k += (size_t)gridDim.x * blockDim.x)
-        y[k] = a * x[k] + b * y[k];
+        y[k] = b == 0.0 ? a * x[k] : a * x[k] + b * y[k];
 }
 
 // out[i] = a_i . b_i for i < gridDim.y, a_i = a + i sa, b_i = b + i sb.  gridDim.x blocks share a dot

@@ -67,3 +67,33 @@ def test_context_on_used_memory(nx, ny, precision):
         assert np.linalg.norm(Phi - ref.Phi) <= tol * np.linalg.norm(ref.Phi)
         first = out if first is None else first
         assert all(np.array_equal(a, b) for a, b in zip(out, first)), hex(word)
+
+
+def test_newton_updates_ignore_what_their_buffers_held():
+    """Right-hand sides are formed as -R in buffers that hold anything: fresh memory full of NaN (unknown
+    frequency, hyper-time), or the NaN product of an earlier call (dense and GMRES updates)."""
+    from paper_2508_06302_gb300 import fse
+    v, m = I.van_der_pol(omega_n=10.0, eps=0.2, F=(10.0,)), I.chain(6)
+    wv, wm = 10.0 / 2.7, 1.1 * m.omega_n1
+    Zv, Zm = I.random_coeffs(v.n, 7, 0.3, seed=3), I.random_coeffs(m.n, 5, 1e-3, seed=3)
+    z = np.random.default_rng(1).standard_normal((5, 2 * m.n)) * 1e-3
+    out = []
+    for word in WORDS:
+        release = fill_device(word)
+        with fse.Context(v, 2, [8], [3], [2.7], 24, newton_tol=0.0, newton_maxit=8) as ctx:
+            Z, rho, rn, rc = ctx.newton_step_unknown(Zv, wv, [2.7], [0])
+        with fse.Context(m, 2, [5], [2], [I.GOLDEN], 24, newton_tol=0.0, newton_maxit=8) as ctx:
+            zn = ctx.newton_step_hypertime(z, wm)[0]
+            ctx.jacobian_apply_hypertime(np.full((1,) + z.shape, np.nan))
+            zh = ctx.newton_step_hypertime(z, wm)[0]
+            ctx.residual_jacobian(Zm, wm)
+            Zd = []
+            for solver in ("dense", "gmres"):
+                ctx.set_linear_solver(solver)
+                ctx.jacobian_apply(np.full((2, Zm.size), np.nan))
+                Zd.append(ctx.newton_step(Zm, wm)[0])
+        release()
+        out.append((Z, rho, zn, zh, *Zd))
+        assert all(np.all(np.isfinite(a)) for a in out[-1]), hex(word)
+        assert np.array_equal(zn, zh)
+        assert all(np.array_equal(a, b) for a, b in zip(out[-1], out[0])), hex(word)
