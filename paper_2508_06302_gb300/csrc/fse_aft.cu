@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(256) k_phi_rows(int N, PhiView<T> F, const dou
 // panel of one trajectory: the panel's part of zin goes to shared memory in the panel's column order, a warp
 // takes the X and V rows of two dofs.  Bound by the FP64 FMAs (349 M for the 1872-dof shell's 64
 // trajectories = 0.55 ms) or by reading the tangents.  Converting loads and a warp per row: 1.28 ms there,
-// 0.75 ms this way; 243-dof plate, 256 trajectories, 484 -> 143 us.
+// 0.65 ms this way; 243-dof plate, 256 trajectories, 484 -> 143 us.
 constexpr int PHI_ROWS = 16;
 __global__ void __launch_bounds__(256) k_phi_apply(PhiView<float> F, const double* __restrict__ zin, double* zout) {
     extern __shared__ double zs[];

@@ -40,10 +40,13 @@ CASES = [  # model, samples, harmonics, precision
     (lambda: I.chain(129), 5, 2, "mixed_fp32"), (lambda: I.chain(153), 16, 7, "mixed_fp32"),   # 32 lanes; 1.498 M
     (lambda: I.chain(154), 16, 7, "mixed_fp32"), (lambda: I.chain(578), 3, 1, "mixed_fp32"),   # staged
     (lambda: blocks(60, 40), 7, 3, "mixed_fp32"), (lambda: blocks(240, 150, 9, 2), 9, 4, "mixed_fp32"),
-    # DFT: lanes over the samples up to 23 states and, with many samples, beyond; tiles of 32 states
+    # DFT: lanes over the samples up to 23 states, 47 with at most 32 samples and, with many samples, beyond;
+    # tiles of 32 states, four warps each up to 16 samples or with many tiles, else eight
     (lambda: I.chain(11), 40, 19, "fp64"), (lambda: I.chain(12), 40, 19, "fp64"), (lambda: I.chain(18), 225, 112, "fp64"),
     (lambda: I.chain(16), 9, 4, "fp64"), (lambda: I.chain(17), 9, 4, "fp64"), (lambda: I.chain(63), 131, 65, "fp64"),
     (lambda: I.chain(64), 131, 65, "fp64"), (lambda: I.chain(50), 2, 0, "fp64"),
+    (lambda: I.chain(23), 32, 15, "fp64"), (lambda: I.chain(23), 33, 16, "fp64"), (lambda: I.chain(24), 32, 15, "fp64"),
+    (lambda: I.chain(24), 16, 7, "fp64"), (lambda: I.chain(24), 17, 8, "fp64"), (lambda: I.chain(33), 7, 3, "fp64"),
 ]
 
 
